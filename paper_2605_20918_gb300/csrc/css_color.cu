@@ -2,11 +2,14 @@
 // CSS probe signs.  Paper: CSS construction paragraph after Eq. 2 (greedy multicolouring,
 // Welsh-Powell order) and Fig. 1(b,c).
 //
-// Jones-Plassmann with the priority (degree desc, SplitMix64(seed, id) desc, id asc) colours a
-// vertex in the first round in which all of its higher-priority neighbours are coloured, and
-// gives it the smallest colour none of them uses.  That is exactly the sequential greedy
-// colouring in priority order, so the result is bit-identical to it.
+// Jones-Plassmann with the priority (degree desc, SplitMix64(seed, id) desc, id asc): a vertex
+// is coloured once all of its higher-priority neighbours (its parents) are, with the smallest
+// colour none of them uses.  That is exactly the sequential greedy colouring in priority order,
+// whatever the order in which ready vertices are taken, so the result is bit-identical to it.
+#include <algorithm>
+
 #include "css_internal.cuh"
+#include "css_pipe.cuh"
 
 namespace {
 
@@ -16,39 +19,40 @@ struct __align__(32) q4 {
   long long x, y, z, w;
 };
 
+// minimum image of the difference of two coordinates of [0, Lq): a select instead of a 64-bit
+// remainder, which is tens of instructions
 __device__ __forceinline__ int64_t min_image(int64_t d, int64_t Lq) {
-  int64_t r = d % Lq;
-  if (r > Lq / 2) r -= Lq;
-  if (r < -(Lq / 2)) r += Lq;
-  return r;
+  if (d > Lq / 2) d -= Lq;
+  if (d < -(Lq / 2)) d += Lq;
+  return d;
 }
 
-__device__ __forceinline__ bool higher(int32_t du, uint64_t ku, int32_t u, int32_t dv, uint64_t kv, int32_t v) {
+// u before v in the greedy order; the hashes are only taken between vertices of equal degree
+__device__ __forceinline__ bool higher(uint64_t seed, int32_t du, int32_t u, int32_t dv, int32_t v) {
   if (du != dv) return du > dv;
+  const uint64_t ku = css_splitmix64(seed, (uint64_t)u), kv = css_splitmix64(seed, (uint64_t)v);
   if (ku != kv) return ku > kv;
   return u < v;
 }
 
+// Fixed-point coordinates wrapped into [0, Lq)^3, and the cell of each molecule.
 __global__ void k_quantise(int32_t n, const double* __restrict__ xyz, int64_t Lq, int32_t nc, q4* __restrict__ q,
                            int32_t* __restrict__ cell) {
   int32_t i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
-  int64_t a = __double2ll_rn(xyz[3 * (int64_t)i] * (double)kFix);
-  int64_t b = __double2ll_rn(xyz[3 * (int64_t)i + 1] * (double)kFix);
-  int64_t c = __double2ll_rn(xyz[3 * (int64_t)i + 2] * (double)kFix);
-  q[i] = q4{a, b, c, 0};
-  if (nc >= 3) {
-    int64_t w[3] = {a % Lq, b % Lq, c % Lq};
-    int32_t ci[3];
+  int64_t w[3];
+  for (int d = 0; d < 3; ++d) {
+    w[d] = __double2ll_rn(xyz[3 * (int64_t)i + d] * (double)kFix) % Lq;
+    if (w[d] < 0) w[d] += Lq;
+  }
+  q[i] = q4{w[0], w[1], w[2], 0};
+  int32_t ci[3] = {0, 0, 0};
+  if (nc >= 3)
     for (int d = 0; d < 3; ++d) {
-      if (w[d] < 0) w[d] += Lq;
-      int64_t t = (w[d] * nc) / Lq;
+      const int64_t t = (w[d] * nc) / Lq;
       ci[d] = (int32_t)(t >= nc ? nc - 1 : t);
     }
-    cell[i] = (ci[0] * nc + ci[1]) * nc + ci[2];
-  } else {
-    cell[i] = 0;
-  }
+  cell[i] = (ci[0] * nc + ci[1]) * nc + ci[2];
 }
 
 __global__ void k_cell_count(int32_t n, const int32_t* __restrict__ cell, int32_t* __restrict__ cnt) {
@@ -66,57 +70,60 @@ __global__ void k_cell_fill(int32_t n, const int32_t* __restrict__ cell, const i
   }
 }
 
-// insertion-sort each cell's members by id (the fill order above is arbitrary)
-__global__ void k_cell_sort(int32_t ncells, const int32_t* __restrict__ start, int32_t* __restrict__ members) {
-  int32_t c = blockIdx.x * blockDim.x + threadIdx.x;
-  if (c >= ncells) return;
-  int32_t s = start[c], e = start[c + 1];
-  for (int32_t i = s + 1; i < e; ++i) {
-    int32_t v = members[i];
-    int32_t j = i - 1;
-    while (j >= s && members[j] > v) {
-      members[j + 1] = members[j];
-      --j;
-    }
-    members[j + 1] = v;
-  }
-}
-
-// pass 0: count neighbours, pass 1: write them.  Candidates come from the 27 cells around
-// the molecule (or from all molecules when the box holds fewer than 3 cells per edge).
+// Neighbours of every molecule, one warp each: the lanes test the candidates of the 27 cells
+// around it (or of all molecules when the box holds fewer than 3 cells per edge) 32 at a time.
+// Pass 0 counts them into deg; pass 1 writes those of higher priority (the parents, in any order)
+// from adj_ptr[i] on and their number to np[i].  A thread per molecule left the chip idle below
+// ~10^5 molecules (2.1 ms a pass at 4,001 molecules).
 template <int PASS>
 __global__ void k_neighbours(int32_t n, const q4* __restrict__ q, const int32_t* __restrict__ cell, int32_t nc,
                              const int32_t* __restrict__ cstart, const int32_t* __restrict__ members, int64_t Lq,
-                             int64_t R2, int32_t* __restrict__ deg, const int32_t* __restrict__ adj_ptr,
-                             int32_t* __restrict__ adj) {
-  int32_t i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n) return;
-  q4 qi = q[i];
-  int32_t count = 0;
-  int32_t out = PASS ? adj_ptr[i] : 0;
+                             int64_t R2, uint64_t seed, int32_t* __restrict__ deg,
+                             const int32_t* __restrict__ adj_ptr, int32_t* __restrict__ np, int32_t* __restrict__ adj) {
+  const int32_t i = (int32_t)(((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5);
+  const int lane = threadIdx.x & 31;
+  if (i >= n) return;  // whole warp
+  const q4 qi = q[i];
+  const int32_t di = PASS ? deg[i] : 0;
+  int32_t count = 0;  // PASS 0: this lane's neighbours; PASS 1: parents written by the warp
+  const int32_t out = PASS ? adj_ptr[i] : 0;
+  // every lane of the warp calls this; j < 0: no candidate
   auto test = [&](int32_t j) {
-    if (j == i) return;
-    q4 qj = q[j];
-    int64_t dx = min_image(qi.x - qj.x, Lq), dy = min_image(qi.y - qj.y, Lq), dz = min_image(qi.z - qj.z, Lq);
-    if (dx * dx + dy * dy + dz * dz < R2) {
-      if (PASS) adj[out + count] = j;
-      ++count;
+    bool take = false;
+    if (j >= 0 && j != i) {
+      const q4 qj = q[j];
+      const int64_t dx = min_image(qi.x - qj.x, Lq), dy = min_image(qi.y - qj.y, Lq), dz = min_image(qi.z - qj.z, Lq);
+      take = dx * dx + dy * dy + dz * dz < R2;
     }
+    if (!PASS) {
+      count += take;
+      return;
+    }
+    take = take && higher(seed, deg[j], j, di, i);
+    const unsigned m = __ballot_sync(0xffffffffu, take);
+    if (take) adj[out + count + __popc(m & ((1u << lane) - 1u))] = j;
+    count += __popc(m);
   };
   if (nc < 3) {
-    for (int32_t j = 0; j < n; ++j) test(j);
+    for (int32_t j = 0; j < n; j += 32) test(j + lane < n ? j + lane : -1);
   } else {
-    int32_t c = cell[i];
-    int32_t cx = c / (nc * nc), cy = (c / nc) % nc, cz = c % nc;
+    const int32_t c = cell[i];
+    const int32_t cx = c / (nc * nc), cy = (c / nc) % nc, cz = c % nc;
     for (int dx = -1; dx <= 1; ++dx)
       for (int dy = -1; dy <= 1; ++dy)
         for (int dz = -1; dz <= 1; ++dz) {
-          int32_t x = (cx + dx + nc) % nc, y = (cy + dy + nc) % nc, z = (cz + dz + nc) % nc;
-          int32_t cc = (x * nc + y) * nc + z;
-          for (int32_t k = cstart[cc]; k < cstart[cc + 1]; ++k) test(members[k]);
+          const int32_t x = (cx + dx + nc) % nc, y = (cy + dy + nc) % nc, z = (cz + dz + nc) % nc;
+          const int32_t cc = (x * nc + y) * nc + z;
+          const int32_t e = cstart[cc + 1];
+          for (int32_t k = cstart[cc]; k < e; k += 32) test(k + lane < e ? members[k + lane] : -1);
         }
   }
-  if (!PASS) deg[i] = count;
+  if (!PASS) {
+    for (int o = 16; o > 0; o >>= 1) count += __shfl_xor_sync(0xffffffffu, count, o);
+    if (lane == 0) deg[i] = count;
+  } else if (lane == 0) {
+    np[i] = count;
+  }
 }
 
 // ---------------------------------------------------------------- exclusive scan
@@ -177,60 +184,118 @@ css_status css_scan_i32(css_ctx* ctx, const int32_t* in, int32_t* out, int64_t n
 namespace {
 
 // ---------------------------------------------------------------- Jones-Plassmann
-__global__ void k_jp_init(int32_t n, const int32_t* __restrict__ adj_ptr, uint64_t seed, int32_t* __restrict__ deg,
-                          uint64_t* __restrict__ key, int32_t* __restrict__ colour) {
-  int32_t i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n) return;
-  deg[i] = adj_ptr[i + 1] - adj_ptr[i];
-  key[i] = css_splitmix64(seed, (uint64_t)i);
-  colour[i] = -1;
+// Degrees of an explicit graph, and the parents of every vertex (one warp each) from adj_ptr[v]
+// on with their number in np[v].
+__global__ void k_degrees(int32_t n, const int32_t* __restrict__ adj_ptr, int32_t* __restrict__ deg) {
+  const int32_t v = blockIdx.x * blockDim.x + threadIdx.x;
+  if (v < n) deg[v] = adj_ptr[v + 1] - adj_ptr[v];
 }
-
-// One Jones-Plassmann round, one warp per uncoloured vertex v (lanes walk v's neighbours): v is
-// ready when every higher-priority neighbour is coloured (a colour, once set, never changes);
-// then it takes the smallest colour none of them uses, searched 256 colours at a time with the
-// lanes' bit masks OR-reduced over the warp.  Vertices not ready count into *remaining.
-__global__ void k_jp_round(int32_t n, const int32_t* __restrict__ adj_ptr, const int32_t* __restrict__ adj,
-                           const int32_t* __restrict__ deg, const uint64_t* __restrict__ key, int32_t* colour,
-                           int32_t* __restrict__ remaining) {
+__global__ void k_parents(int32_t n, const int32_t* __restrict__ adj_ptr, const int32_t* __restrict__ adj,
+                          uint64_t seed, const int32_t* __restrict__ deg, int32_t* __restrict__ np,
+                          int32_t* __restrict__ padj) {
   const int32_t v = (int32_t)(((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5);
   const int lane = threadIdx.x & 31;
   if (v >= n) return;
-  if (__ldcg(&colour[v]) >= 0) return;  // whole warp
-  const int32_t dv = deg[v];
-  const uint64_t kv = key[v];
-  const int32_t s = adj_ptr[v], e = adj_ptr[v + 1];
-  bool blocked = false;
-  for (int32_t k = s + lane; k < e; k += 32) {
-    const int32_t u = adj[k];
-    if (higher(deg[u], key[u], u, dv, kv, v) && __ldcg(&colour[u]) < 0) blocked = true;
+  const int32_t s = adj_ptr[v], e = adj_ptr[v + 1], dv = deg[v];
+  int32_t count = 0;
+  for (int32_t k = s; k < e; k += 32) {
+    const int32_t u = k + lane < e ? adj[k + lane] : -1;
+    const bool take = u >= 0 && higher(seed, deg[u], u, dv, v);
+    const unsigned m = __ballot_sync(0xffffffffu, take);
+    if (take) padj[s + count + __popc(m & ((1u << lane) - 1u))] = u;
+    count += __popc(m);
   }
-  if (__any_sync(0xffffffffu, blocked)) {
-    if (lane == 0) atomicAdd(remaining, 1);
-    return;
-  }
-  for (int32_t base = 0;; base += 256) {
-    uint64_t w[4] = {0, 0, 0, 0};
-    for (int32_t k = s + lane; k < e; k += 32) {
-      const int32_t u = adj[k];
-      if (!higher(deg[u], key[u], u, dv, kv, v)) continue;
-      const int32_t c = __ldcg(&colour[u]) - base;
-      if (c < 0 || c >= 256) continue;
-      w[c >> 6] |= 1ull << (c & 63);
-    }
+  if (lane == 0) np[v] = count;
+}
+
+// The whole colouring in one cooperative launch (all CTAs resident, so a vertex may wait for any
+// other).  Warp w owns vertices [w per, w per + per); each lane watches one parent of its vertex
+// that is not coloured yet (wait[v]: its index among v's parents).  When that parent has its
+// colour, the warp looks at the vertex's remaining parents 32 at a time, moves the watch to the
+// next uncoloured one, or, when there is none, takes the smallest colour none of the parents uses
+// (256 colours at a time, the lanes' bit masks OR-reduced) and publishes it.  A colour is one
+// word that never changes once set, so no ordering between words is needed.
+// Bound by latency: one published colour seen by its dependants is ~1.5 us, and the longest chain
+// of parents is a few hundred vertices.  With one launch per step of that chain, each scanning
+// every vertex, a colouring of 20,000 molecules took 10.0 ms (445 launches); now 1.42 ms in all.
+// Every wait is bounded: a warp that sees 4 s pass without any vertex of the graph being coloured
+// (*done counts them) sets *err and leaves.
+constexpr uint64_t kColourNs = 4000000000ull;
+__global__ void __launch_bounds__(256) k_jp_flow(int32_t n, int32_t per, const int32_t* __restrict__ adj_ptr,
+                                                 const int32_t* __restrict__ np, const int32_t* __restrict__ padj,
+                                                 int32_t* __restrict__ wait, volatile int32_t* colour,
+                                                 int32_t* __restrict__ max_colour, int32_t* done,
+                                                 int32_t* __restrict__ err) {
+  constexpr unsigned FULL = 0xffffffffu;
+  const int lane = threadIdx.x & 31;
+  const int64_t v0 = (((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5) * per;
+  if (v0 >= n) return;
+  const int32_t mine = (int32_t)(n - v0 < per ? n - v0 : per);
+  int32_t left = mine, top = -1, seen = -1;
+  uint64_t t0 = css_pipe::gtime();
+  for (uint32_t sweep = 0; left > 0; ++sweep) {
+    bool moved = false;
+    for (int32_t g = 0; g < mine; g += 32) {
+      const int32_t vl = (int32_t)v0 + g + lane;
+      const bool own = g + lane < mine;
+      int32_t wl = own ? wait[vl] : -1;  // -1: coloured
+      const int32_t sl = own ? adj_ptr[vl] : 0, nl = own ? np[vl] : 0;
+      const bool go = wl >= 0 && (wl >= nl || colour[padj[sl + wl]] >= 0);
+      unsigned todo = __ballot_sync(FULL, go);
+      moved = moved || todo != 0;
+      while (todo) {
+        const int src = __ffs(todo) - 1;
+        todo &= todo - 1;
+        const int32_t v = __shfl_sync(FULL, vl, src), s = __shfl_sync(FULL, sl, src), k = __shfl_sync(FULL, nl, src);
+        int32_t w = __shfl_sync(FULL, wl, src);
+        for (; w < k; w += 32) {
+          const bool open = w + lane < k && colour[padj[s + w + lane]] < 0;
+          const unsigned m = __ballot_sync(FULL, open);
+          if (m) {
+            w += __ffs(m) - 1;
+            break;
+          }
+        }
+        if (w >= k) {  // every parent has its colour
+          int32_t c = -1;
+          for (int32_t base = 0; c < 0; base += 256) {
+            uint64_t used[4] = {0, 0, 0, 0};
+            for (int32_t q = lane; q < k; q += 32) {
+              const int32_t cu = colour[padj[s + q]] - base;
 #pragma unroll
-    for (int q = 0; q < 4; ++q)
-      for (int o = 16; o > 0; o >>= 1) w[q] |= __shfl_xor_sync(0xffffffffu, w[q], o);
-    int32_t off = -1;
-    if (~w[0]) off = __ffsll((long long)~w[0]) - 1;
-    else if (~w[1]) off = 64 + __ffsll((long long)~w[1]) - 1;
-    else if (~w[2]) off = 128 + __ffsll((long long)~w[2]) - 1;
-    else if (~w[3]) off = 192 + __ffsll((long long)~w[3]) - 1;
-    if (off >= 0) {
-      if (lane == 0) colour[v] = base + off;
-      return;
+              for (int z = 0; z < 4; ++z)
+                if (cu >= 64 * z && cu < 64 * (z + 1)) used[z] |= 1ull << (cu & 63);
+            }
+#pragma unroll
+            for (int z = 0; z < 4; ++z) {
+              for (int o = 16; o > 0; o >>= 1) used[z] |= __shfl_xor_sync(FULL, used[z], o);
+              if (c < 0 && ~used[z]) c = base + 64 * z + __ffsll((long long)~used[z]) - 1;
+            }
+          }
+          if (lane == 0) {
+            colour[v] = c;
+            atomicAdd(done, 1);
+          }
+          top = max(top, c);
+          w = -1;
+          --left;
+        }
+        if (lane == src) wait[v] = w;
+        __syncwarp();
+      }
+    }
+    if (!moved && (sweep & 255) == 255) {
+      const int32_t now = __shfl_sync(FULL, *(volatile int32_t*)done, 0);
+      if (now != seen) {
+        seen = now;
+        t0 = css_pipe::gtime();
+      } else if (css_pipe::gtime() - t0 > kColourNs) {
+        if (lane == 0) atomicOr(err, 1);
+        return;
+      }
     }
   }
+  if (lane == 0) atomicMax(max_colour, top);
 }
 
 // An explicit graph must have adj_ptr[0] = 0, non-decreasing adj_ptr and every neighbour in
@@ -253,13 +318,6 @@ __global__ void k_graph_check(int32_t n, const int32_t* __restrict__ adj_ptr, co
   }
 }
 
-__global__ void k_max_colour(int32_t n, const int32_t* __restrict__ colour, int32_t* __restrict__ maxc) {
-  int32_t i = blockIdx.x * blockDim.x + threadIdx.x;
-  int32_t c = i < n ? colour[i] : -1;
-  for (int o = 16; o > 0; o >>= 1) c = max(c, __shfl_xor_sync(0xffffffffu, c, o));
-  if ((threadIdx.x & 31) == 0) atomicMax(maxc, c);
-}
-
 __global__ void k_probe_signs(int64_t count, uint64_t seed, int ones, int8_t* __restrict__ sign) {
   int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= count) return;
@@ -267,8 +325,8 @@ __global__ void k_probe_signs(int64_t count, uint64_t seed, int ones, int8_t* __
 }
 
 // Molecule centres in fixed point, binned into a periodic grid of cells at least r_col wide
-// (about one molecule per cell; any coarser grid is also correct), members of each cell
-// sorted by id.  nc = 1 (one cell) when the box holds fewer than 3 cells per edge.
+// (any coarser grid is also correct), the members of a cell in no particular order (neighbour
+// counts, parent sets and conflict counts do not depend on it).  nc = 1 (one cell) when the box holds fewer than 3 cells per edge.
 struct CellList {
   q4* q;
   int32_t *cell, *cstart, *members;
@@ -303,8 +361,6 @@ css_status build_cells(css_ctx* ctx, int32_t n, const double* xyz, double box, d
   CSS_LAUNCHED(ctx);
   CSS_TRY(css_scan_i32(ctx, ccnt, cl->cstart, ncells, st));
   k_cell_fill<<<nbk, T, 0, st>>>(n, cl->cell, cl->cstart, cfill, cl->members);
-  CSS_LAUNCHED(ctx);
-  k_cell_sort<<<(unsigned)css_ceil_div(ncells, T), T, 0, st>>>(ncells, cl->cstart, cl->members);
   CSS_LAUNCHED(ctx);
   cl->nc = nc;
   cl->Lq = Lq;
@@ -386,72 +442,64 @@ css_status css_color_impl(css_ctx* ctx, int32_t n, const double* xyz, double box
                           const int32_t* adj_ptr_in, const int32_t* adj_in, int32_t* colour, int32_t* n_colours,
                           cudaStream_t st) {
   const int T = 256;
-  const unsigned nbk = (unsigned)css_ceil_div(n, T);
-  const int32_t* adj_ptr = adj_ptr_in;
-  const int32_t* adj = adj_in;
-  int32_t* hbuf = nullptr;
+  const unsigned nbk = (unsigned)css_ceil_div(n, T), nwk = (unsigned)css_ceil_div((int64_t)n * 32, T);
+  int32_t *hbuf, *deg, *np, *wait, *counters, *ptr = nullptr, *padj;
   CSS_TRY(css_pinned(ctx, 64, (void**)&hbuf));
+  CSS_TRY(css_ws(ctx, "col_deg", sizeof(int32_t) * (n + 1), (void**)&deg));
+  CSS_TRY(css_ws(ctx, "col_np", sizeof(int32_t) * n, (void**)&np));
+  CSS_TRY(css_ws(ctx, "col_wait", sizeof(int32_t) * n, (void**)&wait));
+  CSS_TRY(css_ws(ctx, "jp_counters", sizeof(int32_t) * 64, (void**)&counters));
+  CSS_CU(ctx, cudaMemsetAsync(counters, 0, sizeof(int32_t) * 4, st));  // error, malformed graph, -, coloured
+  const int32_t* adj_ptr = adj_ptr_in;
   if (xyz) {
     CellList cl;
     CSS_TRY(build_cells(ctx, n, xyz, box, r_col, &cl, st));
-    int32_t *deg, *ptr;
-    CSS_TRY(css_ws(ctx, "col_deg", sizeof(int32_t) * (n + 1), (void**)&deg));
     CSS_TRY(css_ws(ctx, "col_adjptr", sizeof(int32_t) * (n + 1), (void**)&ptr));
-    k_neighbours<0><<<nbk, T, 0, st>>>(n, cl.q, cl.cell, cl.nc, cl.cstart, cl.members, cl.Lq, cl.R2, deg, nullptr,
-                                       nullptr);
+    k_neighbours<0><<<nwk, T, 0, st>>>(n, cl.q, cl.cell, cl.nc, cl.cstart, cl.members, cl.Lq, cl.R2, seed, deg,
+                                       nullptr, nullptr, nullptr);
     CSS_LAUNCHED(ctx);
     CSS_TRY(css_scan_i32(ctx, deg, ptr, n, st));
+    adj_ptr = ptr;
     CSS_CU(ctx, cudaMemcpyAsync(hbuf, ptr + n, sizeof(int32_t), cudaMemcpyDeviceToHost, st));
     CSS_CU(ctx, cudaStreamSynchronize(st));
-    int64_t nadj = hbuf[0];
-    int32_t* a;
-    CSS_TRY(css_ws(ctx, "col_adj", sizeof(int32_t) * (nadj > 0 ? nadj : 1), (void**)&a));
-    k_neighbours<1><<<nbk, T, 0, st>>>(n, cl.q, cl.cell, cl.nc, cl.cstart, cl.members, cl.Lq, cl.R2, nullptr, ptr,
-                                       a);
+    CSS_TRY(css_ws(ctx, "col_adj", sizeof(int32_t) * (size_t)std::max(hbuf[0], 1), (void**)&padj));
+    k_neighbours<1><<<nwk, T, 0, st>>>(n, cl.q, cl.cell, cl.nc, cl.cstart, cl.members, cl.Lq, cl.R2, seed, deg,
+                                       adj_ptr, np, padj);
     CSS_LAUNCHED(ctx);
-    adj_ptr = ptr;
-    adj = a;
-  }
-  int32_t* deg;
-  uint64_t* key;
-  int32_t* counters;
-  CSS_TRY(css_ws(ctx, "jp_deg", sizeof(int32_t) * n, (void**)&deg));
-  CSS_TRY(css_ws(ctx, "jp_key", sizeof(uint64_t) * n, (void**)&key));
-  CSS_TRY(css_ws(ctx, "jp_counters", sizeof(int32_t) * 64, (void**)&counters));
-  if (!xyz) {  // a caller's graph: refuse a malformed pattern before any round reads through it
-    CSS_CU(ctx, cudaMemsetAsync(counters + 40, 0, sizeof(int32_t), st));
-    k_graph_check<<<nbk, T, 0, st>>>(n, adj_ptr, adj, counters + 40);
+  } else {  // a caller's graph: refuse a malformed pattern before anything reads through it
+    k_graph_check<<<nbk, T, 0, st>>>(n, adj_ptr, adj_in, counters + 1);
     CSS_LAUNCHED(ctx);
-    CSS_CU(ctx, cudaMemcpyAsync(hbuf, counters + 40, sizeof(int32_t), cudaMemcpyDeviceToHost, st));
+    CSS_CU(ctx, cudaMemcpyAsync(hbuf, counters + 1, sizeof(int32_t), cudaMemcpyDeviceToHost, st));
+    CSS_CU(ctx, cudaMemcpyAsync(hbuf + 1, adj_ptr + n, sizeof(int32_t), cudaMemcpyDeviceToHost, st));
     CSS_CU(ctx, cudaStreamSynchronize(st));
     if (hbuf[0] != 0)
       return css_set_arg_error(ctx, "css_color_graph: adj_ptr not non-decreasing from 0 or a neighbour outside [0, n)");
+    CSS_TRY(css_ws(ctx, "col_adj", sizeof(int32_t) * (size_t)std::max(hbuf[1], 1), (void**)&padj));
+    k_degrees<<<nbk, T, 0, st>>>(n, adj_ptr, deg);
+    CSS_LAUNCHED(ctx);
+    k_parents<<<nwk, T, 0, st>>>(n, adj_ptr, adj_in, seed, deg, np, padj);
+    CSS_LAUNCHED(ctx);
   }
-  k_jp_init<<<nbk, T, 0, st>>>(n, adj_ptr, seed, deg, key, colour);
-  CSS_LAUNCHED(ctx);
-  // rounds, checked in groups; every round colours at least the highest-priority uncoloured
-  // vertex, so n rounds always suffice
-  const int group = 8;
-  int64_t rounds = 0;
-  for (;;) {
-    CSS_CU(ctx, cudaMemsetAsync(counters, 0, sizeof(int32_t) * group, st));
-    for (int r = 0; r < group; ++r) {
-      k_jp_round<<<(unsigned)css_ceil_div((int64_t)n * 32, T), T, 0, st>>>(n, adj_ptr, adj, deg, key, colour,
-                                                                           counters + r);
-      CSS_LAUNCHED(ctx);
-    }
-    rounds += group;
-    CSS_CU(ctx, cudaMemcpyAsync(hbuf, counters + group - 1, sizeof(int32_t), cudaMemcpyDeviceToHost, st));
-    CSS_CU(ctx, cudaStreamSynchronize(st));
-    if (hbuf[0] == 0) break;
-    if (rounds > (int64_t)n + group) return css_set_arg_error(ctx, "colouring did not finish (inconsistent graph)");
-  }
-  CSS_CU(ctx, cudaMemsetAsync(counters + 32, 0xff, sizeof(int32_t), st));
-  k_max_colour<<<nbk, T, 0, st>>>(n, colour, counters + 32);
-  CSS_LAUNCHED(ctx);
-  CSS_CU(ctx, cudaMemcpyAsync(hbuf, counters + 32, sizeof(int32_t), cudaMemcpyDeviceToHost, st));
+  CSS_CU(ctx, cudaMemsetAsync(wait, 0, sizeof(int32_t) * n, st));
+  CSS_CU(ctx, cudaMemsetAsync(colour, 0xff, sizeof(int32_t) * n, st));
+  CSS_CU(ctx, cudaMemsetAsync(counters + 2, 0xff, sizeof(int32_t), st));  // largest colour
+  // as many warps as the chip holds at once, a vertex each as far as they go
+  int occ = 0;
+  CSS_CU(ctx, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_jp_flow, T, 0));
+  const int64_t warps = std::min((int64_t)std::max(occ, 1) * ctx->n_sm, css_ceil_div(n, T / 32)) * (T / 32);
+  int32_t per = (int32_t)css_ceil_div(n, warps), n_ = n;
+  volatile int32_t* col_ = colour;
+  int32_t *maxc = counters + 2, *done = counters + 3, *err = counters;
+  void* args[] = {&n_, &per, &adj_ptr, &np, &padj, &wait, &col_, &maxc, &done, &err};
+  CSS_CU(ctx, cudaLaunchCooperativeKernel((void*)k_jp_flow, dim3((unsigned)(warps / (T / 32))), dim3(T), args, 0, st));
+  ++ctx->kernel_launches;
+  CSS_CU(ctx, cudaMemcpyAsync(hbuf, counters, 3 * sizeof(int32_t), cudaMemcpyDeviceToHost, st));
   CSS_CU(ctx, cudaStreamSynchronize(st));
-  *n_colours = hbuf[0] + 1;
+  if (hbuf[0]) {
+    ctx->last_error = "css_color: the colouring did not finish within its time limit";
+    return CSS_ERR_TIMEOUT;
+  }
+  *n_colours = hbuf[2] + 1;
   return CSS_OK;
 }
 
