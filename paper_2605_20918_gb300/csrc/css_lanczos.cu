@@ -12,6 +12,8 @@
 // Small per-colour matrices (A_j, B_j, Grams, Cholesky factors) are FP64; the per-row-chunk
 // partial products are combined in FP64 in a fixed order, so every run is bitwise
 // reproducible (a second pass regenerates the same basis).
+#include <algorithm>
+
 #include "css_lanczos.cuh"
 
 namespace {
@@ -210,7 +212,7 @@ __global__ void k_hpad(int64_t nblocks, int32_t b, int32_t BM, const double* __r
 }
 
 // --------------------------------------------------------------- row-chunk kernels
-// CTA = (chunk of RCHK rows, group of G colours).  The chunk is walked in tiles of RTL rows;
+// CTA = (chunk of rchk rows, group of G colours; row_chunk).  The chunk is walked in tiles of RTL rows;
 // a tile of each array is staged in shared memory as [RTL][G*BP] (b padded to BP, the
 // padding kept at zero), so the global reads of a row are G*b contiguous values.  Every
 // small product (block update, Gram) is register-tiled in 4 x 4 blocks.  Per-tile Gram sums
@@ -218,7 +220,7 @@ __global__ void k_hpad(int64_t nblocks, int32_t b, int32_t BM, const double* __r
 // of floats (error-free TwoSum, so the running sum carries about 44 bits), FP64 tiles into
 // doubles.  The pair is widened to FP64 once per CTA: no FP64 arithmetic in the row loop.
 constexpr int RW = 256;      // threads of a Gram half (see the launch sizes below)
-constexpr int RCHK = 1024;   // rows per CTA
+constexpr int RCHK_MAX = 1024;  // rows per CTA of the largest systems
 
 // colours of a staged tile sit CS = BP + 4 values apart: for BP = 24 the seven colours of a
 // group start in seven different shared-memory banks
@@ -290,6 +292,24 @@ __host__ __device__ inline int row_threads(int b) {
   int t = items > gram ? items : gram;
   if (sym_split<T, BP>() && G * CB * (CB + 1) > t) t = G * CB * (CB + 1);
   return (t + 31) / 32 * 32;
+}
+
+// Rows of one CTA's chunk.  A chunk of 1,024 rows is 3 chunks for a 512-molecule b = 6 system: with
+// its two colour groups six CTAs on 152 SMs, and every FP64 product (2 FMAs per clock and SM) on
+// those few.  So the chunk shrinks until two CTAs per SM (FP32) or four (FP64, whose CTAs run
+// longest) are there, counted for 64 colours, the usual number at a 10 A radius; its least size is
+// one Gram group.  It depends on the rows and the block width only, never on the number of colours
+// of a pass: a colour's partial sums are the same whatever other colours run beside it.  Row work
+// of a step, 1,024-row chunks -> these: b = 6: 64 molecules FP64 1.07 -> 0.127 ms, 512 mixed
+// 0.45 -> 0.18 ms, 4,001 mixed 0.48 -> 0.44 ms; b = 23: 128 molecules FP64 6.4 -> 2.3 ms, 1,000
+// mixed 1.63 -> 1.32 ms.  Twice the CTAs cost FP32 10-30% (a CTA's set-up), half of them FP64 15%.
+template <typename T, int BP>
+inline int32_t row_chunk(int64_t N, int b) {
+  constexpr int GRP = RowTile<T, BP>::GRP;
+  constexpr int64_t ctas = (sizeof(T) == 4 ? 2 : 4) * 152;
+  const int64_t groups = css_ceil_div(64, colours_per_cta<T, BP>(b));
+  const int64_t r = css_ceil_div(css_ceil_div(N * groups, ctas), GRP) * GRP;
+  return (int32_t)std::min<int64_t>(r, RCHK_MAX);
 }
 
 template <typename T, int BP>
@@ -656,7 +676,7 @@ __device__ __forceinline__ RowCtx<T, BP> make_ctx(int32_t b, int32_t ws, int32_t
   return c;
 }
 
-// The row kernels below walk their chunk of RCHK rows in tiles of RTL rows through an NS-stage
+// The row kernels below walk their chunk of rchk rows in tiles of RTL rows through an NS-stage
 // shared-memory ring filled by cp.async.  Padding columns of a stage are zeroed once and never
 // written by a copy; rows past the end of the matrix are zero-filled by the copies themselves.
 template <typename T, int BP>
@@ -666,7 +686,7 @@ struct RowRing {
   __device__ __forceinline__ T* at(int s, int a) const { return base + ((size_t)s * na + a) * tile; }
 };
 
-// Tiles of this CTA's chunk.  fn_issue(stage, tile, r0, nr) issues (does not commit) the copies
+// Tiles of this CTA's chunk of rchk rows.  fn_issue(stage, tile, r0, nr) issues (does not commit) the copies
 // of a tile, fn_mul(stage, tile, r0, nr) is its first phase (a block product in place in its
 // stage), fn_fin(stage, tile, r0, nr, last) its second (stores and Gram sums of that product).
 // Two stages: the barrier-separated schedule, per tile wait, barrier, first phase, barrier, second
@@ -675,9 +695,9 @@ struct RowRing {
 // first phase of tile i + 1 and the second phase of tile i (different stages, so no barrier
 // separates them).
 template <int NS, typename Issue, typename Mul, typename Fin>
-__device__ __forceinline__ void row_pipeline(int64_t N, int32_t rtl, Issue fn_issue, Mul fn_mul, Fin fn_fin) {
+__device__ __forceinline__ void row_pipeline(int64_t N, int32_t rchk, int32_t rtl, Issue fn_issue, Mul fn_mul, Fin fn_fin) {
   static_assert(NS >= 2, "the ring needs a stage in flight besides the one being worked on");
-  const int64_t rbeg = (int64_t)blockIdx.x * RCHK, rend = min(N, rbeg + RCHK);
+  const int64_t rbeg = (int64_t)blockIdx.x * rchk, rend = min(N, rbeg + rchk);
   if (rbeg >= rend) return;
   const int32_t ntile = (int32_t)((rend - rbeg + rtl - 1) / rtl);
   auto r0_of = [&](int32_t i) { return rbeg + (int64_t)i * rtl; };
@@ -732,7 +752,7 @@ __device__ __forceinline__ void row_pipeline(int64_t N, int32_t rtl, Issue fn_is
 // With REORTH the CTA has 2*RW threads: the first RW accumulate Kq, the second RW Kp.
 template <typename T, int BP, bool REORTH>
 __global__ void __launch_bounds__(REORTH ? 2 * RW : RW, 1)
-    k_s1(int64_t N, int32_t b, int32_t ws, int32_t ncb, int32_t cb0, const T* __restrict__ Qp,
+    k_s1(int64_t N, int32_t rchk, int32_t b, int32_t ws, int32_t ncb, int32_t cb0, const T* __restrict__ Qp,
          const T* __restrict__ Q, T* __restrict__ W, const double* __restrict__ Bprev, int first,
          double* __restrict__ partKq, double* __restrict__ partKp) {
   constexpr int RTL = RowTile<T, BP>::RTL3, NS = RowTile<T, BP>::NS3;
@@ -750,7 +770,7 @@ __global__ void __launch_bounds__(REORTH ? 2 * RW : RW, 1)
   c.zero(ring.at(0, 0), 3 * NS * RTL);
   __syncthreads();
   row_pipeline<NS>(
-      N, RTL,
+      N, rchk, RTL,
       [&](int s, int32_t, int64_t r0, int32_t nr) {
         c.template load<RTL>(ring.at(s, 0), Q, r0, nr);
         c.template load<RTL>(ring.at(s, 2), W, r0, nr);
@@ -770,7 +790,7 @@ __global__ void __launch_bounds__(REORTH ? 2 * RW : RW, 1)
 // S3: W1 = W0 - Q_j M1 (- Q_{j-1} M2), stored; partial Gram W1^T W1
 template <typename T, int BP, bool REORTH>
 __global__ void __launch_bounds__(2 * RW, 1)
-    k_s3(int64_t N, int32_t b, int32_t ws, int32_t ncb, const T* __restrict__ Q, const T* __restrict__ Qp,
+    k_s3(int64_t N, int32_t rchk, int32_t b, int32_t ws, int32_t ncb, const T* __restrict__ Q, const T* __restrict__ Qp,
          T* __restrict__ W, const double* __restrict__ M1, const double* __restrict__ M2,
          double* __restrict__ partG) {
   constexpr int RTL = RowTile<T, BP>::RTL3, NS = RowTile<T, BP>::NS3;
@@ -788,7 +808,7 @@ __global__ void __launch_bounds__(2 * RW, 1)
   c.zero(ring.at(0, 0), 3 * NS * RTL);
   __syncthreads();
   row_pipeline<NS>(
-      N, RTL,
+      N, rchk, RTL,
       [&](int s, int32_t, int64_t r0, int32_t nr) {
         c.template load<RTL>(ring.at(s, 0), Q, r0, nr);
         c.template load<RTL>(ring.at(s, 2), W, r0, nr);
@@ -813,7 +833,7 @@ __global__ void __launch_bounds__(2 * RW, 1)
 // colours needs it returns at once.
 template <typename T, int BP, bool GRAM>
 __global__ void __launch_bounds__(384, 2)
-    k_tri(int64_t N, int32_t b, int32_t ws, int32_t ncb, const T* __restrict__ W, T* OUT,
+    k_tri(int64_t N, int32_t rchk, int32_t b, int32_t ws, int32_t ncb, const T* __restrict__ W, T* OUT,
           const double* __restrict__ Rinv, double* __restrict__ partG, const int32_t* __restrict__ need3,
           T* OUT2) {
   constexpr int RTL = RowTile<T, BP>::RTL1, NS = RowTile<T, BP>::NS1;
@@ -844,7 +864,7 @@ __global__ void __launch_bounds__(384, 2)
   c.zero(ring.at(0, 0), (NS + NO) * RTL);
   __syncthreads();
   row_pipeline<NS>(
-      N, RTL,
+      N, rchk, RTL,
       [&](int s, int32_t, int64_t r0, int32_t nr) { c.template load<RTL>(ring.at(s, 0), W, r0, nr); },
       [&](int s, int32_t i, int64_t, int32_t) {
         tile_mul<T, BP, false, false>(c, ring.at(s, 0), sR, sO + (i & (NO - 1)) * RTL * c.pitch, RTL, nullptr, nullptr);
@@ -859,12 +879,24 @@ __global__ void __launch_bounds__(384, 2)
                             reinterpret_cast<double*>(smem_raw));
 }
 
-__global__ void k_reduce(int32_t nch, int32_t ncb, int32_t E, const double* __restrict__ part,
-                         double* __restrict__ out) {
-  int32_t t = blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= ncb * E) return;
+// out = sum of the nch partials of every entry, RD_S of them at a time: thread (x, y) adds the
+// partials y, y + RD_S, ... of entry x of the CTA's 32, the RD_S sums are added in order.  A thread
+// per entry walked all partials alone (35 us for 225 chunks of 65 colours at b = 23).
+constexpr int RD_S = 16;
+__global__ void __launch_bounds__(32 * RD_S) k_reduce(int32_t nch, int64_t n, const double* __restrict__ part,
+                                                      double* __restrict__ out) {
+  __shared__ double sh[RD_S][32];
+  const int64_t t = (int64_t)blockIdx.x * 32 + threadIdx.x;
   double s = 0.0;
-  for (int32_t ch = 0; ch < nch; ++ch) s += part[(size_t)ch * ncb * E + t];
+  if (t < n) {
+#pragma unroll 4
+    for (int32_t ch = threadIdx.y; ch < nch; ch += RD_S) s += part[(size_t)ch * n + t];
+  }
+  sh[threadIdx.y][threadIdx.x] = s;
+  __syncthreads();
+  if (threadIdx.y != 0 || t >= n) return;
+#pragma unroll
+  for (int y = 1; y < RD_S; ++y) s += sh[y][threadIdx.x];
   out[t] = s;
 }
 
@@ -1236,10 +1268,14 @@ css_status run_pass_bp(css_ctx* ctx, const LzArgs& a_in, cudaStream_t st) {
   if (a.use_tc) CSS_TRY(css_hv_tc_schedule(ctx, a, st));
   const int32_t b = a.b, bb = b * b, ncb = a.ncb, m = a.m;
   const int64_t N = (int64_t)a.n_brow * b;
-  const int32_t nch = (int32_t)css_ceil_div(N, RCHK);
   const int32_t G = colours_per_cta<T, BP>(b);
   const int32_t ngr = (int32_t)css_ceil_div(ncb, G);
   const bool reorth = (a.flags & CSS_REORTH_LOCAL) != 0;
+  // FP32, 16 < b <= 24, env CSS_ROWS_STREAM=1: the streaming row passes of css_rows.cu (their
+  // partials come in chunks of their own)
+  const bool rp = sizeof(T) == 4 && BP == 24 && css_rowpass_supported(true, b) && ctx->rows_stream;
+  const int32_t rchk = rp ? RCHK_MAX : row_chunk<T, BP>(N, b);
+  const int32_t nch = (int32_t)css_ceil_div(N, rchk);
   T* Qp = (T*)a.Q0;
   T* Qc = (T*)a.Q1;
   T* W = (T*)a.W;
@@ -1268,10 +1304,12 @@ css_status run_pass_bp(css_ctx* ctx, const LzArgs& a_in, cudaStream_t st) {
   double* sRi210 = sRi10 + (size_t)ncb * bb;  // R0^-1 R1^-1 R2^-1
   // per colour: "a third CholeskyQR pass is needed" in the running step (after the matrices)
   int32_t* need3 = reinterpret_cast<int32_t*>(sRi210 + (size_t)ncb * bb);
-  // FP32, 16 < b <= 24, env CSS_ROWS_STREAM=1: the streaming row passes of css_rows.cu
-  constexpr bool kF32 = sizeof(T) == 4;
-  const bool rp = kF32 && BP == 24 && css_rowpass_supported(true, b) && ctx->rows_stream;
   const unsigned rblocks_bb = (unsigned)css_ceil_div((int64_t)ncb * bb, 256);
+  auto reduce = [&](const double* part, double* out) -> css_status {
+    k_reduce<<<(unsigned)css_ceil_div((int64_t)ncb * bb, 32), dim3(32, RD_S), 0, st>>>(nch, (int64_t)ncb * bb, part, out);
+    CSS_LAUNCHED(ctx);
+    return CSS_OK;
+  };
   const int64_t pb = a.pair_off_h[a.cb0], pe = a.pair_off_h[a.cb0 + ncb];
   const unsigned sblocks = (unsigned)css_ceil_div((pe - pb) * bb, 256);
   auto s1 = reorth ? k_s1<T, BP, true> : k_s1<T, BP, false>;
@@ -1288,11 +1326,10 @@ css_status run_pass_bp(css_ctx* ctx, const LzArgs& a_in, cudaStream_t st) {
     // into W (times the identity) with its Gram, and B_0 is the product of the three factors
     k_eye<<<rblocks_bb, 256, 0, st>>>(ncb, b, sR1i);
     CSS_LAUNCHED(ctx);
-    k_tri<T, BP, true><<<rgrid, th1, sm_tri, st>>>(N, b, a.ws, ncb, (const T*)a.start, W, sR1i,
+    k_tri<T, BP, true><<<rgrid, th1, sm_tri, st>>>(N, rchk, b, a.ws, ncb, (const T*)a.start, W, sR1i,
                                                                      partKq, nullptr, nullptr);
     CSS_LAUNCHED(ctx);
-    k_reduce<<<rblocks_bb, 256, 0, st>>>(nch, ncb, bb, partKq, sG);
-    CSS_LAUNCHED(ctx);
+    CSS_TRY(reduce(partKq, sG));
     k_gtrace<<<(unsigned)css_ceil_div(ncb, 128), 128, 0, st>>>(ncb, b, sG, sH);
     CSS_LAUNCHED(ctx);
     const unsigned gb = (unsigned)css_ceil_div(ncb, 4);
@@ -1300,21 +1337,19 @@ css_status run_pass_bp(css_ctx* ctx, const LzArgs& a_in, cudaStream_t st) {
                                   a.nblk, nullptr);
     CSS_LAUNCHED(ctx);
     CSS_CU(ctx, cudaMemcpyAsync(sC1, sR1, sizeof(double) * ncb * bb, cudaMemcpyDeviceToDevice, st));
-    k_tri<T, BP, true><<<rgrid, th1, sm_tri, st>>>(N, b, a.ws, ncb, W, W, sR1i, partKq, nullptr, nullptr);
+    k_tri<T, BP, true><<<rgrid, th1, sm_tri, st>>>(N, rchk, b, a.ws, ncb, W, W, sR1i, partKq, nullptr, nullptr);
     CSS_LAUNCHED(ctx);
-    k_reduce<<<rblocks_bb, 256, 0, st>>>(nch, ncb, bb, partKq, sG);
-    CSS_LAUNCHED(ctx);
+    CSS_TRY(reduce(partKq, sG));
     k_chol<1><<<gb, 128, 0, st>>>(ncb, b, a.cb0, 1, 0, sG, sH, a.tau, 0.0, sR1, sR1i, sC1, a.B0, a.done, a.nblk,
                                   nullptr);
     CSS_LAUNCHED(ctx);
-    k_tri<T, BP, true><<<rgrid, th1, sm_tri, st>>>(N, b, a.ws, ncb, W, W, sR1i, partKq, nullptr, nullptr);
+    k_tri<T, BP, true><<<rgrid, th1, sm_tri, st>>>(N, rchk, b, a.ws, ncb, W, W, sR1i, partKq, nullptr, nullptr);
     CSS_LAUNCHED(ctx);
-    k_reduce<<<rblocks_bb, 256, 0, st>>>(nch, ncb, bb, partKq, sG);
-    CSS_LAUNCHED(ctx);
+    CSS_TRY(reduce(partKq, sG));
     k_chol<2><<<gb, 128, 0, st>>>(ncb, b, a.cb0, 1, 0, sG, sH, a.tau, 0.0, sR2, sR2i, sC1, a.B0, a.done, a.nblk,
                                   nullptr);
     CSS_LAUNCHED(ctx);
-    k_tri<T, BP, false><<<rgrid, th1, sm_tri, st>>>(N, b, a.ws, ncb, W, Qc, sR2i, nullptr, nullptr, nullptr);
+    k_tri<T, BP, false><<<rgrid, th1, sm_tri, st>>>(N, rchk, b, a.ws, ncb, W, Qc, sR2i, nullptr, nullptr, nullptr);
     CSS_LAUNCHED(ctx);
   } else {
     k_init_q1<T><<<(unsigned)css_ceil_div(N, 256), 256, 0, st>>>(a.n_brow, b, a.ws, a.cb0, ncb, a.colour, a.sign,
@@ -1324,11 +1359,10 @@ css_status run_pass_bp(css_ctx* ctx, const LzArgs& a_in, cudaStream_t st) {
   // Vc[c][j] = Q_j^T u (the u block is only read: the first-step form of the three-term kernel)
   auto project_u = [&](const T* Qj, int32_t j) -> css_status {
     if (!a.ucol) return CSS_OK;
-    k_s1<T, BP, false><<<rgrid, RW, sm_s1, st>>>(N, b, a.ws, ncb, a.cb0, nullptr, Qj, (T*)a.ucol, nullptr, 1,
+    k_s1<T, BP, false><<<rgrid, RW, sm_s1, st>>>(N, rchk, b, a.ws, ncb, a.cb0, nullptr, Qj, (T*)a.ucol, nullptr, 1,
                                                   partKq, nullptr);
     CSS_LAUNCHED(ctx);
-    k_reduce<<<rblocks_bb, 256, 0, st>>>(nch, ncb, bb, partKq, sV);
-    CSS_LAUNCHED(ctx);
+    CSS_TRY(reduce(partKq, sV));
     k_store_v<<<rblocks_bb, 256, 0, st>>>(ncb, b, a.cb0, m * b, j, sV, a.Vc);
     CSS_LAUNCHED(ctx);
     return CSS_OK;
@@ -1386,11 +1420,9 @@ css_status run_pass_bp(css_ctx* ctx, const LzArgs& a_in, cudaStream_t st) {
       // Kq = Q_j^T W0, Kp = Q_{j-1}^T W0 with W0 = W - Q_{j-1} B_{j-1}^T
       CSS_TRY(css_rowpass(ctx, 0, N, b, a.ws, ncb, a.cb0, first, ro, q, qp, wv, nullptr, a.Bblk_prev, nullptr, nullptr,
                           partKq, partKp, st));
-      k_reduce<<<rblocks_bb, 256, 0, st>>>(nch, ncb, bb, partKq, sA);
-      CSS_LAUNCHED(ctx);
+      CSS_TRY(reduce(partKq, sA));
       if (reorth && !first) {
-        k_reduce<<<rblocks_bb, 256, 0, st>>>(nch, ncb, bb, partKp, sKp);
-        CSS_LAUNCHED(ctx);
+        CSS_TRY(reduce(partKp, sKp));
       }
       k_store_A<<<rblocks_bb, 256, 0, st>>>(ncb, b, a.cb0, m, j, sA, a.Ablk);
       CSS_LAUNCHED(ctx);
@@ -1398,8 +1430,7 @@ css_status run_pass_bp(css_ctx* ctx, const LzArgs& a_in, cudaStream_t st) {
       // W1 = W - Q_j Kq - Q_{j-1} (B_{j-1}^T + Kp) over W, and its Gram
       CSS_TRY(css_rowpass(ctx, 1, N, b, a.ws, ncb, a.cb0, first, ro, q, qp, wv, wv, sA, a.Bblk_prev,
                           (reorth && !first) ? sKp : nullptr, partKq, nullptr, st));
-      k_reduce<<<rblocks_bb, 256, 0, st>>>(nch, ncb, bb, partKq, sG);
-      CSS_LAUNCHED(ctx);
+      CSS_TRY(reduce(partKq, sG));
       k_hnorm<<<(unsigned)css_ceil_div(ncb, 8), 256, 0, st>>>(ncb, b, a.cb0, j, sA, a.Bblk_prev, sG, sH);
       CSS_LAUNCHED(ctx);
       // shifted CholeskyQR3 on W1 without storing the intermediates: the Grams of W1 R0^-1 and
@@ -1408,14 +1439,12 @@ css_status run_pass_bp(css_ctx* ctx, const LzArgs& a_in, cudaStream_t st) {
       CSS_CU(ctx, cudaMemcpyAsync(sC1, sR1, sizeof(double) * ncb * bb, cudaMemcpyDeviceToDevice, st));
       CSS_TRY(css_rowpass(ctx, 2, N, b, a.ws, ncb, a.cb0, first, ro, nullptr, nullptr, wv, nullptr, sR1i, nullptr,
                           nullptr, partKq, nullptr, st));
-      k_reduce<<<rblocks_bb, 256, 0, st>>>(nch, ncb, bb, partKq, sG);
-      CSS_LAUNCHED(ctx);
+      CSS_TRY(reduce(partKq, sG));
       CSS_TRY(chol(1, j, sR2, sR2i, 0.0, nullptr));
       CSS_TRY(css_small_mm(ctx, ncb, b, sR1i, sR2i, sRi10, st));
       CSS_TRY(css_rowpass(ctx, 2, N, b, a.ws, ncb, a.cb0, first, ro, nullptr, nullptr, wv, nullptr, sRi10, nullptr,
                           nullptr, partKq, nullptr, st));
-      k_reduce<<<rblocks_bb, 256, 0, st>>>(nch, ncb, bb, partKq, sG);
-      CSS_LAUNCHED(ctx);
+      CSS_TRY(reduce(partKq, sG));
       CSS_TRY(chol(2, j, sR1, sR1i, 0.0, nullptr));
       CSS_TRY(css_small_mm(ctx, ncb, b, sRi10, sR1i, sRi210, st));
       CSS_TRY(css_rowpass(ctx, 3, N, b, a.ws, ncb, a.cb0, first, ro, nullptr, nullptr, wv, (float*)Qp, sRi210, nullptr,
@@ -1431,43 +1460,38 @@ css_status run_pass_bp(css_ctx* ctx, const LzArgs& a_in, cudaStream_t st) {
       continue;
     }
     // three-term update and the projections onto Q_j (and Q_{j-1})
-    s1<<<rgrid, reorth ? 2 * RW : RW, sm_s1, st>>>(N, b, a.ws, ncb, a.cb0, Qp, Qc, W, a.Bblk_prev, j == 0 ? 1 : 0,
+    s1<<<rgrid, reorth ? 2 * RW : RW, sm_s1, st>>>(N, rchk, b, a.ws, ncb, a.cb0, Qp, Qc, W, a.Bblk_prev, j == 0 ? 1 : 0,
                                                    partKq, partKp);
     CSS_LAUNCHED(ctx);
-    k_reduce<<<rblocks_bb, 256, 0, st>>>(nch, ncb, bb, partKq, sA);
-    CSS_LAUNCHED(ctx);
+    CSS_TRY(reduce(partKq, sA));
     if (reorth) {
-      k_reduce<<<rblocks_bb, 256, 0, st>>>(nch, ncb, bb, partKp, sKp);
-      CSS_LAUNCHED(ctx);
+      CSS_TRY(reduce(partKp, sKp));
     }
     k_store_A<<<rblocks_bb, 256, 0, st>>>(ncb, b, a.cb0, m, j, sA, a.Ablk);
     CSS_LAUNCHED(ctx);
     if (j + 1 == m) break;
     // W1 = W0 - Q_j Kq (- Q_{j-1} Kp) and its Gram
-    s3<<<rgrid, th3, sm_s3, st>>>(N, b, a.ws, ncb, Qc, Qp, W, sA, sKp, partKq);
+    s3<<<rgrid, th3, sm_s3, st>>>(N, rchk, b, a.ws, ncb, Qc, Qp, W, sA, sKp, partKq);
     CSS_LAUNCHED(ctx);
     // shifted CholeskyQR3 of W: R0 from G + sI, then two plain CholeskyQR passes; the third is
     // skipped (need3 clear) when the second pass's input W R0^-1 already has a Gram within
     // kQr2Dev of the identity for every colour: one CholeskyQR pass of so well-conditioned a
     // block gives orthonormal columns to the working precision, as the third pass would
-    k_reduce<<<rblocks_bb, 256, 0, st>>>(nch, ncb, bb, partKq, sG);
-    CSS_LAUNCHED(ctx);
+    CSS_TRY(reduce(partKq, sG));
     k_hnorm<<<(unsigned)css_ceil_div(ncb, 8), 256, 0, st>>>(ncb, b, a.cb0, j, sA, a.Bblk_prev, sG, sH);
     CSS_LAUNCHED(ctx);
     CSS_TRY(chol(0, j, sR1, sR1i, a.shift_rel, rp ? nullptr : need3));
     CSS_CU(ctx, cudaMemcpyAsync(sC1, sR1, sizeof(double) * ncb * bb, cudaMemcpyDeviceToDevice, st));
-    k_tri<T, BP, true><<<rgrid, th1, sm_tri, st>>>(N, b, a.ws, ncb, W, W, sR1i, partKq, nullptr, nullptr);
+    k_tri<T, BP, true><<<rgrid, th1, sm_tri, st>>>(N, rchk, b, a.ws, ncb, W, W, sR1i, partKq, nullptr, nullptr);
     CSS_LAUNCHED(ctx);
-    k_reduce<<<rblocks_bb, 256, 0, st>>>(nch, ncb, bb, partKq, sG);
-    CSS_LAUNCHED(ctx);
+    CSS_TRY(reduce(partKq, sG));
     CSS_TRY(chol(1, j, sR1, sR1i, 0.0, need3));
-    k_tri<T, BP, true><<<rgrid, th1, sm_tri, st>>>(N, b, a.ws, ncb, W, W, sR1i, partKq, need3, Qp);
+    k_tri<T, BP, true><<<rgrid, th1, sm_tri, st>>>(N, rchk, b, a.ws, ncb, W, W, sR1i, partKq, need3, Qp);
     CSS_LAUNCHED(ctx);
-    k_reduce<<<rblocks_bb, 256, 0, st>>>(nch, ncb, bb, partKq, sG);
-    CSS_LAUNCHED(ctx);
+    CSS_TRY(reduce(partKq, sG));
     CSS_TRY(chol(2, j, sR2, sR2i, 0.0, need3));
     // Q_{j+1} = W R2^-1 overwrites Q_{j-1} (done by the second pass when two passes sufficed)
-    k_tri<T, BP, false><<<rgrid, th1, sm_tri, st>>>(N, b, a.ws, ncb, W, Qp, sR2i, nullptr, need3, nullptr);
+    k_tri<T, BP, false><<<rgrid, th1, sm_tri, st>>>(N, rchk, b, a.ws, ncb, W, Qp, sR2i, nullptr, need3, nullptr);
     CSS_LAUNCHED(ctx);
     CSS_TRY(sampled(Qp, j + 1));
     CSS_TRY(project_u(Qp, j + 1));
@@ -1512,8 +1536,18 @@ css_status css_spmm(css_ctx* ctx, const LzArgs& a, const void* V, void* W, cudaS
   return launch_spmm<double>(ctx, a, (const double*)V, (double*)W, st);
 }
 
+namespace {
+template <int BP>
+int32_t min_chunk(int64_t N, int32_t b) {
+  const int32_t f = row_chunk<float, BP>(N, b), d = row_chunk<double, BP>(N, b);
+  return f < d ? f : d;
+}
+}  // namespace
+
 size_t css_lanczos_part_doubles(int64_t N, int32_t b, int32_t ncb) {
-  const int64_t nch = css_ceil_div(N, RCHK);
+  const int32_t chunk = b <= 8 ? min_chunk<8>(N, b) : b <= 16 ? min_chunk<16>(N, b) : b <= 24 ? min_chunk<24>(N, b)
+                                                                                              : min_chunk<32>(N, b);
+  const int64_t nch = css_ceil_div(N, chunk);
   return (size_t)nch * ncb * b * b * 2 + (size_t)nch * ncb + 64;
 }
 
