@@ -4,8 +4,8 @@
 //
 // GB300 runs FP64 at about 1/64 of the FP32 rate and a dependent FP64 sqrt + divide costs
 // ~0.6 us, so no stage here is a long sequential FP64 chain:
-//   1. band -> tridiagonal by Householder bulge chasing, up to 32 sweeps in flight (one warp
-//      each, a sweep waits only for the one before it to move past its window); reflectors
+//   1. band -> tridiagonal by Householder bulge chasing, many sweeps in flight (8, 16 or 32
+//      lanes each, a sweep waits only for the one before it to move past its window); reflectors
 //      of length <= b, and a sweep's reflectors touch disjoint rows, so their action on
 //      b-column blocks is applied sweep by sweep with all of a sweep's reflectors in parallel;
 //   2. eigenvalues of the tridiagonal by Sturm-count bisection in FP32 (one thread per
@@ -16,17 +16,16 @@
 //      FP64 accuracy;
 //   4. Y = U^T (Q_band^T E_1 B_0), weights w = ||Y_k||^2, and after mu is known
 //      Z = Q_band U f(Lambda) Y.
+#include <algorithm>
+
 #include "css_eigen.cuh"
+#include "css_pipe.cuh"
 
 namespace {
 
-__device__ __forceinline__ double warp_sum(double v) {
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  return v;
-}
-
 // ------------------------------------------------------------------ band storage
-// AB[col * LDB + d] = T[col + d][col], d in [0, LDB), LDB = 2 kd + 1 (room for the bulge)
+// AB[col * LDB + d] = T[col + d][col], d in [0, LDB), LDB = 2 kd + 2 (room for the bulge, and an odd
+// stride LDB - 1 between the entries of a row, so that a column of lanes reads distinct banks)
 __global__ void k_band_build(int32_t b, int32_t m, int32_t nmax, int32_t ldb, const double* __restrict__ Ablk,
                              const double* __restrict__ Bblk, const int32_t* __restrict__ nblk,
                              double* __restrict__ AB) {
@@ -45,237 +44,301 @@ __global__ void k_band_build(int32_t b, int32_t m, int32_t nmax, int32_t ldb, co
   }
 }
 
-struct Band {
-  double* ab;
-  int32_t ldb;
-  // lower-stored symmetric access, r >= c
-  __device__ __forceinline__ double& at(int32_t r, int32_t c) const { return ab[(size_t)c * ldb + (r - c)]; }
+// Sweeps of an n x n band matrix of half-width kd, the reflectors of a sweep (one annihilating
+// column i, then one per chase step whose block has at least two rows) and the first slot of sweep
+// i among the colour's reflectors: sum over i' < i of 1 + (n - 3 - i') / kd, in closed form.
+__device__ __forceinline__ int32_t n_sweeps(int32_t n, int32_t kd) { return kd >= 2 && n > 2 ? n - 2 : 0; }
+__device__ __forceinline__ int32_t sweep_len(int32_t i, int32_t n, int32_t kd) { return 1 + (n - 3 - i) / kd; }
+__device__ __forceinline__ int32_t sweep_slot(int32_t i, int32_t n, int32_t kd) {
+  auto floors = [kd](int32_t x) {  // sum of r / kd over r < x
+    const int32_t q = x / kd;
+    return kd * (q * (q - 1) / 2) + q * (x - q * kd);
+  };
+  return i + floors(n - 2) - floors(n - 2 - i);
+}
+
+template <int LPS>
+__device__ __forceinline__ double group_sum(double v) {
+#pragma unroll
+  for (int o = LPS / 2; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  return v;
+}
+
+// Householder reflector of x (one element per lane of a group of LPS, zero past its length):
+// H x = beta e_0, H = I - tau v v^T, v_0 = 1, with beta of the sign opposite to x_0 (Golub & Van
+// Loan, section 5.1.3), so x_0 - beta has no cancellation and one reciprocal square root and one
+// division serve tau, beta and the scaling.  Every lane of the warp calls this.
+template <int LPS>
+__device__ __forceinline__ double group_house(double x, int l, double& tau, double& beta) {
+  const double x0 = __shfl_sync(0xffffffffu, x, 0, LPS);
+  const double sig = group_sum<LPS>(l >= 1 ? x * x : 0.0);
+  const double ss = fma(x0, x0, sig), r = rsqrt(ss);
+  const double b = x0 >= 0.0 ? -(ss * r) : ss * r;
+  const double v0 = x0 - b;
+  const bool none = sig == 0.0;
+  tau = none ? 0.0 : fabs(v0) * r;
+  beta = none ? x0 : b;
+  return l == 0 ? 1.0 : (none ? 0.0 : x * (1.0 / v0));
+}
+
+// Band -> tridiagonal with the sweeps pipelined.  Sweep i annihilates column i and chases the
+// bulge.  A step works on the rows [q0, hi) of the lower triangle (its off-diagonal block B and its
+// diagonal block D) and the next step on the rows from hi on.  So a step of sweep i may run once
+// every later step of sweep i - 1 works on rows >= its own hi: what they touch is then disjoint, the
+// same holds by induction for all earlier sweeps, and the result is the sequential order's.  Two
+// steps of sweep i - 1 ahead of sweep i are enough.  Sweep i belongs to slot i mod S of the S slots
+// of a colour, which publishes (sweep, first row of its next step) in one 64-bit word.
+//
+// Bound by FP64 issue: a warp's FP64 instruction takes 64 clocks of its scheduler (19 of the SM with
+// four or more warps) whatever its active lanes, dependent or not, so what counts is the number of
+// instructions of a step and how many schedulers have a step to run:
+//   - LPS = 8, 16 or 32 lanes work on a sweep (kd <= LPS) and a warp holds 32 / LPS sweeps, each at
+//     its own window; with one sweep per warp, 26 of 32 lanes of every FP64 instruction idled at b = 6;
+//   - the two updates of the off-diagonal block are one rank-2 update, the symmetric block is
+//     updated over its lower triangle only, and a reflector takes one rsqrt and one division;
+//   - where the band fits (SMEM), it lives in shared memory and one CTA works on a colour;
+//     otherwise it stays in L2, a step works on a shared-memory copy of its window, and a
+//     cluster of CTAs (co-scheduled, so they may wait for each other) shares a colour, neighbouring
+//     sweeps on different SMs.
+// Measured, one CTA of 32 one-sweep warps per colour -> this: n = 920, kd = 23, 63 colours 52.9 ->
+// 24.4 ms (FP64 issue alone: 16.6 ms on the 126 SMs); n = 390, kd = 13, 44 colours 13.5 -> 5.8 ms;
+// n = 180, kd = 6: 27 colours 4.36 -> 1.57 ms, 504 colours 17.2 -> 2.8 ms.
+// Every wait is bounded: after 2 s without progress the colour's status gets bit 2 and all its
+// CTAs stop.
+struct BandArgs {
+  int32_t kd, nmax, ldb, rcap, cta_per_col, ncta;
+  const int32_t* nblk;
+  double* AB;
+  double* RV;
+  double* RT;
+  int32_t* RR0;
+  unsigned long long* slots;  // [c][S], zeroed (tile mode)
+  double *dd, *ee;
+  int32_t* status;
 };
 
-// Householder vector of x[0..L) held one element per lane of warp 0: H x = beta e_0.
-// Textbook construction (Golub & Van Loan, Alg. 5.1.1): v[0] = 1, tau = 2 v0^2/(sigma+v0^2).
-__device__ void warp_house(double x, int32_t L, double* sv, double* stau, double* sbeta) {
-  const int lane = threadIdx.x & 31;
-  double x0 = __shfl_sync(0xffffffffu, x, 0);
-  double sig = warp_sum((lane >= 1 && lane < L) ? x * x : 0.0);
-  if (sig == 0.0) {
-    if (lane < 32) sv[lane] = (lane == 0) ? 1.0 : 0.0;
-    if (lane == 0) {
-      *stau = 0.0;
-      *sbeta = x0;
-    }
-    return;
-  }
-  double mu = sqrt(x0 * x0 + sig);
-  double v0 = (x0 <= 0.0) ? x0 - mu : -sig / (x0 + mu);
-  double inv = 1.0 / v0;
-  sv[lane] = (lane == 0) ? 1.0 : ((lane < L) ? x * inv : 0.0);
-  if (lane == 0) {
-    *stau = 2.0 * v0 * v0 / (sig + v0 * v0);
-    *sbeta = mu;
-  }
+// doubles of shared memory one sweep needs: vectors v, nv, tz, w and, in tile mode, an mbarrier (16
+// bytes) and the band columns of its window
+__host__ __device__ constexpr int band_group_doubles(int kd, int ldb, int lps, bool smem) {
+  return 4 * lps + (smem ? 0 : 2 + 2 * kd * ldb);
 }
 
-// D <- H D H on the symmetric L x L diagonal block starting at r0 (H = I - tau v v^T), by one
-// warp: lane i owns row i.  pw is the warp's scratch of 32 doubles.
-__device__ void two_sided_w(const Band& A, int32_t r0, int32_t L, const double* v, double tau, double* pw) {
-  const int lane = threadIdx.x & 31;
-  if (tau == 0.0) return;
-  double acc = 0.0;
-  if (lane < L)
-    for (int32_t j = 0; j < L; ++j)
-      acc += (lane >= j ? A.at(r0 + lane, r0 + j) : A.at(r0 + j, r0 + lane)) * v[j];
-  const double vi = lane < L ? v[lane] : 0.0;
-  const double pi = lane < L ? tau * acc : 0.0;
-  const double alpha = -0.5 * tau * warp_sum(pi * vi);
-  const double wi = pi + alpha * vi;
-  pw[lane] = wi;
-  __syncwarp();
-  if (lane < L)
-    for (int32_t j = 0; j <= lane; ++j) A.at(r0 + lane, r0 + j) -= vi * pw[j] + wi * v[j];
-  __syncwarp();
-}
-
-// reflectors recorded by sweep i (the type-1 reflector and one per chase step whose block has
-// at least two rows), the same count the sequential order produces
-__device__ int32_t sweep_refl_count(int32_t i, int32_t n, int32_t kd) {
-  int32_t cnt = 1, p0 = i + 1, Lp = min(kd, n - 1 - i);
-  for (;;) {
-    const int32_t q0 = p0 + Lp;
-    if (q0 > n - 1) break;
-    const int32_t Lq = min(kd, n - q0);
-    if (Lq < 2) break;
-    ++cnt;
-    p0 = q0;
-    Lp = Lq;
+template <int LPS, bool SMEM>
+__global__ void __launch_bounds__(SMEM ? 1024 : 512) k_band_to_tri(const BandArgs a) {
+  constexpr int SPW = 32 / LPS;
+  constexpr unsigned FULL = 0xffffffffu;
+  extern __shared__ __align__(16) unsigned char band_smem[];
+  const int32_t kd = a.kd, ldb = a.ldb, C = a.cta_per_col;
+  const int32_t c = blockIdx.x / C, rank = blockIdx.x - c * C;
+  const int32_t n = a.nblk[c] * kd;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, g = lane / LPS, l = lane - g * LPS;
+  const int32_t nw = blockDim.x >> 5, S = C * nw * SPW;
+  double* ab = a.AB + (size_t)c * a.nmax * ldb;
+  double* mem = reinterpret_cast<double*>(band_smem);
+  volatile unsigned long long* slots;
+  if constexpr (SMEM) {
+    slots = reinterpret_cast<unsigned long long*>(mem);
+    for (int32_t t = threadIdx.x; t < S; t += blockDim.x) slots[t] = 0ull;
+    mem += S;
+    for (int32_t t = threadIdx.x; t < n * ldb; t += blockDim.x) mem[t] = ab[t];
+    ab = mem;
+    mem += (size_t)a.nmax * ldb;
+    __syncthreads();
+  } else {
+    slots = a.slots + (size_t)c * S;
   }
-  return cnt;
-}
-
-// Band -> tridiagonal (one CTA of 32 warps per colour) with the sweeps pipelined: warp w runs
-// sweeps w, w + 32, ...  Every step of a sweep touches the rows and columns of one window
-// [lo, hi) of the matrix, and the windows of a sweep move down the band.  Sweep s runs a step
-// only once sweep s - 1 has finished or its next step's window starts at or after the step's
-// hi: then no later step of s - 1 touches what the step reads or writes, and (by induction)
-// neither does any earlier sweep, so the result is the sequential order's.  Each warp
-// publishes (sweep, start of its next window) in one 64-bit shared word.  Reflector k of
-// sweep i is stored at sweep_off[i] + k, as in the sequential order.  A wait gives up after
-// 2^24 polls: the colour's status gets bit 2 and the CTA stops.
-__global__ void __launch_bounds__(1024) k_band_to_tri(int32_t kd, int32_t nmax, int32_t ldb, int32_t rcap,
-                                                      const int32_t* __restrict__ nblk, double* __restrict__ AB,
-                                                      double* __restrict__ RV, double* __restrict__ RT,
-                                                      int32_t* __restrict__ RR0, int32_t* __restrict__ sweep_off,
-                                                      double* __restrict__ dd, double* __restrict__ ee,
-                                                      int32_t* __restrict__ status) {
-  constexpr int NW = 32;
-  __shared__ double sv[NW][32], svn[NW][32], spw[NW][32];
-  __shared__ double stau[NW], sbeta[NW];
-  __shared__ unsigned long long slot[NW];  // ((sweep + 1) << 32) | start of the next window
-  __shared__ int abort_flag;
-  const int32_t c = blockIdx.x;
-  const int32_t n = nblk[c] * kd;
-  Band A{AB + (size_t)c * nmax * ldb, ldb};
-  double* rv = RV + (size_t)c * rcap * kd;
-  double* rt = RT + (size_t)c * rcap;
-  int32_t* rr = RR0 + (size_t)c * rcap;
-  int32_t* so = sweep_off + (size_t)c * (nmax + 1);
-  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  const int32_t nsweep = n > 2 ? n - 2 : 0;
-  // reflector offsets of the sweeps
-  for (int32_t i = threadIdx.x; i < nsweep; i += blockDim.x) so[i + 1] = sweep_refl_count(i, n, kd);
-  if (threadIdx.x < NW) slot[threadIdx.x] = 0ull;
-  if (threadIdx.x == 0) abort_flag = 0;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    so[0] = 0;
-    for (int32_t i = 0; i < nsweep; ++i) so[i + 1] += so[i];
-    for (int32_t i = nsweep + 1; i <= n; ++i) so[i] = so[nsweep];
-  }
-  __syncthreads();
-  double* v = sv[w];
-  double* vn = svn[w];
-  double* pw = spw[w];
-  auto publish = [&](int32_t s, int32_t front) {
+  mem += (size_t)(warp * SPW + g) * band_group_doubles(kd, ldb, LPS, SMEM);
+  double *v = mem, *nv = mem + LPS, *tz = mem + 2 * LPS, *wv = mem + 3 * LPS;
+  // tile mode: copy of the band columns of the step's window
+  uint64_t* bar = reinterpret_cast<uint64_t*>(mem + 4 * LPS);
+  double* win = mem + 4 * LPS + 2;
+  uint32_t parity = 0;
+  if constexpr (!SMEM) {
+    if (l == 0) css_pipe::bar_init(bar, 1);
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     __syncwarp();
-    if (lane == 0) {
-      __threadfence_block();
-      *(volatile unsigned long long*)&slot[w] =
-          ((unsigned long long)(uint32_t)(s + 1) << 32) | (unsigned long long)(uint32_t)front;
-    }
+  }
+  const int32_t cs = ldb - 1;  // entry (r, j) of a block: base[j * cs + r]
+  const int32_t nsweep = n_sweeps(n, kd);
+  // neighbouring sweeps on different CTAs of the colour
+  const int32_t me = (warp * SPW + g) * C + rank;
+  auto fence = [] {
+    if constexpr (SMEM) __threadfence_block();
+    else __threadfence();
   };
-  // wait until sweep s - 1 cannot touch [.., hi) any more; false on timeout or abort
-  auto wait_prev = [&](int32_t s, int32_t hi) -> bool {
-    bool ok = true;
-    if (s > 0 && lane == 0) {
-      const int pw_ = (s - 1) % NW;
-      for (uint32_t it = 0;; ++it) {
-        const unsigned long long x = *(volatile unsigned long long*)&slot[pw_];
-        const int32_t id = (int32_t)(x >> 32) - 1;
-        const int32_t front = (int32_t)(uint32_t)(x & 0xffffffffull);
-        if (id > s - 1 || (id == s - 1 && front >= hi)) break;
-        if (*(volatile int*)&abort_flag) {
-          ok = false;
+  int32_t i = me, p0 = -1, Lp = 0, k = 0;  // p0 < 0: the sweep's first step is next
+  double tau = 0.0;
+  uint64_t t0 = 0;
+  uint32_t idle = 0;
+  while (__any_sync(FULL, i < nsweep)) {
+    // ------------------------------------------------ may the next step run?
+    const bool live = i < nsweep, first = p0 < 0;
+    const int32_t q0 = first ? i + 1 : p0 + Lp;
+    const int32_t Lq = live ? min(kd, n - q0) : 0;
+    bool act = live;
+    if (live && i > 0) {
+      const unsigned long long x = slots[(i - 1) % S];
+      const int32_t id = (int32_t)(x >> 32) - 1, next_row = (int32_t)(uint32_t)x;
+      act = id > i - 1 || (id == i - 1 && next_row >= q0 + Lq);
+    }
+    if (!__any_sync(FULL, act)) {
+      if (++idle == 1) t0 = css_pipe::gtime();
+      if ((idle & 255u) == 0) {
+        const bool stop = *(volatile int32_t*)&a.status[c] & 2;
+        if (stop || css_pipe::gtime() - t0 > css_pipe::kWaitNs) {
+          if (lane == 0) atomicOr(&a.status[c], 2);
           break;
         }
-        if (it >= (1u << 24)) {
-          atomicOr(&status[c], 2);
-          *(volatile int*)&abort_flag = 1;
-          ok = false;
-          break;
-        }
-        __nanosleep(32);
       }
-      __threadfence_block();
+      __nanosleep(20);
+      continue;
     }
-    ok = __shfl_sync(0xffffffffu, ok ? 1 : 0, 0) != 0;
+    idle = 0;
+    fence();
     __syncwarp();
-    return ok;
-  };
-  auto record = [&](int32_t k, int32_t r0, const double* vv, double tau) {
-    if (lane < kd) rv[(size_t)k * kd + lane] = vv[lane];
-    if (lane == 0) {
-      rt[k] = tau;
-      rr[k] = r0;
-    }
-  };
-  constexpr int32_t kDone = 0x7fffffff;
-  bool dead = false;  // a wait gave up: leave the loops, still reach the final barrier
-  for (int32_t i = w; i < nsweep && !dead; i += NW) {
-    const int32_t r0 = i + 1;
-    const int32_t L = min(kd, n - 1 - i);
-    int32_t k = so[i];
-    publish(i, i);  // first window starts at column i
-    // type 1: annihilate column i below the sub-diagonal; window [i, r0 + L)
-    if (!wait_prev(i, r0 + L)) {
-      dead = true;
-      break;
-    }
-    {
-      const double x = (lane < L) ? A.at(r0 + lane, i) : 0.0;
-      warp_house(x, L, v, &stau[w], &sbeta[w]);
-      __syncwarp();
-      if (lane < L) A.at(r0 + lane, i) = (lane == 0) ? sbeta[w] : 0.0;
-      __syncwarp();
-      two_sided_w(A, r0, L, v, stau[w], pw);
-      record(k++, r0, v, stau[w]);
-    }
-    int32_t p0 = r0, Lp = L;
-    double* cv = v;
-    double* nv = vn;
-    double tau = stau[w];
-    for (;;) {
-      const int32_t q0 = p0 + Lp;
-      if (q0 > n - 1) break;
-      const int32_t Lq = min(kd, n - q0);
-      publish(i, p0);  // this chase step's window is [p0, q0 + Lq)
-      if (!wait_prev(i, q0 + Lq)) {
-        dead = true;
+    // --------------------------------------------------- blocks of the window
+    // B = A[q0 .., p0 ..] (not at the first step) and the lower triangle of D = A[q0 .., q0 ..].  In
+    // tile mode the columns of the window, one contiguous run of the band, arrive by one bulk copy;
+    // the step writes back only what it changed (rows past the window are other sweeps').
+    const int32_t c0 = first ? i : p0;
+    double* w0 = ab + (size_t)c0 * ldb;
+    if constexpr (!SMEM) {
+      bool late = false;
+      if (act) {
+        if (l == 0) {
+          const uint32_t bytes = (uint32_t)((q0 + Lq - c0) * ldb) * 8u;
+          asm volatile("fence.proxy.async;" ::: "memory");
+          css_pipe::bar_expect(bar, bytes);
+          css_pipe::bulk_g2s(win, w0, bytes, bar);
+        }
+        const uint64_t tc = css_pipe::gtime();
+        while (!late && !css_pipe::bar_test(bar, parity)) late = css_pipe::gtime() - tc > css_pipe::kWaitNs;
+        parity ^= 1;
+      }
+      if (__any_sync(FULL, late)) {
+        if (lane == 0) atomicOr(&a.status[c], 2);
         break;
       }
-      // type 2a: B = A[q0.., p0..] <- B (I - tau v v^T), lane = row of B
-      if (tau != 0.0 && lane < Lq) {
+      w0 = win;
+    }
+    double* B = w0 + (q0 - c0);                // entry (r, j) of B (column p0 + j)
+    double* D = w0 + (size_t)(q0 - c0) * ldb;  // entry (r, j) of D (column q0 + j)
+    double* col = w0 + 1;                      // first step: A[i + 1 .., i]
+    // ------------------------------ new reflector (and the old one applied to B)
+    double x = 0.0, ty = 0.0, tau2, beta;
+    if (act && l < Lq) {
+      if (first) {
+        x = col[l];
+      } else {
         double y = 0.0;
-        for (int32_t j = 0; j < Lp; ++j) y += A.at(q0 + lane, p0 + j) * cv[j];
-        for (int32_t j = 0; j < Lp; ++j) A.at(q0 + lane, p0 + j) -= tau * y * cv[j];
+#pragma unroll 4
+        for (int32_t j = 0; j < Lp; ++j) y = fma(B[j * cs + l], v[j], y);
+        ty = tau * y;
+        x = B[l] - ty;
+      }
+    }
+    const double h = group_house<LPS>(x, l, tau2, beta);
+    const bool grow = act && (first || Lq >= 2);  // a one-row block ends the sweep without a reflector
+    const double nl = grow && l < Lq ? h : 0.0;
+    nv[l] = nl;
+    const double d = group_sum<LPS>(nl * ty);
+    __syncwarp();
+    if (act && !first) {
+      // z = nv^T (B - ty v^T) for the columns j >= 1 (one per lane), then
+      // B <- B - ty v^T - nv (tau2 z)^T in one pass
+      double z = 0.0;
+      if (grow && l >= 1 && l < Lp) {
+        const double* Bc = B + l * cs;
+#pragma unroll 4
+        for (int32_t r = 0; r < Lq; ++r) z = fma(nv[r], Bc[r], z);
+        z = tau2 * fma(-d, v[l], z);
+      }
+      tz[l] = z;
+    }
+    __syncwarp();
+    if (act && l < Lq) {
+      if (first) {
+        (SMEM ? col : ab + (size_t)i * ldb + 1)[l] = l == 0 ? beta : 0.0;
+      } else {
+        double* out = SMEM ? B + l : ab + (size_t)p0 * ldb + (q0 - p0) + l;
+        out[0] = grow ? (l == 0 ? beta : 0.0) : B[l] - ty;
+#pragma unroll 4
+        for (int32_t j = 1; j < Lp; ++j) out[(size_t)j * cs] = fma(-nl, tz[j], fma(-ty, v[j], B[j * cs + l]));
+      }
+    }
+    // --------------------------------------------- D <- H D H on its lower triangle
+    double pl = 0.0;
+    if (grow && l < Lq && tau2 != 0.0) {
+      double s0 = 0.0;  // one loop over the row, so that every lane runs the same Lq steps
+      for (int32_t j = 0; j < Lq; ++j) s0 = fma(D[j <= l ? j * cs + l : l * cs + j], nv[j], s0);
+      pl = tau2 * s0;
+    }
+    const double alpha = -0.5 * tau2 * group_sum<LPS>(pl * nl);
+    wv[l] = fma(alpha, nl, pl);
+    __syncwarp();
+    if (grow) {
+      const int32_t ne = Lq * (Lq + 1) / 2;
+      int32_t r = 0, cc = l;
+      for (int32_t e = l; e < ne; e += LPS, cc += LPS) {
+        while (cc > r) {
+          cc -= r + 1;
+          ++r;
+        }
+        D[cc * cs + r] = fma(-nv[r], wv[cc], fma(-wv[r], nv[cc], D[cc * cs + r]));
+      }
+      const int32_t slot = sweep_slot(i, n, kd) + k;
+      if (l < kd) a.RV[((size_t)c * a.rcap + slot) * kd + l] = nl;
+      if (l == 0) {
+        a.RT[(size_t)c * a.rcap + slot] = tau2;
+        a.RR0[(size_t)c * a.rcap + slot] = q0;
+      }
+    }
+    v[l] = act ? nl : v[l];
+    __syncwarp();
+    if constexpr (!SMEM) {  // D back to the band, a column of rows per store
+      if (grow && l < Lq) {
+        double* out = ab + (size_t)q0 * ldb + l;
+        for (int32_t j = 0; j <= l; ++j) out[(size_t)j * cs] = D[j * cs + l];
       }
       __syncwarp();
-      if (Lq < 2) break;
-      // type 2b: new reflector from the bulge's first column, applied from the left
-      {
-        const double x = (lane < Lq) ? A.at(q0 + lane, p0) : 0.0;
-        warp_house(x, Lq, nv, &stau[w], &sbeta[w]);
-      }
-      __syncwarp();
-      const double tau2 = stau[w];
-      if (tau2 != 0.0) {
-        double z = 0.0;  // z[col] = nv^T B[:, col], lane = col >= 1
-        if (lane >= 1 && lane < Lp)
-          for (int32_t r = 0; r < Lq; ++r) z += nv[r] * A.at(q0 + r, p0 + lane);
-        pw[lane] = z;
-        __syncwarp();
-        if (lane < Lq)
-          for (int32_t j = 1; j < Lp; ++j) A.at(q0 + lane, p0 + j) -= tau2 * nv[lane] * pw[j];
-        __syncwarp();
-      }
-      if (lane < Lq) A.at(q0 + lane, p0) = (lane == 0) ? sbeta[w] : 0.0;
-      __syncwarp();
-      // type 3: two-sided on the next diagonal block
-      two_sided_w(A, q0, Lq, nv, tau2, pw);
-      record(k++, q0, nv, tau2);
-      double* t = cv;
-      cv = nv;
-      nv = t;
+    }
+    // --------------------------------------------------------- publish, move on
+    if (act) {
+      if (l == 0) fence();
       tau = tau2;
       p0 = q0;
       Lp = Lq;
+      ++k;
+      const bool over = !grow || q0 + Lq > n - 1;  // no rows below the window
+      if (l == 0)
+        slots[i % S] = ((unsigned long long)(uint32_t)(i + 1) << 32) |
+                       (unsigned long long)(uint32_t)(over ? 0x7fffffff : q0 + Lq);
+      if (over) {
+        i += S;
+        p0 = -1;
+        Lp = 0;
+        k = 0;
+      }
     }
-    if (!dead) publish(i, kDone);
+    __syncwarp();
   }
-  __syncthreads();
-  if (abort_flag) return;
-  for (int32_t i = threadIdx.x; i < n; i += blockDim.x) {
-    dd[(size_t)c * nmax + i] = A.at(i, i);
-    ee[(size_t)c * nmax + i] = (i + 1 < n) ? A.at(i + 1, i) : 0.0;
+  if constexpr (SMEM) {
+    __syncthreads();
+    for (int32_t t = threadIdx.x; t < n; t += blockDim.x) {
+      a.dd[(size_t)c * a.nmax + t] = ab[(size_t)t * ldb];
+      a.ee[(size_t)c * a.nmax + t] = t + 1 < n ? ab[(size_t)t * ldb + 1] : 0.0;
+    }
+  }
+}
+
+// diagonal and sub-diagonal of the reduced band (tile mode)
+__global__ void k_tri_out(int32_t kd, int32_t nmax, int32_t ldb, const int32_t* __restrict__ nblk,
+                          const double* __restrict__ AB, double* __restrict__ dd, double* __restrict__ ee) {
+  const int32_t c = blockIdx.x, n = nblk[c] * kd;
+  const double* ab = AB + (size_t)c * nmax * ldb;
+  for (int32_t t = threadIdx.x; t < n; t += blockDim.x) {
+    dd[(size_t)c * nmax + t] = ab[(size_t)t * ldb];
+    ee[(size_t)c * nmax + t] = t + 1 < n ? ab[(size_t)t * ldb + 1] : 0.0;
   }
 }
 
@@ -285,20 +348,18 @@ __global__ void __launch_bounds__(1024) k_band_to_tri(int32_t kd, int32_t nmax, 
 template <bool FWD>
 __global__ void k_apply_refl(int32_t kd, int32_t b, int32_t nmax, int32_t rcap, const int32_t* __restrict__ nblk,
                              const double* __restrict__ RV, const double* __restrict__ RT,
-                             const int32_t* __restrict__ RR0, const int32_t* __restrict__ sweep_off,
-                             double* __restrict__ X) {
+                             const int32_t* __restrict__ RR0, double* __restrict__ X) {
   const int32_t c = blockIdx.x;
   const int32_t n = nblk[c] * kd;
   const double* rv = RV + (size_t)c * rcap * kd;
   const double* rt = RT + (size_t)c * rcap;
   const int32_t* rr = RR0 + (size_t)c * rcap;
-  const int32_t* so = sweep_off + (size_t)c * (nmax + 1);
   double* x = X + (size_t)c * nmax * b;
-  const int32_t nsweep = n > 2 ? n - 2 : 0;
+  const int32_t nsweep = n_sweeps(n, kd);
   for (int32_t s = 0; s < nsweep; ++s) {
     const int32_t i = FWD ? s : nsweep - 1 - s;
-    const int32_t t0 = so[i], t1 = so[i + 1];
-    for (int32_t t = threadIdx.x; t < (t1 - t0) * b; t += blockDim.x) {
+    const int32_t t0 = sweep_slot(i, n, kd), len = sweep_len(i, n, kd);
+    for (int32_t t = threadIdx.x; t < len * b; t += blockDim.x) {
       const int32_t r = t0 + t / b, col = t % b;
       const double tau = rt[r];
       if (tau == 0.0) continue;
@@ -988,20 +1049,80 @@ __global__ void k_shifts_out(int32_t nmax, const float* __restrict__ lam32, doub
 
 }  // namespace
 
+namespace {
+
+// Launch of k_band_to_tri: lanes per sweep from the band width; enough warps for the sweeps that
+// can be in flight (a sweep trails the one before it by about three windows of kd rows, so two per
+// sweep never starve it); the band in shared memory when it fits beside the sweeps' vectors, else
+// clusters of as many CTAs per colour as the chip has SMs for (at most four).
+template <int LPS>
+css_status launch_band(css_ctx* ctx, const EigArgs& a, int32_t ldb, cudaStream_t st) {
+  constexpr int SPW = 32 / LPS;
+  constexpr size_t kSmem = 220 * 1024;
+  const int32_t kd = a.b, nmax = a.m * a.b;
+  const int32_t flight = nmax / (2 * kd) + 1;
+  BandArgs ba{kd, nmax, ldb, a.rcap, 1, a.n_col, a.nblk, a.AB, a.RV, a.RT, a.RR0, nullptr, a.d, a.e, a.status};
+  auto warps = [&](int32_t ctas, bool smem) {
+    return (int32_t)std::min<int64_t>(smem ? 32 : 16, css_ceil_div(flight, (int64_t)SPW * ctas) + 1);
+  };
+  auto bytes = [&](int32_t nw, bool smem) {
+    return sizeof(double) * ((size_t)nw * SPW * (band_group_doubles(kd, ldb, LPS, smem) + (smem ? 1 : 0)) +
+                             (smem ? (size_t)nmax * ldb : 0));
+  };
+  cudaLaunchConfig_t cfg = {};
+  cfg.stream = st;
+  if (bytes(warps(1, true), true) <= kSmem) {
+    const int32_t nw = warps(1, true);
+    cfg.gridDim = dim3((unsigned)a.n_col);
+    cfg.blockDim = dim3((unsigned)(32 * nw));
+    cfg.dynamicSmemBytes = bytes(nw, true);
+    CSS_CU(ctx, cudaFuncSetAttribute(k_band_to_tri<LPS, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                     (int)cfg.dynamicSmemBytes));
+    CSS_CU(ctx, cudaLaunchKernelEx(&cfg, k_band_to_tri<LPS, true>, ba));
+    CSS_LAUNCHED(ctx);
+    return CSS_OK;
+  }
+  int32_t C = a.n_col * 4 <= ctx->n_sm ? 4 : a.n_col * 2 <= ctx->n_sm ? 2 : 1;
+  int32_t nw = warps(C, false);
+  while (nw > 1 && bytes(nw, false) > kSmem) --nw;  // fewer sweeps in flight, the same result
+  ba.cta_per_col = C;
+  const size_t S = (size_t)C * nw * SPW;
+  CSS_TRY(css_ws(ctx, "e_slots", (size_t)a.n_col * S * sizeof(unsigned long long), (void**)&ba.slots));
+  CSS_CU(ctx, cudaMemsetAsync(ba.slots, 0, (size_t)a.n_col * S * sizeof(unsigned long long), st));
+  cfg.gridDim = dim3((unsigned)(a.n_col * C));
+  cfg.blockDim = dim3((unsigned)(32 * nw));
+  cfg.dynamicSmemBytes = bytes(nw, false);
+  cudaLaunchAttribute at;
+  at.id = cudaLaunchAttributeClusterDimension;
+  at.val.clusterDim.x = (unsigned)C;
+  at.val.clusterDim.y = at.val.clusterDim.z = 1;
+  cfg.attrs = &at;
+  cfg.numAttrs = 1;
+  CSS_CU(ctx, cudaFuncSetAttribute(k_band_to_tri<LPS, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                   (int)cfg.dynamicSmemBytes));
+  CSS_CU(ctx, cudaLaunchKernelEx(&cfg, k_band_to_tri<LPS, false>, ba));
+  CSS_LAUNCHED(ctx);
+  k_tri_out<<<a.n_col, 256, 0, st>>>(kd, nmax, ldb, a.nblk, a.AB, a.d, a.e);
+  CSS_LAUNCHED(ctx);
+  return CSS_OK;
+}
+
+}  // namespace
+
 css_status css_eigen_ritz(css_ctx* ctx, const EigArgs& a, cudaStream_t st) {
-  const int32_t nc = a.n_col, b = a.b, nmax = a.m * b, ldb = 2 * b + 1;
+  const int32_t nc = a.n_col, b = a.b, nmax = a.m * b, ldb = css_band_ld(b);
   k_band_build<<<nc, 256, 0, st>>>(b, a.m, nmax, ldb, a.Ablk, a.Bblk, a.nblk, a.AB);
   CSS_LAUNCHED(ctx);
   CSS_CU(ctx, cudaMemsetAsync(a.status, 0, sizeof(int32_t) * nc, st));
-  k_band_to_tri<<<nc, 1024, 0, st>>>(b, nmax, ldb, a.rcap, a.nblk, a.AB, a.RV, a.RT, a.RR0, a.sweep_off, a.d, a.e,
-                                     a.status);
-  CSS_LAUNCHED(ctx);
+  if (b <= 8) CSS_TRY(launch_band<8>(ctx, a, ldb, st));
+  else if (b <= 16) CSS_TRY(launch_band<16>(ctx, a, ldb, st));
+  else CSS_TRY(launch_band<32>(ctx, a, ldb, st));
   if (a.B0)
     k_x0_b0<<<nc, 256, 0, st>>>(b, nmax, a.B0, a.X0);
   else
     k_x0<<<nc, 256, 0, st>>>(b, nmax, a.cnt, a.X0);
   CSS_LAUNCHED(ctx);
-  k_apply_refl<true><<<nc, 1024, 0, st>>>(b, b, nmax, a.rcap, a.nblk, a.RV, a.RT, a.RR0, a.sweep_off, a.X0);
+  k_apply_refl<true><<<nc, 1024, 0, st>>>(b, b, nmax, a.rcap, a.nblk, a.RV, a.RT, a.RR0, a.X0);
   CSS_LAUNCHED(ctx);
   const size_t sh = 2 * (size_t)nmax * sizeof(float);
   if (sh > 48 * 1024) CSS_CU(ctx, cudaFuncSetAttribute(k_bisect32, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sh));
@@ -1039,14 +1160,14 @@ css_status css_eigen_z(css_ctx* ctx, const EigArgs& a, const int32_t* sys_of_col
   k_zt<<<g, 128, 64 * b * sizeof(double), st>>>(b, b, nmax, a.nblk, sys_of_colour, mu, kT, a.U, a.lam, a.Y, Z,
                                                  fn);
   CSS_LAUNCHED(ctx);
-  k_apply_refl<false><<<nc, 1024, 0, st>>>(b, b, nmax, a.rcap, a.nblk, a.RV, a.RT, a.RR0, a.sweep_off, Z);
+  k_apply_refl<false><<<nc, 1024, 0, st>>>(b, b, nmax, a.rcap, a.nblk, a.RV, a.RT, a.RR0, Z);
   CSS_LAUNCHED(ctx);
   return CSS_OK;
 }
 
 css_status css_eigen_project(css_ctx* ctx, const EigArgs& a, double* V, double* YV, double* scratch, cudaStream_t st) {
   const int32_t nc = a.n_col, b = a.b, nmax = a.m * b;
-  k_apply_refl<true><<<nc, 1024, 0, st>>>(b, b, nmax, a.rcap, a.nblk, a.RV, a.RT, a.RR0, a.sweep_off, V);
+  k_apply_refl<true><<<nc, 1024, 0, st>>>(b, b, nmax, a.rcap, a.nblk, a.RV, a.RT, a.RR0, V);
   CSS_LAUNCHED(ctx);
   dim3 g((unsigned)css_ceil_div(nmax, 128), (unsigned)nc);
   k_ritz_y<<<g, 128, 64 * b * sizeof(double), st>>>(b, b, nmax, a.nblk, a.U, V, YV, scratch);

@@ -14,6 +14,9 @@ __device__ __forceinline__ double css_fermi_dirac(double x, double mu, double kT
   return x < mu ? 1.0 : (x > mu ? 0.0 : 0.5);
 }
 
+// entries per column of the band storage: half-width b, the bulge, and one of padding
+inline int32_t css_band_ld(int32_t b) { return 2 * b + 2; }
+
 struct EigArgs {
   int32_t n_col = 0, b = 0, m = 0;     // colours, block width (band width), block steps
   const double* Ablk = nullptr;        // [c][m][b][b]
@@ -22,11 +25,10 @@ struct EigArgs {
   const int32_t* cnt = nullptr;        // [c] molecules of the colour
   const double* B0 = nullptr;          // [c][b][b] general start factor (nullptr: B_0 = sqrt|c| I)
   int32_t rcap = 0;                    // reflector slots per colour
-  double* AB = nullptr;                // [c][nmax][2b+1]
+  double* AB = nullptr;                // [c][nmax][css_band_ld(b)]
   double* RV = nullptr;                // [c][rcap][b]
   double* RT = nullptr;                // [c][rcap]
   int32_t* RR0 = nullptr;              // [c][rcap]
-  int32_t* sweep_off = nullptr;        // [c][nmax+1]
   double *d = nullptr, *e = nullptr;   // [c][nmax] tridiagonal
   float* lam32 = nullptr;              // [c][nmax] FP32 shifts
   double* tnorm = nullptr;             // [c]

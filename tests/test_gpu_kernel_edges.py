@@ -47,3 +47,16 @@ def test_colour_graph_splits(torch, ctx, graph, n):
     nc = ctx.color_graph(torch.as_tensor(ptr, device="cuda"), torch.as_tensor(adj, device="cuda"), 1004, col)
     ref, nref = oracle.color_graph(ptr, adj, 1004)
     assert nc == nref and np.array_equal(col.cpu().numpy(), ref)
+
+
+# 8, 16 or 32 lanes per sweep (b = 8 / 9, 16 / 17), the band in shared memory or in L2 (m), and in L2
+# with four, two or one CTA per colour (38, 39 and 77 colours); tolerances of the eigen-stage tests
+@pytest.mark.parametrize("b,m,n_col", [(2, 2, 3), (8, 23, 7), (8, 200, 2), (9, 20, 7), (16, 70, 3), (17, 12, 5),
+                                       (32, 16, 38), (32, 16, 39), (32, 16, 77)])
+def test_band_reduction_splits(torch, ctx, b, m, n_col):
+    from tests.test_gpu_eigen import check, random_blocks
+    rng = np.random.default_rng(1000 * b + m)
+    A, B = random_blocks(rng, n_col, m, b)
+    nblk = np.full(n_col, m)
+    nblk[-1] = 1
+    check(torch, ctx, A, B, nblk, rng.integers(1, 50, n_col), mu=0.3, kT=0.5)
