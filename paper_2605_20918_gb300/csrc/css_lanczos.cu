@@ -8,7 +8,7 @@
 //     W0 = W - Q_{j-1} B_{j-1}^T;  A_j = sym(Q_j^T W0)                     (k_s1)
 //     W1 = W0 - Q_j (Q_j^T W0) - Q_{j-1} (Q_{j-1}^T W0)  (local reorthogonalisation; k_s3)
 //     W1 = Q_{j+1} B_j by shifted CholeskyQR3: R = chol(W^T W [+ shift]), W R^-1, three times
-//                                                      (k_chol, k_tri)
+//                                                      (k_gram_chol, k_tri)
 // Small per-colour matrices (A_j, B_j, Grams, Cholesky factors) are FP64; the per-row-chunk
 // partial products are combined in FP64 in a fixed order, so every run is bitwise
 // reproducible (a second pass regenerates the same basis).
@@ -827,10 +827,11 @@ __global__ void __launch_bounds__(2 * RW, 1)
 
 // OUT = W R^-1 (R^-1 upper triangular per colour); partial Gram of OUT when GRAM.  OUT may be W.
 // With three or more stages the products of consecutive tiles alternate between two output tiles.
-// need3 (optional): the per-colour flags of k_chol<1>.  The second CholeskyQR pass (OUT2 set)
+// need3 (optional): the per-colour flags of k_gram_chol<1>.  The second CholeskyQR pass (OUT2 set)
 // writes the columns of a colour whose flag is clear to OUT2 (Q_{j+1}) instead of OUT; the third
 // pass (OUT2 null) writes only the columns of colours whose flag is set, and a CTA none of whose
-// colours needs it returns at once.
+// colours needs it returns at once (in the second pass it leaves out the Gram, which only the third
+// uses).
 template <typename T, int BP, bool GRAM>
 __global__ void __launch_bounds__(384, 2)
     k_tri(int64_t N, int32_t rchk, int32_t b, int32_t ws, int32_t ncb, const T* __restrict__ W, T* OUT,
@@ -840,12 +841,12 @@ __global__ void __launch_bounds__(384, 2)
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const RowCtx<T, BP> c = make_ctx<T, BP>(b, ws, ncb);
   bool store_mine = true;  // this thread's column is stored (to OUT)
+  bool gram = GRAM;        // some colour of the CTA has a use for the Gram
   if (need3) {
-    if (!OUT2) {
-      bool any = false;
-      for (int32_t g = 0; g < c.gcount; ++g) any = any || need3[c.cg0 + g] != 0;
-      if (!any) return;  // uniform over the CTA
-    }
+    bool any = false;
+    for (int32_t g = 0; g < c.gcount; ++g) any = any || need3[c.cg0 + g] != 0;
+    if (!OUT2 && !any) return;  // uniform over the CTA
+    gram = GRAM && any;
     if (c.my_col >= 0) {
       const bool n3 = need3[c.cg0 + c.my_col / b] != 0;
       if (OUT2 && !n3) OUT = OUT2;
@@ -872,195 +873,233 @@ __global__ void __launch_bounds__(384, 2)
       [&](int, int32_t i, int64_t r0, int32_t nr, bool last) {
         const T* o = sO + (i & (NO - 1)) * RTL * c.pitch;
         if (store_mine) c.store(OUT, o, r0, nr);
-        if (GRAM) gram_tile<T, BP, true, RTL>(c, role, o, o, i, last, gp, acc);
+        if (gram) gram_tile<T, BP, true, RTL>(c, role, o, o, i, last, gp, acc);
       });
-  if (GRAM)
+  if (gram)
     gram_store<T, BP, true>(c, role, acc, partG + (size_t)blockIdx.x * ncb * b * b,
                             reinterpret_cast<double*>(smem_raw));
 }
 
-// out = sum of the nch partials of every entry, RD_S of them at a time: thread (x, y) adds the
-// partials y, y + RD_S, ... of entry x of the CTA's 32, the RD_S sums are added in order.  A thread
-// per entry walked all partials alone (35 us for 225 chunks of 65 colours at b = 23).
-constexpr int RD_S = 16;
-__global__ void __launch_bounds__(32 * RD_S) k_reduce(int32_t nch, int64_t n, const double* __restrict__ part,
-                                                      double* __restrict__ out) {
-  __shared__ double sh[RD_S][32];
-  const int64_t t = (int64_t)blockIdx.x * 32 + threadIdx.x;
-  double s = 0.0;
-  if (t < n) {
-#pragma unroll 4
-    for (int32_t ch = threadIdx.y; ch < nch; ch += RD_S) s += part[(size_t)ch * n + t];
+// ------------------------------------------------- small per-colour matrices
+// One CTA per colour adds the Gram partials and works on the sum at once.  FP64 adds and FMAs take
+// 64 clocks of a scheduler each (19 of the SM from four warps on), so every entry has a thread of
+// its own, or several that share its partials.
+inline int gram_threads(int32_t b) { return std::max(256, (b * b + 31) / 32 * 32); }
+
+// G[k][l] (row stride GLD, shared memory) = sum over the nch partials of entry k b + l of one colour
+// (part: its first partial, the next one n entries on); S threads share an entry, their sums are
+// added in order.  scratch: blockDim doubles.  Ends with the CTA synchronised.
+constexpr int GLD = CSS_MAX_B + 1;
+__device__ __forceinline__ void sum_partials(const double* __restrict__ part, int32_t nch, int64_t n, int32_t b,
+                                             double (*G)[GLD], double* scratch) {
+  const int32_t E = b * b, T = blockDim.x, S = max(1, T / E), t = threadIdx.x;
+  if (t < S * E) {
+    const int32_t y = t / E;
+    const double* p = part + (t - y * E);
+    double s = 0.0;
+#pragma unroll 8
+    for (int32_t ch = y; ch < nch; ch += S) s += p[(size_t)ch * n];
+    scratch[t] = s;
   }
-  sh[threadIdx.y][threadIdx.x] = s;
   __syncthreads();
-  if (threadIdx.y != 0 || t >= n) return;
-#pragma unroll
-  for (int y = 1; y < RD_S; ++y) s += sh[y][threadIdx.x];
-  out[t] = s;
-}
-
-// Store A_j = (A + A^T)/2 into the projected matrix and keep the symmetrised copy
-__global__ void k_store_A(int32_t ncb, int32_t b, int32_t cb0, int32_t m, int32_t j, double* __restrict__ A,
-                          double* __restrict__ Ablk) {
-  int32_t t = blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= ncb * b * b) return;
-  int32_t lc = t / (b * b), e = t % (b * b), k = e / b, l = e % b;
-  const double* a = A + (size_t)lc * b * b;
-  double v = 0.5 * (a[k * b + l] + a[l * b + k]);
-  Ablk[(((size_t)(cb0 + lc)) * m + j) * b * b + e] = v;
-  // the symmetrised copy goes to a second slot, so no thread reads a value changed here
-  A[(size_t)ncb * b * b + t] = v;
-}
-
-// Cholesky factor and inverse of one colour's Gram matrix, one warp per colour (lane l owns
-// column l).  Three uses make shifted CholeskyQR3 (Fukaya, Kannan, Nakatsukasa, Yamamoto &
-// Yanagisawa, SIAM J. Sci. Comput. 2020), which keeps the new block orthonormal even when it
-// is nearly rank deficient (converged Ritz directions):
-//   MODE 0: R0 = chol(G + s I), s = shift_rel * trace(G)                 (regularised pass)
-//   MODE 1: R1 = chol(G); stores R10 = R1 R0 in Rprod
-//   MODE 2: R2 = chol(G); B_j = R2 R10 stored in the projected matrix; breakdown when
-//           min_k B_kk <= tau ||H Q_j||_F (same rule as a Householder QR's R_kk)
-// A colour already finished, or a failed factorisation, gives R = I and R^-1 = 0, so the
-// colour's next block is zero.
-// ||H Q_j||_F^2 per colour for the breakdown test.  H Q_j = Q_{j-1} B_{j-1}^T + Q_j A_j + W1
-// with orthonormal blocks orthogonal to W1 (the residual after the projections), so its
-// square norm is ||B_{j-1}||^2 + ||A_j||^2 + trace(W1^T W1) (no B term at the first step).
-__global__ void k_hnorm(int32_t ncb, int32_t b, int32_t cb0, int32_t j, const double* __restrict__ Araw,
-                        const double* __restrict__ Bprev, const double* __restrict__ G, double* __restrict__ hq2) {
-  const int32_t lc = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5), lane = threadIdx.x & 31;
-  if (lc >= ncb) return;
-  const int32_t bb = b * b;
-  const double* a = Araw + (size_t)lc * bb;
-  const double* bp = Bprev + (size_t)(cb0 + lc) * bb;
-  const double* g = G + (size_t)lc * bb;
-  double s = 0.0;
-  for (int32_t e = lane; e < bb; e += 32) {
-    s += a[e] * a[e];
-    if (j > 0) s += bp[e] * bp[e];
+  if (t < E) {
+    double s = scratch[t];
+    for (int32_t y = 1; y < S; ++y) s += scratch[y * E + t];
+    G[t / b][t - t / b * b] = s;
   }
-  if (lane < b) s += g[lane * b + lane];
-  for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-  if (lane == 0) hq2[lc] = s;
+  __syncthreads();
 }
 
-// need3 (optional, one flag per colour of the pass): MODE 1 sets a colour's flag when the Gram
-// of its W R0^-1 is not within kQr2Dev of the identity (max entry), clears it otherwise; MODE 2
-// with the flag clear takes R2 = I, so that B_j = R1 R0 (that colour's third CholeskyQR pass is
-// then skipped: its second pass has written Q_{j+1}).  Each colour decides on its own Gram, so
-// its result does not depend on the other colours of the pass.
+// Kq = Q_j^T W0 (blockIdx.y 0: the raw sum to A, its symmetric part A_j to the projected matrix) and
+// Kp = Q_{j-1}^T W0 (blockIdx.y 1) from their partials
+__global__ void k_gram_A(int32_t nch, int32_t ncb, int32_t b, int32_t cb0, int32_t m, int32_t j,
+                         const double* __restrict__ partKq, const double* __restrict__ partKp, double* __restrict__ A,
+                         double* __restrict__ Ablk, double* __restrict__ Kp) {
+  __shared__ double G[CSS_MAX_B][GLD];
+  __shared__ double scratch[1024];
+  const int32_t lc = blockIdx.x, E = b * b, t = threadIdx.x;
+  const bool second = blockIdx.y != 0;
+  sum_partials((second ? partKp : partKq) + (size_t)lc * E, nch, (int64_t)ncb * E, b, G, scratch);
+  if (t >= E) return;
+  const int32_t k = t / b, l = t - k * b;
+  (second ? Kp : A)[(size_t)lc * E + t] = G[k][l];
+  if (!second && Ablk) Ablk[(((size_t)(cb0 + lc)) * m + j) * E + t] = 0.5 * (G[k][l] + G[l][k]);
+}
+
+// Cholesky factor R of one colour's Gram matrix and R^-1, the three uses of shifted CholeskyQR3
+// (Fukaya, Kannan, Nakatsukasa, Yamamoto & Yanagisawa, SIAM J. Sci. Comput. 2020), which keeps the
+// new block orthonormal even when it is nearly rank deficient (converged Ritz directions):
+//   MODE 0: R0 = chol(G + s I), s = shift_rel * trace(G)  (regularised pass); R0 also to Rprod, and
+//           hq2 = ||H Q_j||_F^2 for the breakdown test.  H Q_j = Q_{j-1} B_{j-1}^T + Q_j A_j + W1 with
+//           orthonormal blocks orthogonal to W1 (the residual after the projections), so it is
+//           ||B_{j-1}||^2 + ||A_j||^2 + trace(W1^T W1) (no B term at the first step; the trace alone
+//           for a start block, Araw == nullptr)
+//   MODE 1: R1 = chol(G), R10 = R1 R0 in Rprod.  need3 (optional, a flag per colour): set when G, the
+//           Gram of W R0^-1, is not within kQr2Dev of the identity (max entry), else clear, and the
+//           colour's factorisation ends here with B_j = R10: one CholeskyQR pass of so
+//           well-conditioned a block gives orthonormal columns to the working precision, as the third
+//           would.  Each colour decides on its own Gram, whatever runs beside it.
+//   MODE 2: R2 = chol(G), B_j = R2 R10, for the colours with need3 set (all when it is null)
+// B_j goes to the projected matrix and, when given, to Bprev.  Breakdown when min_k B_kk <= tau
+// ||H Q_j||_F (the rule of a Householder QR's R_kk).  A colour that is finished, breaks down or has no
+// factor gives R^-1 = 0, so its next block is zero.
+//
+// The elimination runs on [G | I] with eight warps: the rows of G in four of them (row i in warp
+// i mod 4, a lane per column), those of I in the others with the same multipliers, which leaves R and
+// R^-T.  The owner of the next pivot row updates it first and takes the pivot's rsqrt while the others
+// update theirs.  Rows live in shared memory: unrolled over register rows the pivot's code appeared
+// nine times and cost more in instruction fetch than the arithmetic.  Sum of the partials and factor
+// together: b = 23, 60 partials 33 us (before, in two launches, 85 us for a warp that ran the factor's
+// dot products and the back substitution one after the other, and 10 for the sum), b = 6 9 us (16).
 constexpr double kQr2Dev = 1e-2;
 template <int MODE>
-__global__ void k_chol(int32_t ncb, int32_t b, int32_t cb0, int32_t m, int32_t j, const double* __restrict__ G,
-                       const double* __restrict__ hq2, double tau, double shift_rel, double* __restrict__ R,
-                       double* __restrict__ Rinv, double* __restrict__ Rprod, double* __restrict__ Bblk,
-                       int32_t* __restrict__ done, int32_t* __restrict__ nblk, int32_t* __restrict__ need3) {
-  __shared__ double sR[4][CSS_MAX_B][CSS_MAX_B + 1];
-  const int32_t warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int32_t lc = blockIdx.x * 4 + warp;
-  if (lc >= ncb) return;
-  const int32_t c = cb0 + lc;
-  double (*r)[CSS_MAX_B + 1] = sR[warp];
-  const double* g = G + (size_t)lc * b * b;
-  double* ro = R + (size_t)lc * b * b;
-  double* ri = Rinv + (size_t)lc * b * b;
-  double* rp = Rprod + (size_t)lc * b * b;
+__global__ void k_gram_chol(int32_t nch, int32_t ncb, int32_t b, int32_t cb0, int32_t m, int32_t j,
+                            const double* __restrict__ part, const double* __restrict__ Araw,
+                            double* __restrict__ Bprev, double tau, double shift_rel, double* __restrict__ hq2,
+                            double* __restrict__ Rinv, double* __restrict__ Rprod, double* __restrict__ Bblk,
+                            int32_t* __restrict__ done, int32_t* __restrict__ nblk, int32_t* __restrict__ need3) {
+  __shared__ double G[CSS_MAX_B][GLD], X[CSS_MAX_B][GLD];
+  __shared__ double scratch[1024];
+  __shared__ double rowG[2][32], rowI[2][32], sinv[2], swarp[8];
+  __shared__ int sbad;
+  constexpr unsigned FULL = 0xffffffffu;
+  const int32_t lc = blockIdx.x, c = cb0 + lc, E = b * b, t = threadIdx.x, lane = t & 31, warp = t >> 5;
+  if (MODE == 2 && need3 && need3[lc] == 0) return;  // finished by its second pass
+  double* ri = Rinv + (size_t)lc * E;
+  double* rp = Rprod + (size_t)lc * E;
+  double* bo = Bblk + ((size_t)c * m + j) * E;
   const bool was_done = done[c] != 0;
-  bool broken = was_done;
-  for (int32_t i = 0; i < b; ++i)
-    if (lane < b) r[i][lane] = 0.0;
-  __syncwarp();
+  auto stop = [&]() {  // no next block for this colour (the whole CTA calls this)
+    if (t < E) {
+      ri[t] = 0.0;
+      if (MODE > 0) bo[t] = 0.0;
+      if (MODE > 0 && Bprev) Bprev[(size_t)c * E + t] = 0.0;
+      if (MODE < 2) rp[t] = t / b == t % b ? 1.0 : 0.0;
+    }
+    if (t == 0) {
+      if (MODE == 0) hq2[lc] = 0.0;
+      if (MODE == 1 && need3) need3[lc] = 0;
+      if (!was_done) {
+        done[c] = 1;
+        nblk[c] = j + 1;
+      }
+    }
+  };
+  if (was_done) {
+    stop();
+    return;
+  }
+  sum_partials(part + (size_t)lc * E, nch, (int64_t)ncb * E, b, G, scratch);
   double shift = 0.0;
-  if (MODE == 0) {
-    double t = (lane < b) ? g[lane * b + lane] : 0.0;
-    for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
-    shift = shift_rel * t;
+  if (MODE == 0) {  // trace(G) in warp 0, the norms of A_j and B_{j-1} in warps 1 to 7
+    if (warp < 8) {
+      double h = 0.0;
+      if (warp == 0) {
+        h = lane < b ? G[lane][lane] : 0.0;
+      } else if (Araw) {
+        for (int32_t e = t - 32; e < E; e += 224) {
+          const double x = Araw[(size_t)lc * E + e], y = j > 0 ? Bprev[(size_t)c * E + e] : 0.0;
+          h = fma(x, x, fma(y, y, h));
+        }
+      }
+      for (int o = 16; o > 0; o >>= 1) h += __shfl_xor_sync(FULL, h, o);
+      if (lane == 0) swarp[warp] = h;
+    }
+    __syncthreads();
+    shift = shift_rel * swarp[0];
+    if (t == 0) {
+      double h = swarp[0];
+      for (int w = 1; w < 8; ++w) h += swarp[w];
+      hq2[lc] = h;
+    }
   }
-  const bool two_pass = MODE == 2 && need3 && need3[lc] == 0;
+  bool last = MODE == 2;  // this pass ends the colour's factorisation
   if (MODE == 1 && need3) {
-    double dev = broken ? 1.0 : 0.0;
-    if (lane < b && !broken)
-      for (int32_t i = 0; i < b; ++i) dev = fmax(dev, fabs(g[i * b + lane] - (i == lane ? 1.0 : 0.0)));
-    for (int o = 16; o > 0; o >>= 1) dev = fmax(dev, __shfl_xor_sync(0xffffffffu, dev, o));
-    if (lane == 0) need3[lc] = dev <= kQr2Dev ? 0 : 1;
+    const int32_t k = t / b, l = t - k * b;
+    last = !__syncthreads_or(t < E && !(fabs(G[t < E ? k : 0][l] - (k == l ? 1.0 : 0.0)) <= kQr2Dev));
+    if (t == 0) need3[lc] = last ? 0 : 1;
   }
-  if (two_pass) {
-    if (lane < b)
-      for (int32_t i = 0; i < b; ++i) r[i][lane] = i == lane ? 1.0 : 0.0;
-  } else if (!broken) {
-    for (int32_t k = 0; k < b && !broken; ++k) {
-      double sv = 0.0;
-      if (lane < b && lane >= k) {
-        sv = g[k * b + lane] + ((lane == k) ? shift : 0.0);
-        for (int32_t i = 0; i < k; ++i) sv -= r[i][k] * r[i][lane];
+  // ------------------------------------------------------ elimination on [G | I]
+  const bool half = warp >= 4;  // rows of I
+  const int w4 = warp & 3;
+  double (*M)[GLD] = half ? X : G;
+  if (t < E) {
+    X[t / b][t % b] = t / b == t % b ? 1.0 : 0.0;
+    if (MODE == 0 && t / b == t % b) G[t / b][t / b] += shift;
+  }
+  if (t == 0) sbad = 0;
+  __syncthreads();
+  // the owner of row k scales it (rows of G) or hands it over as it is (rows of I)
+  auto pivot = [&](int32_t k, double row) {
+    if (!half) {
+      const double piv = __shfl_sync(FULL, row, k);
+      const double inv = rsqrt(piv);
+      row = lane >= k ? row * inv : 0.0;
+      rowG[k & 1][lane] = row;
+      if (lane < b) G[k][lane] = row;
+      if (lane == 0) {
+        sinv[k & 1] = inv;
+        if (!(piv > 0.0)) sbad = 1;
       }
-      const double piv = __shfl_sync(0xffffffffu, sv, k);
-      if (!(piv > 0.0)) {
-        broken = true;
-        break;
+    } else {
+      rowI[k & 1][lane] = row;
+    }
+  };
+#pragma unroll 1
+  for (int32_t k = -1; k < b; ++k) {
+    if (warp < 8) {
+      const int p = k & 1;
+      double x = 0.0;
+      if (k >= 0) x = half ? rowI[p][lane] * sinv[p] : rowG[p][lane];
+      const int32_t nx = k + 1;
+      if (nx < b && (nx & 3) == w4) {  // the next pivot row first
+        double row = lane < b ? M[nx][lane] : 0.0;
+        if (k >= 0) row = fma(-rowG[p][nx], x, row);
+        pivot(nx, row);
       }
-      const double inv = 1.0 / sqrt(piv);
-      if (lane < b && lane >= k) r[k][lane] = sv * inv;
-      __syncwarp();
-    }
-  }
-  __syncwarp();
-  // the new sub-diagonal block and the breakdown test
-  if (MODE == 2 && !broken && lane < b) {
-    for (int32_t i = 0; i < b; ++i) {
-      double sv = 0.0;
-      for (int32_t k2 = i; k2 <= lane; ++k2) sv += r[i][k2] * rp[k2 * b + lane];
-      Bblk[(((size_t)c) * m + j) * b * b + i * b + lane] = (i <= lane) ? sv : 0.0;
-    }
-  }
-  if (MODE == 2 && !broken) {
-    double dk = 1e300;
-    if (lane < b) {
-      double sv = 0.0;
-      for (int32_t k2 = lane; k2 < b; ++k2) sv += (k2 == lane ? r[lane][lane] : 0.0) * rp[k2 * b + lane];
-      dk = sv;  // (R2 R10)_kk = R2_kk R10_kk for upper-triangular factors
-    }
-    for (int o = 16; o > 0; o >>= 1) dk = fmin(dk, __shfl_xor_sync(0xffffffffu, dk, o));
-    if (!(dk > tau * sqrt(hq2[lc]))) broken = true;
-  }
-  if (broken) {
-    if (lane < b)
-      for (int32_t i = 0; i < b; ++i) {
-        ro[i * b + lane] = (i == lane) ? 1.0 : 0.0;
-        ri[i * b + lane] = 0.0;
-        if (MODE == 1) rp[i * b + lane] = (i == lane) ? 1.0 : 0.0;
-        if (MODE == 2) Bblk[(((size_t)c) * m + j) * b * b + i * b + lane] = 0.0;
+      if (k >= 0 && lane < b) {
+#pragma unroll 1
+        for (int32_t i = nx + 1 + ((w4 - nx - 1) & 3); i < b; i += 4) M[i][lane] = fma(-rowG[p][i], x, M[i][lane]);
+        if (half && (k & 3) == w4) X[k][lane] = x;  // row k of R^-T
       }
-    if (!was_done && lane == 0) {
-      done[c] = 1;
-      nblk[c] = j + 1;
+    }
+    __syncthreads();
+  }
+  if (sbad) {
+    stop();
+    return;
+  }
+  const int32_t k = t / b, l = t - k * b;  // R is in G (zero below its diagonal), R^-T in X
+  const double xr = t < E && k <= l ? X[l][k] : 0.0;
+  if (MODE == 0) {
+    if (t < E) {
+      ri[t] = xr;
+      rp[t] = G[k][l];
     }
     return;
   }
-  // inverse of the upper-triangular factor: lane l solves R x = e_l
-  if (lane < b) {
-    double x[CSS_MAX_B];
-    for (int32_t i = b - 1; i >= 0; --i) {
-      double sv = (i == lane) ? 1.0 : 0.0;
-      for (int32_t k2 = i + 1; k2 <= lane; ++k2) sv -= r[i][k2] * x[k2];
-      x[i] = (i <= lane) ? sv / r[i][i] : 0.0;
+  // product of the factors so far
+  double prod = 0.0;
+  if (t < E && k <= l)
+    for (int32_t q = k; q <= l; ++q) prod = fma(G[k][q], rp[q * b + l], prod);
+  if (last) {  // the breakdown test on the diagonal of B_j
+    const double limit = tau * sqrt(hq2[lc]);
+    if (t < E && k == l && !(prod > limit)) sbad = 1;
+    __syncthreads();
+    if (sbad) {
+      stop();
+      return;
     }
-    for (int32_t i = 0; i < b; ++i) {
-      ri[i * b + lane] = (i <= lane) ? x[i] : 0.0;
-      ro[i * b + lane] = r[i][lane];
-    }
+  } else {
+    __syncthreads();  // every thread has read Rprod
   }
-  __syncwarp();
-  if (MODE == 1 && lane < b) {
-    // R10 = R1 R0 (R0 is the factor of the previous pass, passed in Rprod's slot on entry)
-    double col[CSS_MAX_B];
-    for (int32_t i = 0; i < b; ++i) {
-      double sv = 0.0;
-      for (int32_t k2 = i; k2 <= lane; ++k2) sv += r[i][k2] * rp[k2 * b + lane];
-      col[i] = (i <= lane) ? sv : 0.0;
+  if (t < E) {
+    ri[t] = xr;
+    rp[t] = prod;
+    if (last) {
+      bo[t] = prod;
+      if (Bprev) Bprev[(size_t)c * E + t] = prod;
     }
-    __syncwarp();
-    for (int32_t i = 0; i < b; ++i) rp[i * b + lane] = col[i];
   }
 }
 
@@ -1072,22 +1111,14 @@ __global__ void k_eye(int32_t ncb, int32_t b, double* __restrict__ M) {
   M[t] = (e / b == e % b) ? 1.0 : 0.0;
 }
 
-// hq2[lc] = trace of the Gram G[lc] = ||W_c||_F^2 (breakdown scale of a start block)
-__global__ void k_gtrace(int32_t ncb, int32_t b, const double* __restrict__ G, double* __restrict__ hq2) {
-  const int32_t lc = blockIdx.x * blockDim.x + threadIdx.x;
-  if (lc >= ncb) return;
-  double s = 0.0;
-  for (int32_t k = 0; k < b; ++k) s += G[((size_t)lc * b + k) * b + k];
-  hq2[lc] = s;
-}
-
-// Vc[cb0 + lc][j b + k][l] = P[lc][k][l]
-__global__ void k_store_v(int32_t ncb, int32_t b, int32_t cb0, int32_t nmax, int32_t j, const double* __restrict__ P,
-                          double* __restrict__ Vc) {
-  const int32_t t = blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= ncb * b * b) return;
-  const int32_t lc = t / (b * b), e = t % (b * b), k = e / b, l = e % b;
-  Vc[((size_t)(cb0 + lc) * nmax + (size_t)j * b + k) * b + l] = P[t];
+// Vc[cb0 + lc][j b + k][l] = (Q_j^T u)[k][l] from its partials
+__global__ void k_gram_v(int32_t nch, int32_t ncb, int32_t b, int32_t cb0, int32_t nmax, int32_t j,
+                         const double* __restrict__ part, double* __restrict__ Vc) {
+  __shared__ double G[CSS_MAX_B][GLD];
+  __shared__ double scratch[1024];
+  const int32_t lc = blockIdx.x, E = b * b, t = threadIdx.x;
+  sum_partials(part + (size_t)lc * E, nch, (int64_t)ncb * E, b, G, scratch);
+  if (t < E) Vc[((size_t)(cb0 + lc) * nmax + (size_t)j * b) * b + t] = G[t / b][t % b];
 }
 
 // Q_1 = R_c / sqrt|c| for the colours of the batch (the rest of Q is zeroed by the caller)
@@ -1290,23 +1321,29 @@ css_status run_pass_bp(css_ctx* ctx, const LzArgs& a_in, cudaStream_t st) {
   const int th3 = row_threads<T, BP, RTL3>(b), th1 = row_threads<T, BP, RTL1>(b);
   double* partKq = a.part;
   double* partKp = a.part + (size_t)nch * ncb * bb;
-  double* sA = a.small;                          // [2][ncb][bb]: raw, symmetrised
-  double* sH = a.small + 2 * (size_t)ncb * bb;   // [ncb]
-  double* sG = sH + ncb;                         // [ncb][bb]
-  double* sR1 = sG + (size_t)ncb * bb;
-  double* sR1i = sR1 + (size_t)ncb * bb;
-  double* sR2 = sR1i + (size_t)ncb * bb;
-  double* sR2i = sR2 + (size_t)ncb * bb;
-  double* sC1 = sR2i + (size_t)ncb * bb;
-  double* sKp = sC1 + (size_t)ncb * bb;
-  double* sV = sKp + (size_t)ncb * bb;  // Q_j^T u of the running step (the tenth small matrix)
-  double* sRi10 = sV + (size_t)ncb * bb;     // R0^-1 R1^-1 (FP32 row passes)
-  double* sRi210 = sRi10 + (size_t)ncb * bb;  // R0^-1 R1^-1 R2^-1
+  double* sA = a.small;                        // [ncb][bb] Q_j^T W0
+  double* sKp = sA + (size_t)ncb * bb;         // Q_{j-1}^T W0
+  double* sRi = sKp + (size_t)ncb * bb;        // R^-1 of the running CholeskyQR pass
+  double* sC1 = sRi + (size_t)ncb * bb;        // product of the factors so far
+  double* sRi10 = sC1 + (size_t)ncb * bb;      // R0^-1 R1^-1, R0^-1 R1^-1 R2^-1 and a copy of R0^-1
+  double* sRi210 = sRi10 + (size_t)ncb * bb;   // (streaming row passes)
+  double* sRi0 = sRi210 + (size_t)ncb * bb;
+  double* sH = sRi0 + (size_t)ncb * bb;        // [ncb] ||H Q_j||_F^2
   // per colour: "a third CholeskyQR pass is needed" in the running step (after the matrices)
-  int32_t* need3 = reinterpret_cast<int32_t*>(sRi210 + (size_t)ncb * bb);
-  const unsigned rblocks_bb = (unsigned)css_ceil_div((int64_t)ncb * bb, 256);
-  auto reduce = [&](const double* part, double* out) -> css_status {
-    k_reduce<<<(unsigned)css_ceil_div((int64_t)ncb * bb, 32), dim3(32, RD_S), 0, st>>>(nch, (int64_t)ncb * bb, part, out);
+  int32_t* need3 = reinterpret_cast<int32_t*>(sH + ncb);
+  const int gth = gram_threads(b);
+  // A_j (and Q_{j-1}^T W0) from the partials of S1
+  auto gram_A = [&](int32_t j, bool both, double* Ablk) -> css_status {
+    k_gram_A<<<dim3((unsigned)ncb, both ? 2 : 1), gth, 0, st>>>(nch, ncb, b, a.cb0, m, j, partKq, partKp, sA, Ablk, sKp);
+    CSS_LAUNCHED(ctx);
+    return CSS_OK;
+  };
+  // a CholeskyQR pass's factor from the Gram partials: B_j of step j, or (start) B_0 of the start block
+  auto chol = [&](int mode, int32_t j, double* Ri, int32_t* n3, bool start) -> css_status {
+    auto kern = mode == 0 ? k_gram_chol<0> : mode == 1 ? k_gram_chol<1> : k_gram_chol<2>;
+    kern<<<(unsigned)ncb, gth, 0, st>>>(nch, ncb, b, a.cb0, start ? 1 : m, start ? 0 : j, partKq, start ? nullptr : sA,
+                                        start ? nullptr : a.Bblk_prev, a.tau, a.shift_rel, sH, Ri, sC1,
+                                        start ? a.B0 : a.Bblk, a.done, a.nblk, n3);
     CSS_LAUNCHED(ctx);
     return CSS_OK;
   };
@@ -1324,32 +1361,16 @@ css_status run_pass_bp(css_ctx* ctx, const LzArgs& a_in, cudaStream_t st) {
   if (a.start) {
     // Q_1 B_0 = start by the shifted CholeskyQR3 of the steps below: the start block is copied
     // into W (times the identity) with its Gram, and B_0 is the product of the three factors
-    k_eye<<<rblocks_bb, 256, 0, st>>>(ncb, b, sR1i);
+    k_eye<<<(unsigned)css_ceil_div((int64_t)ncb * bb, 256), 256, 0, st>>>(ncb, b, sRi);
     CSS_LAUNCHED(ctx);
-    k_tri<T, BP, true><<<rgrid, th1, sm_tri, st>>>(N, rchk, b, a.ws, ncb, (const T*)a.start, W, sR1i,
-                                                                     partKq, nullptr, nullptr);
-    CSS_LAUNCHED(ctx);
-    CSS_TRY(reduce(partKq, sG));
-    k_gtrace<<<(unsigned)css_ceil_div(ncb, 128), 128, 0, st>>>(ncb, b, sG, sH);
-    CSS_LAUNCHED(ctx);
-    const unsigned gb = (unsigned)css_ceil_div(ncb, 4);
-    k_chol<0><<<gb, 128, 0, st>>>(ncb, b, a.cb0, 1, 0, sG, sH, a.tau, a.shift_rel, sR1, sR1i, sC1, a.B0, a.done,
-                                  a.nblk, nullptr);
-    CSS_LAUNCHED(ctx);
-    CSS_CU(ctx, cudaMemcpyAsync(sC1, sR1, sizeof(double) * ncb * bb, cudaMemcpyDeviceToDevice, st));
-    k_tri<T, BP, true><<<rgrid, th1, sm_tri, st>>>(N, rchk, b, a.ws, ncb, W, W, sR1i, partKq, nullptr, nullptr);
-    CSS_LAUNCHED(ctx);
-    CSS_TRY(reduce(partKq, sG));
-    k_chol<1><<<gb, 128, 0, st>>>(ncb, b, a.cb0, 1, 0, sG, sH, a.tau, 0.0, sR1, sR1i, sC1, a.B0, a.done, a.nblk,
-                                  nullptr);
-    CSS_LAUNCHED(ctx);
-    k_tri<T, BP, true><<<rgrid, th1, sm_tri, st>>>(N, rchk, b, a.ws, ncb, W, W, sR1i, partKq, nullptr, nullptr);
-    CSS_LAUNCHED(ctx);
-    CSS_TRY(reduce(partKq, sG));
-    k_chol<2><<<gb, 128, 0, st>>>(ncb, b, a.cb0, 1, 0, sG, sH, a.tau, 0.0, sR2, sR2i, sC1, a.B0, a.done, a.nblk,
-                                  nullptr);
-    CSS_LAUNCHED(ctx);
-    k_tri<T, BP, false><<<rgrid, th1, sm_tri, st>>>(N, rchk, b, a.ws, ncb, W, Qc, sR2i, nullptr, nullptr, nullptr);
+    const T* in = (const T*)a.start;
+    for (int mode = 0; mode < 3; ++mode) {
+      k_tri<T, BP, true><<<rgrid, th1, sm_tri, st>>>(N, rchk, b, a.ws, ncb, in, W, sRi, partKq, nullptr, nullptr);
+      CSS_LAUNCHED(ctx);
+      CSS_TRY(chol(mode, 0, sRi, nullptr, true));
+      in = W;
+    }
+    k_tri<T, BP, false><<<rgrid, th1, sm_tri, st>>>(N, rchk, b, a.ws, ncb, W, Qc, sRi, nullptr, nullptr, nullptr);
     CSS_LAUNCHED(ctx);
   } else {
     k_init_q1<T><<<(unsigned)css_ceil_div(N, 256), 256, 0, st>>>(a.n_brow, b, a.ws, a.cb0, ncb, a.colour, a.sign,
@@ -1362,8 +1383,7 @@ css_status run_pass_bp(css_ctx* ctx, const LzArgs& a_in, cudaStream_t st) {
     k_s1<T, BP, false><<<rgrid, RW, sm_s1, st>>>(N, rchk, b, a.ws, ncb, a.cb0, nullptr, Qj, (T*)a.ucol, nullptr, 1,
                                                   partKq, nullptr);
     CSS_LAUNCHED(ctx);
-    CSS_TRY(reduce(partKq, sV));
-    k_store_v<<<rblocks_bb, 256, 0, st>>>(ncb, b, a.cb0, m * b, j, sV, a.Vc);
+    k_gram_v<<<(unsigned)ncb, gth, 0, st>>>(nch, ncb, b, a.cb0, m * b, j, partKq, a.Vc);
     CSS_LAUNCHED(ctx);
     return CSS_OK;
   };
@@ -1384,18 +1404,6 @@ css_status run_pass_bp(css_ctx* ctx, const LzArgs& a_in, cudaStream_t st) {
     } else {
       return CSS_OK;
     }
-    CSS_LAUNCHED(ctx);
-    return CSS_OK;
-  };
-  auto chol = [&](int mode, int32_t j, double* R, double* Ri, double shift, int32_t* n3) -> css_status {
-    const unsigned gb = (unsigned)css_ceil_div(ncb, 4);
-    if (mode == 0)
-      k_chol<0><<<gb, 128, 0, st>>>(ncb, b, a.cb0, m, j, sG, sH, a.tau, shift, R, Ri, sC1, a.Bblk, a.done, a.nblk,
-                                    n3);
-    else if (mode == 1)
-      k_chol<1><<<gb, 128, 0, st>>>(ncb, b, a.cb0, m, j, sG, sH, a.tau, 0.0, R, Ri, sC1, a.Bblk, a.done, a.nblk, n3);
-    else
-      k_chol<2><<<gb, 128, 0, st>>>(ncb, b, a.cb0, m, j, sG, sH, a.tau, 0.0, R, Ri, sC1, a.Bblk, a.done, a.nblk, n3);
     CSS_LAUNCHED(ctx);
     return CSS_OK;
   };
@@ -1420,40 +1428,26 @@ css_status run_pass_bp(css_ctx* ctx, const LzArgs& a_in, cudaStream_t st) {
       // Kq = Q_j^T W0, Kp = Q_{j-1}^T W0 with W0 = W - Q_{j-1} B_{j-1}^T
       CSS_TRY(css_rowpass(ctx, 0, N, b, a.ws, ncb, a.cb0, first, ro, q, qp, wv, nullptr, a.Bblk_prev, nullptr, nullptr,
                           partKq, partKp, st));
-      CSS_TRY(reduce(partKq, sA));
-      if (reorth && !first) {
-        CSS_TRY(reduce(partKp, sKp));
-      }
-      k_store_A<<<rblocks_bb, 256, 0, st>>>(ncb, b, a.cb0, m, j, sA, a.Ablk);
-      CSS_LAUNCHED(ctx);
+      CSS_TRY(gram_A(j, reorth && !first, a.Ablk));
       if (j + 1 == m) break;
       // W1 = W - Q_j Kq - Q_{j-1} (B_{j-1}^T + Kp) over W, and its Gram
       CSS_TRY(css_rowpass(ctx, 1, N, b, a.ws, ncb, a.cb0, first, ro, q, qp, wv, wv, sA, a.Bblk_prev,
                           (reorth && !first) ? sKp : nullptr, partKq, nullptr, st));
-      CSS_TRY(reduce(partKq, sG));
-      k_hnorm<<<(unsigned)css_ceil_div(ncb, 8), 256, 0, st>>>(ncb, b, a.cb0, j, sA, a.Bblk_prev, sG, sH);
-      CSS_LAUNCHED(ctx);
       // shifted CholeskyQR3 on W1 without storing the intermediates: the Grams of W1 R0^-1 and
       // W1 R0^-1 R1^-1 are taken from W1 itself, and Q_{j+1} = W1 R0^-1 R1^-1 R2^-1
-      CSS_TRY(chol(0, j, sR1, sR1i, a.shift_rel, rp ? nullptr : need3));
-      CSS_CU(ctx, cudaMemcpyAsync(sC1, sR1, sizeof(double) * ncb * bb, cudaMemcpyDeviceToDevice, st));
-      CSS_TRY(css_rowpass(ctx, 2, N, b, a.ws, ncb, a.cb0, first, ro, nullptr, nullptr, wv, nullptr, sR1i, nullptr,
+      CSS_TRY(chol(0, j, sRi0, nullptr, false));
+      CSS_TRY(css_rowpass(ctx, 2, N, b, a.ws, ncb, a.cb0, first, ro, nullptr, nullptr, wv, nullptr, sRi0, nullptr,
                           nullptr, partKq, nullptr, st));
-      CSS_TRY(reduce(partKq, sG));
-      CSS_TRY(chol(1, j, sR2, sR2i, 0.0, nullptr));
-      CSS_TRY(css_small_mm(ctx, ncb, b, sR1i, sR2i, sRi10, st));
+      CSS_TRY(chol(1, j, sRi, nullptr, false));
+      CSS_TRY(css_small_mm(ctx, ncb, b, sRi0, sRi, sRi10, st));
       CSS_TRY(css_rowpass(ctx, 2, N, b, a.ws, ncb, a.cb0, first, ro, nullptr, nullptr, wv, nullptr, sRi10, nullptr,
                           nullptr, partKq, nullptr, st));
-      CSS_TRY(reduce(partKq, sG));
-      CSS_TRY(chol(2, j, sR1, sR1i, 0.0, nullptr));
-      CSS_TRY(css_small_mm(ctx, ncb, b, sRi10, sR1i, sRi210, st));
+      CSS_TRY(chol(2, j, sRi, nullptr, false));
+      CSS_TRY(css_small_mm(ctx, ncb, b, sRi10, sRi, sRi210, st));
       CSS_TRY(css_rowpass(ctx, 3, N, b, a.ws, ncb, a.cb0, first, ro, nullptr, nullptr, wv, (float*)Qp, sRi210, nullptr,
                           nullptr, nullptr, nullptr, st));
       CSS_TRY(sampled(Qp, j + 1));
       CSS_TRY(project_u(Qp, j + 1));
-      CSS_CU(ctx, cudaMemcpy2DAsync(a.Bblk_prev + (size_t)a.cb0 * bb, bb * sizeof(double),
-                                    a.Bblk + ((size_t)a.cb0 * m + j) * bb, (size_t)m * bb * sizeof(double),
-                                    bb * sizeof(double), ncb, cudaMemcpyDeviceToDevice, st));
       T* t = Qp;
       Qp = Qc;
       Qc = t;
@@ -1463,42 +1457,24 @@ css_status run_pass_bp(css_ctx* ctx, const LzArgs& a_in, cudaStream_t st) {
     s1<<<rgrid, reorth ? 2 * RW : RW, sm_s1, st>>>(N, rchk, b, a.ws, ncb, a.cb0, Qp, Qc, W, a.Bblk_prev, j == 0 ? 1 : 0,
                                                    partKq, partKp);
     CSS_LAUNCHED(ctx);
-    CSS_TRY(reduce(partKq, sA));
-    if (reorth) {
-      CSS_TRY(reduce(partKp, sKp));
-    }
-    k_store_A<<<rblocks_bb, 256, 0, st>>>(ncb, b, a.cb0, m, j, sA, a.Ablk);
-    CSS_LAUNCHED(ctx);
+    CSS_TRY(gram_A(j, reorth, a.Ablk));
     if (j + 1 == m) break;
     // W1 = W0 - Q_j Kq (- Q_{j-1} Kp) and its Gram
     s3<<<rgrid, th3, sm_s3, st>>>(N, rchk, b, a.ws, ncb, Qc, Qp, W, sA, sKp, partKq);
     CSS_LAUNCHED(ctx);
-    // shifted CholeskyQR3 of W: R0 from G + sI, then two plain CholeskyQR passes; the third is
-    // skipped (need3 clear) when the second pass's input W R0^-1 already has a Gram within
-    // kQr2Dev of the identity for every colour: one CholeskyQR pass of so well-conditioned a
-    // block gives orthonormal columns to the working precision, as the third pass would
-    CSS_TRY(reduce(partKq, sG));
-    k_hnorm<<<(unsigned)css_ceil_div(ncb, 8), 256, 0, st>>>(ncb, b, a.cb0, j, sA, a.Bblk_prev, sG, sH);
+    // shifted CholeskyQR3 of W: R0 from G + sI, then one or two plain CholeskyQR passes (k_gram_chol)
+    CSS_TRY(chol(0, j, sRi, nullptr, false));
+    k_tri<T, BP, true><<<rgrid, th1, sm_tri, st>>>(N, rchk, b, a.ws, ncb, W, W, sRi, partKq, nullptr, nullptr);
     CSS_LAUNCHED(ctx);
-    CSS_TRY(chol(0, j, sR1, sR1i, a.shift_rel, rp ? nullptr : need3));
-    CSS_CU(ctx, cudaMemcpyAsync(sC1, sR1, sizeof(double) * ncb * bb, cudaMemcpyDeviceToDevice, st));
-    k_tri<T, BP, true><<<rgrid, th1, sm_tri, st>>>(N, rchk, b, a.ws, ncb, W, W, sR1i, partKq, nullptr, nullptr);
+    CSS_TRY(chol(1, j, sRi, need3, false));
+    k_tri<T, BP, true><<<rgrid, th1, sm_tri, st>>>(N, rchk, b, a.ws, ncb, W, W, sRi, partKq, need3, Qp);
     CSS_LAUNCHED(ctx);
-    CSS_TRY(reduce(partKq, sG));
-    CSS_TRY(chol(1, j, sR1, sR1i, 0.0, need3));
-    k_tri<T, BP, true><<<rgrid, th1, sm_tri, st>>>(N, rchk, b, a.ws, ncb, W, W, sR1i, partKq, need3, Qp);
-    CSS_LAUNCHED(ctx);
-    CSS_TRY(reduce(partKq, sG));
-    CSS_TRY(chol(2, j, sR2, sR2i, 0.0, need3));
+    CSS_TRY(chol(2, j, sRi, need3, false));
     // Q_{j+1} = W R2^-1 overwrites Q_{j-1} (done by the second pass when two passes sufficed)
-    k_tri<T, BP, false><<<rgrid, th1, sm_tri, st>>>(N, rchk, b, a.ws, ncb, W, Qp, sR2i, nullptr, need3, nullptr);
+    k_tri<T, BP, false><<<rgrid, th1, sm_tri, st>>>(N, rchk, b, a.ws, ncb, W, Qp, sRi, nullptr, need3, nullptr);
     CSS_LAUNCHED(ctx);
     CSS_TRY(sampled(Qp, j + 1));
     CSS_TRY(project_u(Qp, j + 1));
-    // B_{j} for the next step's three-term update, in the batch's local layout
-    CSS_CU(ctx, cudaMemcpy2DAsync(a.Bblk_prev + (size_t)a.cb0 * bb, bb * sizeof(double),
-                                  a.Bblk + ((size_t)a.cb0 * m + j) * bb, (size_t)m * bb * sizeof(double),
-                                  bb * sizeof(double), ncb, cudaMemcpyDeviceToDevice, st));
     T* t = Qp;
     Qp = Qc;
     Qc = t;
@@ -1551,9 +1527,9 @@ size_t css_lanczos_part_doubles(int64_t N, int32_t b, int32_t ncb) {
   return (size_t)nch * ncb * b * b * 2 + (size_t)nch * ncb + 64;
 }
 
-// twelve per-colour b x b matrices, the breakdown scales and the colours' CholeskyQR flags
+// seven per-colour b x b matrices, the breakdown scales and the colours' CholeskyQR flags
 size_t css_lanczos_small_doubles(int32_t b, int32_t ncb) {
-  return (size_t)ncb * b * b * 12 + ncb + (ncb + 1) / 2 + 64;
+  return (size_t)ncb * b * b * 7 + ncb + (ncb + 1) / 2 + 64;
 }
 
 int32_t css_spmm_bm(int32_t b) { return b <= 8 ? 8 : b <= 12 ? 12 : b <= 16 ? 16 : b <= 24 ? 24 : 32; }
