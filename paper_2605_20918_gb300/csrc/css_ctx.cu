@@ -95,8 +95,6 @@ css_status css_create(css_ctx** out, int device) {
   ctx->test_spmm_empty_extra = eextra > 0 && eextra < 4 ? eextra : 0;
   const char* tc = getenv("CSS_HV_TC");
   ctx->hv_tc = tc && tc[0] == '1';
-  const char* rs = getenv("CSS_ROWS_STREAM");
-  ctx->rows_stream = rs && rs[0] == '1';
   const char* gr = getenv("CSS_GRAPH");
   ctx->graph = gr && gr[0] == '0' ? 0 : (gr && gr[0] == '1' ? 1 : -1);
   *out = ctx;

@@ -598,6 +598,11 @@ css_status ws_get(css_ctx* ctx, const char* name, size_t count, Tp** p) {
   return css_ws(ctx, name, count * sizeof(Tp), (void**)p);
 }
 
+css_status rows_timeout(css_ctx* ctx) {
+  ctx->last_error = "block-Lanczos: a bounded wait on the row passes' ring of tiles timed out";
+  return CSS_ERR_TIMEOUT;
+}
+
 struct Timer {
   css_ctx* ctx;
   cudaStream_t st;
@@ -915,6 +920,7 @@ css_status css_density_impl(css_ctx* ctx, int32_t n_sys, const css_sys_desc* sys
   la.done = done;
   la.part = part;
   la.small = small;
+  la.err = misc + 12;
   la.tau = f32 ? 1e-5 : 1e-10;
   la.shift_rel = f32 ? 1e-5 : 1e-12;
   // FP32 Krylov vectors lose local orthogonality at the FP32 level, which biases the trace of
@@ -1144,6 +1150,7 @@ css_status css_density_impl(css_ctx* ctx, int32_t n_sys, const css_sys_desc* sys
     int32_t* hm;
     CSS_TRY(css_pinned(ctx, 64 * sizeof(int32_t), (void**)&hm));
     CSS_CU(ctx, cudaMemcpyAsync(hm, misc + 16, 2 * sizeof(int32_t), cudaMemcpyDeviceToHost, st));
+    CSS_CU(ctx, cudaMemcpyAsync(hm + 2, misc + 12, sizeof(int32_t), cudaMemcpyDeviceToHost, st));
     CSS_CU(ctx, cudaStreamSynchronize(st));
     ctx->last_lam = ea.lam;
     ctx->last_wgt = ea.wgt;
@@ -1156,14 +1163,15 @@ css_status css_density_impl(css_ctx* ctx, int32_t n_sys, const css_sys_desc* sys
     ctx->last_m = m;
     ctx->info.n_colours = n_col;
     ctx->info.n_breakdown = hm[0];
-    const int32_t st_bits = hm[1];
+    const int32_t st_bits = hm[1], rows_err = hm[2], broken = hm[0];
     if (use_tc) CSS_TRY(css_hv_tc_check(ctx, st));
     if (use_dup || use_split) CSS_TRY(css_spmm_dup_check(ctx, st));
+    if (rows_err) return rows_timeout(ctx);
     if (st_bits & 2) {
       ctx->last_error = "css_density: a wait between pipelined band-reduction sweeps timed out";
       return CSS_ERR_TIMEOUT;
     }
-    return hm[0] > 0 ? CSS_WARN_BREAKDOWN : CSS_OK;
+    return broken > 0 ? CSS_WARN_BREAKDOWN : CSS_OK;
   }
   double *dmu, *dkT, *dhalf, *dmu_in, *dtol, *mupart;
   int32_t* dsolve;
@@ -1292,7 +1300,7 @@ css_status css_density_impl(css_ctx* ctx, int32_t n_sys, const css_sys_desc* sys
   CSS_CU(ctx, cudaStreamSynchronize(st));
   const int32_t* hmisc = (const int32_t*)(hres + 3 * n_sys);
   const int32_t mu_err = hmisc[0];
-  const int32_t n_break = hmisc[8];
+  const int32_t n_break = hmisc[8], rows_err = hmisc[4], st_bits = hmisc[9];
   bool finite = true;
   for (int32_t s = 0; s < n_sys; ++s) {
     if (trP) trP[s] = hres[2 * s];
@@ -1330,11 +1338,12 @@ css_status css_density_impl(css_ctx* ctx, int32_t n_sys, const css_sys_desc* sys
   }
   if (use_tc) CSS_TRY(css_hv_tc_check(ctx, st));
   if (use_dup || use_split) CSS_TRY(css_spmm_dup_check(ctx, st));
+  if (rows_err) return rows_timeout(ctx);
   if (mu_err) {
     ctx->last_error = "css_density: grid barrier of the mu bisection timed out";
     return CSS_ERR_TIMEOUT;
   }
-  if (hmisc[9] & 2) {
+  if (st_bits & 2) {
     ctx->last_error = "css_density: a wait between pipelined band-reduction sweeps timed out";
     return CSS_ERR_TIMEOUT;
   }
@@ -1971,6 +1980,7 @@ css_status css_density_nonorth(css_ctx* ctx, const css_bsr* S, const double* Sin
   la.done = done;
   la.part = part;
   la.small = small;
+  la.err = misc + 12;
   la.tau = f32 ? 1e-5 : 1e-10;
   la.shift_rel = f32 ? 1e-5 : 1e-12;
   la.flags = f32 ? (flags | CSS_REORTH_LOCAL) : flags;
@@ -2135,6 +2145,7 @@ css_status css_density_nonorth(css_ctx* ctx, const css_bsr* S, const double* Sin
   ctx->info.n_colours = nc;
   ctx->info.n_breakdown = hm[16];
   ctx->info.m = m;
+  if (hm[12]) return rows_timeout(ctx);
   if (hm[8]) {
     ctx->last_error = "css_density_nonorth: grid barrier of the mu bisection timed out";
     return CSS_ERR_TIMEOUT;

@@ -74,9 +74,6 @@ struct css_ctx {
   // FP32 H * V on the tensor cores where the block width allows it (env CSS_HV_TC=1 at
   // css_create; the default is the CUDA-core kernel)
   bool hv_tc = false;
-  // env CSS_ROWS_STREAM=1 at css_create: the streaming FP32 row passes of css_rows.cu (11
-  // passes per step) instead of the tiled row kernels (14 passes, faster as measured)
-  bool rows_stream = false;
   // side streams (and their fork / join events) on which the per-system block-Lanczos passes
   // of a batch run concurrently; created on first use, destroyed with the context
   std::vector<cudaStream_t> side;

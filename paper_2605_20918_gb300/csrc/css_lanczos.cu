@@ -1302,11 +1302,10 @@ css_status run_pass_bp(css_ctx* ctx, const LzArgs& a_in, cudaStream_t st) {
   const int32_t G = colours_per_cta<T, BP>(b);
   const int32_t ngr = (int32_t)css_ceil_div(ncb, G);
   const bool reorth = (a.flags & CSS_REORTH_LOCAL) != 0;
-  // FP32, 16 < b <= 24, env CSS_ROWS_STREAM=1: the streaming row passes of css_rows.cu (their
-  // partials come in chunks of their own)
-  const bool rp = sizeof(T) == 4 && BP == 24 && css_rowpass_supported(true, b) && ctx->rows_stream;
-  const int32_t rchk = rp ? RCHK_MAX : row_chunk<T, BP>(N, b);
-  const int32_t nch = (int32_t)css_ceil_div(N, rchk);
+  // FP32 with b = 6: the row passes of css_rows.cu, with Gram partials in chunks of their own
+  const bool rows = sizeof(T) == 4 && reorth && css_rows_supported(true, b);
+  const int32_t rchk = row_chunk<T, BP>(N, b);
+  const int32_t nch = (int32_t)css_ceil_div(N, rchk), nch_r = rows ? (int32_t)css_ceil_div(N, css_rows_chunk(N, b)) : 0;
   T* Qp = (T*)a.Q0;
   T* Qc = (T*)a.Q1;
   T* W = (T*)a.W;
@@ -1320,28 +1319,26 @@ css_status run_pass_bp(css_ctx* ctx, const LzArgs& a_in, cudaStream_t st) {
   const size_t sm_tri = (NS1 + (NS1 == 2 ? 1 : 2)) * RTL1 * pitch_bytes + mat;
   const int th3 = row_threads<T, BP, RTL3>(b), th1 = row_threads<T, BP, RTL1>(b);
   double* partKq = a.part;
-  double* partKp = a.part + (size_t)nch * ncb * bb;
+  double* partKp = a.part + (size_t)std::max(nch, nch_r) * ncb * bb;
   double* sA = a.small;                        // [ncb][bb] Q_j^T W0
   double* sKp = sA + (size_t)ncb * bb;         // Q_{j-1}^T W0
   double* sRi = sKp + (size_t)ncb * bb;        // R^-1 of the running CholeskyQR pass
   double* sC1 = sRi + (size_t)ncb * bb;        // product of the factors so far
-  double* sRi10 = sC1 + (size_t)ncb * bb;      // R0^-1 R1^-1, R0^-1 R1^-1 R2^-1 and a copy of R0^-1
-  double* sRi210 = sRi10 + (size_t)ncb * bb;   // (streaming row passes)
-  double* sRi0 = sRi210 + (size_t)ncb * bb;
+  double* sRi0 = sC1 + (size_t)ncb * bb;       // R0^-1 (row passes of css_rows.cu)
   double* sH = sRi0 + (size_t)ncb * bb;        // [ncb] ||H Q_j||_F^2
   // per colour: "a third CholeskyQR pass is needed" in the running step (after the matrices)
   int32_t* need3 = reinterpret_cast<int32_t*>(sH + ncb);
   const int gth = gram_threads(b);
-  // A_j (and Q_{j-1}^T W0) from the partials of S1
-  auto gram_A = [&](int32_t j, bool both, double* Ablk) -> css_status {
-    k_gram_A<<<dim3((unsigned)ncb, both ? 2 : 1), gth, 0, st>>>(nch, ncb, b, a.cb0, m, j, partKq, partKp, sA, Ablk, sKp);
+  // A_j (and Q_{j-1}^T W0) from the n partials of S1
+  auto gram_A = [&](int32_t n, int32_t j, bool both, double* Ablk) -> css_status {
+    k_gram_A<<<dim3((unsigned)ncb, both ? 2 : 1), gth, 0, st>>>(n, ncb, b, a.cb0, m, j, partKq, partKp, sA, Ablk, sKp);
     CSS_LAUNCHED(ctx);
     return CSS_OK;
   };
   // a CholeskyQR pass's factor from the Gram partials: B_j of step j, or (start) B_0 of the start block
-  auto chol = [&](int mode, int32_t j, double* Ri, int32_t* n3, bool start) -> css_status {
+  auto chol = [&](int32_t n, int mode, int32_t j, double* Ri, int32_t* n3, bool start) -> css_status {
     auto kern = mode == 0 ? k_gram_chol<0> : mode == 1 ? k_gram_chol<1> : k_gram_chol<2>;
-    kern<<<(unsigned)ncb, gth, 0, st>>>(nch, ncb, b, a.cb0, start ? 1 : m, start ? 0 : j, partKq, start ? nullptr : sA,
+    kern<<<(unsigned)ncb, gth, 0, st>>>(n, ncb, b, a.cb0, start ? 1 : m, start ? 0 : j, partKq, start ? nullptr : sA,
                                         start ? nullptr : a.Bblk_prev, a.tau, a.shift_rel, sH, Ri, sC1,
                                         start ? a.B0 : a.Bblk, a.done, a.nblk, n3);
     CSS_LAUNCHED(ctx);
@@ -1367,7 +1364,7 @@ css_status run_pass_bp(css_ctx* ctx, const LzArgs& a_in, cudaStream_t st) {
     for (int mode = 0; mode < 3; ++mode) {
       k_tri<T, BP, true><<<rgrid, th1, sm_tri, st>>>(N, rchk, b, a.ws, ncb, in, W, sRi, partKq, nullptr, nullptr);
       CSS_LAUNCHED(ctx);
-      CSS_TRY(chol(mode, 0, sRi, nullptr, true));
+      CSS_TRY(chol(nch, mode, 0, sRi, nullptr, true));
       in = W;
     }
     k_tri<T, BP, false><<<rgrid, th1, sm_tri, st>>>(N, rchk, b, a.ws, ncb, W, Qc, sRi, nullptr, nullptr, nullptr);
@@ -1421,55 +1418,62 @@ css_status run_pass_bp(css_ctx* ctx, const LzArgs& a_in, cudaStream_t st) {
     if (a.ev_spmm) CSS_CU(ctx, cudaEventRecordWithFlags(a.ev_spmm[2 * j], st, ev_flags));
     CSS_TRY(launch_spmm<T>(ctx, a, Qc, W, st));
     if (a.ev_spmm) CSS_CU(ctx, cudaEventRecordWithFlags(a.ev_spmm[2 * j + 1], st, ev_flags));
-    if (rp) {
-      const int first = j == 0 ? 1 : 0, ro = reorth ? 1 : 0;
-      const float *q = (const float*)Qc, *qp = (const float*)Qp;
-      float* wv = (float*)W;
-      // Kq = Q_j^T W0, Kp = Q_{j-1}^T W0 with W0 = W - Q_{j-1} B_{j-1}^T
-      CSS_TRY(css_rowpass(ctx, 0, N, b, a.ws, ncb, a.cb0, first, ro, q, qp, wv, nullptr, a.Bblk_prev, nullptr, nullptr,
-                          partKq, partKp, st));
-      CSS_TRY(gram_A(j, reorth && !first, a.Ablk));
+    if (rows) {
+      CssRows r;
+      r.N = N;
+      r.b = b;
+      r.ws = a.ws;
+      r.ncb = ncb;
+      r.cb0 = a.cb0;
+      r.first = j == 0;
+      r.Q = (const float*)Qc;
+      r.Qp = (const float*)Qp;
+      r.W = (const float*)W;
+      r.Bprev = a.Bblk_prev;
+      r.part1 = partKq;
+      r.part2 = partKp;
+      r.need3 = need3;
+      r.err = a.err;
+      CSS_TRY(css_rows(ctx, 0, r, st));
+      CSS_TRY(gram_A(nch_r, j, j > 0, a.Ablk));
       if (j + 1 == m) break;
-      // W1 = W - Q_j Kq - Q_{j-1} (B_{j-1}^T + Kp) over W, and its Gram
-      CSS_TRY(css_rowpass(ctx, 1, N, b, a.ws, ncb, a.cb0, first, ro, q, qp, wv, wv, sA, a.Bblk_prev,
-                          (reorth && !first) ? sKp : nullptr, partKq, nullptr, st));
-      // shifted CholeskyQR3 on W1 without storing the intermediates: the Grams of W1 R0^-1 and
-      // W1 R0^-1 R1^-1 are taken from W1 itself, and Q_{j+1} = W1 R0^-1 R1^-1 R2^-1
-      CSS_TRY(chol(0, j, sRi0, nullptr, false));
-      CSS_TRY(css_rowpass(ctx, 2, N, b, a.ws, ncb, a.cb0, first, ro, nullptr, nullptr, wv, nullptr, sRi0, nullptr,
-                          nullptr, partKq, nullptr, st));
-      CSS_TRY(chol(1, j, sRi, nullptr, false));
-      CSS_TRY(css_small_mm(ctx, ncb, b, sRi0, sRi, sRi10, st));
-      CSS_TRY(css_rowpass(ctx, 2, N, b, a.ws, ncb, a.cb0, first, ro, nullptr, nullptr, wv, nullptr, sRi10, nullptr,
-                          nullptr, partKq, nullptr, st));
-      CSS_TRY(chol(2, j, sRi, nullptr, false));
-      CSS_TRY(css_small_mm(ctx, ncb, b, sRi10, sRi, sRi210, st));
-      CSS_TRY(css_rowpass(ctx, 3, N, b, a.ws, ncb, a.cb0, first, ro, nullptr, nullptr, wv, (float*)Qp, sRi210, nullptr,
-                          nullptr, nullptr, nullptr, st));
+      r.M1 = sA;
+      r.M2 = sKp;
+      r.out = (float*)W;
+      CSS_TRY(css_rows(ctx, 1, r, st));
+      CSS_TRY(chol(nch_r, 0, j, sRi0, nullptr, false));
+      r.M1 = sRi0;
+      CSS_TRY(css_rows(ctx, 2, r, st));
+      CSS_TRY(chol(nch_r, 1, j, sRi, need3, false));
+      r.M2 = sRi;
+      r.out = (float*)Qp;
+      r.out2 = (float*)W;
+      CSS_TRY(css_rows(ctx, 3, r, st));
+      CSS_TRY(chol(nch_r, 2, j, sRi, need3, false));
+      r.M1 = sRi;
+      CSS_TRY(css_rows(ctx, 4, r, st));
       CSS_TRY(sampled(Qp, j + 1));
       CSS_TRY(project_u(Qp, j + 1));
-      T* t = Qp;
-      Qp = Qc;
-      Qc = t;
+      std::swap(Qp, Qc);
       continue;
     }
     // three-term update and the projections onto Q_j (and Q_{j-1})
     s1<<<rgrid, reorth ? 2 * RW : RW, sm_s1, st>>>(N, rchk, b, a.ws, ncb, a.cb0, Qp, Qc, W, a.Bblk_prev, j == 0 ? 1 : 0,
                                                    partKq, partKp);
     CSS_LAUNCHED(ctx);
-    CSS_TRY(gram_A(j, reorth, a.Ablk));
+    CSS_TRY(gram_A(nch, j, reorth, a.Ablk));
     if (j + 1 == m) break;
     // W1 = W0 - Q_j Kq (- Q_{j-1} Kp) and its Gram
     s3<<<rgrid, th3, sm_s3, st>>>(N, rchk, b, a.ws, ncb, Qc, Qp, W, sA, sKp, partKq);
     CSS_LAUNCHED(ctx);
     // shifted CholeskyQR3 of W: R0 from G + sI, then one or two plain CholeskyQR passes (k_gram_chol)
-    CSS_TRY(chol(0, j, sRi, nullptr, false));
+    CSS_TRY(chol(nch, 0, j, sRi, nullptr, false));
     k_tri<T, BP, true><<<rgrid, th1, sm_tri, st>>>(N, rchk, b, a.ws, ncb, W, W, sRi, partKq, nullptr, nullptr);
     CSS_LAUNCHED(ctx);
-    CSS_TRY(chol(1, j, sRi, need3, false));
+    CSS_TRY(chol(nch, 1, j, sRi, need3, false));
     k_tri<T, BP, true><<<rgrid, th1, sm_tri, st>>>(N, rchk, b, a.ws, ncb, W, W, sRi, partKq, need3, Qp);
     CSS_LAUNCHED(ctx);
-    CSS_TRY(chol(2, j, sRi, need3, false));
+    CSS_TRY(chol(nch, 2, j, sRi, need3, false));
     // Q_{j+1} = W R2^-1 overwrites Q_{j-1} (done by the second pass when two passes sufficed)
     k_tri<T, BP, false><<<rgrid, th1, sm_tri, st>>>(N, rchk, b, a.ws, ncb, W, Qp, sRi, nullptr, need3, nullptr);
     CSS_LAUNCHED(ctx);
@@ -1523,13 +1527,14 @@ int32_t min_chunk(int64_t N, int32_t b) {
 size_t css_lanczos_part_doubles(int64_t N, int32_t b, int32_t ncb) {
   const int32_t chunk = b <= 8 ? min_chunk<8>(N, b) : b <= 16 ? min_chunk<16>(N, b) : b <= 24 ? min_chunk<24>(N, b)
                                                                                               : min_chunk<32>(N, b);
-  const int64_t nch = css_ceil_div(N, chunk);
+  int64_t nch = css_ceil_div(N, chunk);
+  if (css_rows_supported(true, b)) nch = std::max(nch, css_ceil_div(N, css_rows_chunk(N, b)));
   return (size_t)nch * ncb * b * b * 2 + (size_t)nch * ncb + 64;
 }
 
-// seven per-colour b x b matrices, the breakdown scales and the colours' CholeskyQR flags
+// five per-colour b x b matrices, the breakdown scales and the colours' CholeskyQR flags
 size_t css_lanczos_small_doubles(int32_t b, int32_t ncb) {
-  return (size_t)ncb * b * b * 7 + ncb + (ncb + 1) / 2 + 64;
+  return (size_t)ncb * b * b * 5 + ncb + (ncb + 1) / 2 + 64;
 }
 
 int32_t css_spmm_bm(int32_t b) { return b <= 8 ? 8 : b <= 12 ? 12 : b <= 16 ? 16 : b <= 24 ? 24 : 32; }

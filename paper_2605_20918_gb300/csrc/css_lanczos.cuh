@@ -26,6 +26,7 @@ struct LzArgs {
   int32_t* done = nullptr;           // [colour] recurrence stopped
   double* part = nullptr;            // per-chunk partial products
   double* small = nullptr;           // per-colour small matrices of the batch
+  int32_t* err = nullptr;            // set when a bounded wait of the row passes runs out
   double tau = 1e-10;                // breakdown threshold relative to ||H Q_j||_F
   double shift_rel = 1e-12;          // shifted-CholeskyQR shift relative to trace(W^T W)
   uint32_t flags = 0;
@@ -92,13 +93,21 @@ int css_spmm_split_variants();
 css_status css_spmm_split_prepare(css_ctx* ctx, int32_t b, int32_t nnzb, const double* H, const void** Hs,
                                   cudaStream_t st);
 css_status css_spmm_split(css_ctx* ctx, const LzArgs& a, const double* V, double* W, int variant, cudaStream_t st);
-// FP32 row passes of a Lanczos step for 16 < b <= 24 (css_rows.cu); mode 0 S1, 1 S3, 2 TRIG, 3 TRI
-bool css_rowpass_supported(bool fp32, int32_t b);
-css_status css_rowpass(css_ctx* ctx, int mode, int64_t N, int32_t b, int32_t ws, int32_t ncb, int32_t cb0, int first,
-                       int reorth, const float* Q, const float* Qp, const float* W, float* OUT, const double* M1,
-                       const double* Bprev, const double* Kp, double* part1, double* part2, cudaStream_t st);
-css_status css_small_mm(css_ctx* ctx, int32_t ncb, int32_t b, const double* A, const double* B, double* Cm,
-                        cudaStream_t st);
+// FP32 row passes of a Lanczos step with local reorthogonalisation for b = 6 (css_rows.cu); mode 0 S1,
+// 1 S3, 2 T0, 3 T1, 4 T2
+struct CssRows {
+  int64_t N = 0;
+  int32_t b = 0, ws = 0, ncb = 0, cb0 = 0, first = 0;
+  const float *Q = nullptr, *Qp = nullptr, *W = nullptr;
+  float *out = nullptr, *out2 = nullptr;
+  const double *M1 = nullptr, *M2 = nullptr, *Bprev = nullptr;
+  const int32_t* need3 = nullptr;
+  double *part1 = nullptr, *part2 = nullptr;
+  int* err = nullptr;
+};
+bool css_rows_supported(bool fp32, int32_t b);
+int32_t css_rows_chunk(int64_t N, int32_t b);  // rows per Gram partial
+css_status css_rows(css_ctx* ctx, int mode, const CssRows& p, cudaStream_t st);
 // W = M V for a BSR matrix prepared by css_spmm_prepare (a.Hval, a.Hlo_diag, a.row_ptr,
 // a.col_idx, a.n_brow, a.b) and N x a.w blocks V, W of row stride a.ws in the vector precision
 css_status css_spmm(css_ctx* ctx, const LzArgs& a, const void* V, void* W, cudaStream_t st);

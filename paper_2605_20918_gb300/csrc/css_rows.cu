@@ -1,297 +1,448 @@
-// Row passes of one FP32 block-Lanczos step for block widths 17..24 (paper: the three-term
-// recurrence and block QR of the block-Lanczos paragraph after Eq. 4).  Each pass streams the
-// N x w Krylov blocks once and applies, per colour c, a small b x b matrix and/or accumulates a
-// b x b Gram matrix:
-//   S1    W0 = W - Q_{j-1} B_{j-1}^T (not stored);  Kq = Q_j^T W0,  Kp = Q_{j-1}^T W0
-//   S3    W1 = W - Q_j Kq - Q_{j-1} (B_{j-1}^T + Kp), stored over W;  Gram W1^T W1
-//   TRIG  Gram of W1 M (M = R0^-1 or R0^-1 R1^-1 of the shifted CholeskyQR3), not stored
-//   TRI   Q_{j+1} = W1 M (M = R0^-1 R1^-1 R2^-1), stored
-// so a step reads the three N x w blocks twice and W1 three more times and writes two blocks
-// (11 passes; the CholeskyQR intermediates W1 R^-1 are recomputed, not stored).
+// Row passes of one FP32 block-Lanczos step with local reorthogonalisation, block width 6
+// (paper: the three-term recurrence and block QR of the block-Lanczos paragraph after Eq. 4).  Each
+// pass streams N x w Krylov blocks once and applies, per colour c, small b x b matrices and / or
+// accumulates b x b Gram matrices:
+//   S1  W0 = W - Q_{j-1} B_{j-1}^T (not stored);  Kq = Q_j^T W0,  Kp = Q_{j-1}^T W0
+//   S3  W1 = W0 - Q_j Kq - Q_{j-1} Kp, over W (W0 recomputed: B_{j-1}^T + Kp in one FP32 matrix would
+//       round Kp, the correction of B's own rounding, away);  Gram W1^T W1
+//   T0  V = W1 R0^-1 (not stored);  Gram V^T V
+//   T1  Q_{j+1} = (W1 R0^-1) R1^-1;  when some colour needs a third CholeskyQR pass also over W, with
+//       its Gram
+//   T2  Q_{j+1} = W R2^-1 for those colours
+// S1 and T0 store nothing: W0 and V are recomputed by the next pass, with the same FMAs, which costs
+// less than a pass over memory.  A step moves ten N x w blocks instead of twelve.
 //
-// Thread (colour c of the CTA's group, column k) holds column k of the colour's b x b matrix
-// in registers and row k of its Gram accumulator.  Rows are staged in shared memory with the
-// colour's columns padded to 24 (cp.async, a four-stage ring of 8-row sub-chunks), so a thread
-// reads the b values of a row of its colour with six 16-byte broadcast loads: four FMAs per
-// shared-memory load for the products and for the Grams.  Gram sums are taken in FP32 over 32
-// rows and added into an unevaluated hi + lo pair (TwoSum), widened to FP64 once per CTA; the
-// per-CTA partials are summed in FP64 in a fixed order (k_reduce), so every run is bitwise
-// reproducible.
+// The rows of a group of colours (a multiple of 16 bytes in every row) arrive in a ring of tiles filled
+// by two producer warps with 16-byte cp.async copies; the same warps write finished tiles back.
+// mbarriers with bounded waits connect them to the other warps.  (One bulk copy per row segment of
+// ~300 bytes instead took ~62 clocks of an SM each whatever its size, 1.3 TB/s in all.)
+#include <algorithm>
+
 #include "css_lanczos.cuh"
+#include "css_pipe.cuh"
 
 namespace {
 
-constexpr int RP_KP = 24;      // padded colour width
-constexpr int RP_RS = 8;       // rows per sub-chunk
-constexpr int RP_NST = 4;      // cp.async ring depth (sub-chunks)
-constexpr int RP_RCH = 1024;   // rows per CTA (the chunking of the Gram partials)
-constexpr int RP_GRAM_RS = 32; // rows per FP32 Gram sum before the compensated update
+using namespace css_pipe;
 
-enum { RP_S1 = 0, RP_S3 = 1, RP_TRIG = 2, RP_TRI = 3 };
+enum { R_S1 = 0, R_S3 = 1, R_T0 = 2, R_T1 = 3, R_T2 = 4 };
 
-struct RpArgs {
+struct RowsArgs {
   int64_t N;
-  int32_t b, ws, ncb, cb0, first;
-  const float* Q;   // Q_j            (S1, S3)
-  const float* Qp;  // Q_{j-1}        (S1, S3; unused when first)
-  const float* W;   // W or W1        (all)
-  float* OUT;       // S3: W1 (may be W), TRI: Q_{j+1}
-  const double* M1;     // S1: B_{j-1} [cb0 + lc] (used transposed); S3: Kq [lc]; TRIG/TRI: M [lc]
-  const double* Bprev;  // S3: B_{j-1} [cb0 + lc]
-  const double* Kp;     // S3: Kp [lc]
-  double* part1;        // Gram partials [chunk][lc][b][b]: S1 Kq, S3 / TRIG the Gram
-  double* part2;        // S1 Kp
-  int reorth;
+  int32_t rchk, ws, ncb, cb0, G, first;
+  const float* Q;        // Q_j        (S1, S3)
+  const float* Qp;       // Q_{j-1}    (S1, S3; unused when first)
+  const float* W;        // W or W1
+  float* out;            // S3: W; T1, T2: Q_{j+1}
+  float* out2;           // T1: W, when a colour of the group needs the third pass
+  const double* M1;      // S3: Kq [lc]; T0, T1: R0^-1 [lc]; T2: R2^-1 [lc]
+  const double* M2;      // S3: Kp [lc]; T1: R1^-1 [lc]
+  const double* Bprev;   // S1, S3: B_{j-1} [cb0 + lc]
+  const int32_t* need3;  // T1, T2
+  double* part1;         // Gram partials [chunk][lc][b][b]
+  double* part2;         // S1: Kp
+  int* err;
 };
 
-// arrays staged per sub-chunk: S1 Q, Qp, W; S3 Q, Qp, W; TRIG / TRI W
-// colours per CTA: 8 per thread set in S1 (two Grams, 384 threads), 10 in S3 (two matrix
-// columns and a Gram per thread need more registers: 240 threads), 16 in the single-matrix passes
-template <int MODE>
-struct RpCfg {
-  static constexpr int NSET = MODE == RP_S1 ? 2 : 1;  // S1: one thread set per Gram
-  static constexpr int CG = MODE == RP_S1 ? 8 : MODE == RP_S3 ? 10 : 16;
-  static constexpr int THREADS = NSET * CG * RP_KP;
-  static constexpr int NA = (MODE == RP_S1 || MODE == RP_S3) ? 3 : 1;
-  static constexpr int PITCH = CG * RP_KP;            // floats per staged row
-  static constexpr int STAGE = NA * RP_RS * PITCH;    // floats per stage
-  static constexpr bool GRAM = MODE != RP_TRI;
-  static constexpr size_t SMEM = sizeof(float) * ((size_t)RP_NST * STAGE + 2 * RP_RS * PITCH);
-};
+__device__ __forceinline__ unsigned long long pack2(float x, float y) {
+  unsigned long long r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(x), "f"(y));
+  return r;
+}
+__device__ __forceinline__ unsigned long long dup2(float x) { return pack2(x, x); }
+__device__ __forceinline__ float lo2(unsigned long long v) { return __uint_as_float((unsigned)v); }
+__device__ __forceinline__ float hi2(unsigned long long v) { return __uint_as_float((unsigned)(v >> 32)); }
+// two IEEE FMAs, element by element
+__device__ __forceinline__ void fma2(unsigned long long& c, unsigned long long a, unsigned long long b) {
+  asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(c) : "l"(a), "l"(b));
+}
+// hi + lo += x (Knuth's TwoSum: the error of the sum goes to lo)
+__device__ __forceinline__ void add_comp(float& hi, float& lo, float x) {
+  const float t = __fadd_rn(hi, x), z = __fsub_rn(t, hi);
+  lo = __fadd_rn(lo, __fadd_rn(__fsub_rn(hi, __fsub_rn(t, z)), __fsub_rn(x, z)));
+  hi = t;
+}
+__device__ __forceinline__ void copy16(void* dst, const void* src) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(su32(dst)), "l"(src) : "memory");
+}
+// this thread's arrival on b once all its copies so far have landed
+__device__ __forceinline__ void arrive_copies(uint64_t* b) {
+  asm volatile("cp.async.mbarrier.arrive.noinc.shared::cta.b64 [%0];" ::"r"(su32(b)) : "memory");
+}
+constexpr int kProducers = 2;  // warps
 
-__device__ __forceinline__ void cp4(float* dst, const float* src, bool valid) {
-  const unsigned d = (unsigned)__cvta_generic_to_shared(dst);
-  asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;\n" ::"r"(d), "l"(src), "r"(valid ? 4 : 0) : "memory");
-}
-__device__ __forceinline__ void cp_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
-template <int N>
-__device__ __forceinline__ void cp_wait() { asm volatile("cp.async.wait_group %0;\n" ::"n"(N) : "memory"); }
+// words of a staged row: the group's columns, rounded so that consecutive rows are an odd number of
+// 16-byte units apart (lane-per-row accesses of 16 bytes hit distinct banks)
+__host__ __device__ constexpr int row_pitch(int cols) { return 4 * (((cols + 3) / 4) | 1); }
 
-// sum_l x[l] m[l] over the 24 padded columns of a staged row (six broadcast 16-byte loads),
-// in four interleaved partial sums (short dependency chains), combined in a fixed order
-__device__ __forceinline__ float row_dot(const float* x, const float (&m)[RP_KP]) {
-  float s0 = 0.0f, s1 = 0.0f, s2 = 0.0f, s3 = 0.0f;
-#pragma unroll
-  for (int q = 0; q < RP_KP / 4; ++q) {
-    const float4 v = *reinterpret_cast<const float4*>(x + 4 * q);
-    s0 = fmaf(v.x, m[4 * q], s0);
-    s1 = fmaf(v.y, m[4 * q + 1], s1);
-    s2 = fmaf(v.z, m[4 * q + 2], s2);
-    s3 = fmaf(v.w, m[4 * q + 3], s3);
-  }
-  return (s0 + s1) + (s2 + s3);
-}
-__device__ __forceinline__ void row_axpy(const float* y, float a, float (&g)[RP_KP]) {
-#pragma unroll
-  for (int q = 0; q < RP_KP / 4; ++q) {
-    const float4 v = *reinterpret_cast<const float4*>(y + 4 * q);
-    g[4 * q] = fmaf(a, v.x, g[4 * q]);
-    g[4 * q + 1] = fmaf(a, v.y, g[4 * q + 1]);
-    g[4 * q + 2] = fmaf(a, v.z, g[4 * q + 2]);
-    g[4 * q + 3] = fmaf(a, v.w, g[4 * q + 3]);
-  }
-}
-// Knuth's TwoSum of the FP32 chunk sums into (hi, lo)
-__device__ __forceinline__ void gram_flush(float (&g)[RP_KP], float (&hi)[RP_KP], float (&lo)[RP_KP]) {
-#pragma unroll
-  for (int l = 0; l < RP_KP; ++l) {
-    const float x = g[l];
-    const float t = __fadd_rn(hi[l], x);
-    const float z = __fsub_rn(t, hi[l]);
-    lo[l] = __fadd_rn(lo[l], __fadd_rn(__fsub_rn(hi[l], __fsub_rn(t, z)), __fsub_rn(x, z)));
-    hi[l] = t;
-    g[l] = 0.0f;
-  }
-}
-
-template <int MODE>
-__global__ void __launch_bounds__(RpCfg<MODE>::THREADS, 1) k_rowpass(const RpArgs a) {
-  using C = RpCfg<MODE>;
-  extern __shared__ __align__(16) float rsm[];
-  float* stage = rsm;                          // [NST][NA][RS][PITCH]
-  float* sO = rsm + (size_t)RP_NST * C::STAGE;  // [2][RS][PITCH]
-  const int tid = threadIdx.x;
-  const int set = tid / (C::CG * RP_KP), t2 = tid - set * (C::CG * RP_KP);
-  const int cl = t2 / RP_KP, k = t2 - cl * RP_KP;
-  const int32_t lc = blockIdx.y * C::CG + cl;
-  const bool valid = lc < a.ncb && k < a.b;
-  const size_t col = valid ? (size_t)lc * a.b + k : 0;
-  const int soff = cl * RP_KP + k;  // this thread's element in a staged row
-  const int64_t rbeg = (int64_t)blockIdx.x * RP_RCH, rend = min(a.N, rbeg + RP_RCH);
-  const int nsub = (int)((rend - rbeg + RP_RS - 1) / RP_RS);
-  const bool first = a.first != 0;
-  // this thread's column of the colour's matrices (zero beyond b and for idle threads)
-  float m1[RP_KP], m2[RP_KP];
-#pragma unroll
-  for (int l = 0; l < RP_KP; ++l) {
-    float x = 0.0f, y = 0.0f;
-    if (valid && l < a.b) {
-      const size_t bb = (size_t)a.b * a.b;
-      if (MODE == RP_S1) {
-        x = first ? 0.0f : (float)a.M1[(size_t)(a.cb0 + lc) * bb + (size_t)k * a.b + l];  // B^T[l][k]
-      } else if (MODE == RP_S3) {
-        x = (float)a.M1[(size_t)lc * bb + (size_t)l * a.b + k];
-        if (!first)
-          y = (float)(a.Bprev[(size_t)(a.cb0 + lc) * bb + (size_t)k * a.b + l] +
-                      (a.Kp ? a.Kp[(size_t)lc * bb + (size_t)l * a.b + k] : 0.0));
-      } else {
-        x = (float)a.M1[(size_t)lc * bb + (size_t)l * a.b + k];
-      }
+// A CTA's tiles: ns stages of NA arrays of R rows, "full" barriers (the producers' copies) and "done"
+// barriers (the consumers' arrivals).
+template <int NA, int R>
+struct Ring {
+  float* base;
+  uint64_t *full, *done;
+  volatile int* abort;
+  int* err;
+  int32_t ns, pitch, ntile;
+  int64_t r0, rend;
+  __device__ __forceinline__ float* stage(int32_t t) const { return base + (size_t)(t % ns) * NA * R * pitch; }
+  __device__ __forceinline__ int32_t rows(int32_t t) const { return (int32_t)min((int64_t)R, rend - r0 - (int64_t)t * R); }
+  __device__ __forceinline__ bool wait_full(int32_t t) const { return bar_wait(&full[t % ns], (t / ns) & 1, abort, err); }
+  __device__ __forceinline__ void arrive(int32_t t) const { bar_arrive(&done[t % ns]); }
+  __device__ __forceinline__ void init(int32_t consumers) const {  // one thread
+    for (int s = 0; s < ns; ++s) {
+      bar_init(&full[s], 32 * kProducers);
+      bar_init(&done[s], consumers);
     }
-    m1[l] = x;
-    m2[l] = y;
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
-  float g[RP_KP], hi[RP_KP], lo[RP_KP];
-#pragma unroll
-  for (int l = 0; l < RP_KP; ++l) g[l] = hi[l] = lo[l] = 0.0f;
-
-  // each thread copies its own element of every staged row (rows past the end: zero)
-  auto issue = [&](int sc) {
-    if (sc < nsub) {
-      float* st = stage + (size_t)(sc % RP_NST) * C::STAGE;
-      const int64_t r0 = rbeg + (int64_t)sc * RP_RS;
-      const float* src[3] = {C::NA == 3 ? a.Q : a.W, a.Qp, a.W};
-#pragma unroll
-      for (int ar = 0; ar < C::NA; ++ar) {
-        const bool need = !(ar == 1 && first) && set == 0;  // one copy per element (set 0)
-#pragma unroll
-        for (int r = 0; r < RP_RS; ++r) {
-          const bool in = valid && need && r0 + r < rend;
-          float* d = st + ((size_t)ar * RP_RS + r) * C::PITCH + soff;
-          if (set == 0) cp4(d, src[ar] + (size_t)(in ? r0 + r : 0) * a.ws + col, in);
+  // producer warp pw: its part of every tile as the stages become free and, with OUT, of the stores of
+  // the tile's array 0 to out (and out2) once the consumers are done with it.  cpr: 16-byte chunks of a
+  // row's columns, which start at col0
+  template <bool OUT>
+  __device__ void produce(int pw, const float* const* src, int na, float* out, float* out2, int32_t ws, int32_t col0,
+                          int32_t cpr) const {
+    // a thread keeps its chunk of the row and walks down the rows, rp at a time, so that a copy is two
+    // pointer steps (dividing a running index took ~110 clocks of the warp per copy)
+    const int tid = pw * 32 + (threadIdx.x & 31), rp = 32 * kProducers / cpr;
+    const int32_t rb = tid / cpr, c = tid - rb * cpr;
+    const bool mine = rb < rp;
+    const size_t go = (size_t)rb * ws + col0 + 4 * c, gs = (size_t)rp * ws;
+    const int32_t so = rb * pitch + 4 * c, ss = rp * pitch;
+    auto load = [&](int32_t t) {
+      float* st = stage(t) + so;
+      const size_t g = (size_t)(r0 + (int64_t)t * R) * ws + go;
+      const int32_t nr = mine ? rows(t) : 0;
+      for (int a = 0; a < na; ++a) {
+        const float* s = src[a] + g;
+        float* d = st + (size_t)a * R * pitch;
+#pragma unroll 4
+        for (int32_t r = rb; r < nr; r += rp, s += gs, d += ss) copy16(d, s);
+      }
+      arrive_copies(&full[t % ns]);
+    };
+    for (int32_t t = 0; t < ns && t < ntile; ++t) load(t);
+    for (int32_t t = 0; t < ntile; ++t) {
+      if (!OUT && t + ns >= ntile) break;
+      const bool ok = bar_wait(&done[t % ns], (t / ns) & 1, abort, err);
+      if (!__all_sync(0xffffffffu, ok)) break;
+      if (OUT) {
+        const float* d = stage(t) + so;
+        float* o = out + ((size_t)(r0 + (int64_t)t * R) * ws + go);
+        const ptrdiff_t o2 = out2 ? out2 - out : 0;
+        const int32_t nr = mine ? rows(t) : 0;
+#pragma unroll 4
+        for (int32_t r = rb; r < nr; r += rp, o += gs, d += ss) {
+          const float4 v = *reinterpret_cast<const float4*>(d);
+          *reinterpret_cast<float4*>(o) = v;
+          if (o2) *reinterpret_cast<float4*>(o + o2) = v;
         }
       }
+      if (t + ns < ntile) load(t + ns);  // each thread refills the chunks that it stored
     }
-    cp_commit();
-  };
-  for (int s = 0; s < RP_NST - 1; ++s) issue(s);
-
-  for (int sc = 0; sc < nsub; ++sc) {
-    cp_wait<RP_NST - 2>();
-    __syncthreads();  // sub-chunk sc is staged; every thread is done with sub-chunk sc - 1
-    issue(sc + RP_NST - 1);
-    const float* st = stage + (size_t)(sc % RP_NST) * C::STAGE;
-    float* so = sO + (size_t)(sc & 1) * RP_RS * C::PITCH;
-    const int64_t r0 = rbeg + (int64_t)sc * RP_RS;
-    const float* rowbase = st + cl * RP_KP;
-    if (MODE == RP_S1) {
-      // W0 = W - Q_{j-1} B^T: each thread set takes half of the rows
-      constexpr int H = RP_RS / C::NSET;
-#pragma unroll
-      for (int rr = 0; rr < H; ++rr) {
-        const int r = set * H + rr;
-        float o = st[((size_t)2 * RP_RS + r) * C::PITCH + soff];
-        if (!first) o = o - row_dot(rowbase + ((size_t)RP_RS + r) * C::PITCH, m1);
-        so[r * C::PITCH + soff] = o;
-      }
-    } else if (MODE == RP_S3) {
-#pragma unroll
-      for (int r = 0; r < RP_RS; ++r) {
-        float o = st[((size_t)2 * RP_RS + r) * C::PITCH + soff] - row_dot(rowbase + (size_t)r * C::PITCH, m1);
-        if (!first) o = o - row_dot(rowbase + ((size_t)RP_RS + r) * C::PITCH, m2);
-        so[r * C::PITCH + soff] = o;
-        if (valid && r0 + r < rend) a.OUT[(size_t)(r0 + r) * a.ws + col] = o;
-      }
-    } else {
-#pragma unroll
-      for (int r = 0; r < RP_RS; ++r) {
-        const float o = row_dot(rowbase + (size_t)r * C::PITCH, m1);
-        if (MODE == RP_TRIG) so[r * C::PITCH + soff] = o;
-        if (MODE == RP_TRI && valid && r0 + r < rend) a.OUT[(size_t)(r0 + r) * a.ws + col] = o;
-      }
-    }
-    if (C::GRAM) {
-      __syncthreads();  // the products of this sub-chunk are in sO
-      // S1: Gram row k of Q_j^T W0 (set 0) or Q_{j-1}^T W0 (set 1); S3 / TRIG: of W1^T W1
-      const bool active = MODE != RP_S1 || set == 0 || (a.reorth && !first);
-#pragma unroll
-      for (int r = 0; r < RP_RS; ++r) {
-        float x;
-        if (MODE == RP_S1) x = st[((size_t)(set == 0 ? 0 : 1) * RP_RS + r) * C::PITCH + soff];
-        else x = so[r * C::PITCH + soff];
-        if (active) row_axpy(so + r * C::PITCH + cl * RP_KP, x, g);
-      }
-      if (((sc + 1) * RP_RS) % RP_GRAM_RS == 0 || sc + 1 == nsub) gram_flush(g, hi, lo);
-    }
+    asm volatile("cp.async.wait_all;" ::: "memory");
   }
-  cp_wait<0>();
-  if (C::GRAM && valid) {
-    double* part = (MODE == RP_S1 && set == 1) ? a.part2 : a.part1;
-    if (MODE != RP_S1 || set == 0 || (a.reorth && !first)) {
-      double* o = part + (((size_t)blockIdx.x * a.ncb + lc) * a.b + k) * a.b;
+};
+
+// ------------------------------------------------------------------------- b = 6
+// One warp per colour, two rows of a tile per lane: the matrices of the colour and its Gram accumulators live in
+// registers and a row's six values are three 8-byte shared loads, so 32 rows of a colour cost a warp
+// ~100 packed FMAs and 9 shared loads in S1.  A lane sums 32 rows in FP32, then the 32 lanes' sums are
+// added into one hi + lo pair per entry with TwoSum, widened to FP64 once per CTA.  The general tiled
+// kernels (css_lanczos.cu) moved each value through 4-byte copies, staged tiles and barriers: row work
+// of a step 5.33 -> 1.91 ms at 60,000 molecules (S1 339 us, S3 463, T0 125, T1 249: 4.6-5.0 TB/s of what
+// each must move), 0.40 -> 0.145 at 4,001, 0.144 -> 0.067 at 512.  What it took: two rows per lane (one
+// row left the waits and shared-memory latency of a tile exposed: 2.36 ms), ten colours so that a lane
+// has 168 registers (twelve spilled in S1 and S3: 2.22 ms).
+constexpr int B6_R = 64;      // rows per tile, two per lane
+constexpr int B6_GMAX = 10;   // colours (warps) per CTA, an even number: 16-byte columns
+template <int MODE>
+struct B6Cfg {
+  static constexpr int NA = MODE <= R_S3 ? 3 : 1;
+  static constexpr int NS = MODE <= R_S3 ? 4 : 8;
+  static size_t smem(int G) {
+    return (size_t)NS * NA * B6_R * row_pitch(6 * G) * 4 + (size_t)G * 18 * 33 * 4 + (2 * NS + 2) * 8;
+  }
+};
+
+// index of the pair {(k, 2 i), (k, 2 i + 1)} of a symmetric 6 x 6 matrix kept for 2 i + 1 >= k
+__host__ __device__ constexpr int sym_pair(int k, int i) {
+  return (k >> 1 == 0 ? 3 * k : k >> 1 == 1 ? 6 + 2 * (k - 2) : 10 + (k - 4)) + i - (k >> 1);
+}
+
+template <int MODE>
+__global__ void __launch_bounds__(32 * (B6_GMAX + kProducers), 1) k_rows6(const RowsArgs a) {
+  using C = B6Cfg<MODE>;
+  constexpr int NA = C::NA, NS = C::NS, R = B6_R;
+  constexpr bool OUT = MODE == R_S3 || MODE == R_T1 || MODE == R_T2;
+  constexpr bool SYM = MODE != R_S1;
+  extern __shared__ __align__(128) unsigned char rows_smem[];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int32_t g0 = blockIdx.y * a.G, gcount = min(a.G, a.ncb - g0);
+  Ring<NA, R> ring;
+  ring.full = reinterpret_cast<uint64_t*>(rows_smem);
+  ring.done = ring.full + NS;
+  ring.abort = reinterpret_cast<volatile int*>(ring.done + NS);
+  ring.base = reinterpret_cast<float*>(rows_smem + (2 * NS + 2) * 8);
+  ring.err = a.err;
+  ring.ns = NS;
+  ring.pitch = row_pitch(6 * a.G);
+  ring.r0 = (int64_t)blockIdx.x * a.rchk;
+  ring.rend = min(a.N, ring.r0 + a.rchk);
+  ring.ntile = (int32_t)((ring.rend - ring.r0 + R - 1) / R);
+  bool any3 = false;
+  if (MODE >= R_T1)
+    for (int32_t g = 0; g < gcount; ++g) any3 = any3 || a.need3[g0 + g] != 0;
+  if (MODE == R_T2 && !any3) return;  // uniform over the CTA
+  if (threadIdx.x == 0) {
+    ring.init(gcount);
+    *ring.abort = *(volatile int*)a.err ? 1 : 0;
+  }
+  __syncthreads();
+  if (*ring.abort) return;
+  const int32_t lc = g0 + warp;
+  const bool use_p = MODE <= R_S3 && !a.first;
+  constexpr int NACC = MODE == R_S1 ? 36 : 12;
+  unsigned long long acc[NACC];
 #pragma unroll
-      for (int l = 0; l < RP_KP; ++l)
-        if (l < a.b) o[l] = (double)hi[l] + (double)lo[l];
+  for (int i = 0; i < NACC; ++i) acc[i] = 0ull;
+  if (warp >= a.G) {  // producers
+    const float* src[3] = {a.W, a.Q, a.Qp};
+    ring.template produce<OUT>(warp - a.G, src, MODE <= R_S3 ? (use_p ? 3 : 2) : 1, a.out,
+                               MODE == R_T1 && any3 ? a.out2 : nullptr, a.ws, g0 * 6, (gcount * 24 + 15) / 16);
+  } else if (warp < gcount) {
+    // the colour's matrices, negated where they are subtracted, as pairs over the output column
+    constexpr int NM1 = MODE == R_S1 ? 1 : MODE == R_S3 ? 18 : 12, NM2 = MODE == R_S3 ? 18 : MODE == R_T1 ? 12 : 1;
+    unsigned long long m1[NM1], m2[NM2], mb[MODE <= R_S3 ? 12 : 1];
+    const double* M1 = MODE == R_S1 ? nullptr : a.M1 + (size_t)lc * 36;
+    const double* M2 = (MODE == R_S3 || MODE == R_T1) ? a.M2 + (size_t)lc * 36 : nullptr;
+    const double* Bp = MODE <= R_S3 ? a.Bprev + (size_t)(a.cb0 + lc) * 36 : nullptr;
+    int n1 = 0, n2 = 0, nb = 0;
+#pragma unroll
+    for (int l = 0; l < 6; ++l)
+#pragma unroll
+      for (int i = 0; i < 3; ++i) {
+        const int k = 2 * i;
+        if (MODE <= R_S3 && k <= l)  // -B^T: entries (l, k) with k <= l
+          mb[nb++] = use_p ? pack2(-(float)Bp[k * 6 + l], k + 1 <= l ? -(float)Bp[(k + 1) * 6 + l] : 0.0f) : 0ull;
+        if (MODE == R_S1) continue;
+        if (MODE == R_S3) {
+          m1[n1++] = pack2(-(float)M1[l * 6 + k], -(float)M1[l * 6 + k + 1]);
+          m2[n2++] = use_p ? pack2(-(float)M2[l * 6 + k], -(float)M2[l * 6 + k + 1]) : 0ull;
+        } else if (k + 1 >= l) {  // upper triangle
+          m1[n1++] = pack2((float)M1[l * 6 + k], (float)M1[l * 6 + k + 1]);
+          if (MODE == R_T1) m2[n2++] = pack2((float)M2[l * 6 + k], (float)M2[l * 6 + k + 1]);
+        }
+      }
+    // y = x R^-1 over the upper triangle
+    auto tri = [&](const unsigned long long (&x)[3], const unsigned long long* mm, unsigned long long (&y)[3]) {
+#pragma unroll
+      for (int i = 0; i < 3; ++i) y[i] = 0ull;
+      int n = 0;
+#pragma unroll
+      for (int l = 0; l < 6; ++l) {
+        const unsigned long long xl = dup2(l & 1 ? hi2(x[l >> 1]) : lo2(x[l >> 1]));
+#pragma unroll
+        for (int i = 0; i < 3; ++i)
+          if (2 * i + 1 >= l) fma2(y[i], xl, mm[n++]);
+      }
+    };
+    const bool n3 = MODE >= R_T1 && a.need3[lc] != 0;
+    const bool gram = MODE <= R_T0 || (MODE == R_T1 && n3);
+    // the lanes' sums into the entries' hi + lo pairs, rows 3 h .. 3 h + 2 of the Gram at a time: lane e
+    // adds entry e of those 18 over all lanes
+    float* red = ring.base + (size_t)NS * NA * R * ring.pitch + (size_t)warp * 18 * 33;
+    float hi[2][2] = {}, lo[2][2] = {};
+    auto flush = [&]() {
+#pragma unroll
+      for (int g = 0; g < (MODE == R_S1 ? 2 : 1); ++g)
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+          __syncwarp();
+#pragma unroll
+          for (int k = 3 * h; k < 3 * h + 3; ++k)
+#pragma unroll
+            for (int i = 0; i < 3; ++i) {
+              if (SYM && 2 * i + 1 < k) continue;
+              unsigned long long& v = acc[(SYM ? sym_pair(k, i) : g * 18 + 3 * k + i) % NACC];
+              red[(6 * (k - 3 * h) + 2 * i) * 33 + lane] = lo2(v);
+              red[(6 * (k - 3 * h) + 2 * i + 1) * 33 + lane] = hi2(v);
+              v = 0ull;
+            }
+          __syncwarp();
+          if (lane < 18 && (!SYM || lane % 6 >= 3 * h + lane / 6)) {
+#pragma unroll 8
+            for (int i = 0; i < 32; ++i) add_comp(hi[g][h], lo[g][h], red[lane * 33 + i]);
+          }
+        }
+    };
+    const bool pad = OUT && warp + 1 == gcount && (gcount & 1);  // two columns past the last colour
+    for (int32_t t = 0; t < ring.ntile; ++t) {
+      if (!ring.wait_full(t)) break;
+      const int32_t nr = ring.rows(t);
+      float* row0 = ring.stage(t) + (size_t)lane * ring.pitch + 6 * warp;
+      unsigned long long w2[2][3], q2[2][3], p2[2][3];
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        const bool valid = lane + 32 * h < nr;
+        const float* row = row0 + h * 32 * ring.pitch;
+#pragma unroll
+        for (int i = 0; i < 3; ++i) {
+          w2[h][i] = valid ? *reinterpret_cast<const unsigned long long*>(row + 2 * i) : 0ull;
+          if (MODE <= R_S3) {
+            q2[h][i] = valid ? *reinterpret_cast<const unsigned long long*>(row + R * ring.pitch + 2 * i) : 0ull;
+            p2[h][i] = valid && use_p ? *reinterpret_cast<const unsigned long long*>(row + 2 * R * ring.pitch + 2 * i) : 0ull;
+          }
+        }
+      }
+      if (!OUT) {  // the tile is in registers: its stage is free
+        __syncwarp();
+        if (lane == 0) ring.arrive(t);
+      }
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        unsigned long long(&w)[3] = w2[h], (&q)[3] = q2[h], (&p)[3] = p2[h], o[3];
+        float* row = row0 + h * 32 * ring.pitch;
+        if (MODE <= R_S3) {  // W0 = W - Q_{j-1} B^T
+          int n = 0;
+#pragma unroll
+          for (int l = 0; l < 6; ++l) {
+            const unsigned long long x = dup2(l & 1 ? hi2(p[l >> 1]) : lo2(p[l >> 1]));
+#pragma unroll
+            for (int i = 0; i < 3; ++i)
+              if (2 * i <= l) fma2(w[i], x, mb[n++]);
+          }
+        }
+        if (MODE == R_S1) {
+#pragma unroll
+          for (int k = 0; k < 6; ++k) {
+            const unsigned long long xq = dup2(k & 1 ? hi2(q[k >> 1]) : lo2(q[k >> 1]));
+            const unsigned long long xp = dup2(k & 1 ? hi2(p[k >> 1]) : lo2(p[k >> 1]));
+#pragma unroll
+            for (int i = 0; i < 3; ++i) {
+              fma2(acc[(3 * k + i) % NACC], xq, w[i]);
+              fma2(acc[(18 + 3 * k + i) % NACC], xp, w[i]);
+            }
+          }
+        } else {
+          if (MODE == R_S3) {
+#pragma unroll
+            for (int i = 0; i < 3; ++i) o[i] = w[i];
+#pragma unroll
+            for (int l = 0; l < 6; ++l) {
+              const unsigned long long x = dup2(l & 1 ? hi2(q[l >> 1]) : lo2(q[l >> 1]));
+#pragma unroll
+              for (int i = 0; i < 3; ++i) fma2(o[i], x, m1[(3 * l + i) % NM1]);
+            }
+#pragma unroll
+            for (int l = 0; l < 6; ++l) {
+              const unsigned long long x = dup2(l & 1 ? hi2(p[l >> 1]) : lo2(p[l >> 1]));
+#pragma unroll
+              for (int i = 0; i < 3; ++i) fma2(o[i], x, m2[(3 * l + i) % NM2]);
+            }
+          } else {
+            tri(w, m1, o);
+            if (MODE == R_T1) {
+              unsigned long long v[3];
+#pragma unroll
+              for (int i = 0; i < 3; ++i) v[i] = o[i];
+              tri(v, m2, o);
+            }
+          }
+          if (OUT) {
+            if (MODE != R_T2 || n3)
+#pragma unroll
+              for (int i = 0; i < 3; ++i) *reinterpret_cast<unsigned long long*>(row + 2 * i) = o[i];
+            if (pad) *reinterpret_cast<unsigned long long*>(row + 6) = 0ull;
+            if (h == 1) {
+              __syncwarp();
+              if (lane == 0) ring.arrive(t);
+            }
+          }
+          if (gram) {
+#pragma unroll
+            for (int k = 0; k < 6; ++k) {
+              const unsigned long long x = dup2(k & 1 ? hi2(o[k >> 1]) : lo2(o[k >> 1]));
+#pragma unroll
+              for (int i = k >> 1; i < 3; ++i) fma2(acc[sym_pair(k, i) % NACC], x, o[i]);
+            }
+          }
+        }
+      }
+      if (gram && ((t & 15) == 15 || t + 1 == ring.ntile)) flush();
+    }
+    if (!gram || *ring.abort || lane >= 18) return;
+#pragma unroll
+    for (int g = 0; g < (MODE == R_S1 ? 2 : 1); ++g) {
+      double* part = (g ? a.part2 : a.part1) + ((size_t)blockIdx.x * a.ncb + lc) * 36;
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        const int k = 3 * h + lane / 6, l = lane % 6;
+        const double v = (double)hi[g][h] + (double)lo[g][h];
+        if (SYM && l < k) continue;
+        part[6 * k + l] = v;
+        if (SYM && l > k) part[6 * l + k] = v;
+      }
     }
   }
 }
 
-// C[lc] = A[lc] B[lc] for b x b FP64 matrices (products of the CholeskyQR factors' inverses)
-__global__ void k_small_mm(int32_t ncb, int32_t b, const double* __restrict__ A, const double* __restrict__ B,
-                           double* __restrict__ Cm) {
-  const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  const int64_t bb = (int64_t)b * b;
-  if (t >= (int64_t)ncb * bb) return;
-  const int64_t lc = t / bb;
-  const int32_t e = (int32_t)(t - lc * bb), i = e / b, j = e - i * b;
-  const double* a = A + lc * bb;
-  const double* bm = B + lc * bb;
-  double s = 0.0;
-  for (int32_t l = 0; l < b; ++l) s = fma(a[i * b + l], bm[l * b + j], s);
-  Cm[t] = s;
+// Rows per CTA: chunks for one to three waves of a CTA per SM over `groups` groups of colours (a full
+// count: the chunk may not depend on the colours of the call, or a colour's sums would), more waves
+// where a CTA still has `most` rows, so that its start and end (~5 us) stay small.
+int32_t pick_chunk(int64_t N, int groups, int R, int32_t most) {
+  const int64_t waves = std::min<int64_t>(3, std::max<int64_t>(1, N * groups / (152ll * most)));
+  const int64_t nch = std::max<int64_t>(1, 152 * waves / groups);
+  return (int32_t)std::max<int64_t>(css_ceil_div(css_ceil_div(N, nch), R) * R, R);
+}
+
+template <int MODE>
+css_status launch_rows6(css_ctx* ctx, RowsArgs& r, cudaStream_t st) {
+  const int32_t ngr = (int32_t)css_ceil_div(r.ncb, B6_GMAX);
+  r.G = (int32_t)css_ceil_div(css_ceil_div(r.ncb, ngr), 2) * 2;  // even groups of nearly equal size
+  const size_t sm = B6Cfg<MODE>::smem(r.G);
+  CSS_CU(ctx, cudaFuncSetAttribute(k_rows6<MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
+  const dim3 grid((unsigned)css_ceil_div(r.N, r.rchk), (unsigned)css_ceil_div(r.ncb, r.G));
+  k_rows6<MODE><<<grid, 32 * (r.G + kProducers), sm, st>>>(r);
+  CSS_LAUNCHED(ctx);
+  return CSS_OK;
 }
 
 }  // namespace
 
-bool css_rowpass_supported(bool fp32, int32_t b) { return fp32 && b > 16 && b <= RP_KP; }
+bool css_rows_supported(bool fp32, int32_t b) { return fp32 && b == 6; }
 
-int32_t css_rowpass_chunks(int64_t N) { return (int32_t)css_ceil_div(N, RP_RCH); }
-
-template <int MODE>
-static css_status launch_rp(css_ctx* ctx, const RpArgs& a, cudaStream_t st) {
-  using C = RpCfg<MODE>;
-  CSS_CU(ctx, cudaFuncSetAttribute(k_rowpass<MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)C::SMEM));
-  const dim3 grid((unsigned)css_ceil_div(a.N, RP_RCH), (unsigned)css_ceil_div(a.ncb, C::CG));
-  k_rowpass<MODE><<<grid, C::THREADS, C::SMEM, st>>>(a);
-  CSS_LAUNCHED(ctx);
-  return CSS_OK;
+int32_t css_rows_chunk(int64_t N, int32_t b) {
+  (void)b;
+  return pick_chunk(N, 7, B6_R, 2048);
 }
 
-// One FP32 Lanczos step after H V (W = H Q_j in a.W): the three-term update, A_j, the local
-// reorthogonalisation and the shifted CholeskyQR3 of the new block, with the small FP64 factor
-// work done by the callbacks of css_lanczos.cu.  See the header comment for the passes.
-css_status css_rowpass(css_ctx* ctx, int mode, int64_t N, int32_t b, int32_t ws, int32_t ncb, int32_t cb0, int first,
-                       int reorth, const float* Q, const float* Qp, const float* W, float* OUT, const double* M1,
-                       const double* Bprev, const double* Kp, double* part1, double* part2, cudaStream_t st) {
-  RpArgs a;
-  a.N = N;
-  a.b = b;
-  a.ws = ws;
-  a.ncb = ncb;
-  a.cb0 = cb0;
-  a.first = first;
-  a.reorth = reorth;
-  a.Q = Q;
-  a.Qp = Qp;
-  a.W = W;
-  a.OUT = OUT;
-  a.M1 = M1;
-  a.Bprev = Bprev;
-  a.Kp = Kp;
-  a.part1 = part1;
-  a.part2 = part2;
+css_status css_rows(css_ctx* ctx, int mode, const CssRows& p, cudaStream_t st) {
+  RowsArgs r;
+  r.N = p.N;
+  r.rchk = css_rows_chunk(p.N, p.b);
+  r.ws = p.ws;
+  r.ncb = p.ncb;
+  r.cb0 = p.cb0;
+  r.G = 0;
+  r.first = p.first;
+  r.Q = p.Q;
+  r.Qp = p.Qp;
+  r.W = p.W;
+  r.out = p.out;
+  r.out2 = p.out2;
+  r.M1 = p.M1;
+  r.M2 = p.M2;
+  r.Bprev = p.Bprev;
+  r.need3 = p.need3;
+  r.part1 = p.part1;
+  r.part2 = p.part2;
+  r.err = p.err;
   switch (mode) {
-    case RP_S1: return launch_rp<RP_S1>(ctx, a, st);
-    case RP_S3: return launch_rp<RP_S3>(ctx, a, st);
-    case RP_TRIG: return launch_rp<RP_TRIG>(ctx, a, st);
-    default: return launch_rp<RP_TRI>(ctx, a, st);
+    case R_S1: return launch_rows6<R_S1>(ctx, r, st);
+    case R_S3: return launch_rows6<R_S3>(ctx, r, st);
+    case R_T0: return launch_rows6<R_T0>(ctx, r, st);
+    case R_T1: return launch_rows6<R_T1>(ctx, r, st);
+    default: return launch_rows6<R_T2>(ctx, r, st);
   }
-}
-
-css_status css_small_mm(css_ctx* ctx, int32_t ncb, int32_t b, const double* A, const double* B, double* Cm,
-                        cudaStream_t st) {
-  const int64_t n = (int64_t)ncb * b * b;
-  k_small_mm<<<(unsigned)css_ceil_div(n, 256), 256, 0, st>>>(ncb, b, A, B, Cm);
-  CSS_LAUNCHED(ctx);
-  return CSS_OK;
 }

@@ -60,3 +60,22 @@ def test_band_reduction_splits(torch, ctx, b, m, n_col):
     nblk = np.full(n_col, m)
     nblk[-1] = 1
     check(torch, ctx, A, B, nblk, rng.integers(1, 50, n_col), mu=0.3, kT=0.5)
+
+
+# FP32 row passes: rows that leave part of a tile (n b mod 64), one, an odd number and more than one
+# group of colours, and a Krylov space that is exhausted before depth m (nearly dependent blocks, then
+# breakdown); fixed mid-gap mu, the mixed-precision tolerance of the parity tests
+@pytest.mark.parametrize("kind,n,nc,m", [("minimal", 33, 1, 5), ("minimal", 33, 11, 5), ("minimal", 64, 21, 5),
+                                         ("minimal", 75, 75, 4), ("minimal", 9, 9, 12)])
+def test_fp32_row_pass_splits(torch, css, ctx, kind, n, nc, m):
+    from paper_2605_20918_gb300 import synth
+    from tests.test_gpu_parity import MIXED_P_TOL, gpu_density
+    g = synth.water_box(n)
+    H = synth.hamiltonian(g, kind)
+    col = (np.arange(n) % nc).astype(np.int32)
+    s = oracle.probes(col, H.b, 1005)
+    kw = dict(kT=0.05, n_elec=synth.n_electrons(n), m=m, mu=-4.0, solve_mu=False)
+    ref = oracle.density(H, col, s, nc, **kw)
+    got = gpu_density(torch, css, ctx, H, col, s, nc, precision=css.CSS_MIXED_FP32, **kw)
+    scale = max(1.0, float(np.abs(ref["P"]).max()))
+    assert float(np.abs(got["P"] - ref["P"]).max()) < MIXED_P_TOL * scale
