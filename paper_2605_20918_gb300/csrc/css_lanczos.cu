@@ -1302,7 +1302,7 @@ css_status run_pass_bp(css_ctx* ctx, const LzArgs& a_in, cudaStream_t st) {
   const int32_t G = colours_per_cta<T, BP>(b);
   const int32_t ngr = (int32_t)css_ceil_div(ncb, G);
   const bool reorth = (a.flags & CSS_REORTH_LOCAL) != 0;
-  // FP32 with b = 6: the row passes of css_rows.cu, with Gram partials in chunks of their own
+  // FP32 with b = 6 or 23: the row passes of css_rows.cu, with Gram partials in chunks of their own
   const bool rows = sizeof(T) == 4 && reorth && css_rows_supported(true, b);
   const int32_t rchk = row_chunk<T, BP>(N, b);
   const int32_t nch = (int32_t)css_ceil_div(N, rchk), nch_r = rows ? (int32_t)css_ceil_div(N, css_rows_chunk(N, b)) : 0;

@@ -93,7 +93,7 @@ int css_spmm_split_variants();
 css_status css_spmm_split_prepare(css_ctx* ctx, int32_t b, int32_t nnzb, const double* H, const void** Hs,
                                   cudaStream_t st);
 css_status css_spmm_split(css_ctx* ctx, const LzArgs& a, const double* V, double* W, int variant, cudaStream_t st);
-// FP32 row passes of a Lanczos step with local reorthogonalisation for b = 6 (css_rows.cu); mode 0 S1,
+// FP32 row passes of a Lanczos step with local reorthogonalisation for b = 6 and 23 (css_rows.cu); mode 0 S1,
 // 1 S3, 2 T0, 3 T1, 4 T2
 struct CssRows {
   int64_t N = 0;

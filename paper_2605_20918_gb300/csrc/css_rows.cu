@@ -1,4 +1,4 @@
-// Row passes of one FP32 block-Lanczos step with local reorthogonalisation, block width 6
+// Row passes of one FP32 block-Lanczos step with local reorthogonalisation, block widths 6 and 23
 // (paper: the three-term recurrence and block QR of the block-Lanczos paragraph after Eq. 4).  Each
 // pass streams N x w Krylov blocks once and applies, per colour c, small b x b matrices and / or
 // accumulates b x b Gram matrices:
@@ -13,7 +13,7 @@
 // less than a pass over memory.  A step moves ten N x w blocks instead of twelve.
 //
 // The rows of a group of colours (a multiple of 16 bytes in every row) arrive in a ring of tiles filled
-// by two producer warps with 16-byte cp.async copies; the same warps write finished tiles back.
+// by one or two producer warps with 16-byte cp.async copies; the same warps write finished tiles back.
 // mbarriers with bounded waits connect them to the other warps.  (One bulk copy per row segment of
 // ~300 bytes instead took ~62 clocks of an SM each whatever its size, 1.3 TB/s in all.)
 #include <algorithm>
@@ -69,15 +69,13 @@ __device__ __forceinline__ void copy16(void* dst, const void* src) {
 __device__ __forceinline__ void arrive_copies(uint64_t* b) {
   asm volatile("cp.async.mbarrier.arrive.noinc.shared::cta.b64 [%0];" ::"r"(su32(b)) : "memory");
 }
-constexpr int kProducers = 2;  // warps
-
 // words of a staged row: the group's columns, rounded so that consecutive rows are an odd number of
 // 16-byte units apart (lane-per-row accesses of 16 bytes hit distinct banks)
 __host__ __device__ constexpr int row_pitch(int cols) { return 4 * (((cols + 3) / 4) | 1); }
 
 // A CTA's tiles: ns stages of NA arrays of R rows, "full" barriers (the producers' copies) and "done"
-// barriers (the consumers' arrivals).
-template <int NA, int R>
+// barriers (the consumers' arrivals); NP producer warps.
+template <int NA, int R, int NP>
 struct Ring {
   float* base;
   uint64_t *full, *done;
@@ -91,7 +89,7 @@ struct Ring {
   __device__ __forceinline__ void arrive(int32_t t) const { bar_arrive(&done[t % ns]); }
   __device__ __forceinline__ void init(int32_t consumers) const {  // one thread
     for (int s = 0; s < ns; ++s) {
-      bar_init(&full[s], 32 * kProducers);
+      bar_init(&full[s], 32 * NP);
       bar_init(&done[s], consumers);
     }
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -104,7 +102,7 @@ struct Ring {
                           int32_t cpr) const {
     // a thread keeps its chunk of the row and walks down the rows, rp at a time, so that a copy is two
     // pointer steps (dividing a running index took ~110 clocks of the warp per copy)
-    const int tid = pw * 32 + (threadIdx.x & 31), rp = 32 * kProducers / cpr;
+    const int tid = pw * 32 + (threadIdx.x & 31), rp = 32 * NP / cpr;
     const int32_t rb = tid / cpr, c = tid - rb * cpr;
     const bool mine = rb < rp;
     const size_t go = (size_t)rb * ws + col0 + 4 * c, gs = (size_t)rp * ws;
@@ -155,6 +153,7 @@ struct Ring {
 // row left the waits and shared-memory latency of a tile exposed: 2.36 ms), ten colours so that a lane
 // has 168 registers (twelve spilled in S1 and S3: 2.22 ms).
 constexpr int B6_R = 64;      // rows per tile, two per lane
+constexpr int B6_NP = 2;      // producer warps
 constexpr int B6_GMAX = 10;   // colours (warps) per CTA, an even number: 16-byte columns
 template <int MODE>
 struct B6Cfg {
@@ -171,7 +170,7 @@ __host__ __device__ constexpr int sym_pair(int k, int i) {
 }
 
 template <int MODE>
-__global__ void __launch_bounds__(32 * (B6_GMAX + kProducers), 1) k_rows6(const RowsArgs a) {
+__global__ void __launch_bounds__(32 * (B6_GMAX + B6_NP), 1) k_rows6(const RowsArgs a) {
   using C = B6Cfg<MODE>;
   constexpr int NA = C::NA, NS = C::NS, R = B6_R;
   constexpr bool OUT = MODE == R_S3 || MODE == R_T1 || MODE == R_T2;
@@ -179,7 +178,7 @@ __global__ void __launch_bounds__(32 * (B6_GMAX + kProducers), 1) k_rows6(const 
   extern __shared__ __align__(128) unsigned char rows_smem[];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int32_t g0 = blockIdx.y * a.G, gcount = min(a.G, a.ncb - g0);
-  Ring<NA, R> ring;
+  Ring<NA, R, B6_NP> ring;
   ring.full = reinterpret_cast<uint64_t*>(rows_smem);
   ring.done = ring.full + NS;
   ring.abort = reinterpret_cast<volatile int*>(ring.done + NS);
@@ -387,6 +386,309 @@ __global__ void __launch_bounds__(32 * (B6_GMAX + kProducers), 1) k_rows6(const 
   }
 }
 
+// ------------------------------------------------------------------------ b = 23
+// Four colours (92 columns: whole 16-byte chunks) and tiles of 64 rows per CTA.  A tile is worked on in
+// two phases between CTA barriers:
+//   products: a warp takes one colour of 32 rows, a row per lane.  The row's 23 values come from the
+//     ring by 16-byte loads (a colour starts at one of four offsets within a chunk: four forms of the
+//     load, one of the arithmetic), the matrices by broadcast loads shared by 32 rows, an output pair
+//     per packed FMA; triangular matrices skip their zero half.  Results go back to the ring for the
+//     store and, 24 columns per colour, to a copy for the Gram.
+//   Grams: a thread owns an 8 x 8 block of a colour's 24 x 24 and every 8th row (S1: the blocks of Kq
+//     and of Kp together), four or six 16-byte loads for 32 or 64 packed FMAs.  After 32 rows the eight
+//     lanes of a block add their sums by halves (each keeps one row of the block) into hi + lo pairs.
+// Bound by the return path of shared memory: a 16-byte load is 512 bytes to a warp, four clocks of the
+// SM, broadcast or not, so the products' two packed FMAs per load (4 clocks of one scheduler) leave
+// the FMA pipe at a quarter; HBM is at 2 TB/s.  Row work of a step at 10,000 molecules 9.34 -> 6.71 ms
+// (S1 2.47, S3 2.20, T0 0.82, T1 0.88), at 1,000 1.08 -> 0.81 ms, against the tiled kernels.
+constexpr int B23_R = 64, B23_G = 4, B23_GP = 100;  // rows per tile, colours per CTA, pitch of the Gram copies
+template <int MODE>
+struct B23Cfg {
+  static constexpr int NA = MODE <= R_S3 ? 3 : 1;
+  static constexpr int NS = MODE <= R_S3 ? 2 : 4;
+  static constexpr int NP = 3;                          // producer warps
+  static constexpr int CW = MODE == R_S1 ? 9 : 8;       // consumer warps
+  static constexpr int NM = MODE == R_S3 ? 3 : MODE == R_T1 ? 2 : 1;  // matrices per colour
+  static constexpr int NG = MODE == R_S1 ? 3 : MODE == R_T2 ? 0 : 1;  // Gram copies
+  static constexpr size_t smem = (size_t)NS * NA * B23_R * row_pitch(92) * 4 + (size_t)NG * B23_R * B23_GP * 4 +
+                                 (size_t)NM * B23_G * 23 * 24 * 4 + (2 * NS + 2) * 8;
+};
+
+// the 23 values at chunk + O floats of a staged row, zero past them
+template <int O>
+__device__ __forceinline__ void load_row(const float* chunk, float (&x)[24]) {
+  constexpr int NC = (O + 23 + 3) / 4;
+  float4 v[NC];
+#pragma unroll
+  for (int i = 0; i < NC; ++i) v[i] = *reinterpret_cast<const float4*>(chunk + 4 * i);
+#pragma unroll
+  for (int i = 0; i < 23; ++i) {
+    const float4 q = v[(i + O) / 4];
+    x[i] = (i + O) % 4 == 0 ? q.x : (i + O) % 4 == 1 ? q.y : (i + O) % 4 == 2 ? q.z : q.w;
+  }
+  x[23] = 0.0f;
+}
+template <int O>
+__device__ __forceinline__ void store_row(float* chunk, const unsigned long long (&o)[12]) {
+  auto at = [&](int i) { return i & 1 ? hi2(o[i >> 1]) : lo2(o[i >> 1]); };
+#pragma unroll
+  for (int i = 0; i < 23; ++i) {
+    constexpr int first = (4 - O) % 4;  // first value on a chunk boundary
+    if (i >= first && (i - first) % 4 == 0 && i + 3 < 23)
+      *reinterpret_cast<float4*>(chunk + O + i) = make_float4(at(i), at(i + 1), at(i + 2), at(i + 3));
+    else if (i < first || i >= first + (23 - first) / 4 * 4)
+      chunk[O + i] = at(i);
+  }
+}
+__device__ __forceinline__ void load_row_of(int c, const float* row, float (&x)[24]) {  // colour c starts at 23 c
+  if (c == 0) load_row<0>(row, x);
+  else if (c == 1) load_row<3>(row + 20, x);
+  else if (c == 2) load_row<2>(row + 44, x);
+  else load_row<1>(row + 68, x);
+}
+__device__ __forceinline__ void store_row_of(int c, float* row, const unsigned long long (&o)[12]) {
+  if (c == 0) store_row<0>(row, o);
+  else if (c == 1) store_row<3>(row + 20, o);
+  else if (c == 2) store_row<2>(row + 44, o);
+  else store_row<1>(row + 68, o);
+}
+// o += x M, M [23][24] in shared memory; TRI 1: M(l, k) = 0 for k > l, TRI 2: for k < l
+template <int TRI>
+__device__ __forceinline__ void mul_row(unsigned long long (&o)[12], const float (&x)[24], const float* M) {
+#pragma unroll
+  for (int l = 0; l < 23; ++l) {
+    const unsigned long long xx = dup2(x[l]);
+#pragma unroll
+    for (int c = 0; c < 6; ++c) {
+      if ((TRI == 1 && 4 * c > l) || (TRI == 2 && 4 * c + 3 < l)) continue;
+      const ulonglong2 m = *reinterpret_cast<const ulonglong2*>(M + 24 * l + 4 * c);
+      fma2(o[2 * c], xx, m.x);
+      fma2(o[2 * c + 1], xx, m.y);
+    }
+  }
+}
+
+// The sums of an 8 x 8 block (32 pairs, row k in pairs 4 k .. 4 k + 3) over the S lanes that share it:
+// each step the lanes of a pair keep one half of what is left and give away the other.  Lane s of the
+// S ends with pairs 32 / S * rev(s) .. of the block, added into its hi + lo pairs; v is cleared.
+template <int S>
+__device__ __forceinline__ void block_flush(unsigned long long (&v)[32], float (&hi)[64 / S], float (&lo)[64 / S]) {
+  const int lane = threadIdx.x & 31;
+  int n = 16;
+#pragma unroll
+  for (int o = S / 2; o > 0; o >>= 1, n >>= 1) {
+    const bool up = lane & o;
+#pragma unroll
+    for (int i = 0; i < 16; ++i) {
+      if (i >= n) continue;
+      const unsigned long long keep = up ? v[i + n] : v[i], give = up ? v[i] : v[i + n];
+      const unsigned long long got = __shfl_xor_sync(0xffffffffu, give, o);
+      asm("add.rn.f32x2 %0, %1, %2;" : "=l"(v[i]) : "l"(keep), "l"(got));
+    }
+  }
+#pragma unroll
+  for (int i = 0; i < 32 / S; ++i) {
+    add_comp(hi[2 * i], lo[2 * i], lo2(v[i]));
+    add_comp(hi[2 * i + 1], lo[2 * i + 1], hi2(v[i]));
+  }
+#pragma unroll
+  for (int i = 0; i < 32; ++i) v[i] = 0ull;
+}
+
+template <int MODE>
+__global__ void __launch_bounds__(32 * (B23Cfg<MODE>::CW + B23Cfg<MODE>::NP), 1) k_rows23(const RowsArgs a) {
+  using C = B23Cfg<MODE>;
+  constexpr int NA = C::NA, NS = C::NS, R = B23_R, CT = 32 * C::CW, MM = 23 * 24;
+  constexpr bool OUT = MODE == R_S3 || MODE == R_T1 || MODE == R_T2;
+  extern __shared__ __align__(128) unsigned char rows_smem[];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int32_t g0 = blockIdx.y * B23_G, gcount = min(B23_G, a.ncb - g0);
+  Ring<NA, R, C::NP> ring;
+  ring.full = reinterpret_cast<uint64_t*>(rows_smem);
+  ring.done = ring.full + NS;
+  ring.abort = reinterpret_cast<volatile int*>(ring.done + NS);
+  ring.base = reinterpret_cast<float*>(rows_smem + (2 * NS + 2) * 8);
+  ring.err = a.err;
+  ring.ns = NS;
+  ring.pitch = row_pitch(92);
+  ring.r0 = (int64_t)blockIdx.x * a.rchk;
+  ring.rend = min(a.N, ring.r0 + a.rchk);
+  ring.ntile = (int32_t)((ring.rend - ring.r0 + R - 1) / R);
+  float* sG = ring.base + (size_t)NS * NA * R * ring.pitch;  // Gram copies [array][row][24 c + k]
+  float* sM = sG + (size_t)C::NG * R * B23_GP;               // matrices [matrix][colour][l][k]
+  bool any3 = false;
+  if (MODE >= R_T1)
+    for (int32_t g = 0; g < gcount; ++g) any3 = any3 || a.need3[g0 + g] != 0;
+  if (MODE == R_T2 && !any3) return;  // uniform over the CTA
+  const bool use_p = MODE <= R_S3 && !a.first;
+  const bool gram = MODE <= R_T0 || (MODE == R_T1 && any3);
+  if (threadIdx.x == 0) {
+    ring.init(1);
+    *ring.abort = *(volatile int*)a.err ? 1 : 0;
+  }
+  // the colours' matrices (negated where they are subtracted)
+  for (int32_t e = threadIdx.x; e < B23_G * MM; e += blockDim.x) {
+    const int32_t g = e / MM, rem = e - g * MM, l = rem / 24, k = rem - 24 * l;
+    const bool in = g < gcount && k < 23;
+    const size_t o = (size_t)(g0 + (in ? g : 0)) * 529;
+    if (MODE <= R_S3)  // -B^T
+      sM[e] = in && use_p && k <= l ? -(float)a.Bprev[(size_t)(a.cb0 + g0 + g) * 529 + k * 23 + l] : 0.0f;
+    if (MODE == R_S3) {
+      sM[B23_G * MM + e] = in ? -(float)a.M1[o + l * 23 + k] : 0.0f;
+      sM[2 * B23_G * MM + e] = in && use_p ? -(float)a.M2[o + l * 23 + k] : 0.0f;
+    }
+    if (MODE >= R_T0) sM[e] = in ? (float)a.M1[o + l * 23 + k] : 0.0f;
+    if (MODE == R_T1) sM[B23_G * MM + e] = in ? (float)a.M2[o + l * 23 + k] : 0.0f;
+  }
+  // rows past the end of the last tile and columns past the last colour stay zero in the Gram copies
+  for (int32_t e = threadIdx.x; e < C::NG * R * B23_GP; e += blockDim.x) sG[e] = 0.0f;
+  __syncthreads();
+  if (*ring.abort) return;
+  if (warp >= C::CW) {
+    const float* src[3] = {a.W, a.Q, a.Qp};
+    ring.template produce<OUT>(warp - C::CW, src, MODE <= R_S3 ? (use_p ? 3 : 2) : 1, a.out,
+                               MODE == R_T1 && any3 ? a.out2 : nullptr, a.ws, g0 * 23, (gcount * 23 + 3) / 4);
+    return;
+  }
+  auto sync = [] { asm volatile("bar.sync 1, %0;" ::"n"(CT) : "memory"); };
+  // products: warps 0 to 7
+  const int pc = warp & 3, pr = 32 * (warp >> 2) + lane;
+  const bool prod = warp < 8 && pc < gcount;
+  const bool n3 = MODE >= R_T1 && prod && a.need3[g0 + pc] != 0;
+  // Grams: this thread's block and rows
+  constexpr int S = 8;
+  const int gs = threadIdx.x & (S - 1), blk = threadIdx.x / S;
+  const int gc = MODE == R_S1 ? blk / 9 : blk / 6, gb = MODE == R_S1 ? blk % 9 : blk % 6;
+  const int kb = MODE == R_S1 ? gb / 3 : gb < 3 ? 0 : gb < 5 ? 1 : 2;
+  const int lb = MODE == R_S1 ? gb % 3 : gb < 3 ? gb : gb < 5 ? gb - 2 : 2;
+  unsigned long long vq[32], vp[MODE == R_S1 ? 32 : 1];
+  float hq[64 / S] = {}, lq[64 / S] = {}, hp[MODE == R_S1 ? 8 : 1] = {}, lp[MODE == R_S1 ? 8 : 1] = {};
+#pragma unroll
+  for (int i = 0; i < 32; ++i) {
+    vq[i] = 0ull;
+    if (MODE == R_S1) vp[i % (MODE == R_S1 ? 32 : 1)] = 0ull;
+  }
+  // a warp whose wait gives up still runs every barrier, so that no other waits for it
+#pragma unroll 1
+  for (int32_t t = 0; t < ring.ntile; ++t) {
+    const bool ok = ring.wait_full(t);
+    float* st = ring.stage(t);
+    if (prod && ok) {
+      const bool valid = pr < ring.rows(t);
+      float* row = st + (size_t)pr * ring.pitch;
+      float* grow = sG + (size_t)pr * B23_GP + 24 * pc;
+      float x[24];
+      unsigned long long o[12];
+      auto zero_past_end = [&]() {
+        if (!valid)
+#pragma unroll
+          for (int i = 0; i < 24; ++i) x[i] = 0.0f;
+      };
+      auto to_gram = [&](int array, auto val) {
+#pragma unroll
+        for (int i = 0; i < 6; ++i)
+          *reinterpret_cast<ulonglong2*>(grow + (size_t)array * R * B23_GP + 4 * i) = make_ulonglong2(val(2 * i), val(2 * i + 1));
+      };
+      load_row_of(pc, row, x);  // W
+      zero_past_end();
+      if (MODE <= R_S3) {
+#pragma unroll
+        for (int i = 0; i < 12; ++i) o[i] = pack2(x[2 * i], x[2 * i + 1]);
+        if (use_p) {
+          load_row_of(pc, row + 2 * (size_t)R * ring.pitch, x);  // Q_{j-1}
+          zero_past_end();
+          mul_row<1>(o, x, sM + pc * MM);
+          if (MODE == R_S1) to_gram(2, [&](int i) { return pack2(x[2 * i], x[2 * i + 1]); });
+        }
+        if (MODE == R_S1) {
+          to_gram(0, [&](int i) { return o[i]; });
+          load_row_of(pc, row + (size_t)R * ring.pitch, x);  // Q_j
+          zero_past_end();
+          to_gram(1, [&](int i) { return pack2(x[2 * i], x[2 * i + 1]); });
+        } else {
+          float q[24];
+          load_row_of(pc, row + (size_t)R * ring.pitch, q);
+          if (!valid)
+#pragma unroll
+            for (int i = 0; i < 24; ++i) q[i] = 0.0f;
+          mul_row<0>(o, q, sM + (B23_G + pc) * MM);
+          if (use_p) mul_row<0>(o, x, sM + (2 * B23_G + pc) * MM);
+        }
+      } else {
+#pragma unroll
+        for (int i = 0; i < 12; ++i) o[i] = 0ull;
+        mul_row<2>(o, x, sM + pc * MM);
+        if (MODE == R_T1) {
+#pragma unroll
+          for (int i = 0; i < 12; ++i) {
+            x[2 * i] = lo2(o[i]);
+            x[2 * i + 1] = hi2(o[i]);
+            o[i] = 0ull;
+          }
+          mul_row<2>(o, x, sM + (B23_G + pc) * MM);
+        }
+      }
+      if (OUT) {
+        if (MODE != R_T2 || n3) store_row_of(pc, row, o);
+        if (pc + 1 == gcount)
+          for (int32_t i = 23 * gcount; i & 3; ++i) row[i] = 0.0f;  // columns past the last colour
+      }
+      if (MODE != R_S1 && gram) to_gram(0, [&](int i) { return o[i]; });
+    }
+    sync();  // products of the tile are in place; the ring's stage is read (or finished)
+    if (threadIdx.x == 0) ring.arrive(t);
+    if (!gram) continue;
+    if (ok && gc < B23_G) {  // whole warps
+      const float* y0 = sG + (size_t)gs * B23_GP + 24 * gc + 8 * lb;
+      const float* x0 = sG + (size_t)gs * B23_GP + 24 * gc + 8 * kb + (MODE == R_S1 ? R * B23_GP : 0);
+#pragma unroll(MODE == R_S1 ? 1 : 2)
+      for (int i = 0; i < R / S; ++i, y0 += S * B23_GP, x0 += S * B23_GP) {
+        const ulonglong2 ya = *reinterpret_cast<const ulonglong2*>(y0), yb = *reinterpret_cast<const ulonglong2*>(y0 + 4);
+        auto rank1 = [&](const float* xr, unsigned long long* v) {
+          const float4 xa = *reinterpret_cast<const float4*>(xr), xb = *reinterpret_cast<const float4*>(xr + 4);
+          const float xv[8] = {xa.x, xa.y, xa.z, xa.w, xb.x, xb.y, xb.z, xb.w};
+#pragma unroll
+          for (int k = 0; k < 8; ++k) {
+            const unsigned long long xx = dup2(xv[k]);
+            fma2(v[4 * k], xx, ya.x);
+            fma2(v[4 * k + 1], xx, ya.y);
+            fma2(v[4 * k + 2], xx, yb.x);
+            fma2(v[4 * k + 3], xx, yb.y);
+          }
+        };
+        rank1(x0, vq);
+        if constexpr (MODE == R_S1) rank1(x0 + R * B23_GP, vp);
+      }
+      constexpr int FL = 32 / (R / S);  // tiles of 32 rows per lane
+      if (t % FL == FL - 1 || t + 1 == ring.ntile) {
+        block_flush<S>(vq, hq, lq);
+        if constexpr (MODE == R_S1) block_flush<S>(vp, hp, lp);
+      }
+    }
+    sync();  // the Gram copies are free for the next tile
+  }
+  if (!gram || *ring.abort || gc >= gcount) return;
+  if (MODE == R_T1 && a.need3[g0 + gc] == 0) return;
+  // the pairs block_flush left in this lane: p0, p0 + 1, ...
+  int p0 = 0;
+#pragma unroll
+  for (int o = S / 2, n = 16; o > 0; o >>= 1, n >>= 1) p0 += gs & o ? n : 0;
+#pragma unroll
+  for (int gram2 = 0; gram2 < (MODE == R_S1 ? 2 : 1); ++gram2) {
+    double* part = (gram2 ? a.part2 : a.part1) + ((size_t)blockIdx.x * a.ncb + g0 + gc) * 529;
+#pragma unroll
+    for (int i = 0; i < 64 / S; ++i) {
+      const int k = 8 * kb + (p0 + i / 2) / 4, l = 8 * lb + 2 * ((p0 + i / 2) % 4) + (i & 1);
+      const float h = gram2 ? hp[i % (MODE == R_S1 ? 8 : 1)] : hq[i], w = gram2 ? lp[i % (MODE == R_S1 ? 8 : 1)] : lq[i];
+      if (k < 23 && l < 23) {
+        const double v = (double)h + (double)w;
+        part[k * 23 + l] = v;
+        if (MODE != R_S1 && kb != lb) part[l * 23 + k] = v;
+      }
+    }
+  }
+}
+
 // Rows per CTA: chunks for one to three waves of a CTA per SM over `groups` groups of colours (a full
 // count: the chunk may not depend on the colours of the call, or a colour's sums would), more waves
 // where a CTA still has `most` rows, so that its start and end (~5 us) stay small.
@@ -403,18 +705,32 @@ css_status launch_rows6(css_ctx* ctx, RowsArgs& r, cudaStream_t st) {
   const size_t sm = B6Cfg<MODE>::smem(r.G);
   CSS_CU(ctx, cudaFuncSetAttribute(k_rows6<MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
   const dim3 grid((unsigned)css_ceil_div(r.N, r.rchk), (unsigned)css_ceil_div(r.ncb, r.G));
-  k_rows6<MODE><<<grid, 32 * (r.G + kProducers), sm, st>>>(r);
+  k_rows6<MODE><<<grid, 32 * (r.G + B6_NP), sm, st>>>(r);
   CSS_LAUNCHED(ctx);
   return CSS_OK;
 }
 
+template <int MODE>
+css_status launch_rows23(css_ctx* ctx, RowsArgs& r, cudaStream_t st) {
+  using C = B23Cfg<MODE>;
+  CSS_CU(ctx, cudaFuncSetAttribute(k_rows23<MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)C::smem));
+  const dim3 grid((unsigned)css_ceil_div(r.N, r.rchk), (unsigned)css_ceil_div(r.ncb, B23_G));
+  k_rows23<MODE><<<grid, 32 * (C::CW + C::NP), C::smem, st>>>(r);
+  CSS_LAUNCHED(ctx);
+  return CSS_OK;
+}
+
+template <int MODE>
+css_status launch_rows(css_ctx* ctx, int32_t b, RowsArgs& r, cudaStream_t st) {
+  return b == 6 ? launch_rows6<MODE>(ctx, r, st) : launch_rows23<MODE>(ctx, r, st);
+}
+
 }  // namespace
 
-bool css_rows_supported(bool fp32, int32_t b) { return fp32 && b == 6; }
+bool css_rows_supported(bool fp32, int32_t b) { return fp32 && (b == 6 || b == 23); }
 
 int32_t css_rows_chunk(int64_t N, int32_t b) {
-  (void)b;
-  return pick_chunk(N, 7, B6_R, 2048);
+  return b == 6 ? pick_chunk(N, 7, B6_R, 2048) : pick_chunk(N, 17, B23_R, 2048);
 }
 
 css_status css_rows(css_ctx* ctx, int mode, const CssRows& p, cudaStream_t st) {
@@ -439,10 +755,10 @@ css_status css_rows(css_ctx* ctx, int mode, const CssRows& p, cudaStream_t st) {
   r.part2 = p.part2;
   r.err = p.err;
   switch (mode) {
-    case R_S1: return launch_rows6<R_S1>(ctx, r, st);
-    case R_S3: return launch_rows6<R_S3>(ctx, r, st);
-    case R_T0: return launch_rows6<R_T0>(ctx, r, st);
-    case R_T1: return launch_rows6<R_T1>(ctx, r, st);
-    default: return launch_rows6<R_T2>(ctx, r, st);
+    case R_S1: return launch_rows<R_S1>(ctx, p.b, r, st);
+    case R_S3: return launch_rows<R_S3>(ctx, p.b, r, st);
+    case R_T0: return launch_rows<R_T0>(ctx, p.b, r, st);
+    case R_T1: return launch_rows<R_T1>(ctx, p.b, r, st);
+    default: return launch_rows<R_T2>(ctx, p.b, r, st);
   }
 }

@@ -63,10 +63,11 @@ def test_band_reduction_splits(torch, ctx, b, m, n_col):
 
 
 # FP32 row passes: rows that leave part of a tile (n b mod 64), one, an odd number and more than one
-# group of colours, and a Krylov space that is exhausted before depth m (nearly dependent blocks, then
+# group of colours (b = 23: groups of four, whose columns start at four offsets within 16 bytes), and a Krylov space that is exhausted before depth m (nearly dependent blocks, then
 # breakdown); fixed mid-gap mu, the mixed-precision tolerance of the parity tests
 @pytest.mark.parametrize("kind,n,nc,m", [("minimal", 33, 1, 5), ("minimal", 33, 11, 5), ("minimal", 64, 21, 5),
-                                         ("minimal", 75, 75, 4), ("minimal", 9, 9, 12)])
+                                         ("minimal", 75, 75, 4), ("minimal", 9, 9, 12), ("dzp", 9, 1, 5),
+                                         ("dzp", 14, 5, 5), ("dzp", 20, 20, 4), ("dzp", 6, 6, 8)])
 def test_fp32_row_pass_splits(torch, css, ctx, kind, n, nc, m):
     from paper_2605_20918_gb300 import synth
     from tests.test_gpu_parity import MIXED_P_TOL, gpu_density
