@@ -847,7 +847,6 @@ css_status css_density_impl(css_ctx* ctx, int32_t n_sys, const css_sys_desc* sys
   CSS_TRY(ws_get(ctx, "e_AB", (size_t)n_col * nmax * css_band_ld(b), &ea.AB));
   CSS_TRY(ws_get(ctx, "e_RV", (size_t)n_col * ea.rcap * b, &ea.RV));
   CSS_TRY(ws_get(ctx, "e_RT", (size_t)n_col * ea.rcap, &ea.RT));
-  CSS_TRY(ws_get(ctx, "e_RR0", (size_t)n_col * ea.rcap, &ea.RR0));
   CSS_TRY(ws_get(ctx, "e_d", (size_t)n_col * nmax, &ea.d));
   CSS_TRY(ws_get(ctx, "e_e", (size_t)n_col * nmax, &ea.e));
   CSS_TRY(ws_get(ctx, "e_l32", (size_t)n_col * nmax, &ea.lam32));
@@ -1543,7 +1542,6 @@ css_status css_eigen_blocks(css_ctx* ctx, int32_t n_col, int32_t b, int32_t m, c
   CSS_TRY(ws_get(ctx, "e_AB", (size_t)n_col * nmax * css_band_ld(b), &ea.AB));
   CSS_TRY(ws_get(ctx, "e_RV", (size_t)n_col * ea.rcap * b, &ea.RV));
   CSS_TRY(ws_get(ctx, "e_RT", (size_t)n_col * ea.rcap, &ea.RT));
-  CSS_TRY(ws_get(ctx, "e_RR0", (size_t)n_col * ea.rcap, &ea.RR0));
   CSS_TRY(ws_get(ctx, "e_d", (size_t)n_col * nmax, &ea.d));
   CSS_TRY(ws_get(ctx, "e_e", (size_t)n_col * nmax, &ea.e));
   CSS_TRY(ws_get(ctx, "e_l32", (size_t)n_col * nmax, &ea.lam32));
@@ -2008,7 +2006,6 @@ css_status css_density_nonorth(css_ctx* ctx, const css_bsr* S, const double* Sin
   CSS_TRY(ws_get(ctx, "e_AB", (size_t)nc * nmax * css_band_ld(b), &ea.AB));
   CSS_TRY(ws_get(ctx, "e_RV", (size_t)nc * ea.rcap * b, &ea.RV));
   CSS_TRY(ws_get(ctx, "e_RT", (size_t)nc * ea.rcap, &ea.RT));
-  CSS_TRY(ws_get(ctx, "e_RR0", (size_t)nc * ea.rcap, &ea.RR0));
   CSS_TRY(ws_get(ctx, "e_d", (size_t)nc * nmax, &ea.d));
   CSS_TRY(ws_get(ctx, "e_e", (size_t)nc * nmax, &ea.e));
   CSS_TRY(ws_get(ctx, "e_l32", (size_t)nc * nmax, &ea.lam32));

@@ -111,7 +111,6 @@ struct BandArgs {
   double* AB;
   double* RV;
   double* RT;
-  int32_t* RR0;
   unsigned long long* slots;  // [c][S], zeroed (tile mode)
   double *dd, *ee;
   int32_t* status;
@@ -288,10 +287,7 @@ __global__ void __launch_bounds__(SMEM ? 1024 : 512) k_band_to_tri(const BandArg
       }
       const int32_t slot = sweep_slot(i, n, kd) + k;
       if (l < kd) a.RV[((size_t)c * a.rcap + slot) * kd + l] = nl;
-      if (l == 0) {
-        a.RT[(size_t)c * a.rcap + slot] = tau2;
-        a.RR0[(size_t)c * a.rcap + slot] = q0;
-      }
+      if (l == 0) a.RT[(size_t)c * a.rcap + slot] = tau2;
     }
     v[l] = act ? nl : v[l];
     __syncwarp();
@@ -342,37 +338,60 @@ __global__ void k_tri_out(int32_t kd, int32_t nmax, int32_t ldb, const int32_t* 
   }
 }
 
-// Apply the recorded reflectors to an n x b block X ([c][nmax][b]): FWD applies them in
-// generation order (X <- Q^T X), otherwise in reverse (X <- Q X).  A sweep's reflectors act
-// on disjoint rows, so one thread per (reflector of the sweep, column) works in parallel.
+// Apply the recorded reflectors to columns of an n x b block X ([c][nmax][b]): FWD applies them in
+// generation order (X <- Q^T X), otherwise in reverse (X <- Q X).  A sweep's reflectors act on
+// disjoint rows, so one thread per (reflector of the sweep, column) works in parallel; the columns
+// are independent, so a colour's are shared out to gridDim.y CTAs of cw columns.  The columns live in
+// shared memory and the next sweep's reflectors arrive (cp.async) while this one's are applied.
+// Bound by FP64 issue (2 kd FMAs per reflector and column).  One CTA per colour, reading both from
+// global memory: n = 920, 63 colours 7.3 ms, n = 180 0.42 ms; now 3.6 and 0.22.
 template <bool FWD>
-__global__ void k_apply_refl(int32_t kd, int32_t b, int32_t nmax, int32_t rcap, const int32_t* __restrict__ nblk,
-                             const double* __restrict__ RV, const double* __restrict__ RT,
-                             const int32_t* __restrict__ RR0, double* __restrict__ X) {
-  const int32_t c = blockIdx.x;
+__global__ void __launch_bounds__(1024) k_apply_refl(int32_t kd, int32_t b, int32_t cw, int32_t nmax, int32_t rcap,
+                                                     const int32_t* __restrict__ nblk, const double* __restrict__ RV,
+                                                     const double* __restrict__ RT, double* __restrict__ X) {
+  extern __shared__ __align__(16) double refl_smem[];
+  const int32_t c = blockIdx.x, j0 = blockIdx.y * cw, w = min(cw, b - j0);
   const int32_t n = nblk[c] * kd;
   const double* rv = RV + (size_t)c * rcap * kd;
   const double* rt = RT + (size_t)c * rcap;
-  const int32_t* rr = RR0 + (size_t)c * rcap;
-  double* x = X + (size_t)c * nmax * b;
+  double* xg = X + (size_t)c * nmax * b + j0;
   const int32_t nsweep = n_sweeps(n, kd);
+  const int32_t most = nmax / kd + 1, stage = most * (kd + 1);  // reflectors of a sweep, doubles of a stage
+  double* x = refl_smem;  // [n][w]
+  double* sv = refl_smem + (size_t)nmax * cw;
+  for (int32_t t = threadIdx.x; t < n * w; t += blockDim.x) x[t] = xg[(size_t)(t / w) * b + t % w];
+  auto copy8 = [](double* d, const double* g) {
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(css_pipe::su32(d)), "l"(g) : "memory");
+  };
+  auto fetch = [&](int32_t s) {  // a sweep's reflectors and their taus
+    const int32_t i = FWD ? s : nsweep - 1 - s, t0 = sweep_slot(i, n, kd), len = sweep_len(i, n, kd);
+    double* d = sv + (s & 1) * stage;
+    for (int32_t t = threadIdx.x; t < len * kd; t += blockDim.x) copy8(d + t, rv + (size_t)t0 * kd + t);
+    for (int32_t t = threadIdx.x; t < len; t += blockDim.x) copy8(d + most * kd + t, rt + t0 + t);
+  };
+  if (nsweep > 0) fetch(0);
+  asm volatile("cp.async.commit_group;" ::: "memory");
   for (int32_t s = 0; s < nsweep; ++s) {
-    const int32_t i = FWD ? s : nsweep - 1 - s;
-    const int32_t t0 = sweep_slot(i, n, kd), len = sweep_len(i, n, kd);
-    for (int32_t t = threadIdx.x; t < len * b; t += blockDim.x) {
-      const int32_t r = t0 + t / b, col = t % b;
-      const double tau = rt[r];
-      if (tau == 0.0) continue;
-      const int32_t r0 = rr[r];
-      const int32_t L = min(kd, n - r0);
-      const double* v = rv + (size_t)r * kd;
+    asm volatile("cp.async.wait_group 0;" ::: "memory");
+    __syncthreads();  // this sweep's reflectors are there, and the previous sweep is done
+    if (s + 1 < nsweep) fetch(s + 1);
+    asm volatile("cp.async.commit_group;" ::: "memory");
+    const int32_t i = FWD ? s : nsweep - 1 - s, len = sweep_len(i, n, kd);
+    const double* d = sv + (s & 1) * stage;
+    for (int32_t t = threadIdx.x; t < len * w; t += blockDim.x) {
+      const int32_t r = t / w, r0 = i + 1 + r * kd, L = min(kd, n - r0);
+      const double* v = d + r * kd;
+      double* xr = x + (size_t)r0 * w + (t - r * w);
       double s2 = 0.0;
-      for (int32_t l = 0; l < L; ++l) s2 += v[l] * x[(size_t)(r0 + l) * b + col];
-      s2 *= tau;
-      for (int32_t l = 0; l < L; ++l) x[(size_t)(r0 + l) * b + col] -= s2 * v[l];
+#pragma unroll 4
+      for (int32_t l = 0; l < L; ++l) s2 = fma(v[l], xr[l * w], s2);
+      s2 *= d[most * kd + r];
+#pragma unroll 4
+      for (int32_t l = 0; l < L; ++l) xr[l * w] = fma(-s2, v[l], xr[l * w]);
     }
-    __syncthreads();
   }
+  __syncthreads();
+  for (int32_t t = threadIdx.x; t < n * w; t += blockDim.x) xg[(size_t)(t / w) * b + t % w] = x[t];
 }
 
 // X0 = E_1 B_0 = [B_0; 0] for a general start factor B_0 [c][b][b]
@@ -448,7 +467,8 @@ __global__ void k_bisect32(int32_t kd, int32_t nmax, const int32_t* __restrict__
   if (threadIdx.x == 0) tnorm[c] = fmax(span, 1e-100);
   const float flo = (float)(glo - 1e-3 * span - 1e-30), fhi = (float)(ghi + 1e-3 * span + 1e-30);
   const float pivmin = (float)fmax(1e-30, 1e-30 * gem);
-  for (int32_t k = threadIdx.x; k < n; k += blockDim.x) {
+  const int32_t k = blockIdx.y * blockDim.x + threadIdx.x;  // one eigenvalue per thread
+  if (k < n) {
     float a = flo, z = fhi;
     for (int it = 0; it < 80; ++it) {
       float mid = 0.5f * (a + z);
@@ -955,38 +975,50 @@ __global__ void __launch_bounds__(256) k_inviter_cl(int32_t kd, int32_t nmax, co
   if (failed) atomicOr(&status[c], 1);  // an eigenvalue outside its window after every attempt
 }
 
-// Y[k][col] = sum_i U[i][k] X[i][col], w[k] = ||Y[k]||^2 (one thread per k)
-__global__ void k_ritz_y(int32_t kd, int32_t b, int32_t nmax, const int32_t* __restrict__ nblk,
-                         const double* __restrict__ U, const double* __restrict__ X, double* __restrict__ Y,
-                         double* __restrict__ wgt) {
-  extern __shared__ double shx[];
+// Y[k][col] = sum_i U[i][k] X[i][col], w[k] = ||Y[k]||^2 (one thread per k).  B: the block width (0:
+// any, up to 32), so that the b running sums are registers and no test of b stands between the FMAs;
+// eight rows of U are loaded ahead of their FMAs.
+template <int B>
+__global__ void __launch_bounds__(128) k_ritz_y(int32_t kd, int32_t b_, int32_t nmax, const int32_t* __restrict__ nblk,
+                                                const double* __restrict__ U, const double* __restrict__ X,
+                                                double* __restrict__ Y, double* __restrict__ wgt) {
+  constexpr int NB = B ? B : CSS_MAX_B;
+  constexpr int CH = 64;
+  __shared__ double shx[CH * NB];
+  const int32_t b = B ? B : b_;
   const int32_t c = blockIdx.y;
   const int32_t n = nblk[c] * kd;
   const int32_t k = blockIdx.x * blockDim.x + threadIdx.x;
-  const double* u = U + (size_t)c * nmax * nmax;
+  const double* u = U + (size_t)c * nmax * nmax + min(k, nmax - 1);
   const double* x = X + (size_t)c * nmax * b;
-  double acc[CSS_MAX_B];
+  double acc[NB];
 #pragma unroll
-  for (int a = 0; a < CSS_MAX_B; ++a) acc[a] = 0.0;
-  const int32_t CH = 64;
-  for (int32_t i0 = 0; i0 < n; i0 += CH) {
-    const int32_t ie = min(n, i0 + CH);
-    __syncthreads();
-    for (int32_t t = threadIdx.x; t < (ie - i0) * b; t += blockDim.x) shx[t] = x[(size_t)i0 * b + t];
-    __syncthreads();
-    if (k < n)
-      for (int32_t i = i0; i < ie; ++i) {
-        const double uk = u[(size_t)i * nmax + k];
+  for (int a = 0; a < NB; ++a) acc[a] = 0.0;
+  if ((int32_t)(blockIdx.x * blockDim.x) < n)  // the whole CTA
+    for (int32_t i0 = 0; i0 < n; i0 += CH) {
+      const int32_t ie = min(n, i0 + CH);
+      __syncthreads();
+      for (int32_t t = threadIdx.x; t < (ie - i0) * b; t += blockDim.x) shx[t] = x[(size_t)i0 * b + t];
+      __syncthreads();
+      for (int32_t i = i0; i < ie; i += 8) {
+        double uk[8];
 #pragma unroll
-        for (int a = 0; a < CSS_MAX_B; ++a)
-          if (a < b) acc[a] = fma(uk, shx[(i - i0) * b + a], acc[a]);
+        for (int q = 0; q < 8; ++q) uk[q] = i + q < ie ? u[(size_t)(i + q) * nmax] : 0.0;
+#pragma unroll
+        for (int q = 0; q < 8; ++q) {
+          if (i + q >= ie) break;
+          const double* xr = shx + (i + q - i0) * b;
+#pragma unroll
+          for (int a = 0; a < NB; ++a)
+            if (B || a < b) acc[a] = fma(uk[q], xr[a], acc[a]);
+        }
       }
-  }
+    }
   if (k < n) {
     double w = 0.0;
 #pragma unroll
-    for (int a = 0; a < CSS_MAX_B; ++a)
-      if (a < b) {
+    for (int a = 0; a < NB; ++a)
+      if (B || a < b) {
         Y[((size_t)c * nmax + k) * b + a] = acc[a];
         w = fma(acc[a], acc[a], w);
       }
@@ -996,48 +1028,62 @@ __global__ void k_ritz_y(int32_t kd, int32_t b, int32_t nmax, const int32_t* __r
   }
 }
 
-// Zt[i][col] = sum_k U[i][k] g(lam_k) Y[k][col] (one thread per row i).  fn bit 1: g = x^(-1/2)
-// (inverse square root of an overlap, positive Ritz values; NaN otherwise) instead of the Fermi
-// function; bit 0: g multiplied by x (the energy-weighted density matrix, T_c Z_c).
-__global__ void k_zt(int32_t kd, int32_t b, int32_t nmax, const int32_t* __restrict__ nblk,
-                     const int32_t* __restrict__ sys_of_colour, const double* __restrict__ mu,
-                     const double* __restrict__ kT, const double* __restrict__ U, const double* __restrict__ lam,
-                     const double* __restrict__ Y, double* __restrict__ Z, int fn) {
-  extern __shared__ double shy[];
+// Zt[i][col] = sum_k U[i][k] g(lam_k) Y[k][col] (one thread per row i; U in 128 x 32 tiles through
+// shared memory, so that its rows are read whole).  fn bit 1: g = x^(-1/2) (inverse square root of an
+// overlap, positive Ritz values; NaN otherwise) instead of the Fermi function; bit 0: g multiplied by x
+// (the energy-weighted density matrix, T_c Z_c).
+template <int B>
+__global__ void __launch_bounds__(128) k_zt(int32_t kd, int32_t b_, int32_t nmax, const int32_t* __restrict__ nblk,
+                                            const int32_t* __restrict__ sys_of_colour, const double* __restrict__ mu,
+                                            const double* __restrict__ kT, const double* __restrict__ U,
+                                            const double* __restrict__ lam, const double* __restrict__ Y,
+                                            double* __restrict__ Z, int fn) {
+  constexpr int NB = B ? B : CSS_MAX_B;
+  constexpr int CH = 32, ROWS = 128;
+  __shared__ double shy[CH * NB], sg[CH];
+  __shared__ double su[ROWS][CH + 1];
+  const int32_t b = B ? B : b_;
   const int32_t c = blockIdx.y;
   const int32_t n = nblk[c] * kd;
-  const int32_t i = blockIdx.x * blockDim.x + threadIdx.x;
+  const int32_t ib = blockIdx.x * ROWS, i = ib + threadIdx.x;
   const double* u = U + (size_t)c * nmax * nmax;
   const int32_t s = sys_of_colour[c];
   const double m_ = mu[s], t_ = kT[s];
-  double acc[CSS_MAX_B];
+  double acc[NB];
 #pragma unroll
-  for (int a = 0; a < CSS_MAX_B; ++a) acc[a] = 0.0;
-  const int32_t CH = 64;
-  for (int32_t k0 = 0; k0 < n; k0 += CH) {
-    const int32_t ke = min(n, k0 + CH);
-    __syncthreads();
-    for (int32_t t = threadIdx.x; t < (ke - k0) * b; t += blockDim.x) {
-      const int32_t kk = k0 + t / b;
-      const double l = lam[(size_t)c * nmax + kk];
-      double fw = (fn & 2) ? (l > 0.0 ? 1.0 / sqrt(l) : __longlong_as_double(0x7ff8000000000000ll))
-                           : css_fermi_dirac(l, m_, t_);
-      if (fn & 1) fw *= l;
-      shy[t] = fw * Y[((size_t)c * nmax) * b + (size_t)k0 * b + t];
-    }
-    __syncthreads();
-    if (i < n)
-      for (int32_t kk = k0; kk < ke; ++kk) {
-        const double uk = u[(size_t)i * nmax + kk];
-#pragma unroll
-        for (int a = 0; a < CSS_MAX_B; ++a)
-          if (a < b) acc[a] = fma(uk, shy[(kk - k0) * b + a], acc[a]);
+  for (int a = 0; a < NB; ++a) acc[a] = 0.0;
+  if (ib < n)  // the whole CTA
+    for (int32_t k0 = 0; k0 < n; k0 += CH) {
+      const int32_t ke = min(n, k0 + CH);
+      __syncthreads();
+      if (threadIdx.x < ke - k0) {
+        const double l = lam[(size_t)c * nmax + k0 + threadIdx.x];
+        double fw = (fn & 2) ? (l > 0.0 ? 1.0 / sqrt(l) : __longlong_as_double(0x7ff8000000000000ll))
+                             : css_fermi_dirac(l, m_, t_);
+        if (fn & 1) fw *= l;
+        sg[threadIdx.x] = fw;
       }
-  }
+      for (int32_t t = threadIdx.x; t < ROWS * CH; t += blockDim.x) {
+        const int32_t r = t / CH, k = t - r * CH;
+        su[r][k] = ib + r < n && k0 + k < ke ? u[(size_t)(ib + r) * nmax + k0 + k] : 0.0;
+      }
+      __syncthreads();
+      for (int32_t t = threadIdx.x; t < (ke - k0) * b; t += blockDim.x)
+        shy[t] = sg[t / b] * Y[((size_t)c * nmax + k0) * b + t];
+      __syncthreads();
+      if (i < n)
+#pragma unroll 4
+        for (int32_t k = 0; k < ke - k0; ++k) {
+          const double uk = su[threadIdx.x][k];
+#pragma unroll
+          for (int a = 0; a < NB; ++a)
+            if (B || a < b) acc[a] = fma(uk, shy[k * b + a], acc[a]);
+        }
+    }
   if (i < nmax) {
 #pragma unroll
-    for (int a = 0; a < CSS_MAX_B; ++a)
-      if (a < b) Z[((size_t)c * nmax + i) * b + a] = (i < n) ? acc[a] : 0.0;
+    for (int a = 0; a < NB; ++a)
+      if (B || a < b) Z[((size_t)c * nmax + i) * b + a] = (i < n) ? acc[a] : 0.0;
   }
 }
 
@@ -1051,6 +1097,34 @@ __global__ void k_shifts_out(int32_t nmax, const float* __restrict__ lam32, doub
 
 namespace {
 
+// Launch of k_apply_refl: the column split that fills the last wave of CTAs best (the largest share of
+// the columns on one SM is smallest), within shared memory
+template <bool FWD>
+css_status launch_refl(css_ctx* ctx, const EigArgs& a, double* X, cudaStream_t st) {
+  const int32_t kd = a.b, b = a.b, nmax = a.m * a.b;
+  auto bytes = [&](int32_t cw) {
+    return sizeof(double) * ((size_t)nmax * cw + 2 * (size_t)(nmax / kd + 1) * (kd + 1));
+  };
+  int32_t best = 1;
+  double least = 1e300;
+  for (int32_t cw = b; cw >= 1; --cw) {
+    const int64_t splits = css_ceil_div(b, cw);
+    if (bytes(cw) > 200 * 1024 || splits > 12) continue;
+    const double load = (double)css_ceil_div((int64_t)a.n_col * splits, ctx->n_sm) * cw;
+    if (load < 0.95 * least) {
+      least = load;
+      best = cw;
+    }
+  }
+  const int32_t tasks = (nmax / kd + 1) * best;
+  const unsigned threads = (unsigned)std::min<int32_t>(1024, (tasks + 31) / 32 * 32);
+  CSS_CU(ctx, cudaFuncSetAttribute(k_apply_refl<FWD>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes(best)));
+  k_apply_refl<FWD><<<dim3((unsigned)a.n_col, (unsigned)css_ceil_div(b, best)), threads, bytes(best), st>>>(
+      kd, b, best, nmax, a.rcap, a.nblk, a.RV, a.RT, X);
+  CSS_LAUNCHED(ctx);
+  return CSS_OK;
+}
+
 // Launch of k_band_to_tri: lanes per sweep from the band width; enough warps for the sweeps that
 // can be in flight (a sweep trails the one before it by about three windows of kd rows, so two per
 // sweep never starve it); the band in shared memory when it fits beside the sweeps' vectors, else
@@ -1061,7 +1135,7 @@ css_status launch_band(css_ctx* ctx, const EigArgs& a, int32_t ldb, cudaStream_t
   constexpr size_t kSmem = 220 * 1024;
   const int32_t kd = a.b, nmax = a.m * a.b;
   const int32_t flight = nmax / (2 * kd) + 1;
-  BandArgs ba{kd, nmax, ldb, a.rcap, 1, a.n_col, a.nblk, a.AB, a.RV, a.RT, a.RR0, nullptr, a.d, a.e, a.status};
+  BandArgs ba{kd, nmax, ldb, a.rcap, 1, a.n_col, a.nblk, a.AB, a.RV, a.RT, nullptr, a.d, a.e, a.status};
   auto warps = [&](int32_t ctas, bool smem) {
     return (int32_t)std::min<int64_t>(smem ? 32 : 16, css_ceil_div(flight, (int64_t)SPW * ctas) + 1);
   };
@@ -1122,11 +1196,10 @@ css_status css_eigen_ritz(css_ctx* ctx, const EigArgs& a, cudaStream_t st) {
   else
     k_x0<<<nc, 256, 0, st>>>(b, nmax, a.cnt, a.X0);
   CSS_LAUNCHED(ctx);
-  k_apply_refl<true><<<nc, 1024, 0, st>>>(b, b, nmax, a.rcap, a.nblk, a.RV, a.RT, a.RR0, a.X0);
-  CSS_LAUNCHED(ctx);
+  CSS_TRY(launch_refl<true>(ctx, a, a.X0, st));
   const size_t sh = 2 * (size_t)nmax * sizeof(float);
   if (sh > 48 * 1024) CSS_CU(ctx, cudaFuncSetAttribute(k_bisect32, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sh));
-  k_bisect32<<<nc, 256, sh, st>>>(b, nmax, a.nblk, a.d, a.e, a.lam32, a.tnorm);
+  k_bisect32<<<dim3((unsigned)nc, (unsigned)css_ceil_div(nmax, 128)), 128, sh, st>>>(b, nmax, a.nblk, a.d, a.e, a.lam32, a.tnorm);
   CSS_LAUNCHED(ctx);
   k_inviter_p1<<<dim3((unsigned)css_ceil_div(nmax, 128), (unsigned)nc), 128, 0, st>>>(
       b, nmax, a.nblk, a.d, a.e, a.lam32, a.tnorm, 1e-4, a.U, a.F, a.lam, a.flag, a.gid);
@@ -1148,7 +1221,8 @@ css_status css_eigen_ritz(css_ctx* ctx, const EigArgs& a, cudaStream_t st) {
     CSS_LAUNCHED(ctx);
   }
   dim3 g((unsigned)css_ceil_div(nmax, 128), (unsigned)nc);
-  k_ritz_y<<<g, 128, 64 * b * sizeof(double), st>>>(b, b, nmax, a.nblk, a.U, a.X0, a.Y, a.wgt);
+  (b == 6 ? k_ritz_y<6> : b == 23 ? k_ritz_y<23> : k_ritz_y<0>)<<<g, 128, 0, st>>>(b, b, nmax, a.nblk, a.U, a.X0, a.Y,
+                                                                                     a.wgt);
   CSS_LAUNCHED(ctx);
   return CSS_OK;
 }
@@ -1157,20 +1231,19 @@ css_status css_eigen_z(css_ctx* ctx, const EigArgs& a, const int32_t* sys_of_col
                        const double* kT, double* Z, cudaStream_t st, int fn) {
   const int32_t nc = a.n_col, b = a.b, nmax = a.m * b;
   dim3 g((unsigned)css_ceil_div(nmax, 128), (unsigned)nc);
-  k_zt<<<g, 128, 64 * b * sizeof(double), st>>>(b, b, nmax, a.nblk, sys_of_colour, mu, kT, a.U, a.lam, a.Y, Z,
-                                                 fn);
+  (b == 6 ? k_zt<6> : b == 23 ? k_zt<23> : k_zt<0>)<<<g, 128, 0, st>>>(b, b, nmax, a.nblk, sys_of_colour, mu, kT, a.U,
+                                                                         a.lam, a.Y, Z, fn);
   CSS_LAUNCHED(ctx);
-  k_apply_refl<false><<<nc, 1024, 0, st>>>(b, b, nmax, a.rcap, a.nblk, a.RV, a.RT, a.RR0, Z);
-  CSS_LAUNCHED(ctx);
+  CSS_TRY(launch_refl<false>(ctx, a, Z, st));
   return CSS_OK;
 }
 
 css_status css_eigen_project(css_ctx* ctx, const EigArgs& a, double* V, double* YV, double* scratch, cudaStream_t st) {
   const int32_t nc = a.n_col, b = a.b, nmax = a.m * b;
-  k_apply_refl<true><<<nc, 1024, 0, st>>>(b, b, nmax, a.rcap, a.nblk, a.RV, a.RT, a.RR0, V);
-  CSS_LAUNCHED(ctx);
+  CSS_TRY(launch_refl<true>(ctx, a, V, st));
   dim3 g((unsigned)css_ceil_div(nmax, 128), (unsigned)nc);
-  k_ritz_y<<<g, 128, 64 * b * sizeof(double), st>>>(b, b, nmax, a.nblk, a.U, V, YV, scratch);
+  (b == 6 ? k_ritz_y<6> : b == 23 ? k_ritz_y<23> : k_ritz_y<0>)<<<g, 128, 0, st>>>(b, b, nmax, a.nblk, a.U, V, YV,
+                                                                                     scratch);
   CSS_LAUNCHED(ctx);
   return CSS_OK;
 }

@@ -28,7 +28,6 @@ struct EigArgs {
   double* AB = nullptr;                // [c][nmax][css_band_ld(b)]
   double* RV = nullptr;                // [c][rcap][b]
   double* RT = nullptr;                // [c][rcap]
-  int32_t* RR0 = nullptr;              // [c][rcap]
   double *d = nullptr, *e = nullptr;   // [c][nmax] tridiagonal
   float* lam32 = nullptr;              // [c][nmax] FP32 shifts
   double* tnorm = nullptr;             // [c]
