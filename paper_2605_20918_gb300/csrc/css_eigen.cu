@@ -10,7 +10,7 @@
 //      b-column blocks is applied sweep by sweep with all of a sweep's reflectors in parallel;
 //   2. eigenvalues of the tridiagonal by Sturm-count bisection in FP32 (one thread per
 //      eigenvalue), used only as shifts;
-//   3. FP64 Rayleigh-quotient inverse iteration: one thread per eigenvalue in lockstep, then
+//   3. Rayleigh-quotient inverse iteration (two FP32 steps, two FP64): one thread per eigenvalue, then
 //      one warp per cluster of close shifts (simultaneous iteration with Gram-Schmidt and a
 //      Rayleigh-Ritz step inside the cluster), which gives eigenvalues and eigenvectors to
 //      FP64 accuracy;
@@ -488,22 +488,165 @@ constexpr int kMaxCluster = 16;
 // at least that residual over the gap to the other eigenvalues.
 constexpr double kResTol = 128.0 * 2.2e-16;
 
-__device__ __forceinline__ double hash_unit(uint64_t a, uint64_t b) {
-  uint64_t z = css_splitmix64(a * 0x9E3779B97F4A7C15ull + 0x5851F42D4C957F2Dull, b);
-  return (double)(z >> 11) * (2.0 / 9007199254740992.0) - 1.0;
+// uniform in [-1, 1)
+__device__ __forceinline__ float hash_unit(uint64_t a, uint64_t b) {
+  const uint64_t z = css_splitmix64(a * 0x9E3779B97F4A7C15ull + 0x5851F42D4C957F2Dull, b);
+  return (float)(int32_t)(z >> 32) * 4.656612873077393e-10f;
 }
 
-// Phase 1 of the FP64 inverse iteration: one thread per eigenvalue, all threads of a colour
-// in lockstep (same loop bounds, fixed four iterations: two at the FP32 shift, two with
-// Rayleigh-quotient shifts), so the column-per-thread accesses to U and the scratch F are
-// coalesced across a warp.  Eigenvalues whose shift lies within tol of a neighbour's (a
-// cluster) and results that did not converge or left their window are flagged for phase 2.
-__global__ void __launch_bounds__(128) k_inviter_p1(int32_t kd, int32_t nmax, const int32_t* __restrict__ nblk,
+constexpr int kCB = 8;  // rows per batch
+
+// Scratch of one solve in the caller's column, nmax apart per row: the rows of U (reciprocal pivot and
+// two super-diagonals) and the right-hand side / solution.
+struct Col64 {
+  using T = double;
+  double *u0, *u1, *u2, *x;
+  size_t ld;
+  __device__ __forceinline__ double rhs(int32_t i) const { return x[i * ld]; }
+  __device__ __forceinline__ void put(int32_t i, double a, double b, double c, double r) const {
+    u0[i * ld] = a;
+    u1[i * ld] = b;
+    u2[i * ld] = c;
+    x[i * ld] = r;
+  }
+  __device__ __forceinline__ void get(int32_t i, double& a, double& b, double& c, double& r) const {
+    a = u0[i * ld];
+    b = u1[i * ld];
+    c = u2[i * ld];
+    r = x[i * ld];
+  }
+  __device__ __forceinline__ void put_x(int32_t i, double y) const { x[i * ld] = y; }
+};
+// the same in FP32, in the 8-byte slots of the FP64 u0 and u1 columns
+struct Col32 {
+  using T = float;
+  float2 *p, *q;  // {u0, u1}, {u2, x}
+  size_t ld;
+  __device__ __forceinline__ float rhs(int32_t i) const { return q[i * ld].y; }
+  __device__ __forceinline__ void put(int32_t i, float a, float b, float c, float r) const {
+    p[i * ld] = make_float2(a, b);
+    q[i * ld] = make_float2(c, r);
+  }
+  __device__ __forceinline__ void get(int32_t i, float& a, float& b, float& c, float& r) const {
+    const float2 v = p[i * ld], w = q[i * ld];
+    a = v.x;
+    b = v.y;
+    c = w.x;
+    r = w.y;
+  }
+  __device__ __forceinline__ void put_x(int32_t i, float y) const { q[i * ld].y = y; }
+};
+
+// |x| as an integer of the same order: an integer comparison where an FP64 one would take the FP64 pipe
+__device__ __forceinline__ long long abs_bits(double x) { return __double_as_longlong(x) & 0x7fffffffffffffffll; }
+__device__ __forceinline__ int abs_bits(float x) { return __float_as_int(x) & 0x7fffffff; }
+
+// LU with partial pivoting of T - sigma I fused with the forward elimination of the column's right-hand
+// side (scaled by scl), then the back substitution U y = x; y overwrites the column.  Returns ||y||^2
+// and, with RQ, y^T T y.  Every sweep over the rows loads a batch of rows before the batch's dependent
+// arithmetic, so a warp keeps several loads in flight.  Lanes with st == false store nothing.
+template <bool RQ, typename Col>
+__device__ typename Col::T shifted_solve(const Col& m, const typename Col::T* __restrict__ d,
+                                         const typename Col::T* __restrict__ e, int32_t n, typename Col::T sigma,
+                                         typename Col::T scl, typename Col::T pivmin, bool st, typename Col::T& rq) {
+  using T = typename Col::T;
+  T cd = d[0] - sigma, cs = n > 1 ? e[0] : T(0);
+  T xc = m.rhs(0) * scl;
+  for (int32_t i0 = 0; i0 + 1 < n; i0 += kCB) {
+    T sub[kCB], dg[kCB], sup[kCB], xn[kCB];
+#pragma unroll
+    for (int q = 0; q < kCB; ++q) {
+      const int32_t i = i0 + q;
+      const bool ok = i + 1 < n;
+      sub[q] = ok ? e[i] : T(1);
+      dg[q] = ok ? d[i + 1] : T(0);
+      sup[q] = (i + 2 < n) ? e[i + 1] : T(0);
+      xn[q] = ok ? m.rhs(i + 1) : T(0);
+    }
+#pragma unroll
+    for (int q = 0; q < kCB; ++q) {
+      const int32_t i = i0 + q;
+      if (i + 1 >= n) break;
+      const T dgs = dg[q] - sigma, xs = xn[q] * scl;
+      // neighbouring lanes hold neighbouring shifts and mostly agree on the pivot, so a branch costs
+      // no more than the selects that would replace it
+      T u0, u1, u2, rhs, ncd, ncs, nx;
+      if (abs_bits(cd) >= abs_bits(sub[q])) {
+        if (abs_bits(cd) < abs_bits(pivmin)) cd = cd >= T(0) ? pivmin : -pivmin;
+        u0 = T(1) / cd;  // the pivot's reciprocal serves the multiplier and the back substitution
+        const T l = sub[q] * u0;
+        u1 = cs;
+        u2 = T(0);
+        rhs = xc;
+        ncd = dgs - l * cs;
+        ncs = sup[q];
+        nx = xs - l * xc;
+      } else {
+        u0 = T(1) / sub[q];
+        const T l = cd * u0;
+        u1 = dgs;
+        u2 = sup[q];
+        rhs = xs;
+        ncd = cs - l * dgs;
+        ncs = -l * sup[q];
+        nx = xc - l * xs;
+      }
+      if (st) m.put(i, u0, u1, u2, rhs);
+      cd = ncd;
+      cs = ncs;
+      xc = nx;
+    }
+  }
+  if (fabs(cd) < pivmin) cd = cd >= T(0) ? pivmin : -pivmin;
+  // back substitution, rows n-1 down to 0, in batches
+  T y1 = xc / cd, y2 = T(0);
+  T ss = y1 * y1;
+  rq = RQ ? ss * d[n - 1] : T(0);
+  if (st) m.put_x(n - 1, y1);
+  for (int32_t i0 = n - 2; i0 >= 0; i0 -= kCB) {
+    T r[kCB], a0[kCB], a1[kCB], a2[kCB], dv[kCB], ev[kCB];
+#pragma unroll
+    for (int q = 0; q < kCB; ++q) {
+      const int32_t i = i0 - q, j = i >= 0 ? i : 0;
+      m.get(j, a0[q], a1[q], a2[q], r[q]);
+      if (RQ) {
+        dv[q] = d[j];
+        ev[q] = e[j];
+      }
+    }
+#pragma unroll
+    for (int q = 0; q < kCB; ++q) {
+      const int32_t i = i0 - q;
+      if (i < 0) break;
+      const T y = (r[q] - a1[q] * y1 - a2[q] * y2) * a0[q];
+      if (st) m.put_x(i, y);
+      ss += y * y;
+      if (RQ) rq += y * (dv[q] * y + T(2) * (ev[q] * y1));
+      y2 = y1;
+      y1 = y;
+    }
+  }
+  return ss;
+}
+
+// Phase 1 of the inverse iteration: one thread per eigenvalue, all threads of a colour in lockstep
+// (same loop bounds, fixed four iterations), so the column-per-thread accesses to the scratch are
+// coalesced across a warp.  The first two iterations run at the FP32 shift and in FP32: they only have
+// to bring the random start vector to the eigenvector within FP32 rounding over the gap (which is at
+// least 1e-4 ||T|| here), from where the two FP64 iterations with Rayleigh-quotient shifts converge
+// cubically.  Eigenvalues whose shift lies within tol of a neighbour's (a cluster) and results that did
+// not converge or left their window are flagged for phase 2.
+// Bound by FP64 issue (64 clocks of a scheduler per instruction, ~19 a row and solve).  With all four
+// iterations, the start vector and separate Rayleigh-quotient passes in FP64 n = 920, 63 colours took
+// 14.8 ms and n = 180, 62 colours 1.29 ms; now 8.7 and 0.61 (four CTAs per SM: with the 168 registers
+// the compiler takes otherwise, 10.3 ms).
+__global__ void __launch_bounds__(128, 4) k_inviter_p1(int32_t kd, int32_t nmax, const int32_t* __restrict__ nblk,
                                                     const double* __restrict__ dd, const double* __restrict__ ee,
                                                     const float* __restrict__ lam32, const double* __restrict__ tnorm,
                                                     double rel_cluster, double* __restrict__ U,
                                                     double* __restrict__ F, double* __restrict__ lam,
                                                     int32_t* __restrict__ flag, const int32_t* __restrict__ gid) {
+  extern __shared__ float p1_smem[];
   const int32_t c = blockIdx.y;
   const uint64_t cseed = gid ? (uint64_t)gid[c] : (uint64_t)c;  // the colour's own id seeds its start vectors
   const int32_t n = nblk[c] * kd;
@@ -512,19 +655,18 @@ __global__ void __launch_bounds__(128) k_inviter_p1(int32_t kd, int32_t nmax, co
   const double* d = dd + (size_t)c * nmax;
   const double* e = ee + (size_t)c * nmax;
   const float* l32 = lam32 + (size_t)c * nmax;
-  double* u = U + (size_t)c * nmax * nmax;
-  double* f_u0 = F + (size_t)c * 5 * nmax * nmax;
-  double* f_u1 = f_u0 + (size_t)nmax * nmax;
-  double* f_u2 = f_u1 + (size_t)nmax * nmax;
-  double* f_x = f_u2 + (size_t)nmax * nmax;
-  int32_t* fl = flag + (size_t)c * nmax;
+  float *d32 = p1_smem, *e32 = p1_smem + nmax;
+  for (int32_t i = threadIdx.x; i < n; i += blockDim.x) {
+    d32[i] = (float)d[i];
+    e32[i] = i + 1 < n ? (float)e[i] : 0.0f;
+  }
+  __syncthreads();
   const double tn = tnorm[c];
   const double tol = rel_cluster * tn;
-  const double pivmin = 2.2e-16 * tn;
   const double res_tol = kResTol * tn;
   const bool valid = k < n;
   bool in_cluster = false;
-  double win_lo = 0.0, win_hi = 0.0, sigma = 0.0;
+  double win_lo = 0.0, win_hi = 0.0;
   if (valid) {
     const double lk = (double)l32[k];
     const double g_lo = k > 0 ? lk - (double)l32[k - 1] : tn;
@@ -532,93 +674,52 @@ __global__ void __launch_bounds__(128) k_inviter_p1(int32_t kd, int32_t nmax, co
     in_cluster = g_lo <= tol || g_hi <= tol;
     win_lo = lk - 0.25 * g_lo - 2e-6 * tn;
     win_hi = lk + 0.25 * g_hi + 2e-6 * tn;
-    sigma = lk;
   }
   const bool work = valid && !in_cluster;
-  // start vector, normalised
-  double nrm = 0.0;
-  for (int32_t i = 0; i < n; ++i) {
-    const double x = work ? hash_unit(cseed * 1000003ull + (uint64_t)k, (uint64_t)i) : 0.0;
-    if (work) f_x[(size_t)i * nmax + k] = x;
-    nrm += x * x;
+  if (!__any_sync(0xffffffffu, work)) {
+    if (valid) flag[(size_t)c * nmax + k] = 1;
+    return;
   }
-  double inv = work ? 1.0 / sqrt(nrm) : 0.0;
-  double growth = 0.0;
-  for (int it = 0; it < 4; ++it) {
-    // factor T - sigma I with partial pivoting and eliminate on x in the same sweep; the rows
-    // of U are stored, x is overwritten by L^-1 P x (scaled by inv)
-    double cd = d[0] - sigma, cs = n > 1 ? e[0] : 0.0;
-    double xc = work ? f_x[k] * inv : 0.0;  // current row's right-hand side
-    for (int32_t i = 0; i + 1 < n; ++i) {
-      const double sub = e[i], dg = d[i + 1] - sigma, sup = (i + 2 < n) ? e[i + 1] : 0.0;
-      const double xn = work ? f_x[(size_t)(i + 1) * nmax + k] * inv : 0.0;
-      double u0, u1, u2, rhs_i, ncd, ncs, nx;
-      if (fabs(cd) >= fabs(sub)) {
-        if (fabs(cd) < pivmin) cd = cd >= 0 ? pivmin : -pivmin;
-        u0 = 1.0 / cd;  // the pivot's reciprocal serves the multiplier and the back substitution
-        const double l = sub * u0;
-        u1 = cs;
-        u2 = 0.0;
-        rhs_i = xc;
-        ncd = dg - l * cs;
-        ncs = sup;
-        nx = xn - l * xc;
-      } else {
-        u0 = 1.0 / sub;
-        const double l = cd * u0;
-        u1 = dg;
-        u2 = sup;
-        rhs_i = xn;
-        ncd = cs - l * dg;
-        ncs = -l * sup;
-        nx = xc - l * xn;
-      }
-      if (work) {
-        f_u0[(size_t)i * nmax + k] = u0;
-        f_u1[(size_t)i * nmax + k] = u1;
-        f_u2[(size_t)i * nmax + k] = u2;
-        f_x[(size_t)i * nmax + k] = rhs_i;
-      }
-      cd = ncd;
-      cs = ncs;
-      xc = nx;
+  // idle lanes shadow the colour's last column and store nothing
+  const size_t nn = (size_t)nmax * nmax, col = valid ? k : n - 1;
+  double* f = F + (size_t)c * 5 * nn + col;
+  const Col64 m{f, f + nn, f + 2 * nn, f + 3 * nn, (size_t)nmax};
+  const Col32 m32{reinterpret_cast<float2*>(f), reinterpret_cast<float2*>(f + nn), (size_t)nmax};
+  if (work)
+    for (int32_t i = 0; i < n; ++i) m32.put_x(i, hash_unit(cseed * 1000003ull + (uint64_t)k, (uint64_t)i));
+  float ss = (float)n * (1.0f / 3.0f), none;  // the start vector's expected square norm
+  for (int it = 0; it < 2; ++it)
+    ss = shifted_solve<false>(m32, d32, e32, n, l32[col], rsqrtf(ss), 1.2e-7f * (float)tn, work, none);
+  // its Rayleigh quotient, and the vector in FP64
+  double s2 = 0.0, rq = 0.0, prev = 0.0;
+  for (int32_t i0 = 0; i0 < n; i0 += kCB) {
+    float x[kCB];
+#pragma unroll
+    for (int q = 0; q < kCB; ++q) x[q] = i0 + q < n ? m32.rhs(i0 + q) : 0.0f;
+#pragma unroll
+    for (int q = 0; q < kCB; ++q) {
+      const int32_t i = i0 + q;
+      if (i >= n) break;
+      const double y = (double)x[q];
+      if (work) m.put_x(i, y);
+      s2 += y * y;
+      rq += y * (d[i] * y + (i > 0 ? 2.0 * (e[i - 1] * prev) : 0.0));
+      prev = y;
     }
-    if (fabs(cd) < pivmin) cd = cd >= 0 ? pivmin : -pivmin;
-    // backward substitution U y = x, then the norm
-    double y1 = 0.0, y2 = 0.0, ss = 0.0;
-    for (int32_t i = n - 1; i >= 0; --i) {
-      double r, u0;  // u0: the reciprocal of the row's pivot
-      if (i == n - 1) {
-        r = xc;
-        u0 = 1.0 / cd;
-      } else {
-        r = work ? f_x[(size_t)i * nmax + k] : 0.0;
-        u0 = work ? f_u0[(size_t)i * nmax + k] : 1.0;
-        if (work) r -= f_u1[(size_t)i * nmax + k] * y1;
-        if (work && i + 2 < n) r -= f_u2[(size_t)i * nmax + k] * y2;
-      }
-      const double y = work ? r * u0 : 0.0;
-      if (work) f_x[(size_t)i * nmax + k] = y;
-      ss += y * y;
-      y2 = y1;
-      y1 = y;
-    }
-    growth = sqrt(ss);
-    inv = work ? 1.0 / growth : 0.0;
-    // Rayleigh quotient of the normalised vector
-    double rq = 0.0, prev = 0.0;
-    for (int32_t i = 0; i < n; ++i) {
-      const double xi = work ? f_x[(size_t)i * nmax + k] * inv : 0.0;
-      rq += xi * (d[i] * xi + 2.0 * (i > 0 ? e[i - 1] * prev : 0.0));
-      prev = xi;
-    }
-    if (it >= 1) sigma = rq;
+  }
+  double sigma = rq / s2, scl = rsqrt(s2), growth = 0.0;
+  for (int it = 0; it < 2; ++it) {
+    const double y2 = shifted_solve<true>(m, d, e, n, sigma, scl, 2.2e-16 * tn, work, rq);
+    growth = sqrt(y2);
+    scl = 1.0 / growth;
+    sigma = rq / y2;
   }
   if (!valid) return;
   const bool ok = work && growth * res_tol > 1.0 && sigma >= win_lo && sigma <= win_hi;
-  fl[k] = ok ? 0 : 1;
+  flag[(size_t)c * nmax + k] = ok ? 0 : 1;
   if (!ok) return;
-  for (int32_t i = 0; i < n; ++i) u[(size_t)i * nmax + k] = f_x[(size_t)i * nmax + k] * inv;
+  double* u = U + (size_t)c * nn + k;
+  for (int32_t i = 0; i < n; ++i) u[(size_t)i * nmax] = m.x[(size_t)i * nmax] * scl;
   lam[(size_t)c * nmax + k] = sigma;
 }
 
@@ -627,106 +728,8 @@ __global__ void __launch_bounds__(128) k_inviter_p1(int32_t kd, int32_t nmax, co
 // of the scratch X and its LU factors columns k0 + j of U0..U2, so the lanes of a warp touch
 // contiguous addresses of a row.  Every member solves with its own shift, then the members are
 // orthonormalised by modified Gram-Schmidt in member order (simultaneous inverse iteration);
-// Rayleigh-Ritz inside the cluster gives the final pairs.  Every sweep over the rows loads a
-// batch of rows before the batch's dependent arithmetic, so one warp keeps several loads in
-// flight.
-constexpr int kCB = 8;  // rows per batch
-
-struct ClusterCols {
-  const double* d;
-  const double* e;
-  double* u0;
-  double* u1;
-  double* u2;
-  double* x;
-  int32_t n, nmax;
-};
-
-// LU with partial pivoting of T - sigma I fused with the forward elimination of column col of
-// X (scaled by scl), then the back substitution U y = x; y overwrites the column.  Returns ||y||.
-// Lanes with st == false compute but store nothing.
-__device__ double cl_solve(const ClusterCols& m, int32_t col, double sigma, double scl, double pivmin, bool st) {
-  const int32_t n = m.n, nmax = m.nmax;
-  double cd = m.d[0] - sigma, cs = n > 1 ? m.e[0] : 0.0;
-  double xc = m.x[col] * scl;
-  for (int32_t i0 = 0; i0 + 1 < n; i0 += kCB) {
-    double sub[kCB], dg[kCB], sup[kCB], xn[kCB];
-#pragma unroll
-    for (int q = 0; q < kCB; ++q) {
-      const int32_t i = i0 + q;
-      const bool ok = i + 1 < n;
-      sub[q] = ok ? m.e[i] : 1.0;
-      dg[q] = ok ? m.d[i + 1] - sigma : 0.0;
-      sup[q] = (i + 2 < n) ? m.e[i + 1] : 0.0;
-      xn[q] = ok ? m.x[(size_t)(i + 1) * nmax + col] * scl : 0.0;
-    }
-#pragma unroll
-    for (int q = 0; q < kCB; ++q) {
-      const int32_t i = i0 + q;
-      if (i + 1 >= n) break;
-      double u0, u1, u2, rhs, ncd, ncs, nx;
-      if (fabs(cd) >= fabs(sub[q])) {
-        if (fabs(cd) < pivmin) cd = cd >= 0 ? pivmin : -pivmin;
-        u0 = 1.0 / cd;  // the pivot's reciprocal serves the multiplier and the back substitution
-        const double l = sub[q] * u0;
-        u1 = cs;
-        u2 = 0.0;
-        rhs = xc;
-        ncd = dg[q] - l * cs;
-        ncs = sup[q];
-        nx = xn[q] - l * xc;
-      } else {
-        u0 = 1.0 / sub[q];
-        const double l = cd * u0;
-        u1 = dg[q];
-        u2 = sup[q];
-        rhs = xn[q];
-        ncd = cs - l * dg[q];
-        ncs = -l * sup[q];
-        nx = xc - l * xn[q];
-      }
-      if (st) {
-        m.u0[(size_t)i * nmax + col] = u0;
-        m.u1[(size_t)i * nmax + col] = u1;
-        m.u2[(size_t)i * nmax + col] = u2;
-        m.x[(size_t)i * nmax + col] = rhs;
-      }
-      cd = ncd;
-      cs = ncs;
-      xc = nx;
-    }
-  }
-  if (fabs(cd) < pivmin) cd = cd >= 0 ? pivmin : -pivmin;
-  // back substitution, rows n-1 down to 0, in batches
-  double y1 = xc / cd, y2 = 0.0;
-  double ss = y1 * y1;
-  if (st) m.x[(size_t)(n - 1) * nmax + col] = y1;
-  for (int32_t i0 = n - 2; i0 >= 0; i0 -= kCB) {
-    double r[kCB], a0[kCB], a1[kCB], a2[kCB];
-#pragma unroll
-    for (int q = 0; q < kCB; ++q) {
-      const int32_t i = i0 - q;
-      const bool ok = i >= 0;
-      const size_t o = (size_t)(ok ? i : 0) * nmax + col;
-      r[q] = ok ? m.x[o] : 0.0;
-      a0[q] = ok ? m.u0[o] : 1.0;
-      a1[q] = ok ? m.u1[o] : 0.0;
-      a2[q] = ok ? m.u2[o] : 0.0;
-    }
-#pragma unroll
-    for (int q = 0; q < kCB; ++q) {
-      const int32_t i = i0 - q;
-      if (i < 0) break;
-      const double y = (r[q] - a1[q] * y1 - a2[q] * y2) * a0[q];
-      if (st) m.x[(size_t)i * nmax + col] = y;
-      ss += y * y;
-      y2 = y1;
-      y1 = y;
-    }
-  }
-  return sqrt(ss);
-}
-
+// Rayleigh-Ritz inside the cluster gives the final pairs.  A single eigenvalue takes its norm and
+// Rayleigh quotient from the solve and skips the orthonormalisation.
 // Work list of phase 2: (colour, first member, members) of every cluster of close shifts (runs
 // cut every kMaxCluster members) that holds a member phase 1 did not finish; one thread per shift,
 // the order of the list does not matter (every item writes only its own columns)
@@ -750,8 +753,11 @@ __global__ void k_cl_items(int32_t kd, int32_t nmax, const int32_t* __restrict__
   items[atomicAdd(count, 1)] = make_int4(c, k, k1 - k + 1, 0);
 }
 
-// one warp per work item of k_cl_items (warps past the list's length return)
-__global__ void __launch_bounds__(256) k_inviter_cl(int32_t kd, int32_t nmax, const int32_t* __restrict__ nblk,
+// one warp, a CTA of its own, per work item of k_cl_items (CTAs past the list's length return), so that
+// the items of small systems spread over the SMs: eight to a CTA, 48 items of 62 colours shared six SMs.
+// With that, the shuffles of the cluster products bounded by the cluster's size and the cheaper solves:
+// n = 180, 62 colours 1.84 -> 0.94 ms, n = 920, 63 colours 10.4 -> 8.2 ms
+__global__ void __launch_bounds__(32) k_inviter_cl(int32_t kd, int32_t nmax, const int32_t* __restrict__ nblk,
                                                     const double* __restrict__ dd, const double* __restrict__ ee,
                                                     const float* __restrict__ lam32,
                                                     const double* __restrict__ tnorm, double rel_cluster,
@@ -759,11 +765,11 @@ __global__ void __launch_bounds__(256) k_inviter_cl(int32_t kd, int32_t nmax, co
                                                     double* __restrict__ lam, int32_t* __restrict__ status,
                                                     const int32_t* __restrict__ gid, const int32_t* __restrict__ count,
                                                     const int4* __restrict__ items) {
-  __shared__ double sC[8][kMaxCluster][kMaxCluster + 1];
-  __shared__ double sV[8][kMaxCluster][kMaxCluster + 1];
+  __shared__ double sC[kMaxCluster][kMaxCluster + 1];
+  __shared__ double sV[kMaxCluster][kMaxCluster + 1];
   constexpr unsigned FULL = 0xffffffffu;
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int32_t item = blockIdx.x * (blockDim.x >> 5) + warp;
+  const int lane = threadIdx.x;
+  const int32_t item = blockIdx.x;
   if (item >= *count) return;  // uniform over the warp
   const int4 it4 = items[item];
   const int32_t c = it4.x, k0 = it4.y, kc = it4.z, k1 = k0 + kc - 1;
@@ -771,15 +777,11 @@ __global__ void __launch_bounds__(256) k_inviter_cl(int32_t kd, int32_t nmax, co
   const int32_t n = nblk[c] * kd;
   const float* l32 = lam32 + (size_t)c * nmax;
   double* u = U + (size_t)c * nmax * nmax;
-  ClusterCols m;
-  m.d = dd + (size_t)c * nmax;
-  m.e = ee + (size_t)c * nmax;
-  m.u0 = F + (size_t)c * 5 * nmax * nmax;
-  m.u1 = m.u0 + (size_t)nmax * nmax;
-  m.u2 = m.u1 + (size_t)nmax * nmax;
-  m.x = m.u2 + (size_t)nmax * nmax;
-  m.n = n;
-  m.nmax = nmax;
+  const double* d = dd + (size_t)c * nmax;
+  const double* e = ee + (size_t)c * nmax;
+  const size_t nn = (size_t)nmax * nmax;
+  double* f0 = F + (size_t)c * 5 * nn;
+  double* xm = f0 + 3 * nn;
   const double tn = tnorm[c];
   const double pivmin = 2.2e-16 * tn;
   const double res_tol = kResTol * tn;
@@ -788,6 +790,7 @@ __global__ void __launch_bounds__(256) k_inviter_cl(int32_t kd, int32_t nmax, co
     {
       const bool act = lane < kc;
       const int32_t col = k0 + (act ? lane : 0);  // idle lanes shadow member 0 and store nothing
+      const Col64 m{f0 + col, f0 + nn + col, f0 + 2 * nn + col, f0 + 3 * nn + col, (size_t)nmax};
       const double g_lo = k0 > 0 ? (double)l32[k0] - (double)l32[k0 - 1] : tn;
       const double g_hi = k1 + 1 < n ? (double)l32[k1 + 1] - (double)l32[k1] : tn;
       const double win_lo = (double)l32[k0] - 0.25 * g_lo - 2e-6 * tn;
@@ -795,23 +798,23 @@ __global__ void __launch_bounds__(256) k_inviter_cl(int32_t kd, int32_t nmax, co
       double lamj = 0.0;
       bool ok_all = false;
       for (int attempt = 0; attempt < 3 && !ok_all; ++attempt) {
-        // start vectors (norm folded into the first solve's right-hand side)
-        double nrm = 0.0;
-        for (int32_t i0 = 0; i0 < n; i0 += kCB) {
-#pragma unroll
-          for (int q = 0; q < kCB; ++q) {
-            const int32_t i = i0 + q;
-            if (i < n) {
-              const double x = hash_unit(cseed * 1000003ull + (uint64_t)col + 7919ull * attempt, (uint64_t)i);
-              if (act) m.x[(size_t)i * nmax + col] = x;
-              nrm += x * x;
-            }
-          }
-        }
-        double scl = 1.0 / sqrt(nrm);
+        // start vectors (their expected norm folded into the first solve's right-hand side)
+        if (act)
+          for (int32_t i = 0; i < n; ++i)
+            xm[(size_t)i * nmax + col] = hash_unit(cseed * 1000003ull + (uint64_t)col + 7919ull * attempt, (uint64_t)i);
+        double scl = sqrt(3.0 / (double)n);
         double sigma = (double)l32[col];
         for (int it = 0; it < 8; ++it) {
-          const double growth = cl_solve(m, col, sigma, scl, pivmin, act);
+          double rq1;
+          const double y2 = kc > 1 ? shifted_solve<false>(m, d, e, n, sigma, scl, pivmin, act, rq1)
+                                   : shifted_solve<true>(m, d, e, n, sigma, scl, pivmin, act, rq1);
+          const double growth = sqrt(y2);
+          if (kc == 1) {
+            scl = 1.0 / growth;
+            if (it >= 1) sigma = rq1 / y2;
+            if (__all_sync(FULL, !act || (it >= 2 && growth * res_tol > 1.0))) break;
+            continue;
+          }
           // modified Gram-Schmidt in member order; pass s subtracts the projection on member s-1
           // (coefficient from pass s-1) and takes the inner products with member s
           double cprev = 0.0, nrm2 = 1.0;
@@ -820,7 +823,7 @@ __global__ void __launch_bounds__(256) k_inviter_cl(int32_t kd, int32_t nmax, co
             for (int32_t i0 = 0; i0 < n; i0 += kCB) {
               double v[kCB];
 #pragma unroll
-              for (int q = 0; q < kCB; ++q) v[q] = (i0 + q < n) ? m.x[(size_t)(i0 + q) * nmax + col] : 0.0;
+              for (int q = 0; q < kCB; ++q) v[q] = (i0 + q < n) ? xm[(size_t)(i0 + q) * nmax + col] : 0.0;
 #pragma unroll
               for (int q = 0; q < kCB; ++q) {
                 if (s > 0) {
@@ -833,7 +836,7 @@ __global__ void __launch_bounds__(256) k_inviter_cl(int32_t kd, int32_t nmax, co
               if (s > 0 && act && lane >= s) {
 #pragma unroll
                 for (int q = 0; q < kCB; ++q)
-                  if (i0 + q < n) m.x[(size_t)(i0 + q) * nmax + col] = v[q];
+                  if (i0 + q < n) xm[(size_t)(i0 + q) * nmax + col] = v[q];
               }
             }
             const double ds = __shfl_sync(FULL, dj, s);
@@ -848,15 +851,15 @@ __global__ void __launch_bounds__(256) k_inviter_cl(int32_t kd, int32_t nmax, co
 #pragma unroll
             for (int q = 0; q < kCB; ++q) {
               const int32_t i = i0 + q;
-              v[q] = i < n ? m.x[(size_t)i * nmax + col] * r : 0.0;
-              dv[q] = i < n ? m.d[i] : 0.0;
-              ev[q] = (i > 0 && i < n) ? m.e[i - 1] : 0.0;
+              v[q] = i < n ? xm[(size_t)i * nmax + col] * r : 0.0;
+              dv[q] = i < n ? d[i] : 0.0;
+              ev[q] = (i > 0 && i < n) ? e[i - 1] : 0.0;
             }
 #pragma unroll
             for (int q = 0; q < kCB; ++q) {
               rq += v[q] * (dv[q] * v[q] + 2.0 * ev[q] * prev);
               prev = v[q];
-              if (act && i0 + q < n) m.x[(size_t)(i0 + q) * nmax + col] = v[q];
+              if (act && i0 + q < n) xm[(size_t)(i0 + q) * nmax + col] = v[q];
             }
           }
           scl = 1.0;
@@ -865,30 +868,31 @@ __global__ void __launch_bounds__(256) k_inviter_cl(int32_t kd, int32_t nmax, co
           if (__all_sync(FULL, !act || conv)) break;
         }
         lamj = sigma;
+        const double fin = kc > 1 ? 1.0 : scl;  // a single vector is normalised as it is written
         if (kc > 1) {
           // Rayleigh-Ritz inside the cluster: C = X^T T X, column j accumulated by lane j
           double cc[kMaxCluster];
 #pragma unroll
           for (int a = 0; a < kMaxCluster; ++a) cc[a] = 0.0;
           double xprev = 0.0;
-          double xcur = m.x[col];
+          double xcur = xm[col];
           for (int32_t i0 = 0; i0 < n; i0 += kCB) {
             double xnx[kCB], dv[kCB], elo[kCB], ehi[kCB];
 #pragma unroll
             for (int q = 0; q < kCB; ++q) {
               const int32_t i = i0 + q;
-              xnx[q] = (i + 1 < n) ? m.x[(size_t)(i + 1) * nmax + col] : 0.0;
-              dv[q] = i < n ? m.d[i] : 0.0;
-              elo[q] = (i > 0 && i < n) ? m.e[i - 1] : 0.0;
-              ehi[q] = (i + 1 < n) ? m.e[i] : 0.0;
+              xnx[q] = (i + 1 < n) ? xm[(size_t)(i + 1) * nmax + col] : 0.0;
+              dv[q] = i < n ? d[i] : 0.0;
+              elo[q] = (i > 0 && i < n) ? e[i - 1] : 0.0;
+              ehi[q] = (i + 1 < n) ? e[i] : 0.0;
             }
 #pragma unroll
             for (int q = 0; q < kCB; ++q) {
               const double tx = dv[q] * xcur + elo[q] * xprev + ehi[q] * xnx[q];
 #pragma unroll
               for (int a = 0; a < kMaxCluster; ++a) {
-                const double xa = __shfl_sync(FULL, xcur, a);
-                if (a < kc) cc[a] = fma(xa, tx, cc[a]);
+                if (a >= kc) break;  // the whole warp
+                cc[a] = fma(__shfl_sync(FULL, xcur, a), tx, cc[a]);
               }
               xprev = xcur;
               xcur = xnx[q];
@@ -897,11 +901,11 @@ __global__ void __launch_bounds__(256) k_inviter_cl(int32_t kd, int32_t nmax, co
           if (act)
 #pragma unroll
             for (int a = 0; a < kMaxCluster; ++a)
-              if (a < kc) sC[warp][a][lane] = cc[a];
+              if (a < kc) sC[a][lane] = cc[a];
           __syncwarp();
           if (lane == 0) {
-            double (*C)[kMaxCluster + 1] = sC[warp];
-            double (*V)[kMaxCluster + 1] = sV[warp];
+            double (*C)[kMaxCluster + 1] = sC;
+            double (*V)[kMaxCluster + 1] = sV;
             for (int32_t a = 0; a < kc; ++a)
               for (int32_t q = 0; q < kc; ++q) V[a][q] = a == q ? 1.0 : 0.0;
             for (int32_t a = 0; a < kc; ++a)
@@ -940,27 +944,27 @@ __global__ void __launch_bounds__(256) k_inviter_cl(int32_t kd, int32_t nmax, co
             }
           }
           __syncwarp();
-          lamj = act ? sC[warp][lane][lane] : 0.0;
+          lamj = act ? sC[lane][lane] : 0.0;
         }
         ok_all = __all_sync(FULL, !act || (lamj >= win_lo && lamj <= win_hi));
         if (!ok_all && attempt < 2) continue;
         // write the eigenvectors: X (rotated by V inside a cluster) into U
         double vcol[kMaxCluster];
 #pragma unroll
-        for (int a = 0; a < kMaxCluster; ++a) vcol[a] = (kc > 1 && act && a < kc) ? sV[warp][a][lane] : 0.0;
+        for (int a = 0; a < kMaxCluster; ++a) vcol[a] = (kc > 1 && act && a < kc) ? sV[a][lane] : 0.0;
         for (int32_t i0 = 0; i0 < n; i0 += kCB) {
           double v[kCB];
 #pragma unroll
-          for (int q = 0; q < kCB; ++q) v[q] = (i0 + q < n) ? m.x[(size_t)(i0 + q) * nmax + col] : 0.0;
+          for (int q = 0; q < kCB; ++q) v[q] = (i0 + q < n) ? xm[(size_t)(i0 + q) * nmax + col] : 0.0;
 #pragma unroll
           for (int q = 0; q < kCB; ++q) {
-            double o = v[q];
+            double o = v[q] * fin;
             if (kc > 1) {
               o = 0.0;
 #pragma unroll
               for (int a = 0; a < kMaxCluster; ++a) {
-                const double xa = __shfl_sync(FULL, v[q], a);
-                if (a < kc) o = fma(xa, vcol[a], o);
+                if (a >= kc) break;  // the whole warp
+                o = fma(__shfl_sync(FULL, v[q], a), vcol[a], o);
               }
             }
             if (act && i0 + q < n) u[(size_t)(i0 + q) * nmax + col] = o;
@@ -1201,7 +1205,7 @@ css_status css_eigen_ritz(css_ctx* ctx, const EigArgs& a, cudaStream_t st) {
   if (sh > 48 * 1024) CSS_CU(ctx, cudaFuncSetAttribute(k_bisect32, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sh));
   k_bisect32<<<dim3((unsigned)nc, (unsigned)css_ceil_div(nmax, 128)), 128, sh, st>>>(b, nmax, a.nblk, a.d, a.e, a.lam32, a.tnorm);
   CSS_LAUNCHED(ctx);
-  k_inviter_p1<<<dim3((unsigned)css_ceil_div(nmax, 128), (unsigned)nc), 128, 0, st>>>(
+  k_inviter_p1<<<dim3((unsigned)css_ceil_div(nmax, 128), (unsigned)nc), 128, 2 * (size_t)nmax * sizeof(float), st>>>(
       b, nmax, a.nblk, a.d, a.e, a.lam32, a.tnorm, 1e-4, a.U, a.F, a.lam, a.flag, a.gid);
   CSS_LAUNCHED(ctx);
   // phase 2 on a compact list: one warp per flagged cluster of any colour
@@ -1213,8 +1217,8 @@ css_status css_eigen_ritz(css_ctx* ctx, const EigArgs& a, cudaStream_t st) {
   k_cl_items<<<dim3((unsigned)css_ceil_div(nmax, 128), (unsigned)nc), 128, 0, st>>>(b, nmax, a.nblk, a.lam32, a.tnorm,
                                                                                    1e-4, a.flag, cl_count, cl_items);
   CSS_LAUNCHED(ctx);
-  k_inviter_cl<<<(unsigned)css_ceil_div((int64_t)nc * nmax, 8), 256, 0, st>>>(
-      b, nmax, a.nblk, a.d, a.e, a.lam32, a.tnorm, 1e-4, a.U, a.F, a.lam, a.status, a.gid, cl_count, cl_items);
+  k_inviter_cl<<<(unsigned)(nc * nmax), 32, 0, st>>>(b, nmax, a.nblk, a.d, a.e, a.lam32, a.tnorm, 1e-4, a.U, a.F, a.lam,
+                                                   a.status, a.gid, cl_count, cl_items);
   CSS_LAUNCHED(ctx);
   if (ctx->debug_eig == 1) {
     k_shifts_out<<<nc, 256, 0, st>>>(nmax, a.lam32, a.lam);
