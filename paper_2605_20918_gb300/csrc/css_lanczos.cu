@@ -55,12 +55,16 @@ __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commi
 template <int N>
 __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;\n" ::"n"(N) : "memory"); }
 
-template <typename T, int BM, int TC, int NT>
+// B: the block width when the products are instantiated for it (FP64, b = 6 and 23: the zero rows and
+// columns of the padded block are left out, 576 -> 529 and 64 -> 36 of its FMAs at 64 clocks of a
+// scheduler each), 0 for any b <= BM.
+template <typename T, int BM, int TC, int NT, int B>
 __global__ void __launch_bounds__(NT) k_spmm(int32_t b, const int32_t* __restrict__ row_ptr,
                                               const int32_t* __restrict__ col_idx, const T* __restrict__ Ht,
                                               const T* __restrict__ V, T* __restrict__ W, int32_t ws, int32_t w,
                                               const T* __restrict__ Hlo_t, int32_t jbase) {
   using C = SpmmCfg<T, BM, TC, NT>;
+  constexpr int KA = B ? B : BM;  // rows and columns of a block that are multiplied
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int32_t I = blockIdx.x;
   const int32_t t = threadIdx.x;
@@ -81,7 +85,7 @@ __global__ void __launch_bounds__(NT) k_spmm(int32_t b, const int32_t* __restric
     T* vd = stage_v(s) + TC * t;
     const T* vsrc = V + (size_t)J * b * ws + (col < w ? col : 0);
 #pragma unroll
-    for (int k = 0; k < BM; ++k)
+    for (int k = 0; k < KA; ++k)
       cp_async_chunk<C::CH>(vd + (size_t)k * C::CT, vsrc + (size_t)(k < b ? k : 0) * ws, k < b ? cbytes : 0);
     cp_async_commit();
   };
@@ -92,13 +96,13 @@ __global__ void __launch_bounds__(NT) k_spmm(int32_t b, const int32_t* __restric
   constexpr bool PACK = sizeof(T) == 4;
   constexpr int AP = PACK ? BM / 2 : 1;
   unsigned long long acc2[AP][TC];
-  T acc[PACK ? 1 : BM][TC];
+  T acc[PACK ? 1 : KA][TC];
 #pragma unroll
   for (int a = 0; a < AP; ++a)
 #pragma unroll
     for (int u = 0; u < TC; ++u) acc2[a][u] = 0ull;
 #pragma unroll
-  for (int a = 0; a < (PACK ? 1 : BM); ++a)
+  for (int a = 0; a < (PACK ? 1 : KA); ++a)
 #pragma unroll
     for (int u = 0; u < TC; ++u) acc[a][u] = T(0);
   if (nsteps > 0) {
@@ -137,12 +141,12 @@ __global__ void __launch_bounds__(NT) k_spmm(int32_t b, const int32_t* __restric
           }
         } else {
 #pragma unroll 4
-          for (int k = 0; k < BM; ++k) {
+          for (int k = 0; k < KA; ++k) {
             T v[TC];
 #pragma unroll
             for (int u = 0; u < TC; ++u) v[u] = vs[(size_t)k * C::CT + u];
 #pragma unroll
-            for (int a = 0; a < BM; ++a) {
+            for (int a = 0; a < KA; ++a) {
               const T h = hs[k * BM + a];
 #pragma unroll
               for (int u = 0; u < TC; ++u) acc[a][u] = fma(h, v[u], acc[a][u]);
@@ -164,7 +168,7 @@ __global__ void __launch_bounds__(NT) k_spmm(int32_t b, const int32_t* __restric
     }
   };
 #pragma unroll
-  for (int a = 0; a < BM; ++a) {
+  for (int a = 0; a < KA; ++a) {
     if (a >= b) break;
     if (cbytes == C::CH) {
       if constexpr (C::CH == 16 && sizeof(T) == 4) {
@@ -1199,10 +1203,10 @@ css_status smem_optin(css_ctx* ctx, K kern, size_t bytes) {
   return CSS_OK;
 }
 
-template <typename T, int BM, int TC, int NT>
+template <typename T, int BM, int TC, int NT, int B>
 css_status launch_spmm_t(css_ctx* ctx, const LzArgs& a, const T* V, T* W, cudaStream_t st) {
   using C = SpmmCfg<T, BM, TC, NT>;
-  auto kern = k_spmm<T, BM, TC, NT>;
+  auto kern = k_spmm<T, BM, TC, NT, B>;
   CSS_TRY(smem_optin(ctx, kern, C::smem));
   dim3 grid((unsigned)a.n_brow, (unsigned)css_ceil_div(a.w, C::CT));
   kern<<<grid, C::NT, C::smem, st>>>(a.b, a.row_ptr, a.col_idx, (const T*)a.Hval, V, W, a.ws, a.w,
@@ -1215,19 +1219,23 @@ css_status launch_spmm_t(css_ctx* ctx, const LzArgs& a, const T* V, T* W, cudaSt
 // same order, so the choice changes the speed only, never the result
 constexpr int kSpmmVariants = 5;
 
-template <typename T, int BM>
+template <typename T, int BM, int B = 0>
 css_status launch_spmm_bm(css_ctx* ctx, const LzArgs& a, const T* V, T* W, int v, cudaStream_t st) {
   constexpr int TCW = (sizeof(T) == 4 && BM < 32) ? 4 : (sizeof(T) == 4 || BM < 32) ? 2 : 1;  // widest
   constexpr int TCN = TCW > 1 ? TCW / 2 : 1;
-  if (v == 0) return launch_spmm_t<T, BM, TCW, 128>(ctx, a, V, W, st);
-  if (v == 1) return launch_spmm_t<T, BM, TCN, 256>(ctx, a, V, W, st);
-  if (v == 2) return launch_spmm_t<T, BM, TCN, 128>(ctx, a, V, W, st);
-  if (v == 3) return launch_spmm_t<T, BM, TCW, 64>(ctx, a, V, W, st);  // more, smaller CTAs per SM
-  return launch_spmm_t<T, BM, TCW, 96>(ctx, a, V, W, st);
+  if (v == 0) return launch_spmm_t<T, BM, TCW, 128, B>(ctx, a, V, W, st);
+  if (v == 1) return launch_spmm_t<T, BM, TCN, 256, B>(ctx, a, V, W, st);
+  if (v == 2) return launch_spmm_t<T, BM, TCN, 128, B>(ctx, a, V, W, st);
+  if (v == 3) return launch_spmm_t<T, BM, TCW, 64, B>(ctx, a, V, W, st);  // more, smaller CTAs per SM
+  return launch_spmm_t<T, BM, TCW, 96, B>(ctx, a, V, W, st);
 }
 
 template <typename T>
 css_status launch_spmm_v(css_ctx* ctx, const LzArgs& a, const T* V, T* W, int v, cudaStream_t st) {
+  if constexpr (sizeof(T) == 8) {
+    if (a.b == 6) return launch_spmm_bm<T, 8, 6>(ctx, a, V, W, v, st);
+    if (a.b == 23) return launch_spmm_bm<T, 24, 23>(ctx, a, V, W, v, st);
+  }
   switch (css_spmm_bm(a.b)) {
     case 8: return launch_spmm_bm<T, 8>(ctx, a, V, W, v, st);
     case 12: return launch_spmm_bm<T, 12>(ctx, a, V, W, v, st);
