@@ -864,10 +864,19 @@ css_status css_density_impl(css_ctx* ctx, int32_t n_sys, const css_sys_desc* sys
   // FP32 with b = 6 or 23: the exact-width H * V unless a padded variant is asked for
   const bool use_dup = !use_tc && ctx->spmm_variant < 0 && css_spmm_dup_supported(f32, b);
   const void* Hsplit = nullptr;
+  // FP64 with b <= 24: exact digit products on the tensor cores, unless a padded variant is asked for or
+  // the digits would not fit their bounds
+  int32_t rows_max = 0;
+  for (int32_t s = 0; s < n_sys; ++s) rows_max = std::max(rows_max, sys[s].H.n_brow);
+  const bool use_int = prec == CSS_FP64 && ctx->spmm_variant < 0 && css_hv_int_supported(b, rows_max, nnzb);
+  const void* Hdig = nullptr;
+  const int32_t* Hexp = nullptr;
   if (use_tc)
     CSS_TRY(css_hv_tc_prepare(ctx, b, n_brow, nnzb, row_ptr, col_idx, Hval, &Htc, &Hd3, st));
   else if (use_split)
     CSS_TRY(css_spmm_split_prepare(ctx, b, nnzb, Hval, &Hsplit, st));
+  else if (use_int)
+    CSS_TRY(css_hv_int_prepare(ctx, b, n_brow, nnzb, row_ptr, col_idx, brow, Hval, &Hdig, &Hexp, st));
   else if (use_dup)
     CSS_TRY(css_spmm_dup_prepare(ctx, b, n_brow, nnzb, row_ptr, col_idx, Hval, &Hdup, &Hlodup, st));
   else
@@ -926,7 +935,7 @@ css_status css_density_impl(css_ctx* ctx, int32_t n_sys, const css_sys_desc* sys
   auto vec_need = [&](int32_t k) -> size_t {
     const int32_t ws = (int32_t)css_ceil_div((int64_t)k * b, 8) * 8;
     return 3 * (size_t)Nmax * ws * s_vec + css_lanczos_part_doubles(Nmax, b, k) * 8 * 2 +
-           css_lanczos_small_doubles(b, k) * 8;
+           css_lanczos_small_doubles(b, k) * 8 + (use_int ? css_hv_int_v_bytes(rows_max, b, k * b) : 0);
   };
   const size_t reserve = (size_t)2 << 30;
   while (ncb > 1 && vec_need(ncb) + reserve > free_b) ncb = (ncb + 1) / 2;
@@ -938,6 +947,8 @@ css_status css_density_impl(css_ctx* ctx, int32_t n_sys, const css_sys_desc* sys
   CSS_TRY(css_ws(ctx, "W", (size_t)Nmax * ws * s_vec, &Wv));
   CSS_TRY(ws_get(ctx, "lz_part", css_lanczos_part_doubles(Nmax, b, ncb) * 2, &part));
   CSS_TRY(ws_get(ctx, "lz_small", css_lanczos_small_doubles(b, ncb), &small));
+  void* vdig = nullptr;
+  if (use_int) CSS_TRY(css_ws(ctx, "v_digits", css_hv_int_v_bytes(rows_max, b, ncb * b), &vdig));
 
   LzArgs la;
   la.fp32 = f32;
@@ -951,6 +962,10 @@ css_status css_density_impl(css_ctx* ctx, int32_t n_sys, const css_sys_desc* sys
   la.Hdup = Hdup;
   la.Hlo_dup = Hlodup;
   la.Hsplit = Hsplit;
+  la.Hdig = Hdig;
+  la.Hexp = Hexp;
+  la.Hexp_n = (int64_t)n_brow * b;
+  la.Vdig = vdig;
   la.use_tc = use_tc;
   la.tc_H = Htc;
   la.tc_Hd3 = Hd3;
@@ -1004,7 +1019,7 @@ css_status css_density_impl(css_ctx* ctx, int32_t n_sys, const css_sys_desc* sys
     // reserve (sets already held from an earlier call count as free)
     size_t free2 = 0, total2 = 0, held = 0;
     CSS_CU(ctx, cudaMemGetInfo(&free2, &total2));
-    static const char* const kSideNames[] = {"sQ0_", "sQ1_", "sW_", "spart_", "ssmall_"};
+    static const char* const kSideNames[] = {"sQ0_", "sQ1_", "sW_", "spart_", "ssmall_", "svdig_"};
     for (auto& kv : ctx->bufs)
       for (const char* pre : kSideNames)
         if (kv.first.rfind(pre, 0) == 0) held += kv.second.bytes;
@@ -1013,7 +1028,7 @@ css_status css_density_impl(css_ctx* ctx, int32_t n_sys, const css_sys_desc* sys
     if (nside < 2) nside = 0;
   }
   struct SideWs {
-    void *Q0, *Q1, *W;
+    void *Q0, *Q1, *W, *vdig;
     double *part, *small;
   };
   std::vector<SideWs> sws(nside);
@@ -1040,6 +1055,9 @@ css_status css_density_impl(css_ctx* ctx, int32_t n_sys, const css_sys_desc* sys
       CSS_TRY(ws_get(ctx, nm, css_lanczos_part_doubles(Nmax, b, ncb) * 2, &sws[k].part));
       snprintf(nm, sizeof(nm), "ssmall_%d", k);
       CSS_TRY(ws_get(ctx, nm, css_lanczos_small_doubles(b, ncb), &sws[k].small));
+      snprintf(nm, sizeof(nm), "svdig_%d", k);
+      sws[k].vdig = nullptr;
+      if (use_int) CSS_TRY(css_ws(ctx, nm, css_hv_int_v_bytes(rows_max, b, ncb * b), &sws[k].vdig));
     }
   }
   // systems by decreasing size, dealt round-robin to the side streams
@@ -1066,6 +1084,7 @@ css_status css_density_impl(css_ctx* ctx, int32_t n_sys, const css_sys_desc* sys
         lb.W = sws[k].W;
         lb.part = sws[k].part;
         lb.small = sws[k].small;
+        lb.Vdig = sws[k].vdig;
         lb.row0 = row_off[s];
         lb.n_brow = sys[s].H.n_brow;
         lb.row_ptr = row_ptr + row_off[s];

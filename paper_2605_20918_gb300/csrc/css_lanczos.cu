@@ -1257,6 +1257,7 @@ css_status launch_spmm(css_ctx* ctx, const LzArgs& a, const T* V, T* W, cudaStre
     if (a.use_tc) return tune_only ? CSS_OK : css_hv_tc(ctx, a, V, W, st);
     dup = a.Hdup != nullptr;
   } else {
+    if (a.Hdig) return tune_only ? CSS_OK : css_hv_int(ctx, a, V, W, st);
     dup = a.Hsplit != nullptr;
   }
   // the exact-width kernel (FP32) or the split-FP64 one (css_spmm.cu) when H was prepared for

@@ -58,6 +58,12 @@ struct LzArgs {
   const void* Hlo_dup = nullptr;
   // FP64 H * V in FP32 pairs (css_spmm.cu) when Hsplit is set: hi and lo parts of every block
   const void* Hsplit = nullptr;
+  // FP64 H * V by exact digit products (css_hv_int.cu) when Hdig is set: the digits of every block, the
+  // exponents of the combined matrix's rows and columns, and a buffer of css_hv_int_v_bytes for the digits of V
+  const void* Hdig = nullptr;
+  const int32_t* Hexp = nullptr;
+  int64_t Hexp_n = 0;  // from a row's exponent to its column's
+  void* Vdig = nullptr;
   bool use_tc = false;
   const void* tc_H = nullptr;
   const void* tc_Hd3 = nullptr;
@@ -93,6 +99,13 @@ int css_spmm_split_variants();
 css_status css_spmm_split_prepare(css_ctx* ctx, int32_t b, int32_t nnzb, const double* H, const void** Hs,
                                   cudaStream_t st);
 css_status css_spmm_split(css_ctx* ctx, const LzArgs& a, const double* V, double* W, int variant, cudaStream_t st);
+// FP64 H * V by exact digit products on the tensor cores (css_hv_int.cu); n_brow: the largest pass's rows
+bool css_hv_int_supported(int32_t b, int32_t n_brow, int32_t nnzb);
+size_t css_hv_int_v_bytes(int32_t n_brow, int32_t b, int32_t w);
+css_status css_hv_int_prepare(css_ctx* ctx, int32_t b, int32_t n_brow, int32_t nnzb, const int32_t* row_ptr,
+                              const int32_t* col_idx, const int32_t* brow, const double* H, const void** Hdig,
+                              const int32_t** Hexp, cudaStream_t st);
+css_status css_hv_int(css_ctx* ctx, const LzArgs& a, const double* V, double* W, cudaStream_t st);
 // FP32 row passes of a Lanczos step with local reorthogonalisation for b = 6 and 23 (css_rows.cu); mode 0 S1,
 // 1 S3, 2 T0, 3 T1, 4 T2
 struct CssRows {

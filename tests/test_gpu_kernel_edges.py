@@ -80,3 +80,42 @@ def test_fp32_row_pass_splits(torch, css, ctx, kind, n, nc, m):
     got = gpu_density(torch, css, ctx, H, col, s, nc, precision=css.CSS_MIXED_FP32, **kw)
     scale = max(1.0, float(np.abs(ref["P"]).max()))
     assert float(np.abs(got["P"] - ref["P"]).max()) < MIXED_P_TOL * scale
+
+
+def _dense_bsr(n, b, scale, seed):
+    """Symmetric matrix with every block present; row and column i scaled by scale[i]."""
+    from paper_2605_20918_gb300 import synth
+    rng = np.random.default_rng(seed)
+    A = rng.standard_normal((n * b, n * b)) / np.sqrt(n * b)
+    A = (A + A.T) * np.sqrt(scale)[:, None] * np.sqrt(scale)[None, :]
+    A[np.arange(n * b), np.arange(n * b)] += rng.uniform(-20.0, 20.0, n * b) * scale
+    val = np.ascontiguousarray(A.reshape(n, b, n, b).transpose(0, 2, 1, 3)).reshape(n * n, b, b)
+    ptr = (np.arange(n + 1) * n).astype(np.int32)
+    return synth.BSR(n, b, ptr, np.tile(np.arange(n, dtype=np.int32), n), val)
+
+
+# FP64 H*V from exact digit products: block widths at the edges of the 8-row and 16-column tiles and past
+# the rule's last (b = 25), one to nine tiles of 16 columns (a partly filled last one, a second CTA), rows
+# with fewer, as many and more blocks than one exact sum takes (146 / b), rows graded over eight decades.  A fixed mu; the
+# tolerance of the FP64 parity tests
+@pytest.mark.parametrize("n,b,nc,m,grade", [(1, 1, 1, 1, 0), (150, 1, 9, 6, 0), (37, 6, 24, 5, 0), (24, 6, 3, 5, 8),
+                                            (19, 8, 2, 4, 0), (18, 9, 5, 4, 0), (9, 16, 9, 3, 8), (9, 17, 1, 4, 0),
+                                            (13, 23, 4, 5, 0), (7, 24, 3, 3, 0), (7, 25, 3, 3, 0)])
+def test_fp64_digit_products(torch, css, monkeypatch, n, b, nc, m, grade):
+    from tests.test_gpu_parity import FP64_TOL, gpu_density
+    scale = 10.0 ** np.linspace(0.0, -grade, n * b)
+    H = _dense_bsr(n, b, scale, 100 * n + b)
+    col = (np.arange(n) % nc).astype(np.int32)
+    s = oracle.probes(col, b, 1005)
+    kw = dict(kT=0.5, n_elec=float(n * b), m=m, mu=0.1, solve_mu=False)
+    ref = oracle.density(H, col, s, nc, **kw)
+    for variant in (None, "0"):  # the default and the general (DFMA) kernel
+        if variant is not None:
+            monkeypatch.setenv("CSS_SPMM_VARIANT", variant)
+        c = css.Context(0)
+        try:
+            got = gpu_density(torch, css, c, H, col, s, nc, precision=css.CSS_FP64, **kw)
+        finally:
+            c.close()
+        assert float(np.abs(got["P"] - ref["P"]).max()) < FP64_TOL, variant
+        assert abs(got["trP"] - ref["trP"]) < 1e-8
