@@ -58,11 +58,11 @@ typedef enum {
                         /* on-site blocks in three parts) accumulated in FP32, for 17 <= b <= 24 */
                         /* (other b: CSS_ERR_UNSUPPORTED); the other sparse products of        */
                         /* css_hprime and css_density_nonorth stay on the FP32 FMA pipe        */
-  CSS_FP64_SPLIT = 3    /* as CSS_FP64, with the H*V of the block-Lanczos recurrence on the FP32 */
-                        /* FMA pipe: H and V as pairs hi + lo of FP32 numbers, each product by */
-                        /* an error-free FMA split, sums by TwoSum into hi + lo (about 2^-47   */
-                        /* relative per term against 2^-53); b = 6 or 23 (other b:            */
-                        /* CSS_ERR_UNSUPPORTED); other sparse products stay FP64             */
+  CSS_FP64_SPLIT = 3    /* as CSS_FP64, with leave to take the H*V of the block-Lanczos recurrence */
+                        /* in FP32 pairs on the FMA pipe (hi + lo, error-free products, TwoSum   */
+                        /* sums: about 2^-47 relative per term against 2^-53); b = 6 or 23       */
+                        /* (other b: CSS_ERR_UNSUPPORTED).  Systems whose 8-bit digits of H fit  */
+                        /* 8 GiB run the exact digit products of CSS_FP64, which are faster      */
 } css_precision;
 
 /* css_density flags */

@@ -4,7 +4,8 @@
 // (2024) 297).
 //
 // The GB300 runs FP64 FMAs at 1/64 of its FP32 rate (a warp instruction per 16 clocks of an SM), which
-// bounded the DFMA kernel (css_lanczos.cu k_spmm): 5.38 ms for 128 molecules at b = 23.  A bf16 holds an
+// bounded the DFMA kernel (css_lanczos.cu k_spmm): 5.38 ms a launch for 128 molecules at b = 23, 48.7 us for 64
+at b = 6.  Here they take 0.79 ms (digits of V and exponents included) and 36 us.  A bf16 holds an
 // 8-bit signed digit exactly and the products of two digits sum exactly in an FP32 accumulator up to
 // 2^24, so bf16 tensor-core products of digits are integer arithmetic.
 //
@@ -23,8 +24,9 @@
 // tcgen05 tile of M = 128 in tensor memory would need once per 24 columns of N with a K of 23 per
 // block: the digit products are many small MMAs, not one large one.
 // A CTA takes one block row I and eight tiles of 16 columns, a warp each.  The digits of H_IJ (10.5 KB,
-// shared by the warps) and of V_J (7 KB per warp) arrive in MMA fragment order through a three-stage
-// cp.async ring, so that a thread copies the very 16 bytes of V it will load.
+// shared by the warps) and of V_J (7 KB per warp) arrive in MMA fragment order through a
+// cp.async ring of three stages (six for b <= 16 when the CTAs do not fill the chip and nothing else hides a
+// copy's latency); a thread copies the very 16 bytes of V it will load.
 #include <algorithm>
 
 #include "css_lanczos.cuh"
@@ -34,7 +36,6 @@ namespace {
 constexpr int kDig = 7;    // digits of an entry
 constexpr int kSum = 8;    // sums S_d over i + j = d
 constexpr int kWarps = 8;  // column tiles per CTA
-constexpr int kStages = 3;
 constexpr int kTile = 16;  // columns of V per warp
 // rows of H and columns of V whose largest entry is below 2^-968 keep 2^-1023 as their last digit
 constexpr int kMinExp = 54;
@@ -52,7 +53,7 @@ template <int NT, int KC>
 struct IntCfg {
   static constexpr int HB = kDig * NT * 32 * KC * 8;    // bytes of the digits of an H block
   static constexpr int VB = kDig * KC * 32 * 16;        // of a V block (16 columns)
-  static constexpr int smem = kStages * (HB + kWarps * VB);
+  static constexpr int smem(int stages) { return stages * (HB + kWarps * VB); }
 };
 inline int nt_of(int32_t b) { return (b + 7) / 8; }
 inline int kc_of(int32_t b) { return (b + 15) / 16; }
@@ -137,19 +138,21 @@ __global__ void __launch_bounds__(256) k_hdigits(int64_t nb, int32_t b, const in
   }
 }
 
-// largest biased exponent of every column of the scaled V (vexp cleared before): 64 rows by 128 columns a CTA
-__global__ void __launch_bounds__(128) k_vcol_exp(int64_t N, int32_t w, int32_t ws, const double* __restrict__ V,
+// largest biased exponent of every column of the scaled V (vexp cleared before): 16 ng rows by 128 columns a CTA
+__global__ void __launch_bounds__(128) k_vcol_exp(int64_t N, int32_t ng, int32_t w, int32_t ws, const double* __restrict__ V,
                                                   const int32_t* __restrict__ hcol, int32_t* __restrict__ vexp) {
   const int32_t col = blockIdx.y * 128 + threadIdx.x;
   if (col >= w) return;
-  const int64_t r0 = (int64_t)blockIdx.x * 64;
-  const int32_t nr = (int32_t)(N - r0 < 64 ? N - r0 : 64);
-  const double* v = V + (size_t)r0 * ws + col;
+  const int64_t r0 = (int64_t)blockIdx.x * ng * 16;
   int e = 0;
-#pragma unroll 8
-  for (int32_t r = 0; r < nr; ++r, v += ws) {
-    const int x = (int)expo(*v);
-    e = max(e, x == 0x7ff ? kNotFinite : x + col_scale(hcol[r0 + r]));
+  for (int64_t r = r0; r < min(N, r0 + ng * 16); r += 16) {
+    const double* v = V + (size_t)r * ws + col;
+#pragma unroll
+    for (int i = 0; i < 16; ++i) {
+      if (r + i >= N) break;
+      const int x = (int)expo(v[(size_t)i * ws]);
+      e = max(e, x == 0x7ff ? kNotFinite : x + col_scale(hcol[r + i]));
+    }
   }
   if (e) atomicMax(&vexp[col], e);
 }
@@ -215,7 +218,7 @@ struct IntArgs {
   double* W;
 };
 
-template <int NT, int KC>
+template <int NT, int KC, int kStages>
 __global__ void __launch_bounds__(32 * kWarps, 1) k_hv_int(const IntArgs a) {
   using C = IntCfg<NT, KC>;
   extern __shared__ __align__(16) unsigned char sm[];
@@ -316,10 +319,13 @@ css_status launch(css_ctx* ctx, const LzArgs& a, const double* V, double* W, int
   const int32_t b = a.b, tiles = (int32_t)css_ceil_div(a.w, kTile);
   const int64_t N = (int64_t)a.n_brow * b;
   const int32_t *hexp = a.Hexp + (size_t)a.row0 * b, *hcol = hexp + a.Hexp_n;
-  CSS_CU(ctx, cudaFuncSetAttribute(k_hv_int<NT, KC>, cudaFuncAttributeMaxDynamicSharedMemorySize, C::smem));
+  constexpr int deep = KC == 1 ? 6 : 3;
+  CSS_CU(ctx, cudaFuncSetAttribute(k_hv_int<NT, KC, 3>, cudaFuncAttributeMaxDynamicSharedMemorySize, C::smem(3)));
+  CSS_CU(ctx, cudaFuncSetAttribute(k_hv_int<NT, KC, deep>, cudaFuncAttributeMaxDynamicSharedMemorySize, C::smem(deep)));
   CSS_CU(ctx, cudaMemsetAsync(vexp, 0, sizeof(int32_t) * a.w, st));
-  k_vcol_exp<<<dim3((unsigned)css_ceil_div(N, 64), (unsigned)css_ceil_div(a.w, 128)), 128, 0, st>>>(N, a.w, a.ws, V,
-                                                                                                  hcol, vexp);
+  const int32_t ng = N > 16384 ? 4 : 1;
+  k_vcol_exp<<<dim3((unsigned)css_ceil_div(N, 16 * ng), (unsigned)css_ceil_div(a.w, 128)), 128, 0, st>>>(
+      N, ng, a.w, a.ws, V, hcol, vexp);
   CSS_LAUNCHED(ctx);
   for (int32_t t0 = 0; t0 < tiles; t0 += per) {
     const int32_t nt = std::min(per, tiles - t0);
@@ -342,7 +348,11 @@ css_status launch(css_ctx* ctx, const LzArgs& a, const double* V, double* W, int
     r.Hd = static_cast<const unsigned char*>(a.Hdig);
     r.Vd = reinterpret_cast<const unsigned char*>(vd);
     r.W = W;
-    k_hv_int<NT, KC><<<dim3((unsigned)a.n_brow, (unsigned)css_ceil_div(nt, kWarps)), 32 * kWarps, C::smem, st>>>(r);
+    const dim3 grid((unsigned)a.n_brow, (unsigned)css_ceil_div(nt, kWarps));
+    if (grid.x * (int64_t)grid.y <= ctx->n_sm)
+      k_hv_int<NT, KC, deep><<<grid, 32 * kWarps, C::smem(deep), st>>>(r);
+    else
+      k_hv_int<NT, KC, 3><<<grid, 32 * kWarps, C::smem(3), st>>>(r);
     CSS_LAUNCHED(ctx);
   }
   return CSS_OK;
