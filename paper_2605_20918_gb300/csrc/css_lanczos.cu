@@ -1313,8 +1313,10 @@ css_status run_pass_bp(css_ctx* ctx, const LzArgs& a_in, cudaStream_t st) {
   const bool reorth = (a.flags & CSS_REORTH_LOCAL) != 0;
   // FP32 with b = 6 or 23: the row passes of css_rows.cu, with Gram partials in chunks of their own
   const bool rows = sizeof(T) == 4 && reorth && css_rows_supported(true, b);
+  const bool rows64 = css_rows64_supported(sizeof(T) == 4, b, reorth);  // FP64: css_rows64.cu
   const int32_t rchk = row_chunk<T, BP>(N, b);
-  const int32_t nch = (int32_t)css_ceil_div(N, rchk), nch_r = rows ? (int32_t)css_ceil_div(N, css_rows_chunk(N, b)) : 0;
+  const int32_t nch = (int32_t)css_ceil_div(N, rchk), nch_r = rows ? (int32_t)css_ceil_div(N, css_rows_chunk(N, b))
+                                                                      : rows64 ? (int32_t)css_ceil_div(N, css_rows64_chunk(N)) : 0;
   T* Qp = (T*)a.Q0;
   T* Qc = (T*)a.Q1;
   T* W = (T*)a.W;
@@ -1466,6 +1468,35 @@ css_status run_pass_bp(css_ctx* ctx, const LzArgs& a_in, cudaStream_t st) {
       std::swap(Qp, Qc);
       continue;
     }
+    if (rows64) {
+      CssRows64 r;
+      r.N = N;
+      r.ws = a.ws;
+      r.ncb = ncb;
+      r.cb0 = a.cb0;
+      r.first = j == 0;
+      r.Q = (const double*)Qc;
+      r.Qp = (const double*)Qp;
+      r.W = (double*)W;
+      r.out = (double*)Qp;
+      r.M = a.Bblk_prev;
+      r.need3 = need3;
+      r.part = partKq;
+      CSS_TRY(css_rows64(ctx, 0, b, r, st));
+      CSS_TRY(gram_A(nch_r, j, false, a.Ablk));
+      if (j + 1 == m) break;
+      r.M = sA;
+      CSS_TRY(css_rows64(ctx, 1, b, r, st));
+      r.M = sRi;
+      for (int mode = 0; mode < 3; ++mode) {  // shifted CholeskyQR3 (k_gram_chol)
+        CSS_TRY(chol(nch_r, mode, j, sRi, mode ? need3 : nullptr, false));
+        CSS_TRY(css_rows64(ctx, 2 + mode, b, r, st));
+      }
+      CSS_TRY(sampled(Qp, j + 1));
+      CSS_TRY(project_u(Qp, j + 1));
+      std::swap(Qp, Qc);
+      continue;
+    }
     // three-term update and the projections onto Q_j (and Q_{j-1})
     s1<<<rgrid, reorth ? 2 * RW : RW, sm_s1, st>>>(N, rchk, b, a.ws, ncb, a.cb0, Qp, Qc, W, a.Bblk_prev, j == 0 ? 1 : 0,
                                                    partKq, partKp);
@@ -1538,6 +1569,7 @@ size_t css_lanczos_part_doubles(int64_t N, int32_t b, int32_t ncb) {
                                                                                               : min_chunk<32>(N, b);
   int64_t nch = css_ceil_div(N, chunk);
   if (css_rows_supported(true, b)) nch = std::max(nch, css_ceil_div(N, css_rows_chunk(N, b)));
+  if (css_rows64_supported(false, b, false)) nch = std::max(nch, css_ceil_div(N, css_rows64_chunk(N)));
   return (size_t)nch * ncb * b * b * 2 + (size_t)nch * ncb + 64;
 }
 

@@ -121,6 +121,20 @@ struct CssRows {
 bool css_rows_supported(bool fp32, int32_t b);
 int32_t css_rows_chunk(int64_t N, int32_t b);  // rows per Gram partial
 css_status css_rows(css_ctx* ctx, int mode, const CssRows& p, cudaStream_t st);
+// FP64 row passes of a step without local reorthogonalisation for b = 6 and 23 (css_rows64.cu); mode 0 S1,
+// 1 S3, 2 T0, 3 T1, 4 T2
+struct CssRows64 {
+  int64_t N = 0;
+  int32_t ws = 0, ncb = 0, cb0 = 0, first = 0;
+  const double *Q = nullptr, *Qp = nullptr;  // Q_j, Q_{j-1}
+  double *W = nullptr, *out = nullptr;       // W in place; T1, T2: Q_{j+1}
+  const double* M = nullptr;                 // S1: B_{j-1} [cb0 + lc]; S3: Kq; T0, T1, T2: R^-1 [lc]
+  const int32_t* need3 = nullptr;
+  double* part = nullptr;                    // Gram partials [chunk][lc][b][b]
+};
+bool css_rows64_supported(bool fp32, int32_t b, bool reorth);
+int32_t css_rows64_chunk(int64_t N);  // rows per Gram partial
+css_status css_rows64(css_ctx* ctx, int mode, int32_t b, const CssRows64& a, cudaStream_t st);
 // W = M V for a BSR matrix prepared by css_spmm_prepare (a.Hval, a.Hlo_diag, a.row_ptr,
 // a.col_idx, a.n_brow, a.b) and N x a.w blocks V, W of row stride a.ws in the vector precision
 css_status css_spmm(css_ctx* ctx, const LzArgs& a, const void* V, void* W, cudaStream_t st);

@@ -119,3 +119,22 @@ def test_fp64_digit_products(torch, css, monkeypatch, n, b, nc, m, grade):
             c.close()
         assert float(np.abs(got["P"] - ref["P"]).max()) < FP64_TOL, variant
         assert abs(got["trP"] - ref["trP"]) < 1e-8
+
+
+# FP64 row passes: one row tile partly filled, exactly filled and exceeded, one colour and many, chunks of
+# two tiles with a partly filled last chunk (450 molecules), and a Krylov space that is exhausted before
+# depth m (third CholeskyQR pass, then breakdown); the tolerance of the FP64 parity tests
+@pytest.mark.parametrize("kind,n,nc,m", [("minimal", 1, 1, 1), ("minimal", 16, 1, 5), ("minimal", 33, 11, 5),
+                                         ("minimal", 450, 3, 4), ("minimal", 9, 9, 12), ("dzp", 9, 1, 5),
+                                         ("dzp", 32, 5, 4), ("dzp", 20, 20, 4), ("dzp", 6, 6, 8)])
+def test_fp64_row_pass_splits(torch, css, ctx, kind, n, nc, m):
+    from paper_2605_20918_gb300 import synth
+    from tests.test_gpu_parity import FP64_TOL, gpu_density
+    g = synth.water_box(n)
+    H = synth.hamiltonian(g, kind)
+    col = (np.arange(n) % nc).astype(np.int32)
+    s = oracle.probes(col, H.b, 1005)
+    kw = dict(kT=0.05, n_elec=synth.n_electrons(n), m=m, mu=-4.0, solve_mu=False)
+    ref = oracle.density(H, col, s, nc, **kw)
+    got = gpu_density(torch, css, ctx, H, col, s, nc, precision=css.CSS_FP64, **kw)
+    assert float(np.abs(got["P"] - ref["P"]).max()) < FP64_TOL
