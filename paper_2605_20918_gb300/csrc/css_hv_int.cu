@@ -5,7 +5,7 @@
 //
 // The GB300 runs FP64 FMAs at 1/64 of its FP32 rate (a warp instruction per 16 clocks of an SM), which
 // bounded the DFMA kernel (css_lanczos.cu k_spmm): 5.38 ms a launch for 128 molecules at b = 23, 48.7 us for 64
-at b = 6.  Here they take 0.79 ms (digits of V and exponents included) and 36 us.  A bf16 holds an
+// at b = 6.  Here they take 0.79 ms (digits of V and exponents included) and 36 us.  A bf16 holds an
 // 8-bit signed digit exactly and the products of two digits sum exactly in an FP32 accumulator up to
 // 2^24, so bf16 tensor-core products of digits are integer arithmetic.
 //
