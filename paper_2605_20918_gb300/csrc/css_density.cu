@@ -879,7 +879,7 @@ css_status css_density_impl(css_ctx* ctx, int32_t n_sys, const css_sys_desc* sys
   else if (use_split)
     CSS_TRY(css_spmm_split_prepare(ctx, b, nnzb, Hval, &Hsplit, st));
   else if (use_int)
-    CSS_TRY(css_hv_int_prepare(ctx, b, n_brow, nnzb, row_ptr, col_idx, brow, Hval, &Hdig, &Hexp, st));
+    CSS_TRY(css_hv_int_prepare(ctx, b, n_brow, nnzb, row_ptr, col_idx, Hval, &Hdig, &Hexp, st));
   else if (use_dup)
     CSS_TRY(css_spmm_dup_prepare(ctx, b, n_brow, nnzb, row_ptr, col_idx, Hval, &Hdup, &Hlodup, st));
   else
@@ -1962,9 +1962,7 @@ css_status css_density_nonorth(css_ctx* ctx, const css_bsr* S, const double* Sin
   k_block_transpose<<<(unsigned)css_ceil_div((int64_t)S->nnzb * bb, T), T, 0, st>>>(S->nnzb, b, strans, Sinv_val,
                                                                                     sinvT);
   CSS_LAUNCHED(ctx);
-  const void *hpv, *hplo, *siv, *silo, *sv, *slo, *sitv, *sitlo;
-  CSS_TRY(css_spmm_prepare_as(ctx, "no_hp", f32, b, n_brow, Hp->nnzb, Hp->row_ptr, Hp->col_idx, Hp->val, &hpv, &hplo,
-                              st));
+  const void *hpv = nullptr, *hplo = nullptr, *siv, *silo, *sv, *slo, *sitv, *sitlo;
   CSS_TRY(css_spmm_prepare_as(ctx, "no_si", f32, b, n_brow, S->nnzb, S->row_ptr, S->col_idx, Sinv_val, &siv, &silo,
                               st));
   CSS_TRY(css_spmm_prepare_as(ctx, "no_s", f32, b, n_brow, S->nnzb, S->row_ptr, S->col_idx, S->val, &sv, &slo, st));
@@ -1979,6 +1977,20 @@ css_status css_density_nonorth(css_ctx* ctx, const css_bsr* S, const double* Sin
   if (7 * vbytes + ((size_t)1 << 30) > free_b + ctx->ws_bytes) {
     ctx->last_error = "css_density_nonorth: the Krylov blocks of all colours do not fit in device memory";
     return CSS_ERR_NOMEM;
+  }
+  // the recurrence's H'*V as in css_density_impl, where the digits fit beside the Krylov blocks
+  const size_t vd_bytes = css_hv_int_v_bytes(n_brow, b, nc * b);
+  const bool use_int = prec == CSS_FP64 && ctx->spmm_variant < 0 && css_hv_int_supported(b, n_brow, Hp->nnzb) &&
+                       7 * vbytes + vd_bytes + ((size_t)9 << 30) <= free_b + ctx->ws_bytes;
+  const void* Hdig = nullptr;
+  const int32_t* Hexp = nullptr;
+  void* vdig = nullptr;
+  if (use_int) {
+    CSS_TRY(css_hv_int_prepare(ctx, b, n_brow, Hp->nnzb, Hp->row_ptr, Hp->col_idx, Hp->val, &Hdig, &Hexp, st));
+    CSS_TRY(css_ws(ctx, "v_digits", vd_bytes, &vdig));
+  } else {
+    CSS_TRY(css_spmm_prepare_as(ctx, "no_hp", f32, b, n_brow, Hp->nnzb, Hp->row_ptr, Hp->col_idx, Hp->val, &hpv, &hplo,
+                                st));
   }
   void *R, *R0, *SR, *U, *Q0, *Q1, *Wv;
   CSS_TRY(css_ws(ctx, "no_R", vbytes, &R));
@@ -2034,6 +2046,10 @@ css_status css_density_nonorth(css_ctx* ctx, const css_bsr* S, const double* Sin
   la.col_idx = Hp->col_idx;
   la.Hval = hpv;
   la.Hlo_diag = hplo;
+  la.Hdig = Hdig;
+  la.Hexp = Hexp;
+  la.Hexp_n = N;
+  la.Vdig = vdig;
   la.max_row_blocks = max_row;
   la.colour = colour;
   la.sign = sign;

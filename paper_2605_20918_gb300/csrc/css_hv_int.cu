@@ -93,48 +93,52 @@ __global__ void __launch_bounds__(256) k_hrow_exp(int32_t b, const int32_t* __re
   }
 }
 
-// largest biased exponent of every column of the row-scaled H (hcol cleared before): a thread per column
-// of a block
-__global__ void __launch_bounds__(256) k_hcol_exp(int64_t nb, int32_t b, const int32_t* __restrict__ brow,
+// largest biased exponent of every column of the row-scaled H (hcol cleared before): a CTA per block row, a
+// thread per column of a block
+__global__ void __launch_bounds__(256) k_hcol_exp(int32_t b, const int32_t* __restrict__ row_ptr,
                                                   const int32_t* __restrict__ col_idx, const double* __restrict__ H,
                                                   const int32_t* __restrict__ hexp, int32_t* __restrict__ hcol) {
-  const int64_t t = (int64_t)blockIdx.x * 256 + threadIdx.x, p = t / b;
-  if (p >= nb) return;
-  const int32_t k = (int32_t)(t - p * b);
-  const int32_t* e = hexp + (int64_t)brow[p] * b;
-  int m = -kColBias;
-  for (int32_t a = 0; a < b; ++a) {
-    const double h = H[(p * b + a) * b + k];
-    if (h != 0.0) m = max(m, (int)expo(h) - max(e[a], kMinExp));
+  const int64_t p0 = row_ptr[blockIdx.x], p1 = row_ptr[blockIdx.x + 1];
+  const int32_t* e = hexp + (int64_t)blockIdx.x * b;
+  for (int64_t t = p0 * b + threadIdx.x; t < p1 * b; t += 256) {
+    const int64_t p = t / b;
+    const int32_t k = (int32_t)(t - p * b);
+    int m = -kColBias;
+    for (int32_t a = 0; a < b; ++a) {
+      const double h = H[(p * b + a) * b + k];
+      if (h != 0.0) m = max(m, (int)expo(h) - max(e[a], kMinExp));
+    }
+    if (m > -kColBias) atomicMax(&hcol[(int64_t)col_idx[p] * b + k], m + kColBias);
   }
-  if (m > -kColBias) atomicMax(&hcol[(int64_t)col_idx[p] * b + k], m + kColBias);
 }
 
-// digits of every H block in the order of the B fragments: [block][digit][N tile][K tile][lane][2 words]
+// digits of every H block (a CTA per block row) in the order of the B fragments:
+// [block][digit][N tile][K tile][lane][2 words]
 template <int NT, int KC>
-__global__ void __launch_bounds__(256) k_hdigits(int64_t nb, int32_t b, const int32_t* __restrict__ brow,
+__global__ void __launch_bounds__(256) k_hdigits(int32_t b, const int32_t* __restrict__ row_ptr,
                                                  const int32_t* __restrict__ col_idx, const double* __restrict__ H,
                                                  const int32_t* __restrict__ hexp, const int32_t* __restrict__ hcol,
                                                  uint32_t* __restrict__ out) {
-  const int64_t t = (int64_t)blockIdx.x * 256 + threadIdx.x;
-  const int lane = (int)(t & 31), nt = (int)((t >> 5) % NT);
-  const int64_t p = (t >> 5) / NT;
-  if (p >= nb) return;
-  const int a = 8 * nt + (lane >> 2);
-  const double sc = a < b ? digit_scale(hexp[(int64_t)brow[p] * b + a], 0) : 0.0;
-  const double* h = H + (p * b + a) * b;
-  const int32_t* hc = hcol + (int64_t)col_idx[p] * b;
-  auto at = [&](int k) -> long long {
-    if (a >= b || k >= b) return 0;
-    return __double2ll_rn(h[k] * sc * __hiloint2double((1023 - col_scale(hc[k])) << 20, 0));
-  };
+  const int lane = threadIdx.x & 31;
+  const int64_t p1 = row_ptr[blockIdx.x + 1];
+  for (int64_t t = (int64_t)row_ptr[blockIdx.x] * NT + (threadIdx.x >> 5); t < p1 * NT; t += 8) {
+    const int64_t p = t / NT;
+    const int nt = (int)(t - p * NT), a = 8 * nt + (lane >> 2);
+    const double sc = a < b ? digit_scale(hexp[(int64_t)blockIdx.x * b + a], 0) : 0.0;
+    const double* h = H + (p * b + a) * b;
+    const int32_t* hc = hcol + (int64_t)col_idx[p] * b;
+    auto at = [&](int k) -> long long {
+      if (a >= b || k >= b) return 0;
+      return __double2ll_rn(h[k] * sc * __hiloint2double((1023 - col_scale(hc[k])) << 20, 0));
+    };
 #pragma unroll
-  for (int r = 0; r < 2 * KC; ++r) {
-    const int k = 8 * r + 2 * (lane & 3);
-    uint32_t d[kDig];
-    digits2(at(k), at(k + 1), d);
+    for (int r = 0; r < 2 * KC; ++r) {
+      const int k = 8 * r + 2 * (lane & 3);
+      uint32_t d[kDig];
+      digits2(at(k), at(k + 1), d);
 #pragma unroll
-    for (int s = 0; s < kDig; ++s) out[((((p * kDig + s) * NT + nt) * KC + r / 2) * 32 + lane) * 2 + (r & 1)] = d[s];
+      for (int s = 0; s < kDig; ++s) out[((((p * kDig + s) * NT + nt) * KC + r / 2) * 32 + lane) * 2 + (r & 1)] = d[s];
+    }
   }
 }
 
@@ -358,15 +362,6 @@ css_status launch(css_ctx* ctx, const LzArgs& a, const double* V, double* W, int
   return CSS_OK;
 }
 
-template <int NT, int KC>
-css_status digits_of(css_ctx* ctx, int32_t b, int64_t nnzb, const int32_t* brow, const int32_t* col_idx, const double* H,
-                     const int32_t* hexp, const int32_t* hcol, uint32_t* out, cudaStream_t st) {
-  k_hdigits<NT, KC><<<(unsigned)css_ceil_div(nnzb * NT * 32, 256), 256, 0, st>>>(nnzb, b, brow, col_idx, H, hexp, hcol,
-                                                                                out);
-  CSS_LAUNCHED(ctx);
-  return CSS_OK;
-}
-
 // column tiles of V's digits that go through the buffer at once
 int32_t tiles_at_once(int32_t n_brow, int32_t b, int32_t w) {
   const size_t one = (size_t)n_brow * v_block_bytes(b);
@@ -386,8 +381,8 @@ size_t css_hv_int_v_bytes(int32_t n_brow, int32_t b, int32_t w) {
 }
 
 css_status css_hv_int_prepare(css_ctx* ctx, int32_t b, int32_t n_brow, int32_t nnzb, const int32_t* row_ptr,
-                              const int32_t* col_idx, const int32_t* brow, const double* H, const void** Hdig,
-                              const int32_t** Hexp, cudaStream_t st) {
+                              const int32_t* col_idx, const double* H, const void** Hdig, const int32_t** Hexp,
+                              cudaStream_t st) {
   uint32_t* d;
   int32_t* e;
   CSS_TRY(css_ws(ctx, "h_digits", (size_t)nnzb * h_block_bytes(b), (void**)&d));
@@ -397,13 +392,11 @@ css_status css_hv_int_prepare(css_ctx* ctx, int32_t b, int32_t n_brow, int32_t n
   if (n_brow > 0) {
     k_hrow_exp<<<(unsigned)n_brow, 256, 0, st>>>(b, row_ptr, H, e);
     CSS_LAUNCHED(ctx);
-  }
-  if (nnzb > 0) {
-    k_hcol_exp<<<(unsigned)css_ceil_div((int64_t)nnzb * b, 256), 256, 0, st>>>(nnzb, b, brow, col_idx, H, e, e + n);
+    k_hcol_exp<<<(unsigned)n_brow, 256, 0, st>>>(b, row_ptr, col_idx, H, e, e + n);
     CSS_LAUNCHED(ctx);
-    if (b <= 8) CSS_TRY((digits_of<1, 1>(ctx, b, nnzb, brow, col_idx, H, e, e + n, d, st)));
-    else if (b <= 16) CSS_TRY((digits_of<2, 1>(ctx, b, nnzb, brow, col_idx, H, e, e + n, d, st)));
-    else CSS_TRY((digits_of<3, 2>(ctx, b, nnzb, brow, col_idx, H, e, e + n, d, st)));
+    auto kern = b <= 8 ? k_hdigits<1, 1> : b <= 16 ? k_hdigits<2, 1> : k_hdigits<3, 2>;
+    kern<<<(unsigned)n_brow, 256, 0, st>>>(b, row_ptr, col_idx, H, e, e + n, d);
+    CSS_LAUNCHED(ctx);
   }
   *Hdig = d;
   *Hexp = e;

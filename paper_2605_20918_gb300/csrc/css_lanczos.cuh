@@ -103,8 +103,8 @@ css_status css_spmm_split(css_ctx* ctx, const LzArgs& a, const double* V, double
 bool css_hv_int_supported(int32_t b, int32_t n_brow, int32_t nnzb);
 size_t css_hv_int_v_bytes(int32_t n_brow, int32_t b, int32_t w);
 css_status css_hv_int_prepare(css_ctx* ctx, int32_t b, int32_t n_brow, int32_t nnzb, const int32_t* row_ptr,
-                              const int32_t* col_idx, const int32_t* brow, const double* H, const void** Hdig,
-                              const int32_t** Hexp, cudaStream_t st);
+                              const int32_t* col_idx, const double* H, const void** Hdig, const int32_t** Hexp,
+                              cudaStream_t st);
 css_status css_hv_int(css_ctx* ctx, const LzArgs& a, const double* V, double* W, cudaStream_t st);
 // FP32 row passes of a Lanczos step with local reorthogonalisation for b = 6 and 23 (css_rows.cu); mode 0 S1,
 // 1 S3, 2 T0, 3 T1, 4 T2
