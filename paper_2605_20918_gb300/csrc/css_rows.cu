@@ -387,30 +387,36 @@ __global__ void __launch_bounds__(32 * (B6_GMAX + B6_NP), 1) k_rows6(const RowsA
 }
 
 // ------------------------------------------------------------------------ b = 23
-// Four colours (92 columns: whole 16-byte chunks) and tiles of 64 rows per CTA.  A tile is worked on in
-// two phases between CTA barriers:
-//   products: a warp takes one colour of 32 rows, a row per lane.  The row's 23 values come from the
-//     ring by 16-byte loads (a colour starts at one of four offsets within a chunk: four forms of the
-//     load, one of the arithmetic), the matrices by broadcast loads shared by 32 rows, an output pair
-//     per packed FMA; triangular matrices skip their zero half.  Results go back to the ring for the
-//     store and, 24 columns per colour, to a copy for the Gram.
+// Four colours (92 columns: whole 16-byte chunks) and tiles of 64 rows per CTA (S1: 32).  Warps have roles, and
+// the products of a tile run beside the Grams of the one before it, with one barrier per tile:
+//   products: a warp takes one colour, two rows per lane (S1: two colours, a row per lane).  A row's 23
+//     values come from the ring by 16-byte loads (a colour starts at one of four offsets within a chunk:
+//     four forms of the load, one of the arithmetic), the matrices by broadcast loads shared by 64 rows, an
+//     output pair per packed FMA; triangular matrices skip their zero half.  Results go back to the ring for
+//     the store and, 24 columns per colour, to one of two copies for the Gram.
 //   Grams: a thread owns an 8 x 8 block of a colour's 24 x 24 and every 8th row (S1: the blocks of Kq
 //     and of Kp together), four or six 16-byte loads for 32 or 64 packed FMAs.  After 32 rows the eight
 //     lanes of a block add their sums by halves (each keeps one row of the block) into hi + lo pairs.
-// Bound by the return path of shared memory: a 16-byte load is 512 bytes to a warp, four clocks of the
-// SM, broadcast or not, so the products' two packed FMAs per load (4 clocks of one scheduler) leave
-// the FMA pipe at a quarter; HBM is at 2 TB/s.  Row work of a step at 10,000 molecules 9.34 -> 6.71 ms
-// (S1 2.47, S3 2.20, T0 0.82, T1 0.88), at 1,000 1.08 -> 0.81 ms, against the tiled kernels.
-constexpr int B23_R = 64, B23_G = 4, B23_GP = 100;  // rows per tile, colours per CTA, pitch of the Gram copies
+// Bound by the return path of shared memory (a 16-byte load is 512 bytes to a warp, broadcast or not) and the
+// latency of a product's loads; HBM is at 2 to 3.3 TB/s.  The roles are separate loops, so that the Gram sums are
+// not live across the products: in one loop the products spilled and a step took 0.97 ms at 1,000 molecules
+// instead of 0.65.  Row work of a step at 10,000 molecules: tiled kernels 9.34 ms, both phases on the same
+// warps between two barriers 6.71, now 5.35; at 1,000 1.08, 0.81, 0.65 (S1 191 us, S3 220, T0 70, T1 87).  Slower
+// there: four lanes per Gram block with more producer warps 0.67, or with a row per lane on eight product
+// warps 0.74; S3 in tiles of 32 rows 0.66.
+constexpr int B23_G = 4, B23_GP = 100;  // colours per CTA, pitch of the Gram copies
 template <int MODE>
 struct B23Cfg {
+  static constexpr int R = MODE == R_S1 ? 32 : 64;      // rows per tile
   static constexpr int NA = MODE <= R_S3 ? 3 : 1;
-  static constexpr int NS = MODE <= R_S3 ? 2 : 4;
-  static constexpr int NP = 3;                          // producer warps
-  static constexpr int CW = MODE == R_S1 ? 9 : 8;       // consumer warps
+  static constexpr int NS = MODE == R_S3 ? 2 : 4;
+  // twelve warps (168 registers a lane): products, Grams, producers
+  static constexpr int S = 8;                           // lanes that share a Gram block
+  static constexpr int PW = MODE == R_S1 ? 2 : 4, GW = (MODE == R_S1 ? 36 : 24) * S / 32, NP = 12 - PW - GW;
+  static constexpr int RPL = R / 32;                    // rows per lane of a product
   static constexpr int NM = MODE == R_S3 ? 3 : MODE == R_T1 ? 2 : 1;  // matrices per colour
   static constexpr int NG = MODE == R_S1 ? 3 : MODE == R_T2 ? 0 : 1;  // Gram copies
-  static constexpr size_t smem = (size_t)NS * NA * B23_R * row_pitch(92) * 4 + (size_t)NG * B23_R * B23_GP * 4 +
+  static constexpr size_t smem = (size_t)NS * NA * R * row_pitch(92) * 4 + (size_t)2 * NG * R * B23_GP * 4 +
                                  (size_t)NM * B23_G * 23 * 24 * 4 + (2 * NS + 2) * 8;
 };
 
@@ -452,18 +458,23 @@ __device__ __forceinline__ void store_row_of(int c, float* row, const unsigned l
   else if (c == 2) store_row<2>(row + 44, o);
   else store_row<1>(row + 68, o);
 }
-// o += x M, M [23][24] in shared memory; TRI 1: M(l, k) = 0 for k > l, TRI 2: for k < l
-template <int TRI>
-__device__ __forceinline__ void mul_row(unsigned long long (&o)[12], const float (&x)[24], const float* M) {
+// o += x M for N rows, M [23][24] in shared memory; TRI 1: M(l, k) = 0 for k > l, TRI 2: for k < l
+template <int TRI, int N>
+__device__ __forceinline__ void mul_rows(unsigned long long (&o)[N][12], const float (&x)[N][24], const float* M) {
 #pragma unroll
   for (int l = 0; l < 23; ++l) {
-    const unsigned long long xx = dup2(x[l]);
+    unsigned long long xx[N];
+#pragma unroll
+    for (int n = 0; n < N; ++n) xx[n] = dup2(x[n][l]);
 #pragma unroll
     for (int c = 0; c < 6; ++c) {
       if ((TRI == 1 && 4 * c > l) || (TRI == 2 && 4 * c + 3 < l)) continue;
       const ulonglong2 m = *reinterpret_cast<const ulonglong2*>(M + 24 * l + 4 * c);
-      fma2(o[2 * c], xx, m.x);
-      fma2(o[2 * c + 1], xx, m.y);
+#pragma unroll
+      for (int n = 0; n < N; ++n) {
+        fma2(o[n][2 * c], xx[n], m.x);
+        fma2(o[n][2 * c + 1], xx[n], m.y);
+      }
     }
   }
 }
@@ -496,9 +507,10 @@ __device__ __forceinline__ void block_flush(unsigned long long (&v)[32], float (
 }
 
 template <int MODE>
-__global__ void __launch_bounds__(32 * (B23Cfg<MODE>::CW + B23Cfg<MODE>::NP), 1) k_rows23(const RowsArgs a) {
+__global__ void __launch_bounds__(32 * 12, 1) k_rows23(const RowsArgs a) {
   using C = B23Cfg<MODE>;
-  constexpr int NA = C::NA, NS = C::NS, R = B23_R, CT = 32 * C::CW, MM = 23 * 24;
+  constexpr int NA = C::NA, NS = C::NS, R = C::R, RPL = C::RPL, CT = 32 * (C::PW + C::GW), MM = 23 * 24;
+  constexpr int GB = C::NG * R * B23_GP;  // values of one buffer of Gram copies
   constexpr bool OUT = MODE == R_S3 || MODE == R_T1 || MODE == R_T2;
   extern __shared__ __align__(128) unsigned char rows_smem[];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -514,8 +526,8 @@ __global__ void __launch_bounds__(32 * (B23Cfg<MODE>::CW + B23Cfg<MODE>::NP), 1)
   ring.r0 = (int64_t)blockIdx.x * a.rchk;
   ring.rend = min(a.N, ring.r0 + a.rchk);
   ring.ntile = (int32_t)((ring.rend - ring.r0 + R - 1) / R);
-  float* sG = ring.base + (size_t)NS * NA * R * ring.pitch;  // Gram copies [array][row][24 c + k]
-  float* sM = sG + (size_t)C::NG * R * B23_GP;               // matrices [matrix][colour][l][k]
+  float* sG = ring.base + (size_t)NS * NA * R * ring.pitch;  // Gram copies [tile & 1][array][row][24 c + k]
+  float* sM = sG + (size_t)2 * GB;                           // matrices [matrix][colour][l][k]
   bool any3 = false;
   if (MODE >= R_T1)
     for (int32_t g = 0; g < gcount; ++g) any3 = any3 || a.need3[g0 + g] != 0;
@@ -541,23 +553,111 @@ __global__ void __launch_bounds__(32 * (B23Cfg<MODE>::CW + B23Cfg<MODE>::NP), 1)
     if (MODE == R_T1) sM[B23_G * MM + e] = in ? (float)a.M2[o + l * 23 + k] : 0.0f;
   }
   // rows past the end of the last tile and columns past the last colour stay zero in the Gram copies
-  for (int32_t e = threadIdx.x; e < C::NG * R * B23_GP; e += blockDim.x) sG[e] = 0.0f;
+  for (int32_t e = threadIdx.x; e < 2 * GB; e += blockDim.x) sG[e] = 0.0f;
   __syncthreads();
   if (*ring.abort) return;
-  if (warp >= C::CW) {
+  if (warp >= C::PW + C::GW) {
     const float* src[3] = {a.W, a.Q, a.Qp};
-    ring.template produce<OUT>(warp - C::CW, src, MODE <= R_S3 ? (use_p ? 3 : 2) : 1, a.out,
+    ring.template produce<OUT>(warp - C::PW - C::GW, src, MODE <= R_S3 ? (use_p ? 3 : 2) : 1, a.out,
                                MODE == R_T1 && any3 ? a.out2 : nullptr, a.ws, g0 * 23, (gcount * 23 + 3) / 4);
     return;
   }
   auto sync = [] { asm volatile("bar.sync 1, %0;" ::"n"(CT) : "memory"); };
-  // products: warps 0 to 7
-  const int pc = warp & 3, pr = 32 * (warp >> 2) + lane;
-  const bool prod = warp < 8 && pc < gcount;
-  const bool n3 = MODE >= R_T1 && prod && a.need3[g0 + pc] != 0;
+  auto product = [&](int32_t t, int pc) {
+    const bool n3 = MODE >= R_T1 && a.need3[g0 + pc] != 0;
+    float* st = ring.stage(t);
+    const int nr = ring.rows(t);
+    float* row[RPL];
+    float* grow = sG + (size_t)(t & 1) * GB + (size_t)lane * B23_GP + 24 * pc;
+    float x[RPL][24];
+    unsigned long long o[RPL][12];
+#pragma unroll
+    for (int h = 0; h < RPL; ++h) row[h] = st + (size_t)(lane + 32 * h) * ring.pitch;
+    auto load = [&](int array) {  // rows past the end as zeros
+#pragma unroll
+      for (int h = 0; h < RPL; ++h) {
+        load_row_of(pc, row[h] + (size_t)array * R * ring.pitch, x[h]);
+        if (lane + 32 * h >= nr)
+#pragma unroll
+          for (int i = 0; i < 24; ++i) x[h][i] = 0.0f;
+      }
+    };
+    auto to_gram = [&](int array, auto val) {
+#pragma unroll
+      for (int h = 0; h < RPL; ++h)
+#pragma unroll
+        for (int i = 0; i < 6; ++i)
+          *reinterpret_cast<ulonglong2*>(grow + ((size_t)array * R + 32 * h) * B23_GP + 4 * i) =
+              make_ulonglong2(val(h, 2 * i), val(h, 2 * i + 1));
+    };
+    auto as_x = [&](int h, int i) { return pack2(x[h][2 * i], x[h][2 * i + 1]); };
+    auto as_o = [&](int h, int i) { return o[h][i]; };
+    load(0);  // W
+    if (MODE <= R_S3) {
+#pragma unroll
+      for (int h = 0; h < RPL; ++h)
+#pragma unroll
+        for (int i = 0; i < 12; ++i) o[h][i] = as_x(h, i);
+      if (use_p) {
+        load(2);  // Q_{j-1}
+        mul_rows<1>(o, x, sM + pc * MM);
+        if (MODE == R_S1) to_gram(2, as_x);
+      }
+      if (MODE == R_S1) to_gram(0, as_o);
+      load(1);  // Q_j
+      if (MODE == R_S1) {
+        to_gram(1, as_x);
+      } else {
+        mul_rows<0>(o, x, sM + (B23_G + pc) * MM);
+        if (use_p) {
+          load(2);
+          mul_rows<0>(o, x, sM + (2 * B23_G + pc) * MM);
+        }
+      }
+    } else {
+#pragma unroll
+      for (int h = 0; h < RPL; ++h)
+#pragma unroll
+        for (int i = 0; i < 12; ++i) o[h][i] = 0ull;
+      mul_rows<2>(o, x, sM + pc * MM);
+      if (MODE == R_T1) {
+#pragma unroll
+        for (int h = 0; h < RPL; ++h)
+#pragma unroll
+          for (int i = 0; i < 12; ++i) {
+            x[h][2 * i] = lo2(o[h][i]);
+            x[h][2 * i + 1] = hi2(o[h][i]);
+            o[h][i] = 0ull;
+          }
+        mul_rows<2>(o, x, sM + (B23_G + pc) * MM);
+      }
+    }
+    if (OUT) {
+#pragma unroll
+      for (int h = 0; h < RPL; ++h) {
+        if (MODE != R_T2 || n3) store_row_of(pc, row[h], o[h]);
+        if (pc + 1 == gcount)
+          for (int32_t i = 23 * gcount; i & 3; ++i) row[h][i] = 0.0f;  // columns past the last colour
+      }
+    }
+    if (MODE != R_S1 && gram) to_gram(0, as_o);
+  };
+  // the products of tile t run beside the Grams of tile t - 1, one barrier a tile; a warp whose wait gives
+  // up still runs every barrier, so that no other waits for it
+  if (warp < C::PW) {
+#pragma unroll 1
+    for (int32_t t = 0; t <= ring.ntile; ++t) {
+      if (t < ring.ntile && ring.wait_full(t))
+#pragma unroll 1
+        for (int pc = warp; pc < gcount; pc += C::PW) product(t, pc);
+      sync();  // the Gram copies of tile t are in place, those of tile t - 1 free, the ring's stage is done with
+      if (threadIdx.x == 0 && t < ring.ntile) ring.arrive(t);
+    }
+    return;
+  }
   // Grams: this thread's block and rows
-  constexpr int S = 8;
-  const int gs = threadIdx.x & (S - 1), blk = threadIdx.x / S;
+  constexpr int S = C::S;
+  const int gt = (int)threadIdx.x - 32 * C::PW, gs = gt & (S - 1), blk = gt / S;
   const int gc = MODE == R_S1 ? blk / 9 : blk / 6, gb = MODE == R_S1 ? blk % 9 : blk % 6;
   const int kb = MODE == R_S1 ? gb / 3 : gb < 3 ? 0 : gb < 5 ? 1 : 2;
   const int lb = MODE == R_S1 ? gb % 3 : gb < 3 ? gb : gb < 5 ? gb - 2 : 2;
@@ -568,104 +668,37 @@ __global__ void __launch_bounds__(32 * (B23Cfg<MODE>::CW + B23Cfg<MODE>::NP), 1)
     vq[i] = 0ull;
     if (MODE == R_S1) vp[i % (MODE == R_S1 ? 32 : 1)] = 0ull;
   }
-  // a warp whose wait gives up still runs every barrier, so that no other waits for it
-#pragma unroll 1
-  for (int32_t t = 0; t < ring.ntile; ++t) {
-    const bool ok = ring.wait_full(t);
-    float* st = ring.stage(t);
-    if (prod && ok) {
-      const bool valid = pr < ring.rows(t);
-      float* row = st + (size_t)pr * ring.pitch;
-      float* grow = sG + (size_t)pr * B23_GP + 24 * pc;
-      float x[24];
-      unsigned long long o[12];
-      auto zero_past_end = [&]() {
-        if (!valid)
-#pragma unroll
-          for (int i = 0; i < 24; ++i) x[i] = 0.0f;
-      };
-      auto to_gram = [&](int array, auto val) {
-#pragma unroll
-        for (int i = 0; i < 6; ++i)
-          *reinterpret_cast<ulonglong2*>(grow + (size_t)array * R * B23_GP + 4 * i) = make_ulonglong2(val(2 * i), val(2 * i + 1));
-      };
-      load_row_of(pc, row, x);  // W
-      zero_past_end();
-      if (MODE <= R_S3) {
-#pragma unroll
-        for (int i = 0; i < 12; ++i) o[i] = pack2(x[2 * i], x[2 * i + 1]);
-        if (use_p) {
-          load_row_of(pc, row + 2 * (size_t)R * ring.pitch, x);  // Q_{j-1}
-          zero_past_end();
-          mul_row<1>(o, x, sM + pc * MM);
-          if (MODE == R_S1) to_gram(2, [&](int i) { return pack2(x[2 * i], x[2 * i + 1]); });
-        }
-        if (MODE == R_S1) {
-          to_gram(0, [&](int i) { return o[i]; });
-          load_row_of(pc, row + (size_t)R * ring.pitch, x);  // Q_j
-          zero_past_end();
-          to_gram(1, [&](int i) { return pack2(x[2 * i], x[2 * i + 1]); });
-        } else {
-          float q[24];
-          load_row_of(pc, row + (size_t)R * ring.pitch, q);
-          if (!valid)
-#pragma unroll
-            for (int i = 0; i < 24; ++i) q[i] = 0.0f;
-          mul_row<0>(o, q, sM + (B23_G + pc) * MM);
-          if (use_p) mul_row<0>(o, x, sM + (2 * B23_G + pc) * MM);
-        }
-      } else {
-#pragma unroll
-        for (int i = 0; i < 12; ++i) o[i] = 0ull;
-        mul_row<2>(o, x, sM + pc * MM);
-        if (MODE == R_T1) {
-#pragma unroll
-          for (int i = 0; i < 12; ++i) {
-            x[2 * i] = lo2(o[i]);
-            x[2 * i + 1] = hi2(o[i]);
-            o[i] = 0ull;
-          }
-          mul_row<2>(o, x, sM + (B23_G + pc) * MM);
-        }
-      }
-      if (OUT) {
-        if (MODE != R_T2 || n3) store_row_of(pc, row, o);
-        if (pc + 1 == gcount)
-          for (int32_t i = 23 * gcount; i & 3; ++i) row[i] = 0.0f;  // columns past the last colour
-      }
-      if (MODE != R_S1 && gram) to_gram(0, [&](int i) { return o[i]; });
-    }
-    sync();  // products of the tile are in place; the ring's stage is read (or finished)
-    if (threadIdx.x == 0) ring.arrive(t);
-    if (!gram) continue;
-    if (ok && gc < B23_G) {  // whole warps
-      const float* y0 = sG + (size_t)gs * B23_GP + 24 * gc + 8 * lb;
-      const float* x0 = sG + (size_t)gs * B23_GP + 24 * gc + 8 * kb + (MODE == R_S1 ? R * B23_GP : 0);
+  auto sum_tile = [&](int32_t t) {
+    const float* buf = sG + (size_t)(t & 1) * GB + (size_t)gs * B23_GP + 24 * gc;
+    const float *y0 = buf + 8 * lb, *x0 = buf + 8 * kb + (MODE == R_S1 ? R * B23_GP : 0);
 #pragma unroll(MODE == R_S1 ? 1 : 2)
-      for (int i = 0; i < R / S; ++i, y0 += S * B23_GP, x0 += S * B23_GP) {
-        const ulonglong2 ya = *reinterpret_cast<const ulonglong2*>(y0), yb = *reinterpret_cast<const ulonglong2*>(y0 + 4);
-        auto rank1 = [&](const float* xr, unsigned long long* v) {
-          const float4 xa = *reinterpret_cast<const float4*>(xr), xb = *reinterpret_cast<const float4*>(xr + 4);
-          const float xv[8] = {xa.x, xa.y, xa.z, xa.w, xb.x, xb.y, xb.z, xb.w};
+    for (int i = 0; i < R / S; ++i, y0 += S * B23_GP, x0 += S * B23_GP) {
+      const ulonglong2 ya = *reinterpret_cast<const ulonglong2*>(y0), yb = *reinterpret_cast<const ulonglong2*>(y0 + 4);
+      auto rank1 = [&](const float* xr, unsigned long long* v) {
+        const float4 xa = *reinterpret_cast<const float4*>(xr), xb = *reinterpret_cast<const float4*>(xr + 4);
+        const float xv[8] = {xa.x, xa.y, xa.z, xa.w, xb.x, xb.y, xb.z, xb.w};
 #pragma unroll
-          for (int k = 0; k < 8; ++k) {
-            const unsigned long long xx = dup2(xv[k]);
-            fma2(v[4 * k], xx, ya.x);
-            fma2(v[4 * k + 1], xx, ya.y);
-            fma2(v[4 * k + 2], xx, yb.x);
-            fma2(v[4 * k + 3], xx, yb.y);
-          }
-        };
-        rank1(x0, vq);
-        if constexpr (MODE == R_S1) rank1(x0 + R * B23_GP, vp);
-      }
-      constexpr int FL = 32 / (R / S);  // tiles of 32 rows per lane
-      if (t % FL == FL - 1 || t + 1 == ring.ntile) {
-        block_flush<S>(vq, hq, lq);
-        if constexpr (MODE == R_S1) block_flush<S>(vp, hp, lp);
-      }
+        for (int k = 0; k < 8; ++k) {
+          const unsigned long long xx = dup2(xv[k]);
+          fma2(v[4 * k], xx, ya.x);
+          fma2(v[4 * k + 1], xx, ya.y);
+          fma2(v[4 * k + 2], xx, yb.x);
+          fma2(v[4 * k + 3], xx, yb.y);
+        }
+      };
+      rank1(x0, vq);
+      if constexpr (MODE == R_S1) rank1(x0 + R * B23_GP, vp);
     }
-    sync();  // the Gram copies are free for the next tile
+    constexpr int FL = 32 / (R / S);  // tiles of 32 rows per lane
+    if (t % FL == FL - 1 || t + 1 == ring.ntile) {
+      block_flush<S>(vq, hq, lq);
+      if constexpr (MODE == R_S1) block_flush<S>(vp, hp, lp);
+    }
+  };
+#pragma unroll 1
+  for (int32_t t = 0; t <= ring.ntile; ++t) {
+    if (t > 0 && gram) sum_tile(t - 1);
+    sync();
   }
   if (!gram || *ring.abort || gc >= gcount) return;
   if (MODE == R_T1 && a.need3[g0 + gc] == 0) return;
@@ -715,7 +748,7 @@ css_status launch_rows23(css_ctx* ctx, RowsArgs& r, cudaStream_t st) {
   using C = B23Cfg<MODE>;
   CSS_CU(ctx, cudaFuncSetAttribute(k_rows23<MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)C::smem));
   const dim3 grid((unsigned)css_ceil_div(r.N, r.rchk), (unsigned)css_ceil_div(r.ncb, B23_G));
-  k_rows23<MODE><<<grid, 32 * (C::CW + C::NP), C::smem, st>>>(r);
+  k_rows23<MODE><<<grid, 32 * 12, C::smem, st>>>(r);
   CSS_LAUNCHED(ctx);
   return CSS_OK;
 }
@@ -730,7 +763,7 @@ css_status launch_rows(css_ctx* ctx, int32_t b, RowsArgs& r, cudaStream_t st) {
 bool css_rows_supported(bool fp32, int32_t b) { return fp32 && (b == 6 || b == 23); }
 
 int32_t css_rows_chunk(int64_t N, int32_t b) {
-  return b == 6 ? pick_chunk(N, 7, B6_R, 2048) : pick_chunk(N, 17, B23_R, 2048);
+  return b == 6 ? pick_chunk(N, 7, B6_R, 2048) : pick_chunk(N, 17, 64, 2048);
 }
 
 css_status css_rows(css_ctx* ctx, int mode, const CssRows& p, cudaStream_t st) {
