@@ -215,6 +215,95 @@ __global__ void __launch_bounds__(NW * 32, MINB) k_spmm_dup(SdArgs a) {
   }
 }
 
+// b = 6 with the rows of a CTA side by side: warp r of a CTA takes block row blockIdx.x R + r, all for the same
+// 128 columns (4 per lane).  A V_J is 6 rows for 36 FMAs a column, so at b = 6 the ring kernel above is bound by
+// the 16-byte loads of V from L2 (8.3 TB/s at 60,000 molecules, 31% of the FFMA peak).  Rows that follow one
+// another are neighbours in space as the molecules are numbered and share most of their J, so here V goes
+// through L1, which one CTA's warps fill for one another.  A warp's H blocks (144 bytes) come three steps ahead
+// through a ring of its own (nine lanes copy 16 bytes each), its column indices 32 at a time, V one step
+// ahead; no warp waits for another.  The sums are the ring kernel's, FMA by FMA.  Ring kernel -> this, four rows
+// a CTA: 60,000 molecules 1.90 -> 1.68 ms, 4,001 117 -> 92 us, 512 27.0 -> 20.9 us (eight rows 1.71 ms, sixteen 1.78).
+constexpr int S6_NS = 4;  // H blocks in flight and in use per warp
+template <int R, int MINB>
+__global__ void __launch_bounds__(R * 32, MINB) k_spmm6_rows(SdArgs a, int32_t n_brow) {
+  constexpr unsigned FULL = 0xffffffffu;
+  __shared__ __align__(16) float ring[R][S6_NS][36];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int32_t I = blockIdx.x * R + warp;
+  if (I >= n_brow) return;  // whole warp; nothing below involves other warps
+  const int32_t col = blockIdx.y * 128 + lane * 4;
+  const int32_t p0 = a.row_ptr[I], nnz = a.row_ptr[I + 1] - p0, nsteps = nnz + (a.Hlot ? 1 : 0);
+  const float* Vc = a.V + (col < a.w ? col : 0);  // lanes past w read column 0 and store nothing
+  auto copy_h = [&](int32_t q) {
+    if (q < nsteps && lane < 9) {
+      const float* src = (q < nnz ? a.Ht + (size_t)(p0 + q) * 36 : a.Hlot + (size_t)I * 36) + 4 * lane;
+      asm volatile("cp.async.ca.shared.global [%0], [%1], 16;" ::"r"(su32(&ring[warp][q % S6_NS][4 * lane])), "l"(src)
+                   : "memory");
+    }
+    asm volatile("cp.async.commit_group;" ::: "memory");
+  };
+  for (int q = 0; q < S6_NS - 1; ++q) copy_h(q);
+  int32_t jl = lane < nnz ? a.col_idx[p0 + lane] - a.jbase : I, jnext = 0;
+  auto load_v = [&](int32_t J, float4 (&v)[6]) {
+#pragma unroll
+    for (int k = 0; k < 6; ++k) v[k] = __ldg(reinterpret_cast<const float4*>(Vc + ((size_t)J * 6 + k) * a.ws));
+  };
+  unsigned long long acc[3][4];
+#pragma unroll
+  for (int i = 0; i < 3; ++i)
+#pragma unroll
+    for (int u = 0; u < 4; ++u) acc[i][u] = 0ull;
+  float4 v[6], vn[6];
+  if (nsteps > 0) load_v(__shfl_sync(FULL, jl, 0), v);
+#pragma unroll 2
+  for (int32_t q = 0; q < nsteps; ++q) {
+    if ((q & 31) == 16) {  // the next 32 column indices
+      const int32_t n = (q & ~31) + 32 + lane;
+      jnext = n < nnz ? a.col_idx[p0 + n] - a.jbase : I;
+    }
+    if ((q & 31) == 31) jl = jnext;
+    if (q + 1 < nsteps) load_v(__shfl_sync(FULL, jl, (q + 1) & 31), vn);
+    asm volatile("cp.async.wait_group %0;" ::"n"(S6_NS - 2) : "memory");
+    __syncwarp();  // block q is there for every lane, block q - 1 is read
+    copy_h(q + S6_NS - 1);
+    const ulonglong2* h = reinterpret_cast<const ulonglong2*>(ring[warp][q % S6_NS]);
+#pragma unroll
+    for (int k = 0; k < 6; k += 2) {
+      const ulonglong2 h0 = h[3 * (k / 2)], h1 = h[3 * (k / 2) + 1], h2 = h[3 * (k / 2) + 2];
+      const unsigned long long a0[4] = {dup2(v[k].x), dup2(v[k].y), dup2(v[k].z), dup2(v[k].w)};
+      const unsigned long long a1[4] = {dup2(v[k + 1].x), dup2(v[k + 1].y), dup2(v[k + 1].z), dup2(v[k + 1].w)};
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        fma2(acc[0][u], h0.x, a0[u]);
+        fma2(acc[1][u], h0.y, a0[u]);
+        fma2(acc[2][u], h1.x, a0[u]);
+        fma2(acc[0][u], h1.y, a1[u]);
+        fma2(acc[1][u], h2.x, a1[u]);
+        fma2(acc[2][u], h2.y, a1[u]);
+      }
+    }
+#pragma unroll
+    for (int k = 0; k < 6; ++k) v[k] = vn[k];
+  }
+  asm volatile("cp.async.wait_all;" ::: "memory");
+  if (col >= a.w) return;
+  const bool whole = col + 4 <= a.w;
+  float* Wr = a.W + (size_t)I * 6 * a.ws + col;
+#pragma unroll
+  for (int r = 0; r < 6; ++r) {
+    float o[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) o[u] = __uint_as_float((unsigned)(r & 1 ? acc[r >> 1][u] >> 32 : acc[r >> 1][u]));
+    if (whole) {
+      *reinterpret_cast<float4*>(Wr + (size_t)r * a.ws) = make_float4(o[0], o[1], o[2], o[3]);
+    } else {
+#pragma unroll
+      for (int u = 0; u < 4; ++u)
+        if (col + u < a.w) Wr[(size_t)r * a.ws + u] = o[u];
+    }
+  }
+}
+
 // Ht[p][k][r] = H_p[r][k] in FP32 (round to nearest) for r, k < b, zero for the pad row r = b of
 // an odd b.  LO: block p is the diagonal block of row p, and the value the low FP32 part
 // fl32(h - fl32(h)) (zero for a row without a diagonal block).
@@ -243,11 +332,7 @@ __global__ void k_hdup(int64_t nblocks, int32_t b, int32_t RA, const double* __r
   Ht[e] = v;
 }
 
-template <int B, int NW, int MINB>
-css_status launch_dup(css_ctx* ctx, const LzArgs& a, const float* V, float* W, int* err, cudaStream_t st) {
-  using C = SdCfg<B, NW>;
-  auto kern = k_spmm_dup<B, NW, MINB>;
-  static_assert(C::smem <= 48 * 1024, "static shared-memory limit");
+SdArgs dup_args(const css_ctx* ctx, const LzArgs& a, const float* V, float* W, int* err) {
   SdArgs s;
   s.row_ptr = a.row_ptr;
   s.col_idx = a.col_idx;
@@ -260,8 +345,23 @@ css_status launch_dup(css_ctx* ctx, const LzArgs& a, const float* V, float* W, i
   s.jbase = a.row0;
   s.empty_extra = ctx->test_spmm_empty_extra;
   s.err = err;
+  return s;
+}
+
+template <int B, int NW, int MINB>
+css_status launch_dup(css_ctx* ctx, const LzArgs& a, const float* V, float* W, int* err, cudaStream_t st) {
+  using C = SdCfg<B, NW>;
+  static_assert(C::smem <= 48 * 1024, "static shared-memory limit");
   const dim3 grid((unsigned)a.n_brow, (unsigned)css_ceil_div(a.w, C::CT));
-  kern<<<grid, C::NT, C::smem, st>>>(s);
+  k_spmm_dup<B, NW, MINB><<<grid, C::NT, C::smem, st>>>(dup_args(ctx, a, V, W, err));
+  CSS_LAUNCHED(ctx);
+  return CSS_OK;
+}
+
+template <int R, int MINB>
+css_status launch_rows(css_ctx* ctx, const LzArgs& a, const float* V, float* W, int* err, cudaStream_t st) {
+  const dim3 grid((unsigned)css_ceil_div(a.n_brow, R), (unsigned)css_ceil_div(a.w, 128));
+  k_spmm6_rows<R, MINB><<<grid, R * 32, 0, st>>>(dup_args(ctx, a, V, W, err), a.n_brow);
   CSS_LAUNCHED(ctx);
   return CSS_OK;
 }
@@ -565,8 +665,8 @@ css_status css_spmm_dup_prepare(css_ctx* ctx, int32_t b, int32_t n_brow, int32_t
   return CSS_OK;
 }
 
-// launch variants (columns per thread, warps per CTA, CTAs per SM the registers are sized for);
-// every variant sums each output in the same order
+// launch variants (warps per CTA, CTAs per SM the registers are sized for; at b = 6 three of the kernel with
+// rows side by side and the ring kernel); every variant sums each output in the same order
 css_status css_spmm_dup(css_ctx* ctx, const LzArgs& a, const float* V, float* W, int v, cudaStream_t st) {
   if (a.n_brow == 0 || a.w == 0) return CSS_OK;
   if (((uintptr_t)V & 15) || ((uintptr_t)W & 15) || (a.ws & 7))
@@ -583,9 +683,9 @@ css_status css_spmm_dup(css_ctx* ctx, const LzArgs& a, const float* V, float* W,
   }
   if (a.b == 6) {
     switch (v) {
-      case 0: return launch_dup<6, 2, 8>(ctx, a, V, W, err, st);
-      case 1: return launch_dup<6, 4, 4>(ctx, a, V, W, err, st);
-      case 2: return launch_dup<6, 8, 2>(ctx, a, V, W, err, st);
+      case 0: return launch_rows<4, 4>(ctx, a, V, W, err, st);
+      case 1: return launch_rows<8, 2>(ctx, a, V, W, err, st);
+      case 2: return launch_rows<16, 1>(ctx, a, V, W, err, st);
       default: return launch_dup<6, 1, 16>(ctx, a, V, W, err, st);
     }
   }
