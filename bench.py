@@ -38,10 +38,16 @@ SPMM_KERNEL_VERSION = "k_spmm_dup-v2"  # profiles/spmm_traffic.json must name th
 
 def hv_kernel(mixed, b, tc=False):
     """(name, version tag) of the H*V kernel a build runs: the tensor-core one when asked for, the
-    exact-width FP32 kernel for b = 6 and 23, else the padded FFMA/DFMA kernel."""
+    exact-width FP32 kernels for b = 6 and 23, the digit products for FP64 with b <= 24, else the padded
+    FFMA/DFMA kernel."""
     if mixed and (tc or os.environ.get("CSS_HV_TC") == "1") and 16 < b <= 24:
         return "k_hv_tc (H*V on tcgen05, 3xTF32)", "k_hv_tc"
-    if mixed and b in (6, 23) and not os.environ.get("CSS_SPMM_VARIANT"):
+    if not mixed and b <= 24 and not os.environ.get("CSS_SPMM_VARIANT"):
+        return ("k_hv_int (FP64 H*V by exact products of 8-bit digits on the bf16 tensor cores)", "k_hv_int")
+    if mixed and b == 6 and not os.environ.get("CSS_SPMM_VARIANT"):
+        return ("k_spmm6_rows / k_spmm_dup (exact-width H*V on the FP32 FMA pipe, the faster as tuned)",
+                "k_spmm6_rows")
+    if mixed and b == 23 and not os.environ.get("CSS_SPMM_VARIANT"):
         return ("k_spmm_dup (exact-width H*V on the FP32 FMA pipe, packed row pairs, all colours of the "
                 "system as columns)", SPMM_KERNEL_VERSION)
     return ("k_spmm (padded H*V on the " + ("FP32 FMA" if mixed else "FP64 DFMA") +
@@ -534,11 +540,9 @@ def main():
     tc = (os.environ.get("CSS_HV_TC") == "1" or prec == css.CSS_MIXED_3XTF32) and mixed and 16 < H0.b <= 24
     split = prec == css.CSS_FP64_SPLIT
     hv_name, hv_version = hv_kernel(mixed, H0.b, tc)
-    if split:
-        hv_name, hv_version = ("k_spmm_df (FP64-accurate H*V in FP32 hi + lo pairs on the FP32 FMA pipe)",
-                               "k_spmm_df")
-    # the split arithmetic takes 11 FP32 lane operations per FP64-equivalent term (2 flop)
-    peak = (tf32_peak if tc else fp32_peak) if mixed else (fp32_peak / 11.0 if split else FP64_PEAK)
+    digits = hv_version == "k_hv_int"
+    # the digit arithmetic takes 34 bf16 products per FP64-equivalent product
+    peak = (tf32_peak if tc else fp32_peak) if mixed else (pk["bf16_sustained"] / 34.0 if digits else FP64_PEAK)
     traffic = None
     tf = ROOT / "profiles" / "spmm_traffic.json"
     if tf.exists():
@@ -554,19 +558,19 @@ def main():
     line = {"metric": METRIC, "value": value, "unit": "s/P-build", "n_gpus": ws,
             "steps": a.steps, "warmup": a.warmup, "ms_per_step": elapsed / a.steps * 1e3, "higher_is_better": False,
             "scaling": "weak", "vs_baseline": None,
-            "dtype": "f32+f64" if mixed else ("f64 (H*V in f32 pairs)" if split else "f64"),
+            "dtype": "f32+f64" if mixed else "f64",
             "data": "synthetic", "config": cfg,
             "roofline": {"kernel": hv_name,
-                         "bound": "tensor" if tc else ("alu" if mixed or split else "alu_fp64"),
+                         "bound": "tensor" if tc or digits else ("alu" if mixed else "alu_fp64"),
                          "achieved": achieved, "peak": peak, "unit": "TFLOP/s", "frac": achieved / peak,
                          "traffic": None if tc else traffic,
                          "peak_source": (f"dense TF32 tensor peak: measured sustained BF16 {pk['bf16_sustained']:.0f} "
                                          f"TF/s x 1.1/2.25 ({pk['source']})" if tc else
                                          f"FP32 FFMA (CUDA-core) ceiling: {n_sm} SMs x 128 lanes x 2 flop x "
                                          f"{pk['sm_max_mhz']:.0f} MHz" if mixed else
-                                         f"FP32 FFMA ceiling / 11 FP32 operations per FP64-equivalent term "
-                                         f"({n_sm} SMs x 128 lanes x 2 flop x {pk['sm_max_mhz']:.0f} MHz / 11)"
-                                         if split else FP64_PEAK_NOTE),
+                                         f"measured sustained dense BF16 {pk['bf16_sustained']:.0f} TF/s / 34 digit "
+                                         f"products per FP64 product ({pk['source']})"
+                                         if digits else FP64_PEAK_NOTE),
                          "frac_vs_tf32_tensor_peak": achieved / tf32_peak if mixed else None,
                          "launch_ms": spmm_avg, "flops_per_launch": last_inf["spmm_flops"],
                          "alg_bytes_per_launch": last_inf["spmm_bytes"]},
@@ -597,7 +601,7 @@ def main():
         t64 = e0.elapsed_time(e1) / 2e3
         inf64 = ctx.info()
         dP = float((P64 - P[t]).abs().max().item())
-        # the same FP64 build with the recurrence's H*V in FP32 pairs (CSS_FP64_SPLIT, b = 6 or 23):
+        # the same FP64 build with CSS_FP64_SPLIT (b = 6 or 23):
         # one untimed, one timed build, its P against the FP64 P
         split = None
         if Hd.b in (6, 23):
@@ -617,8 +621,8 @@ def main():
                      "max_abs_dP_vs_fp64": float((Psp - P64).abs().max().item()),
                      "dTrP_vs_fp64": rsp["trP"] - r64["trP"],
                      "dE_band_eV_per_molecule_vs_fp64": abs(2 * (rsp["trPH"] - r64["trPH"])) / a.n_mol,
-                     "note": "CSS_FP64_SPLIT: FP64 vectors, the recurrence's H*V with FP32 hi + lo pairs and "
-                             "error-free products on the FP32 FMA pipe"}
+                     "note": "CSS_FP64_SPLIT: FP64 vectors; the recurrence's H*V by exact digit products where the "
+                             "digits of H fit 8 GiB, in FP32 pairs beyond"}
             del Psp
         # FP64 at the mixed run's mu: the error of the mixed arithmetic alone, without the
         # change of mu (any mu in the gap satisfies the electron count)
