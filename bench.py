@@ -538,7 +538,6 @@ def main():
     fp32_peak = fp32_peak_tflops(n_sm, pk["sm_max_mhz"])
     tf32_peak = tf32_peak_tflops(pk)
     tc = (os.environ.get("CSS_HV_TC") == "1" or prec == css.CSS_MIXED_3XTF32) and mixed and 16 < H0.b <= 24
-    split = prec == css.CSS_FP64_SPLIT
     hv_name, hv_version = hv_kernel(mixed, H0.b, tc)
     digits = hv_version == "k_hv_int"
     # the digit arithmetic takes 34 bf16 products per FP64-equivalent product
