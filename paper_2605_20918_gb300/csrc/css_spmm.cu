@@ -222,13 +222,74 @@ __global__ void __launch_bounds__(NW * 32, MINB) k_spmm_dup(SdArgs a) {
 // through L1, which one CTA's warps fill for one another.  A warp's H blocks (144 bytes) come three steps ahead
 // through a ring of its own (nine lanes copy 16 bytes each), its column indices 32 at a time, V one step
 // ahead; no warp waits for another.  The sums are the ring kernel's, FMA by FMA.  Ring kernel -> this, four rows
-// a CTA: 60,000 molecules 1.90 -> 1.68 ms, 4,001 117 -> 92 us, 512 27.0 -> 20.9 us (eight rows 1.71 ms, sixteen 1.78).
+// a CTA: 60,000 molecules (w = 396) 1.90 -> 1.37 ms, 4,001 117 -> 92 us, 512 27.0 -> 20.9 us (eight rows 1.40 ms, sixteen 1.46).
+// The last tile, when at most half of its columns exist, packs rows into a warp instead: as many lanes per row
+// as it has 4-column chunks, each lane with its own row's indices and H blocks by plain loads through L1 (a
+// whole warp for 12 columns cost 1.68 instead of 1.37 ms at w = 396).
 constexpr int S6_NS = 4;  // H blocks in flight and in use per warp
+// acc += H_p V_J for a 6 x 6 block (h: pairs of rows, k ascending) and 4 columns
+__device__ __forceinline__ void block6(unsigned long long (&acc)[3][4], const ulonglong2* h, const float4 (&v)[6]) {
+#pragma unroll
+  for (int k = 0; k < 6; k += 2) {
+    const ulonglong2 h0 = h[3 * (k / 2)], h1 = h[3 * (k / 2) + 1], h2 = h[3 * (k / 2) + 2];
+    const unsigned long long a0[4] = {dup2(v[k].x), dup2(v[k].y), dup2(v[k].z), dup2(v[k].w)};
+    const unsigned long long a1[4] = {dup2(v[k + 1].x), dup2(v[k + 1].y), dup2(v[k + 1].z), dup2(v[k + 1].w)};
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      fma2(acc[0][u], h0.x, a0[u]);
+      fma2(acc[1][u], h0.y, a0[u]);
+      fma2(acc[2][u], h1.x, a0[u]);
+      fma2(acc[0][u], h1.y, a1[u]);
+      fma2(acc[1][u], h2.x, a1[u]);
+      fma2(acc[2][u], h2.y, a1[u]);
+    }
+  }
+}
+__device__ __forceinline__ void store6(const unsigned long long (&acc)[3][4], float* Wr, int32_t ws, int32_t left) {
+#pragma unroll
+  for (int r = 0; r < 6; ++r) {
+    float o[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) o[u] = __uint_as_float((unsigned)(r & 1 ? acc[r >> 1][u] >> 32 : acc[r >> 1][u]));
+    if (left >= 4) {
+      *reinterpret_cast<float4*>(Wr + (size_t)r * ws) = make_float4(o[0], o[1], o[2], o[3]);
+    } else {
+#pragma unroll
+      for (int u = 0; u < 4; ++u)
+        if (u < left) Wr[(size_t)r * ws + u] = o[u];
+    }
+  }
+}
 template <int R, int MINB>
 __global__ void __launch_bounds__(R * 32, MINB) k_spmm6_rows(SdArgs a, int32_t n_brow) {
   constexpr unsigned FULL = 0xffffffffu;
   __shared__ __align__(16) float ring[R][S6_NS][36];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int32_t tail = a.w - (int32_t)blockIdx.y * 128;
+  if (tail <= 64) {  // lanes of a row: its chunks of 4 columns
+    const int32_t L = (tail + 3) / 4, rpw = 32 / L, sub = lane / L;
+    const int32_t I = (blockIdx.x * R + warp) * rpw + sub, col = blockIdx.y * 128 + 4 * (lane - sub * L);
+    const bool valid = sub < rpw && I < n_brow;
+    const int32_t p0 = valid ? a.row_ptr[I] : 0, nnz = valid ? a.row_ptr[I + 1] - p0 : 0;
+    const int32_t nsteps = valid ? nnz + (a.Hlot ? 1 : 0) : 0;
+    const int32_t most = __reduce_max_sync(FULL, nsteps);
+    unsigned long long acc[3][4] = {};
+#pragma unroll 2
+    for (int32_t q = 0; q < most; ++q) {
+      if (q >= nsteps) continue;
+      const int32_t J = q < nnz ? a.col_idx[p0 + q] - a.jbase : I;
+      const float* hs = q < nnz ? a.Ht + (size_t)(p0 + q) * 36 : a.Hlot + (size_t)I * 36;
+      ulonglong2 h[9];
+      float4 v[6];
+#pragma unroll
+      for (int i = 0; i < 9; ++i) h[i] = __ldg(reinterpret_cast<const ulonglong2*>(hs) + i);
+#pragma unroll
+      for (int k = 0; k < 6; ++k) v[k] = __ldg(reinterpret_cast<const float4*>(a.V + ((size_t)J * 6 + k) * a.ws + col));
+      block6(acc, h, v);
+    }
+    if (valid) store6(acc, a.W + (size_t)I * 6 * a.ws + col, a.ws, a.w - col);
+    return;
+  }
   const int32_t I = blockIdx.x * R + warp;
   if (I >= n_brow) return;  // whole warp; nothing below involves other warps
   const int32_t col = blockIdx.y * 128 + lane * 4;
@@ -266,42 +327,12 @@ __global__ void __launch_bounds__(R * 32, MINB) k_spmm6_rows(SdArgs a, int32_t n
     asm volatile("cp.async.wait_group %0;" ::"n"(S6_NS - 2) : "memory");
     __syncwarp();  // block q is there for every lane, block q - 1 is read
     copy_h(q + S6_NS - 1);
-    const ulonglong2* h = reinterpret_cast<const ulonglong2*>(ring[warp][q % S6_NS]);
-#pragma unroll
-    for (int k = 0; k < 6; k += 2) {
-      const ulonglong2 h0 = h[3 * (k / 2)], h1 = h[3 * (k / 2) + 1], h2 = h[3 * (k / 2) + 2];
-      const unsigned long long a0[4] = {dup2(v[k].x), dup2(v[k].y), dup2(v[k].z), dup2(v[k].w)};
-      const unsigned long long a1[4] = {dup2(v[k + 1].x), dup2(v[k + 1].y), dup2(v[k + 1].z), dup2(v[k + 1].w)};
-#pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        fma2(acc[0][u], h0.x, a0[u]);
-        fma2(acc[1][u], h0.y, a0[u]);
-        fma2(acc[2][u], h1.x, a0[u]);
-        fma2(acc[0][u], h1.y, a1[u]);
-        fma2(acc[1][u], h2.x, a1[u]);
-        fma2(acc[2][u], h2.y, a1[u]);
-      }
-    }
+    block6(acc, reinterpret_cast<const ulonglong2*>(ring[warp][q % S6_NS]), v);
 #pragma unroll
     for (int k = 0; k < 6; ++k) v[k] = vn[k];
   }
   asm volatile("cp.async.wait_all;" ::: "memory");
-  if (col >= a.w) return;
-  const bool whole = col + 4 <= a.w;
-  float* Wr = a.W + (size_t)I * 6 * a.ws + col;
-#pragma unroll
-  for (int r = 0; r < 6; ++r) {
-    float o[4];
-#pragma unroll
-    for (int u = 0; u < 4; ++u) o[u] = __uint_as_float((unsigned)(r & 1 ? acc[r >> 1][u] >> 32 : acc[r >> 1][u]));
-    if (whole) {
-      *reinterpret_cast<float4*>(Wr + (size_t)r * a.ws) = make_float4(o[0], o[1], o[2], o[3]);
-    } else {
-#pragma unroll
-      for (int u = 0; u < 4; ++u)
-        if (col + u < a.w) Wr[(size_t)r * a.ws + u] = o[u];
-    }
-  }
+  if (col < a.w) store6(acc, a.W + (size_t)I * 6 * a.ws + col, a.ws, a.w - col);
 }
 
 // Ht[p][k][r] = H_p[r][k] in FP32 (round to nearest) for r, k < b, zero for the pad row r = b of

@@ -138,3 +138,27 @@ def test_fp64_row_pass_splits(torch, css, ctx, kind, n, nc, m):
     ref = oracle.density(H, col, s, nc, **kw)
     got = gpu_density(torch, css, ctx, H, col, s, nc, precision=css.CSS_FP64, **kw)
     assert float(np.abs(got["P"] - ref["P"]).max()) < FP64_TOL
+
+
+# FP32 H*V at b = 6, rows side by side: one column tile of few columns, half a tile (the last that packs rows
+# into a warp), one colour more, full tiles with such tails, and rows that do not fill a CTA; every variant
+# bitwise equal to the ring kernel
+@pytest.mark.parametrize("n,nc", [(1, 1), (33, 1), (75, 10), (75, 11), (75, 22), (130, 32), (130, 33), (130, 64)])
+def test_hv6_rows_equal_the_ring_kernel_bitwise(torch, css, monkeypatch, n, nc):
+    from paper_2605_20918_gb300 import synth
+    from tests.test_gpu_parity import gpu_density
+    g = synth.water_box(n)
+    H = synth.hamiltonian(g, "minimal")
+    col = (np.arange(n) % nc).astype(np.int32)
+    s = oracle.probes(col, H.b, 1005)
+    P = []
+    for v in "3012":
+        monkeypatch.setenv("CSS_SPMM_DUP_VARIANT", v)
+        c = css.Context(0)
+        try:
+            P.append(gpu_density(torch, css, c, H, col, s, nc, kT=0.05, n_elec=synth.n_electrons(n), m=min(n, 4), mu=-4.0,
+                                 solve_mu=False, precision=css.CSS_MIXED_FP32)["P"])
+        finally:
+            c.close()
+    for v in range(1, 4):
+        assert np.array_equal(P[0], P[v]), v
