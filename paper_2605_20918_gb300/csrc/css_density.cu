@@ -1982,12 +1982,15 @@ css_status css_density_nonorth(css_ctx* ctx, const css_bsr* S, const double* Sin
   const size_t vd_bytes = css_hv_int_v_bytes(n_brow, b, nc * b);
   const bool use_int = prec == CSS_FP64 && ctx->spmm_variant < 0 && css_hv_int_supported(b, n_brow, Hp->nnzb) &&
                        7 * vbytes + vd_bytes + ((size_t)9 << 30) <= free_b + ctx->ws_bytes;
-  const void* Hdig = nullptr;
+  const bool use_dup = ctx->spmm_variant < 0 && css_spmm_dup_supported(f32, b);
+  const void *Hdig = nullptr, *hdup = nullptr, *hlodup = nullptr;
   const int32_t* Hexp = nullptr;
   void* vdig = nullptr;
   if (use_int) {
     CSS_TRY(css_hv_int_prepare(ctx, b, n_brow, Hp->nnzb, Hp->row_ptr, Hp->col_idx, Hp->val, &Hdig, &Hexp, st));
     CSS_TRY(css_ws(ctx, "v_digits", vd_bytes, &vdig));
+  } else if (use_dup) {
+    CSS_TRY(css_spmm_dup_prepare(ctx, b, n_brow, Hp->nnzb, Hp->row_ptr, Hp->col_idx, Hp->val, &hdup, &hlodup, st));
   } else {
     CSS_TRY(css_spmm_prepare_as(ctx, "no_hp", f32, b, n_brow, Hp->nnzb, Hp->row_ptr, Hp->col_idx, Hp->val, &hpv, &hplo,
                                 st));
@@ -2050,6 +2053,8 @@ css_status css_density_nonorth(css_ctx* ctx, const css_bsr* S, const double* Sin
   la.Hexp = Hexp;
   la.Hexp_n = N;
   la.Vdig = vdig;
+  la.Hdup = hdup;
+  la.Hlo_dup = hlodup;
   la.max_row_blocks = max_row;
   la.colour = colour;
   la.sign = sign;
@@ -2208,6 +2213,7 @@ css_status css_density_nonorth(css_ctx* ctx, const css_bsr* S, const double* Sin
   CSS_LAUNCHED(ctx);
 
   // -------------------------------------------------------------- read back
+  if (use_dup) CSS_TRY(css_spmm_dup_check(ctx, st));  // its flag comes through the pinned staging too
   double* hres;
   CSS_TRY(css_pinned(ctx, 256, (void**)&hres));
   CSS_CU(ctx, cudaMemcpyAsync(hres, tout, 2 * sizeof(double), cudaMemcpyDeviceToHost, st));
