@@ -202,7 +202,7 @@ constexpr int MU_C = 2 * MU_P;    // of both brackets of a system
 // dynamic shared memory of k_mu: the candidates' sums of every system, the thread sums of one colour,
 // the two brackets and the systems' flags
 inline size_t mu_smem(int32_t n_sys) {
-  return sizeof(double) * ((size_t)n_sys * (MU_C + 4) + (size_t)MU_C * (MU_T + 1)) + sizeof(int) * ((size_t)n_sys + 2);
+  return sizeof(double) * ((size_t)n_sys * (MU_C + 4) + (size_t)MU_C * (MU_T + 1)) + sizeof(int) * (size_t)n_sys;
 }
 
 // Chemical potential of every system s from its Ritz quadrature
@@ -232,7 +232,6 @@ __global__ void __launch_bounds__(MU_T) k_mu(int32_t n_sys, int32_t n_col, int32
   double* lo = ts + MU_C * (MU_T + 1);              // [n_sys][2]
   double* hi = lo + 2 * n_sys;
   int* conv = reinterpret_cast<int*>(hi + 2 * n_sys);
-  int* all_done = conv + n_sys;
   const unsigned G = gridDim.x;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int32_t per = (int32_t)((n_col + G - 1) / G);
@@ -296,7 +295,6 @@ __global__ void __launch_bounds__(MU_T) k_mu(int32_t n_sys, int32_t n_col, int32
   };
   for (int it = 0; it < 100; ++it) {
     for (int32_t t = threadIdx.x; t < n_sys * MU_C; t += blockDim.x) acc[t] = 0.0;
-    if (threadIdx.x == 0) *all_done = 1;
     __syncthreads();
     for (int32_t c = c0; c < c1; ++c) {
       const int32_t s = sys_of_colour[c];
@@ -358,6 +356,7 @@ __global__ void __launch_bounds__(MU_T) k_mu(int32_t n_sys, int32_t n_col, int32
       if (lane == 0) acc[t] = g - half_ne[t / MU_C];
     }
     __syncthreads();
+    bool finished = true;  // this thread's systems
     for (int32_t s = threadIdx.x; s < n_sys; s += blockDim.x) {
       if (conv[s]) continue;
       bool done = true;
@@ -373,10 +372,11 @@ __global__ void __launch_bounds__(MU_T) k_mu(int32_t n_sys, int32_t n_col, int32
         done = done && (z - a <= 1e-13 * fmax(1.0, fabs(0.5 * (a + z))) || stuck);
       }
       if (done) conv[s] = 1;
-      else *all_done = 0;
+      else finished = false;
     }
-    __syncthreads();
-    if (*all_done) break;
+    // a vote, not a flag in shared memory: a flag would need one more barrier between its last read here and
+    // its reset in the next round, or a warp could leave alone in mid-search
+    if (__syncthreads_and(finished)) break;
   }
   if (blockIdx.x == 0)
     for (int32_t s = threadIdx.x; s < n_sys; s += blockDim.x)
