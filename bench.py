@@ -540,8 +540,8 @@ def main():
     tc = (os.environ.get("CSS_HV_TC") == "1" or prec == css.CSS_MIXED_3XTF32) and mixed and 16 < H0.b <= 24
     hv_name, hv_version = hv_kernel(mixed, H0.b, tc)
     digits = hv_version == "k_hv_int"
-    # the digit arithmetic takes 34 bf16 products per FP64-equivalent product
-    peak = (tf32_peak if tc else fp32_peak) if mixed else (pk["bf16_sustained"] / 34.0 if digits else FP64_PEAK)
+    # the digit arithmetic takes 43 bf16 products per FP64-equivalent product
+    peak = (tf32_peak if tc else fp32_peak) if mixed else (pk["bf16_sustained"] / 43.0 if digits else FP64_PEAK)
     traffic = None
     tf = ROOT / "profiles" / "spmm_traffic.json"
     if tf.exists():
@@ -567,7 +567,7 @@ def main():
                                          f"TF/s x 1.1/2.25 ({pk['source']})" if tc else
                                          f"FP32 FFMA (CUDA-core) ceiling: {n_sm} SMs x 128 lanes x 2 flop x "
                                          f"{pk['sm_max_mhz']:.0f} MHz" if mixed else
-                                         f"measured sustained dense BF16 {pk['bf16_sustained']:.0f} TF/s / 34 digit "
+                                         f"measured sustained dense BF16 {pk['bf16_sustained']:.0f} TF/s / 43 digit "
                                          f"products per FP64 product ({pk['source']})"
                                          if digits else FP64_PEAK_NOTE),
                          "frac_vs_tf32_tensor_peak": achieved / tf32_peak if mixed else None,
@@ -621,7 +621,7 @@ def main():
                      "dTrP_vs_fp64": rsp["trP"] - r64["trP"],
                      "dE_band_eV_per_molecule_vs_fp64": abs(2 * (rsp["trPH"] - r64["trPH"])) / a.n_mol,
                      "note": "CSS_FP64_SPLIT: FP64 vectors; the recurrence's H*V by exact digit products where the "
-                             "digits of H fit 8 GiB, in FP32 pairs beyond"}
+                             "digits of H fit 10 GiB, in FP32 pairs beyond"}
             del Psp
         # FP64 at the mixed run's mu: the error of the mixed arithmetic alone, without the
         # change of mu (any mu in the gap satisfies the electron count)

@@ -49,7 +49,11 @@ typedef enum {
 } css_status;
 
 typedef enum {
-  CSS_FP64 = 0,        /* everything in FP64                                               */
+  CSS_FP64 = 0,        /* everything in FP64.  The recurrence's H*V with b <= 24 (digits of H up to */
+                       /* 10 GiB) rounds the entries of H to 2^-63 of a power of two above their row's */
+                       /* and column's largest, those of V to 2^-63 of their column's, multiplies and  */
+                       /* adds exactly and rounds the result once: closer to the exact product in norm */
+                       /* than an FP64 sum; an entry below 2^-10 of its largest keeps under 53 bits    */
   CSS_MIXED_FP32 = 1,  /* H*V, Krylov vectors and block products in FP32 (FP32 accumulate); */
                        /* recurrence coefficients, Cholesky, eigensolve, mu, Z and P in FP64; */
                        /* implies CSS_REORTH_LOCAL (it removes an FP32-level bias of Tr P)   */
@@ -62,7 +66,7 @@ typedef enum {
                         /* in FP32 pairs on the FMA pipe (hi + lo, error-free products, TwoSum   */
                         /* sums: about 2^-47 relative per term against 2^-53); b = 6 or 23       */
                         /* (other b: CSS_ERR_UNSUPPORTED).  Systems whose 8-bit digits of H fit  */
-                        /* 8 GiB run the exact digit products of CSS_FP64, which are faster      */
+                        /* 10 GiB run the exact digit products of CSS_FP64, which are faster      */
 } css_precision;
 
 /* css_density flags */

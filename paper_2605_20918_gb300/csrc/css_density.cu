@@ -865,7 +865,7 @@ css_status css_density_impl(css_ctx* ctx, int32_t n_sys, const css_sys_desc* sys
   const void* Hsplit = nullptr;
   // FP64 (and CSS_FP64_SPLIT) with b <= 24: exact digit products on the tensor cores, unless a padded variant
   // is asked for or the digits would not fit their bounds.  Against the FP32-pair kernel they are faster (256
-  // molecules, b = 23: 2.93 -> 1.70 ms a launch) and closer to the exact products, so that one is left what
+  // molecules, b = 23: 2.93 -> 2.12 ms a launch) and closer to the exact products, so that one is left what
   // exceeds the bounds.
   int32_t rows_max = 0;
   for (int32_t s = 0; s < n_sys; ++s) rows_max = std::max(rows_max, sys[s].H.n_brow);

@@ -1,58 +1,64 @@
-// FP64 H * V on the tensor cores: every entry is cut into seven 8-bit digits, the digit products are
+// FP64 H * V on the tensor cores: every entry is cut into eight 8-bit digits, the digit products are
 // summed exactly, and the sums are put together in 64-bit integers (the Ozaki scheme: Ozaki, Ogita,
 // Oishi & Rump, Numer. Algorithms 59 (2012) 95; its integer form: Ootomo, Ozaki & Yokota, IJHPCA 38
 // (2024) 297).
 //
 // The GB300 runs FP64 FMAs at 1/64 of its FP32 rate (a warp instruction per 16 clocks of an SM), which
 // bounded the DFMA kernel (css_lanczos.cu k_spmm): 5.38 ms a launch for 128 molecules at b = 23, 48.7 us for 64
-// at b = 6.  Here they take 0.79 ms (digits of V and exponents included) and 36 us.  A bf16 holds an
-// 8-bit signed digit exactly and the products of two digits sum exactly in an FP32 accumulator up to
-// 2^24, so bf16 tensor-core products of digits are integer arithmetic.
+// at b = 6.  Here they take 1.00 ms (digits of V and exponents included) and 40 us.  Whole builds are faster than with
+// DFMA at every b that comes here: 2,000 molecules b = 1 19.7 -> 11.4 ms, b = 4 43.8 -> 25.6, b = 9 160 -> 90; 512
+// molecules b = 13 70.8 -> 31.6, b = 16 68.3 -> 32.2, b = 24 144 -> 62; 64 molecules b = 1 6.2 -> 4.8, b = 6 6.57 -> 6.34.
+// A bf16 holds an 8-bit signed digit exactly and the products of two digits sum exactly in an FP32 accumulator
+// up to 2^24, so bf16 tensor-core products of digits are integer arithmetic.
 //
 // Digits: H is scaled by powers of two, its rows by 2^-e (2^e above the row's largest |entry|) and then its
 // columns by 2^-c (so above the largest of the scaled column), and V by 2^c and each of its columns by its
-// largest entry.  A scaled entry times 2^55 rounds to an integer x = sum_s d_s 256^(6 - s) with
-// -128 <= d_s <= 128.  Of the 49 products d_i d'_j the 34 with i + j <= 7 are taken; the others are below
-// 2^-61 of the two maxima.  So an output differs from the exact sum by its own rounding and the rounding of
-// the entries to 2^-56 of those maxima, less than an FP64 sum of such terms loses in its additions; the
-// column scaling keeps that true of graded matrices D A D.  The sums are exact, so the result depends on
-// neither the order of the blocks nor the other columns of the pass.
+// largest entry.  A scaled entry times 2^62 rounds to an integer x = sum_s d_s 256^(7 - s) with
+// |d_0| <= 65 and -128 <= d_s <= 128.  Of the 64 products d_i d'_j the 43 with i + j <= 8 are taken; the others
+// are below 2^-69 of the two maxima.  So an output differs from the exact sum by its own rounding and the
+// rounding of the entries to 2^-63 of those maxima; the column scaling keeps that true of graded matrices
+// D A D.  The sums are exact, so the result depends on neither the order of the blocks nor the other columns of
+// the pass.  The ten bits below those of an FP64 sum are needed: in the recurrence the on-site terms of a row (tens
+// of eV) cancel and leave couplings that an FP64 sum carries to their own 2^-53.  With seven digits (2^-56,
+// 34 products; 0.79 ms) the projected blocks of 20 molecules were off by 4 (b = 13) to 12 times (b = 24) as much as
+// with the DFMA kernel; now by a third to a half.
 // An infinity or NaN in a row of H or a column of V makes that row or column of the result NaN.
 //
 // Shape: mma.sync m16n8k16 with 16 columns of V as M, the rows of an H block as N and the columns of the
-// block as K.  The sums of the eight i + j and of every N tile live in registers (96 at b = 23), which a
+// block as K.  The sums of the nine i + j and of every N tile live in registers (108 at b = 23), which a
 // tcgen05 tile of M = 128 in tensor memory would need once per 24 columns of N with a K of 23 per
 // block: the digit products are many small MMAs, not one large one.
-// A CTA takes one block row I and eight tiles of 16 columns, a warp each.  The digits of H_IJ (10.5 KB,
-// shared by the warps) and of V_J (7 KB per warp) arrive in MMA fragment order through a
-// cp.async ring of three stages (six for b <= 16 when the CTAs do not fill the chip and nothing else hides a
-// copy's latency); a thread copies the very 16 bytes of V it will load.
+// A CTA takes one block row I and eight tiles of 16 columns, a warp each.  The digits of 16 columns of H_IJ (6 KB
+// at b = 23, shared by the warps) and of as many rows of V_J (4 KB per warp) arrive in MMA fragment order through a
+// cp.async ring of five stages at b > 16 (all that shared memory holds), else three (six when the CTAs do not
+// fill the chip and nothing else hides a copy's latency); a thread copies the very 16 bytes of V it will load.
 #include <algorithm>
 
 #include "css_lanczos.cuh"
 
 namespace {
 
-constexpr int kDig = 7;    // digits of an entry
-constexpr int kSum = 8;    // sums S_d over i + j = d
+constexpr int kDig = 8;    // digits of an entry
+constexpr int kSum = 9;    // sums S_d over i + j = d
 constexpr int kWarps = 8;  // column tiles per CTA
 constexpr int kTile = 16;  // columns of V per warp
-// rows of H and columns of V whose largest entry is below 2^-968 keep 2^-1023 as their last digit
-constexpr int kMinExp = 54;
+// rows of H and columns of V whose largest entry is below 2^-961 keep 2^-1023 as their last digit
+constexpr int kMinExp = 61;
 constexpr int kMinCol = -900;    // least column scale of H
 constexpr int kColBias = 4096;   // hcol holds c + kColBias, 0 for a column without entries
 constexpr int kNotFinite = 4096; // exponent of a column of V with an infinity or NaN
 // largest buffer of V's digits: wider blocks of columns go through it in turn, each reading H's digits
-// once more (at 10,000 molecules, b = 23, seven turns)
+// once more (at 10,000 molecules, b = 23, eight turns)
 constexpr size_t kVBytes = (size_t)1 << 30;
-// largest digits of H (2.5 to 4 times its FP64 blocks): beyond, the DFMA kernel runs as before
-constexpr size_t kHBytes = (size_t)8 << 30;
+// largest digits of H (2 times its FP64 blocks at b = 16, 2.9 at 23, 7.1 at 6, 256 at 1): beyond, the DFMA kernel
+// runs as before
+constexpr size_t kHBytes = (size_t)10 << 30;
 
-// NT tiles of 8 rows and KC tiles of 16 columns of an H block
+// NT tiles of 8 rows and KC tiles of 16 columns of an H block; a stage holds one K tile
 template <int NT, int KC>
 struct IntCfg {
-  static constexpr int HB = kDig * NT * 32 * KC * 8;    // bytes of the digits of an H block
-  static constexpr int VB = kDig * KC * 32 * 16;        // of a V block (16 columns)
+  static constexpr int HB = kDig * NT * 32 * 8;  // bytes of the digits of a K tile of an H block
+  static constexpr int VB = kDig * 32 * 16;      // of a V block (16 columns)
   static constexpr int smem(int stages) { return stages * (HB + kWarps * VB); }
 };
 inline int nt_of(int32_t b) { return (b + 7) / 8; }
@@ -61,10 +67,10 @@ inline size_t h_block_bytes(int32_t b) { return (size_t)kDig * nt_of(b) * 32 * k
 inline size_t v_block_bytes(int32_t b) { return (size_t)kDig * kc_of(b) * 32 * 16; }
 
 __device__ __forceinline__ uint32_t expo(double x) { return (uint32_t)(__double2hiint(x) & 0x7ff00000) >> 20; }
-// 2^(55 + c - e) for entries of biased exponent at most E: |x| < 2^e, e = E - 1022; 0 where it would be
+// 2^(62 + c - e) for entries of biased exponent at most E: |x| < 2^e, e = E - 1022; 0 where it would be
 // subnormal (no entry under it then reaches half of the last digit)
 __device__ __forceinline__ double digit_scale(int E, int c) {
-  return __hiloint2double(max(2100 + c - max(E, kMinExp), 0) << 20, 0);
+  return __hiloint2double(max(2107 + c - max(E, kMinExp), 0) << 20, 0);
 }
 __device__ __forceinline__ int col_scale(int hcol) { return hcol ? max(hcol - kColBias, kMinCol) : 0; }
 
@@ -113,7 +119,7 @@ __global__ void __launch_bounds__(256) k_hcol_exp(int32_t b, const int32_t* __re
 }
 
 // digits of every H block (a CTA per block row) in the order of the B fragments:
-// [block][digit][N tile][K tile][lane][2 words]
+// [block][K tile][digit][N tile][lane][2 words]
 template <int NT, int KC>
 __global__ void __launch_bounds__(256) k_hdigits(int32_t b, const int32_t* __restrict__ row_ptr,
                                                  const int32_t* __restrict__ col_idx, const double* __restrict__ H,
@@ -137,7 +143,7 @@ __global__ void __launch_bounds__(256) k_hdigits(int32_t b, const int32_t* __res
       uint32_t d[kDig];
       digits2(at(k), at(k + 1), d);
 #pragma unroll
-      for (int s = 0; s < kDig; ++s) out[((((p * kDig + s) * NT + nt) * KC + r / 2) * 32 + lane) * 2 + (r & 1)] = d[s];
+      for (int s = 0; s < kDig; ++s) out[((((p * KC + r / 2) * kDig + s) * NT + nt) * 32 + lane) * 2 + (r & 1)] = d[s];
     }
   }
 }
@@ -161,7 +167,7 @@ __global__ void __launch_bounds__(128) k_vcol_exp(int64_t N, int32_t ng, int32_t
   if (e) atomicMax(&vexp[col], e);
 }
 
-// digits of 16 columns of V_J (a warp each) in the order of the A fragments: [tile][J][digit][K tile][lane][4
+// digits of 16 columns of V_J (a warp each) in the order of the A fragments: [tile][J][K tile][digit][lane][4
 // words]; columns from col0 on
 template <int KC>
 __global__ void __launch_bounds__(256) k_vdigits(int32_t nJ, int32_t b, int32_t ntile, int32_t col0, int32_t w, int32_t ws,
@@ -188,9 +194,9 @@ __global__ void __launch_bounds__(256) k_vdigits(int32_t nJ, int32_t b, int32_t 
       const int E = r & 1 ? E1 : E0;
       digits2(at(k, c, E), at(k + 1, c, E), d[r]);
     }
-    uint4* o = out + ((((int64_t)tile * nJ + J) * kDig) * KC + kc) * 32 + lane;
+    uint4* o = out + (((int64_t)tile * nJ + J) * KC + kc) * kDig * 32 + lane;
 #pragma unroll
-    for (int s = 0; s < kDig; ++s) o[(size_t)s * KC * 32] = make_uint4(d[0][s], d[1][s], d[2][s], d[3][s]);
+    for (int s = 0; s < kDig; ++s) o[s * 32] = make_uint4(d[0][s], d[1][s], d[2][s], d[3][s]);
   }
 }
 
@@ -230,26 +236,26 @@ __global__ void __launch_bounds__(32 * kWarps, 1) k_hv_int(const IntArgs a) {
   const int32_t I = blockIdx.x, tile = blockIdx.y * kWarps + warp;
   const bool live = tile < a.ntile;
   const int64_t p0 = a.row_ptr[I];
-  const int32_t nq = (int32_t)(a.row_ptr[I + 1] - p0);
-  const unsigned char* vt = a.Vd + (size_t)(live ? tile : 0) * a.nJ * C::VB;
-  auto stage_h = [&](int q) { return sm + (size_t)(q % kStages) * (C::HB + kWarps * C::VB); };
-  auto stage_v = [&](int q) { return stage_h(q) + C::HB + warp * C::VB; };
-  auto load = [&](int32_t q) {
-    if (q < nq) {
-      const unsigned char* h = a.Hd + (size_t)(p0 + q) * C::HB;
-      unsigned char* dh = stage_h(q);
+  const int32_t ns = (int32_t)(a.row_ptr[I + 1] - p0) * KC;  // K tiles of the row
+  const unsigned char* vt = a.Vd + (size_t)(live ? tile : 0) * a.nJ * KC * C::VB;
+  auto stage_h = [&](int s) { return sm + (size_t)(s % kStages) * (C::HB + kWarps * C::VB); };
+  auto stage_v = [&](int s) { return stage_h(s) + C::HB + warp * C::VB; };
+  auto load = [&](int32_t s) {
+    if (s < ns) {
+      const unsigned char* h = a.Hd + (size_t)(p0 * KC + s) * C::HB;
+      unsigned char* dh = stage_h(s);
       for (int i = threadIdx.x; i < C::HB / 16; i += 32 * kWarps) copy16(dh + 16 * i, h + 16 * i);
       if (live) {
-        const unsigned char* v = vt + (size_t)(a.col_idx[p0 + q] - a.row0) * C::VB;
-        unsigned char* dv = stage_v(q);
+        const unsigned char* v = vt + ((size_t)(a.col_idx[p0 + s / KC] - a.row0) * KC + s % KC) * C::VB;
+        unsigned char* dv = stage_v(s);
 #pragma unroll
-        for (int i = 0; i < kDig * KC; ++i) copy16(dv + 16 * (32 * i + lane), v + 16 * (32 * i + lane));
+        for (int i = 0; i < kDig; ++i) copy16(dv + 16 * (32 * i + lane), v + 16 * (32 * i + lane));
       }
     }
     asm volatile("cp.async.commit_group;" ::: "memory");
   };
   float acc[kSum][NT][4];
-  long long hi[NT][4], lo[NT][4];
+  long long hi[NT][4], lo[NT][4];  // sums 0 to 4 and 5 to 8
 #pragma unroll
   for (int n = 0; n < NT; ++n)
 #pragma unroll
@@ -258,41 +264,37 @@ __global__ void __launch_bounds__(32 * kWarps, 1) k_hv_int(const IntArgs a) {
 #pragma unroll
       for (int d = 0; d < kSum; ++d) acc[d][n][i] = 0.0f;
     }
-  for (int q = 0; q < kStages - 1; ++q) load(q);
+  for (int s = 0; s < kStages - 1; ++s) load(s);
   int32_t left = a.flush;
 #pragma unroll 1
-  for (int32_t q = 0; q < nq; ++q) {
+  for (int32_t s = 0; s < ns; ++s) {
     asm volatile("cp.async.wait_group %0;" ::"n"(kStages - 2) : "memory");
-    __syncthreads();  // block q has arrived in every thread, block q - 1 is read
-    load(q + kStages - 1);
+    __syncthreads();  // K tile s has arrived in every thread, s - 1 is read
+    load(s + kStages - 1);
     if (live) {
-      const unsigned char *dh = stage_h(q), *dv = stage_v(q);
+      const unsigned char *dh = stage_h(s), *dv = stage_v(s);
+      uint4 av[kDig];
 #pragma unroll
-      for (int kc = 0; kc < KC; ++kc) {
-        uint4 av[kDig];
+      for (int i = 0; i < kDig; ++i) av[i] = *reinterpret_cast<const uint4*>(dv + 16 * (32 * i + lane));
 #pragma unroll
-        for (int i = 0; i < kDig; ++i) av[i] = *reinterpret_cast<const uint4*>(dv + 16 * (32 * (i * KC + kc) + lane));
+      for (int j = 0; j < kDig; ++j)
 #pragma unroll
-        for (int j = 0; j < kDig; ++j)
+        for (int n = 0; n < NT; ++n) {
+          const uint2 bv = *reinterpret_cast<const uint2*>(dh + 8 * ((j * NT + n) * 32 + lane));
 #pragma unroll
-          for (int n = 0; n < NT; ++n) {
-            const uint2 bv = *reinterpret_cast<const uint2*>(dh + 8 * (((j * NT + n) * KC + kc) * 32 + lane));
-#pragma unroll
-            for (int i = 0; i < kDig; ++i)
-              if (i + j < kSum) mma_bf16(acc[i + j][n], av[i], bv.x, bv.y);
-          }
-      }
-      if (--left == 0 || q + 1 == nq) {  // the sums are below 2^24 so far: take them over
+          for (int i = 0; i < kDig; ++i)
+            if (i + j < kSum) mma_bf16(acc[i + j][n], av[i], bv.x, bv.y);
+        }
+      if ((s + 1) % KC == 0 && (--left == 0 || s + 1 == ns)) {  // the sums are below 2^24 so far: take them over
         left = a.flush;
 #pragma unroll
         for (int n = 0; n < NT; ++n)
 #pragma unroll
           for (int i = 0; i < 4; ++i) {
 #pragma unroll
-            for (int d = 0; d < 4; ++d) {
-              hi[n][i] += (long long)(int)acc[d][n][i] * (1ll << (8 * (3 - d)));
-              lo[n][i] += (long long)(int)acc[4 + d][n][i] * (1ll << (8 * (3 - d)));
-              acc[d][n][i] = acc[4 + d][n][i] = 0.0f;
+            for (int d = 0; d < kSum; ++d) {
+              (d < 5 ? hi : lo)[n][i] += (long long)(int)acc[d][n][i] * (1ll << (8 * (d < 5 ? 4 - d : 8 - d)));
+              acc[d][n][i] = 0.0f;
             }
           }
       }
@@ -311,7 +313,7 @@ __global__ void __launch_bounds__(32 * kWarps, 1) k_hv_int(const IntArgs a) {
       if (EH == 0x7ff || EV == kNotFinite)
         y = __hiloint2double(0x7ff80000, 0);
       else
-        y = join(hi[n][i], lo[n][i], max(EH, kMinExp) + max(EV, kMinExp) - 2 * 1022 - 70);
+        y = join(hi[n][i], lo[n][i], max(EH, kMinExp) + max(EV, kMinExp) - 2 * 1022 - 76);
       a.W[((size_t)I * a.b + r) * a.ws + c] = y;
     }
 }
@@ -323,8 +325,8 @@ css_status launch(css_ctx* ctx, const LzArgs& a, const double* V, double* W, int
   const int32_t b = a.b, tiles = (int32_t)css_ceil_div(a.w, kTile);
   const int64_t N = (int64_t)a.n_brow * b;
   const int32_t *hexp = a.Hexp + (size_t)a.row0 * b, *hcol = hexp + a.Hexp_n;
-  constexpr int deep = KC == 1 ? 6 : 3;
-  CSS_CU(ctx, cudaFuncSetAttribute(k_hv_int<NT, KC, 3>, cudaFuncAttributeMaxDynamicSharedMemorySize, C::smem(3)));
+  constexpr int deep = KC == 1 ? 6 : 5, flat = KC == 1 ? 3 : 5;
+  CSS_CU(ctx, cudaFuncSetAttribute(k_hv_int<NT, KC, flat>, cudaFuncAttributeMaxDynamicSharedMemorySize, C::smem(flat)));
   CSS_CU(ctx, cudaFuncSetAttribute(k_hv_int<NT, KC, deep>, cudaFuncAttributeMaxDynamicSharedMemorySize, C::smem(deep)));
   CSS_CU(ctx, cudaMemsetAsync(vexp, 0, sizeof(int32_t) * a.w, st));
   const int32_t ng = N > 16384 ? 4 : 1;
@@ -343,7 +345,7 @@ css_status launch(css_ctx* ctx, const LzArgs& a, const double* V, double* W, int
     r.col0 = t0 * kTile;
     r.w = a.w;
     r.ws = a.ws;
-    r.flush = 146 / b;  // seven sums of 146 products of 2^14 stay below 2^24
+    r.flush = 145 / b;  // the largest sum (d = 7): 145 (6 128^2 + 2 65 128) is below 2^24
     r.row0 = a.row0;
     r.row_ptr = a.row_ptr;
     r.col_idx = a.col_idx;
@@ -356,7 +358,7 @@ css_status launch(css_ctx* ctx, const LzArgs& a, const double* V, double* W, int
     if (grid.x * (int64_t)grid.y <= ctx->n_sm)
       k_hv_int<NT, KC, deep><<<grid, 32 * kWarps, C::smem(deep), st>>>(r);
     else
-      k_hv_int<NT, KC, 3><<<grid, 32 * kWarps, C::smem(3), st>>>(r);
+      k_hv_int<NT, KC, flat><<<grid, 32 * kWarps, C::smem(flat), st>>>(r);
     CSS_LAUNCHED(ctx);
   }
   return CSS_OK;
