@@ -1111,6 +1111,7 @@ namespace {
 // the columns on one SM is smallest), within shared memory
 template <bool FWD>
 css_status launch_refl(css_ctx* ctx, const EigArgs& a, double* X, cudaStream_t st) {
+  constexpr size_t kSmem = 200 * 1024;  // of a CTA
   const int32_t kd = a.b, b = a.b, nmax = a.m * a.b;
   auto bytes = [&](int32_t cw) {
     return sizeof(double) * ((size_t)nmax * cw + 2 * (size_t)(nmax / kd + 1) * (kd + 1));
@@ -1119,7 +1120,7 @@ css_status launch_refl(css_ctx* ctx, const EigArgs& a, double* X, cudaStream_t s
   double least = 1e300;
   for (int32_t cw = b; cw >= 1; --cw) {
     const int64_t splits = css_ceil_div(b, cw);
-    if (bytes(cw) > 200 * 1024 || splits > 12) continue;
+    if (bytes(cw) > kSmem || splits > 12) continue;
     const double load = (double)css_ceil_div((int64_t)a.n_col * splits, ctx->n_sm) * cw;
     if (load < 0.95 * least) {
       least = load;
@@ -1128,7 +1129,7 @@ css_status launch_refl(css_ctx* ctx, const EigArgs& a, double* X, cudaStream_t s
   }
   const int32_t tasks = (nmax / kd + 1) * best;
   const unsigned threads = (unsigned)std::min<int32_t>(1024, (tasks + 31) / 32 * 32);
-  CSS_CU(ctx, cudaFuncSetAttribute(k_apply_refl<FWD>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes(best)));
+  CSS_TRY(css_smem_limit(ctx, k_apply_refl<FWD>, kSmem));
   k_apply_refl<FWD><<<dim3((unsigned)a.n_col, (unsigned)css_ceil_div(b, best)), threads, bytes(best), st>>>(
       kd, b, best, nmax, a.rcap, a.nblk, a.RV, a.RT, X);
   CSS_LAUNCHED(ctx);
@@ -1160,8 +1161,7 @@ css_status launch_band(css_ctx* ctx, const EigArgs& a, int32_t ldb, cudaStream_t
     cfg.gridDim = dim3((unsigned)a.n_col);
     cfg.blockDim = dim3((unsigned)(32 * nw));
     cfg.dynamicSmemBytes = bytes(nw, true);
-    CSS_CU(ctx, cudaFuncSetAttribute(k_band_to_tri<LPS, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     (int)cfg.dynamicSmemBytes));
+    CSS_TRY(css_smem_limit(ctx, k_band_to_tri<LPS, true>, kSmem));
     CSS_CU(ctx, cudaLaunchKernelEx(&cfg, k_band_to_tri<LPS, true>, ba));
     CSS_LAUNCHED(ctx);
     return CSS_OK;
@@ -1182,8 +1182,7 @@ css_status launch_band(css_ctx* ctx, const EigArgs& a, int32_t ldb, cudaStream_t
   at.val.clusterDim.y = at.val.clusterDim.z = 1;
   cfg.attrs = &at;
   cfg.numAttrs = 1;
-  CSS_CU(ctx, cudaFuncSetAttribute(k_band_to_tri<LPS, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                   (int)cfg.dynamicSmemBytes));
+  CSS_TRY(css_smem_limit(ctx, k_band_to_tri<LPS, false>, kSmem));
   CSS_CU(ctx, cudaLaunchKernelEx(&cfg, k_band_to_tri<LPS, false>, ba));
   CSS_LAUNCHED(ctx);
   k_tri_out<<<a.n_col, 256, 0, st>>>(kd, nmax, ldb, a.nblk, a.AB, a.d, a.e);
@@ -1243,8 +1242,7 @@ css_status css_eigen_ritz(css_ctx* ctx, const EigArgs& a, cudaStream_t st) {
     CSS_CU(ctx, cudaEventRecord(ctx->side_ev[0], st));
     CSS_CU(ctx, cudaStreamWaitEvent(s_refl, ctx->side_ev[0], 0));
     CSS_TRY(launch_refl<true>(ctx, a, a.X0, s_refl));
-    const size_t sh = 2 * (size_t)nmax * sizeof(float);
-    if (sh > 48 * 1024) CSS_CU(ctx, cudaFuncSetAttribute(k_bisect32, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sh));
+    const size_t sh = 2 * (size_t)nmax * sizeof(float);  // 32 KB at the largest nmax, 4096
     k_bisect32<<<dim3((unsigned)nc, (unsigned)css_ceil_div(nmax, 128)), 128, sh, st>>>(b, nmax, a.nblk, a.d, a.e,
                                                                                       a.lam32, a.tnorm);
     CSS_LAUNCHED(ctx);

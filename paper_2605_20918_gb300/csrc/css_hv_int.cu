@@ -326,8 +326,8 @@ css_status launch(css_ctx* ctx, const LzArgs& a, const double* V, double* W, int
   const int64_t N = (int64_t)a.n_brow * b;
   const int32_t *hexp = a.Hexp + (size_t)a.row0 * b, *hcol = hexp + a.Hexp_n;
   constexpr int deep = KC == 1 ? 6 : 5, flat = KC == 1 ? 3 : 5;
-  CSS_CU(ctx, cudaFuncSetAttribute(k_hv_int<NT, KC, flat>, cudaFuncAttributeMaxDynamicSharedMemorySize, C::smem(flat)));
-  CSS_CU(ctx, cudaFuncSetAttribute(k_hv_int<NT, KC, deep>, cudaFuncAttributeMaxDynamicSharedMemorySize, C::smem(deep)));
+  CSS_TRY(css_smem_limit(ctx, k_hv_int<NT, KC, flat>, C::smem(flat)));
+  CSS_TRY(css_smem_limit(ctx, k_hv_int<NT, KC, deep>, C::smem(deep)));
   CSS_CU(ctx, cudaMemsetAsync(vexp, 0, sizeof(int32_t) * a.w, st));
   const int32_t ng = N > 16384 ? 4 : 1;
   k_vcol_exp<<<dim3((unsigned)css_ceil_div(N, 16 * ng), (unsigned)css_ceil_div(a.w, 128)), 128, 0, st>>>(

@@ -131,6 +131,16 @@ __host__ __device__ __forceinline__ uint64_t css_splitmix64(uint64_t seed, uint6
 
 __host__ __device__ __forceinline__ int64_t css_ceil_div(int64_t a, int64_t b) { return (a + b - 1) / b; }
 
+// Let `kern` take up to `bytes` of dynamic shared memory.  The limit belongs to the process, not to a launch, so
+// `bytes` is a constant of the kernel: with each launch's own size, a thread with a small system would lower
+// it between another thread's call here and its launch, which then fails.
+constexpr size_t kSmemMost = 227 * 1024;  // of a CTA
+template <typename K>
+css_status css_smem_limit(css_ctx* ctx, K* kern, size_t bytes) {
+  CSS_CU(ctx, cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes));
+  return CSS_OK;
+}
+
 // ----------------------------------------------------------- internal entry points
 // colouring (css_color.cu)
 css_status css_color_impl(css_ctx* ctx, int32_t n, const double* xyz, double box, double r_col, uint64_t seed,

@@ -1196,18 +1196,11 @@ __global__ void k_accum_x(int64_t p_begin, int64_t p_end, int32_t b, int32_t ws,
   X[(size_t)p * bb + e] += s;
 }
 
-// opt in to more than 48 KB of dynamic shared memory where a launch needs it
-template <typename K>
-css_status smem_optin(css_ctx* ctx, K kern, size_t bytes) {
-  if (bytes > 48 * 1024) CSS_CU(ctx, cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes));
-  return CSS_OK;
-}
-
 template <typename T, int BM, int TC, int NT, int B>
 css_status launch_spmm_t(css_ctx* ctx, const LzArgs& a, const T* V, T* W, cudaStream_t st) {
   using C = SpmmCfg<T, BM, TC, NT>;
   auto kern = k_spmm<T, BM, TC, NT, B>;
-  CSS_TRY(smem_optin(ctx, kern, C::smem));
+  CSS_TRY(css_smem_limit(ctx, kern, C::smem));
   dim3 grid((unsigned)a.n_brow, (unsigned)css_ceil_div(a.w, C::CT));
   kern<<<grid, C::NT, C::smem, st>>>(a.b, a.row_ptr, a.col_idx, (const T*)a.Hval, V, W, a.ws, a.w,
                                      (const T*)a.Hlo_diag, a.row0);
@@ -1359,11 +1352,11 @@ css_status run_pass_bp(css_ctx* ctx, const LzArgs& a_in, cudaStream_t st) {
   const unsigned sblocks = (unsigned)css_ceil_div((pe - pb) * bb, 256);
   auto s1 = reorth ? k_s1<T, BP, true> : k_s1<T, BP, false>;
   auto s3 = reorth ? k_s3<T, BP, true> : k_s3<T, BP, false>;
-  CSS_TRY(smem_optin(ctx, s1, sm_s1));
-  CSS_TRY(smem_optin(ctx, s3, sm_s3));
-  CSS_TRY(smem_optin(ctx, k_tri<T, BP, true>, sm_tri));
-  CSS_TRY(smem_optin(ctx, k_tri<T, BP, false>, sm_tri));
-  if (a.ucol) CSS_TRY(smem_optin(ctx, k_s1<T, BP, false>, sm_s1));
+  CSS_TRY(css_smem_limit(ctx, s1, kSmemMost));
+  CSS_TRY(css_smem_limit(ctx, s3, kSmemMost));
+  CSS_TRY(css_smem_limit(ctx, k_tri<T, BP, true>, kSmemMost));
+  CSS_TRY(css_smem_limit(ctx, k_tri<T, BP, false>, kSmemMost));
+  if (a.ucol) CSS_TRY(css_smem_limit(ctx, k_s1<T, BP, false>, kSmemMost));
   CSS_CU(ctx, cudaMemsetAsync(Qp, 0, vec_bytes, st));
   CSS_CU(ctx, cudaMemsetAsync(Qc, 0, vec_bytes, st));
   if (a.start) {

@@ -736,7 +736,7 @@ css_status launch_rows6(css_ctx* ctx, RowsArgs& r, cudaStream_t st) {
   const int32_t ngr = (int32_t)css_ceil_div(r.ncb, B6_GMAX);
   r.G = (int32_t)css_ceil_div(css_ceil_div(r.ncb, ngr), 2) * 2;  // even groups of nearly equal size
   const size_t sm = B6Cfg<MODE>::smem(r.G);
-  CSS_CU(ctx, cudaFuncSetAttribute(k_rows6<MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
+  CSS_TRY(css_smem_limit(ctx, k_rows6<MODE>, B6Cfg<MODE>::smem(B6_GMAX)));
   const dim3 grid((unsigned)css_ceil_div(r.N, r.rchk), (unsigned)css_ceil_div(r.ncb, r.G));
   k_rows6<MODE><<<grid, 32 * (r.G + B6_NP), sm, st>>>(r);
   CSS_LAUNCHED(ctx);
@@ -746,7 +746,7 @@ css_status launch_rows6(css_ctx* ctx, RowsArgs& r, cudaStream_t st) {
 template <int MODE>
 css_status launch_rows23(css_ctx* ctx, RowsArgs& r, cudaStream_t st) {
   using C = B23Cfg<MODE>;
-  CSS_CU(ctx, cudaFuncSetAttribute(k_rows23<MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)C::smem));
+  CSS_TRY(css_smem_limit(ctx, k_rows23<MODE>, C::smem));
   const dim3 grid((unsigned)css_ceil_div(r.N, r.rchk), (unsigned)css_ceil_div(r.ncb, B23_G));
   k_rows23<MODE><<<grid, 32 * 12, C::smem, st>>>(r);
   CSS_LAUNCHED(ctx);

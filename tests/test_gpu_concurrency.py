@@ -71,3 +71,44 @@ def test_mu_of_many_systems_beside_a_busy_stream(torch, css):
                     assert abs(mu[s] - _mu(lam, w, f["kT"], f["n_elec"])) < 1e-9 * max(1.0, abs(mu[s])), s
             assert np.array_equal(mu, first), rep
     torch.cuda.synchronize()
+
+
+# Two threads with a context each, systems of different sizes: a kernel's limit of dynamic shared memory belongs to
+# the process, so one thread's small launch must not lower it under the other's large one.  Repeated calls
+# are bitwise equal
+@pytest.mark.parametrize("precision", ["CSS_FP64", "CSS_MIXED_FP32"])
+def test_two_threads_with_systems_of_different_sizes(torch, css, precision):
+    import threading
+    from paper_2605_20918_gb300 import synth
+    import oracle
+    jobs = []
+    for n, r_col, m in ((64, 8.0, 30), (8, 4.0, 4)):
+        g = synth.water_box(n)
+        H = synth.hamiltonian(g, "minimal")
+        col, nc = oracle.color(g.pos, g.box, r_col, 1004)
+        jobs.append((css.DeviceBSR.from_host(H), torch.as_tensor(col, device="cuda"),
+                     torch.as_tensor(oracle.probes(col, H.b, 1005), device="cuda"), nc, synth.n_electrons(n), m))
+    torch.cuda.synchronize()
+    failed = []
+
+    def work(Hd, col, sign, nc, ne, m):
+        try:
+            stream = torch.cuda.Stream()
+            P = torch.empty_like(Hd.val)
+            first = None
+            with torch.cuda.stream(stream), css.Context(0) as ctx:
+                for _ in range(150):
+                    ctx.density(Hd, col, sign, nc, P, kT=0.05, n_elec=ne, m=m, precision=getattr(css, precision))
+                    stream.synchronize()
+                    first = P.clone() if first is None else first
+                    if not torch.equal(P, first):
+                        raise AssertionError("results differ between repeats")
+        except Exception as e:
+            failed.append(repr(e))
+
+    threads = [threading.Thread(target=work, args=j) for j in jobs]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert not failed, failed
