@@ -93,6 +93,8 @@ css_status css_create(css_ctx** out, int device) {
   const char* te = getenv("CSS_TEST_SPMM_EMPTY_EXTRA");
   const int eextra = te ? atoi(te) : 0;
   ctx->test_spmm_empty_extra = eextra > 0 && eextra < 4 ? eextra : 0;
+  const char* bh = getenv("CSS_TEST_BAND_HOLD");
+  ctx->test_band_hold = bh && bh[0] == '1';
   const char* tc = getenv("CSS_HV_TC");
   ctx->hv_tc = tc && tc[0] == '1';
   const char* gr = getenv("CSS_GRAPH");

@@ -106,7 +106,7 @@ __device__ __forceinline__ double group_house(double x, int l, double& tau, doub
 // Every wait is bounded: after 2 s without progress the colour's status gets bit 2 and all its
 // CTAs stop.
 struct BandArgs {
-  int32_t kd, nmax, ldb, rcap, cta_per_col, ncta;
+  int32_t kd, nmax, ldb, rcap, cta_per_col, hold;  // hold: tests only, sweeps after the first wait for ever
   const int32_t* nblk;
   double* AB;
   double* RV;
@@ -178,13 +178,13 @@ __global__ void __launch_bounds__(SMEM ? 1024 : 512) k_band_to_tri(const BandArg
     if (live && i > 0) {
       const unsigned long long x = slots[(i - 1) % S];
       const int32_t id = (int32_t)(x >> 32) - 1, next_row = (int32_t)(uint32_t)x;
-      act = id > i - 1 || (id == i - 1 && next_row >= q0 + Lq);
+      act = !a.hold && (id > i - 1 || (id == i - 1 && next_row >= q0 + Lq));
     }
     if (!__any_sync(FULL, act)) {
       if (++idle == 1) t0 = css_pipe::gtime();
       if ((idle & 255u) == 0) {
-        const bool stop = *(volatile int32_t*)&a.status[c] & 2;
-        if (stop || css_pipe::gtime() - t0 > css_pipe::kWaitNs) {
+        const bool stop = (*(volatile int32_t*)&a.status[c] & 2) || css_pipe::gtime() - t0 > css_pipe::kWaitNs;
+        if (__any_sync(FULL, stop)) {  // the lanes leave together: those that stayed would vote without the others
           if (lane == 0) atomicOr(&a.status[c], 2);
           break;
         }
@@ -1146,7 +1146,7 @@ css_status launch_band(css_ctx* ctx, const EigArgs& a, int32_t ldb, cudaStream_t
   constexpr size_t kSmem = 220 * 1024;
   const int32_t kd = a.b, nmax = a.m * a.b;
   const int32_t flight = nmax / (2 * kd) + 1;
-  BandArgs ba{kd, nmax, ldb, a.rcap, 1, a.n_col, a.nblk, a.AB, a.RV, a.RT, nullptr, a.d, a.e, a.status};
+  BandArgs ba{kd, nmax, ldb, a.rcap, 1, ctx->test_band_hold, a.nblk, a.AB, a.RV, a.RT, nullptr, a.d, a.e, a.status};
   auto warps = [&](int32_t ctas, bool smem) {
     return (int32_t)std::min<int64_t>(smem ? 32 : 16, css_ceil_div(flight, (int64_t)SPW * ctas) + 1);
   };

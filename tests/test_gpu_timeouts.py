@@ -1,0 +1,38 @@
+"""Bounded waits that run out return CSS_ERR_TIMEOUT and leave the device usable; the waits are held by test
+hooks read at css_create, nothing faults."""
+import numpy as np
+import pytest
+
+import oracle
+from paper_2605_20918_gb300 import synth
+
+pytestmark = pytest.mark.gpu
+
+
+def _times_out_then_works(monkeypatch, hook, n, kind, m, precision):
+    torch = pytest.importorskip("torch")
+    import paper_2605_20918_gb300 as css
+    g = synth.water_box(n)
+    H = synth.hamiltonian(g, kind)
+    col, nc = oracle.color(g.pos, g.box, 6.0, 1004)
+    sign = oracle.probes(col, H.b, 1005)
+    args = (css.DeviceBSR.from_host(H), torch.as_tensor(col, device="cuda"), torch.as_tensor(sign, device="cuda"), nc)
+    P = torch.empty((H.nnzb, H.b, H.b), dtype=torch.float64, device="cuda")
+    kw = dict(kT=0.05, mu=-4.0, solve_mu=False, m=m, precision=getattr(css, precision))
+    monkeypatch.setenv(hook, "1")
+    bad = css.Context(0)
+    monkeypatch.delenv(hook)
+    with bad, pytest.raises(css.CSSError) as e:
+        bad.density(*args, P, **kw)
+    assert e.value.status == css.CSS_ERR_TIMEOUT
+    torch.cuda.synchronize()  # no sticky CUDA error
+    with css.Context(0) as ctx:
+        ctx.density(*args, P, **kw)
+    ref = oracle.density(H, col, sign, nc, kT=0.05, mu=-4.0, solve_mu=False, m=m)
+    assert float(np.abs(P.cpu().numpy() - ref["P"]).max()) < (1e-10 if precision == "CSS_FP64" else 1e-6)
+
+
+# the sweeps of the band reduction: band in shared memory, and in L2 with several CTAs a colour
+@pytest.mark.parametrize("n,kind,m", [(64, "minimal", 10), (40, "dzp", 26)])
+def test_band_reduction_sweeps(monkeypatch, n, kind, m):
+    _times_out_then_works(monkeypatch, "CSS_TEST_BAND_HOLD", n, kind, m, "CSS_FP64")
