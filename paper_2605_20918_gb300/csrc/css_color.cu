@@ -219,13 +219,13 @@ __global__ void k_parents(int32_t n, const int32_t* __restrict__ adj_ptr, const 
 // of parents is a few hundred vertices.  With one launch per step of that chain, each scanning
 // every vertex, a colouring of 20,000 molecules took 10.0 ms (445 launches); now 1.42 ms in all.
 // Every wait is bounded: a warp that sees 4 s pass without any vertex of the graph being coloured
-// (*done counts them) sets *err and leaves.
+// (*done counts them) sets *err and leaves.  hold: a vertex that is never taken (tests), -1 for none.
 constexpr uint64_t kColourNs = 4000000000ull;
 __global__ void __launch_bounds__(256) k_jp_flow(int32_t n, int32_t per, const int32_t* __restrict__ adj_ptr,
                                                  const int32_t* __restrict__ np, const int32_t* __restrict__ padj,
                                                  int32_t* __restrict__ wait, volatile int32_t* colour,
                                                  int32_t* __restrict__ max_colour, int32_t* done,
-                                                 int32_t* __restrict__ err) {
+                                                 int32_t* __restrict__ err, int32_t hold) {
   constexpr unsigned FULL = 0xffffffffu;
   const int lane = threadIdx.x & 31;
   const int64_t v0 = (((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5) * per;
@@ -240,7 +240,7 @@ __global__ void __launch_bounds__(256) k_jp_flow(int32_t n, int32_t per, const i
       const bool own = g + lane < mine;
       int32_t wl = own ? wait[vl] : -1;  // -1: coloured
       const int32_t sl = own ? adj_ptr[vl] : 0, nl = own ? np[vl] : 0;
-      const bool go = wl >= 0 && (wl >= nl || colour[padj[sl + wl]] >= 0);
+      const bool go = wl >= 0 && vl != hold && (wl >= nl || colour[padj[sl + wl]] >= 0);
       unsigned todo = __ballot_sync(FULL, go);
       moved = moved || todo != 0;
       while (todo) {
@@ -286,10 +286,12 @@ __global__ void __launch_bounds__(256) k_jp_flow(int32_t n, int32_t per, const i
     }
     if (!moved && (sweep & 255) == 255) {
       const int32_t now = __shfl_sync(FULL, *(volatile int32_t*)done, 0);
+      const bool late = now == seen && css_pipe::gtime() - t0 > kColourNs;
       if (now != seen) {
         seen = now;
         t0 = css_pipe::gtime();
-      } else if (css_pipe::gtime() - t0 > kColourNs) {
+      }
+      if (__any_sync(FULL, late)) {  // the lanes leave together: those that stayed would vote without the others
         if (lane == 0) atomicOr(err, 1);
         return;
       }
@@ -490,7 +492,8 @@ css_status css_color_impl(css_ctx* ctx, int32_t n, const double* xyz, double box
   int32_t per = (int32_t)css_ceil_div(n, warps), n_ = n;
   volatile int32_t* col_ = colour;
   int32_t *maxc = counters + 2, *done = counters + 3, *err = counters;
-  void* args[] = {&n_, &per, &adj_ptr, &np, &padj, &wait, &col_, &maxc, &done, &err};
+  int32_t hold_ = ctx->test_colour_hold ? 0 : -1;
+  void* args[] = {&n_, &per, &adj_ptr, &np, &padj, &wait, &col_, &maxc, &done, &err, &hold_};
   CSS_CU(ctx, cudaLaunchCooperativeKernel((void*)k_jp_flow, dim3((unsigned)(warps / (T / 32))), dim3(T), args, 0, st));
   ++ctx->kernel_launches;
   CSS_CU(ctx, cudaMemcpyAsync(hbuf, counters, 3 * sizeof(int32_t), cudaMemcpyDeviceToHost, st));

@@ -70,6 +70,9 @@ struct css_ctx {
   // failure injection for tests (env CSS_TEST_BAND_HOLD = 1 at css_create): no sweep of the band reduction but the
   // first may step, so their bounded waits run out and the call returns CSS_ERR_TIMEOUT
   int test_band_hold = 0;
+  // failure injection for tests (env CSS_TEST_COLOUR_HOLD = 1 at css_create): the colouring never takes vertex 0, so
+  // its bounded waits run out and the call returns CSS_ERR_TIMEOUT
+  int test_colour_hold = 0;
   // failure injection for tests (env CSS_TEST_MU_BARRIER_EXTRA = k at css_create): the grid
   // barrier of the mu bisection waits for k CTAs more than the launch has, so its bounded wait
   // runs out and the call returns CSS_ERR_TIMEOUT; 0 (the default) is the normal barrier

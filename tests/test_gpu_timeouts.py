@@ -36,3 +36,25 @@ def _times_out_then_works(monkeypatch, hook, n, kind, m, precision):
 @pytest.mark.parametrize("n,kind,m", [(64, "minimal", 10), (40, "dzp", 26)])
 def test_band_reduction_sweeps(monkeypatch, n, kind, m):
     _times_out_then_works(monkeypatch, "CSS_TEST_BAND_HOLD", n, kind, m, "CSS_FP64")
+
+
+# the colouring, with a few vertices on many warps and with several per warp: vertex 0 is never coloured, so its own
+# warp, its dependants' and theirs have to give up
+@pytest.mark.parametrize("n", [40, 20_000])
+def test_colouring(monkeypatch, n):
+    torch = pytest.importorskip("torch")
+    import paper_2605_20918_gb300 as css
+    g = synth.water_box(n)
+    xyz = torch.as_tensor(g.pos, device="cuda")
+    col = torch.empty(n, dtype=torch.int32, device="cuda")
+    monkeypatch.setenv("CSS_TEST_COLOUR_HOLD", "1")
+    bad = css.Context(0)
+    monkeypatch.delenv("CSS_TEST_COLOUR_HOLD")
+    with bad, pytest.raises(css.CSSError) as e:
+        bad.color(xyz, g.box, 6.0, 1004, col)
+    assert e.value.status == css.CSS_ERR_TIMEOUT
+    torch.cuda.synchronize()  # no sticky CUDA error
+    with css.Context(0) as ctx:
+        nc = ctx.color(xyz, g.box, 6.0, 1004, col)
+    ref, nref = oracle.color(g.pos, g.box, 6.0, 1004)
+    assert nc == nref and np.array_equal(col.cpu().numpy(), ref)
