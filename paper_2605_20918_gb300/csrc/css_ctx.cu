@@ -97,6 +97,8 @@ css_status css_create(css_ctx** out, int device) {
   ctx->test_band_hold = bh && bh[0] == '1';
   const char* ch = getenv("CSS_TEST_COLOUR_HOLD");
   ctx->test_colour_hold = ch && ch[0] == '1';
+  const char* rh = getenv("CSS_TEST_ROWS_HOLD");
+  ctx->test_rows_hold = rh && rh[0] == '1';
   const char* tc = getenv("CSS_HV_TC");
   ctx->hv_tc = tc && tc[0] == '1';
   const char* gr = getenv("CSS_GRAPH");

@@ -73,6 +73,9 @@ struct css_ctx {
   // failure injection for tests (env CSS_TEST_COLOUR_HOLD = 1 at css_create): the colouring never takes vertex 0, so
   // its bounded waits run out and the call returns CSS_ERR_TIMEOUT
   int test_colour_hold = 0;
+  // failure injection for tests (env CSS_TEST_ROWS_HOLD = 1 at css_create): the stages of the FP32 row passes wait for
+  // one arrival more than they get, so their bounded waits run out and the call returns CSS_ERR_TIMEOUT
+  int test_rows_hold = 0;
   // failure injection for tests (env CSS_TEST_MU_BARRIER_EXTRA = k at css_create): the grid
   // barrier of the mu bisection waits for k CTAs more than the launch has, so its bounded wait
   // runs out and the call returns CSS_ERR_TIMEOUT; 0 (the default) is the normal barrier

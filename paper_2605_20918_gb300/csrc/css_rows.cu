@@ -42,6 +42,7 @@ struct RowsArgs {
   double* part1;         // Gram partials [chunk][lc][b][b]
   double* part2;         // S1: Kp
   int* err;
+  int32_t hold;          // tests: arrivals that a stage waits for beyond those it gets
 };
 
 __device__ __forceinline__ unsigned long long pack2(float x, float y) {
@@ -85,7 +86,10 @@ struct Ring {
   int64_t r0, rend;
   __device__ __forceinline__ float* stage(int32_t t) const { return base + (size_t)(t % ns) * NA * R * pitch; }
   __device__ __forceinline__ int32_t rows(int32_t t) const { return (int32_t)min((int64_t)R, rend - r0 - (int64_t)t * R); }
-  __device__ __forceinline__ bool wait_full(int32_t t) const { return bar_wait(&full[t % ns], (t / ns) & 1, abort, err); }
+  // for a whole warp: whether a wait gave up is one decision of its lanes, which leave the tile loop together
+  __device__ __forceinline__ bool wait_full(int32_t t) const {
+    return __all_sync(0xffffffffu, bar_wait(&full[t % ns], (t / ns) & 1, abort, err));
+  }
   __device__ __forceinline__ void arrive(int32_t t) const { bar_arrive(&done[t % ns]); }
   __device__ __forceinline__ void init(int32_t consumers) const {  // one thread
     for (int s = 0; s < ns; ++s) {
@@ -194,7 +198,7 @@ __global__ void __launch_bounds__(32 * (B6_GMAX + B6_NP), 1) k_rows6(const RowsA
     for (int32_t g = 0; g < gcount; ++g) any3 = any3 || a.need3[g0 + g] != 0;
   if (MODE == R_T2 && !any3) return;  // uniform over the CTA
   if (threadIdx.x == 0) {
-    ring.init(gcount);
+    ring.init(gcount + a.hold);
     *ring.abort = *(volatile int*)a.err ? 1 : 0;
   }
   __syncthreads();
@@ -535,7 +539,7 @@ __global__ void __launch_bounds__(32 * 12, 1) k_rows23(const RowsArgs a) {
   const bool use_p = MODE <= R_S3 && !a.first;
   const bool gram = MODE <= R_T0 || (MODE == R_T1 && any3);
   if (threadIdx.x == 0) {
-    ring.init(1);
+    ring.init(1 + a.hold);
     *ring.abort = *(volatile int*)a.err ? 1 : 0;
   }
   // the colours' matrices (negated where they are subtracted)
@@ -787,6 +791,7 @@ css_status css_rows(css_ctx* ctx, int mode, const CssRows& p, cudaStream_t st) {
   r.part1 = p.part1;
   r.part2 = p.part2;
   r.err = p.err;
+  r.hold = ctx->test_rows_hold;
   switch (mode) {
     case R_S1: return launch_rows<R_S1>(ctx, p.b, r, st);
     case R_S3: return launch_rows<R_S3>(ctx, p.b, r, st);

@@ -58,3 +58,25 @@ def test_colouring(monkeypatch, n):
         nc = ctx.color(xyz, g.box, 6.0, 1004, col)
     ref, nref = oracle.color(g.pos, g.box, 6.0, 1004)
     assert nc == nref and np.array_equal(col.cpu().numpy(), ref)
+
+
+# the FP32 row passes' rings of tiles: one tile per chunk of rows (only the stores wait), and in one chunk more tiles
+# than stages (loads and products wait too)
+@pytest.mark.parametrize("n,kind,m", [(64, "minimal", 6), (40, "dzp", 4), (6000, "minimal", 2), (3000, "dzp", 2)])
+def test_row_passes(monkeypatch, n, kind, m):
+    if n < 1000:
+        return _times_out_then_works(monkeypatch, "CSS_TEST_ROWS_HOLD", n, kind, m, "CSS_MIXED_FP32")
+    torch = pytest.importorskip("torch")
+    import paper_2605_20918_gb300 as css
+    g = synth.water_box(n)
+    H = css.DeviceBSR.from_host(synth.hamiltonian(g, kind))
+    col = torch.arange(n, dtype=torch.int32, device="cuda") % 60
+    sign = torch.ones(n * H.b, dtype=torch.int8, device="cuda")
+    P = torch.empty_like(H.val)
+    monkeypatch.setenv("CSS_TEST_ROWS_HOLD", "1")
+    bad = css.Context(0)
+    monkeypatch.delenv("CSS_TEST_ROWS_HOLD")
+    with bad, pytest.raises(css.CSSError) as e:
+        bad.density(H, col, sign, 60, P, mu=-4.0, solve_mu=False, m=m, precision=css.CSS_MIXED_FP32)
+    assert e.value.status == css.CSS_ERR_TIMEOUT
+    torch.cuda.synchronize()  # no sticky CUDA error
