@@ -1088,9 +1088,8 @@ __global__ void k_gram_chol(int32_t nch, int32_t ncb, int32_t b, int32_t cb0, in
     for (int32_t q = k; q <= l; ++q) prod = fma(G[k][q], rp[q * b + l], prod);
   if (last) {  // the breakdown test on the diagonal of B_j
     const double limit = tau * sqrt(hq2[lc]);
-    if (t < E && k == l && !(prod > limit)) sbad = 1;
-    __syncthreads();
-    if (sbad) {
+    // a vote: setting sbad here would race with the warps that still read it above
+    if (__syncthreads_or(t < E && k == l && !(prod > limit))) {
       stop();
       return;
     }

@@ -162,3 +162,21 @@ def test_hv6_rows_equal_the_ring_kernel_bitwise(torch, css, monkeypatch, n, nc):
             c.close()
     for v in range(1, 4):
         assert np.array_equal(P[0], P[v]), v
+
+
+# CholeskyQR's two ways to end a colour, a pivot that is not positive and a diagonal below the breakdown limit, at
+# the block widths whose factor kernel has the most warps: Krylov spaces that are exhausted before depth m; the
+# status and P of the oracle, and the same bits in repeated calls
+@pytest.mark.parametrize("n,b,nc,m", [(3, 32, 3, 6), (4, 32, 2, 9), (5, 24, 5, 7), (4, 16, 1, 8)])
+def test_breakdown_of_wide_blocks(torch, css, ctx, n, b, nc, m):
+    from tests.test_gpu_parity import FP64_TOL, gpu_density
+    H = _dense_bsr(n, b, np.ones(n * b), 10 * n + b)
+    col = (np.arange(n) % nc).astype(np.int32)
+    s = oracle.probes(col, b, 1005)
+    kw = dict(kT=0.5, n_elec=float(n * b), m=m, mu=0.1, solve_mu=False)
+    ref = oracle.density(H, col, s, nc, **kw)
+    runs = [gpu_density(torch, css, ctx, H, col, s, nc, precision=css.CSS_FP64, **kw) for _ in range(8)]
+    assert float(np.abs(runs[0]["P"] - ref["P"]).max()) < FP64_TOL
+    assert (runs[0]["status"] == css.CSS_WARN_BREAKDOWN) == (ref["n_breakdown"] > 0)
+    for r in runs[1:]:
+        assert r["status"] == runs[0]["status"] and np.array_equal(r["P"], runs[0]["P"])
