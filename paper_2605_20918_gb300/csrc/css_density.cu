@@ -648,6 +648,24 @@ css_status ws_get(css_ctx* ctx, const char* name, size_t count, Tp** p) {
   return css_ws(ctx, name, count * sizeof(Tp), (void**)p);
 }
 
+// bytes that the context holds in buffers whose names start with one of `names`
+size_t ws_held(const css_ctx* ctx, std::initializer_list<const char*> names) {
+  size_t held = 0;
+  for (const auto& kv : ctx->bufs)
+    for (const char* pre : names)
+      if (kv.first.rfind(pre, 0) == 0) {
+        held += kv.second.bytes;
+        break;
+      }
+  return held;
+}
+
+// device memory of the eigen stage, apart from its small arrays
+size_t eigen_bytes(int64_t n_col, int32_t b, int32_t m) {
+  const size_t nmax = (size_t)m * b, rcap = nmax * (m + 2);
+  return (size_t)n_col * (8 * (6 * nmax * nmax + rcap * (b + 1) + nmax * (css_band_ld(b) + 4 * b + 4)) + 40 * nmax);
+}
+
 css_status rows_timeout(css_ctx* ctx) {
   ctx->last_error = "block-Lanczos: a bounded wait on the row passes' ring of tiles timed out";
   return CSS_ERR_TIMEOUT;
@@ -863,29 +881,6 @@ css_status css_density_impl(css_ctx* ctx, int32_t n_sys, const css_sys_desc* sys
   // FP32 with b = 6 or 23: the exact-width H * V unless a padded variant is asked for
   const bool use_dup = !use_tc && ctx->spmm_variant < 0 && css_spmm_dup_supported(f32, b);
   const void* Hsplit = nullptr;
-  // FP64 (and CSS_FP64_SPLIT) with b <= 24: exact digit products on the tensor cores, unless a padded variant
-  // is asked for or the digits would not fit their bounds.  Against the FP32-pair kernel they are faster (256
-  // molecules, b = 23: 2.93 -> 2.12 ms a launch) and closer to the exact products, so that one is left what
-  // exceeds the bounds.
-  int32_t rows_max = 0;
-  for (int32_t s = 0; s < n_sys; ++s) rows_max = std::max(rows_max, sys[s].H.n_brow);
-  const bool use_int = (prec == CSS_FP64 || prec == CSS_FP64_SPLIT) && ctx->spmm_variant < 0 &&
-                       css_hv_int_supported(b, rows_max, nnzb);
-  const bool use_split = prec == CSS_FP64_SPLIT && !use_int;
-  const void* Hdig = nullptr;
-  const int32_t* Hexp = nullptr;
-  if (use_tc)
-    CSS_TRY(css_hv_tc_prepare(ctx, b, n_brow, nnzb, row_ptr, col_idx, Hval, &Htc, &Hd3, st));
-  else if (use_split)
-    CSS_TRY(css_spmm_split_prepare(ctx, b, nnzb, Hval, &Hsplit, st));
-  else if (use_int)
-    CSS_TRY(css_hv_int_prepare(ctx, b, n_brow, nnzb, row_ptr, col_idx, Hval, &Hdig, &Hexp, st));
-  else if (use_dup)
-    CSS_TRY(css_spmm_dup_prepare(ctx, b, n_brow, nnzb, row_ptr, col_idx, Hval, &Hdup, &Hlodup, st));
-  else
-    CSS_TRY(css_spmm_prepare(ctx, f32, b, n_brow, nnzb, row_ptr, col_idx, Hval, &Hv, &Hlo, st));
-  tm.mark();  // 1
-
   // ----------------------------------------------------------- memory plan
   const size_t s_vec = f32 ? 4 : 8;
   double *Ablk, *Bblk, *Bprev, *X;
@@ -934,14 +929,52 @@ css_status css_density_impl(css_ctx* ctx, int32_t n_sys, const css_sys_desc* sys
   }
   size_t free_b = 0, total_b = 0;
   CSS_CU(ctx, cudaMemGetInfo(&free_b, &total_b));
-  int32_t ncb = ncmax;
-  auto vec_need = [&](int32_t k) -> size_t {
+  const size_t reserve = (size_t)2 << 30;
+  const int32_t rows_max = (int32_t)(Nmax / b);
+  auto vec_bytes = [&](int32_t k, bool digits) -> size_t {
     const int32_t ws = (int32_t)css_ceil_div((int64_t)k * b, 8) * 8;
     return 3 * (size_t)Nmax * ws * s_vec + css_lanczos_part_doubles(Nmax, b, k) * 8 * 2 +
-           css_lanczos_small_doubles(b, k) * 8 + (use_int ? css_hv_int_v_bytes(rows_max, b, k * b) : 0);
+           css_lanczos_small_doubles(b, k) * 8 + (digits ? css_hv_int_v_bytes(rows_max, b, k * b) : 0);
   };
-  const size_t reserve = (size_t)2 << 30;
-  while (ncb > 1 && vec_need(ncb) + reserve > free_b) ncb = (ncb + 1) / 2;
+  // colours per pass that fit in `avail` bytes beside the reserve (at least one)
+  auto colours_in = [&](size_t avail, bool digits) {
+    int32_t k = ncmax;
+    while (k > 1 && vec_bytes(k, digits) + reserve > avail) k = (k + 1) / 2;
+    return k;
+  };
+  // FP64 (and CSS_FP64_SPLIT) with b <= 24: exact digit products on the tensor cores, unless a padded variant
+  // is asked for or the digits would not fit their bounds.  Against the FP32-pair kernel they are faster (256
+  // molecules, b = 23: 2.93 -> 2.12 ms a launch) and closer to the exact products, so that one is left what
+  // exceeds the bounds.  The digits (up to 256 times H's blocks at b = 1) are taken where they leave room for the
+  // vectors of at least half as many colours as there would be without them: half as many columns a pass
+  // cost them next to nothing (whole tiles of 128), much fewer read H's digits for each few.  Buffers that
+  // an earlier call left count as free, so that a repeated call decides alike.
+  bool use_int = (prec == CSS_FP64 || prec == CSS_FP64_SPLIT) && ctx->spmm_variant < 0 &&
+                 css_hv_int_supported(b, rows_max, nnzb);
+  const size_t vec_held = ws_held(ctx, {"Q0", "Q1", "W", "lz_part", "lz_small", "v_digits"});
+  if (use_int) {
+    const size_t hd = css_hv_int_h_bytes(b, n_brow, nnzb), avail = free_b + vec_held + ws_held(ctx, {"h_digits", "h_exp"});
+    use_int = hd + vec_bytes(1, true) + reserve <= avail &&
+              2 * colours_in(avail - hd, true) >= colours_in(avail, false);
+  }
+  const bool use_split = prec == CSS_FP64_SPLIT && !use_int;
+  const void* Hdig = nullptr;
+  const int32_t* Hexp = nullptr;
+  const int64_t ws_before = ctx->ws_bytes;
+  if (use_tc)
+    CSS_TRY(css_hv_tc_prepare(ctx, b, n_brow, nnzb, row_ptr, col_idx, Hval, &Htc, &Hd3, st));
+  else if (use_split)
+    CSS_TRY(css_spmm_split_prepare(ctx, b, nnzb, Hval, &Hsplit, st));
+  else if (use_int)
+    CSS_TRY(css_hv_int_prepare(ctx, b, n_brow, nnzb, row_ptr, col_idx, Hval, &Hdig, &Hexp, st));
+  else if (use_dup)
+    CSS_TRY(css_spmm_dup_prepare(ctx, b, n_brow, nnzb, row_ptr, col_idx, Hval, &Hdup, &Hlodup, st));
+  else
+    CSS_TRY(css_spmm_prepare(ctx, f32, b, n_brow, nnzb, row_ptr, col_idx, Hval, &Hv, &Hlo, st));
+  tm.mark();  // 1
+  const size_t grown = (size_t)std::max<int64_t>(ctx->ws_bytes - ws_before, 0);  // by H in the kernel's form
+  const int32_t ncb = colours_in(free_b + vec_held - std::min(grown, free_b), use_int);
+  auto vec_need = [&](int32_t k) { return vec_bytes(k, use_int); };
   const int32_t ws = (int32_t)css_ceil_div((int64_t)ncb * b, 8) * 8;
   void *Q0, *Q1, *Wv;
   double *part, *small;
@@ -1020,12 +1053,9 @@ css_status css_density_impl(css_ctx* ctx, int32_t n_sys, const css_sys_desc* sys
   if (nside > 0) {
     // each side stream needs one more Krylov set; take only as many as fit beside the
     // reserve (sets already held from an earlier call count as free)
-    size_t free2 = 0, total2 = 0, held = 0;
+    size_t free2 = 0, total2 = 0;
+    const size_t held = ws_held(ctx, {"sQ0_", "sQ1_", "sW_", "spart_", "ssmall_", "svdig_"});
     CSS_CU(ctx, cudaMemGetInfo(&free2, &total2));
-    static const char* const kSideNames[] = {"sQ0_", "sQ1_", "sW_", "spart_", "ssmall_", "svdig_"};
-    for (auto& kv : ctx->bufs)
-      for (const char* pre : kSideNames)
-        if (kv.first.rfind(pre, 0) == 0) held += kv.second.bytes;
     const size_t avail = free2 + held > reserve ? free2 + held - reserve : 0;
     nside = (int)std::min<size_t>((size_t)nside, avail / vec_need(ncb));
     if (nside < 2) nside = 0;
@@ -1978,10 +2008,13 @@ css_status css_density_nonorth(css_ctx* ctx, const css_bsr* S, const double* Sin
     ctx->last_error = "css_density_nonorth: the Krylov blocks of all colours do not fit in device memory";
     return CSS_ERR_NOMEM;
   }
-  // the recurrence's H'*V as in css_density_impl, where the digits fit beside the Krylov blocks
+  // the recurrence's H'*V as in css_density_impl, where the digits fit beside the Krylov blocks and the eigen stage
   const size_t vd_bytes = css_hv_int_v_bytes(n_brow, b, nc * b);
   const bool use_int = prec == CSS_FP64 && ctx->spmm_variant < 0 && css_hv_int_supported(b, n_brow, Hp->nnzb) &&
-                       7 * vbytes + vd_bytes + ((size_t)9 << 30) <= free_b + ctx->ws_bytes;
+                       7 * vbytes + vd_bytes + css_hv_int_h_bytes(b, n_brow, Hp->nnzb) + eigen_bytes(nc, b, m) +
+                               ((size_t)1 << 30) <=
+                           free_b + ws_held(ctx, {"no_R", "no_start", "no_SR", "no_u", "no_Q", "no_W", "e_", "h_digits",
+                                                  "h_exp", "v_digits"});
   const bool use_dup = ctx->spmm_variant < 0 && css_spmm_dup_supported(f32, b);
   const void *Hdig = nullptr, *hdup = nullptr, *hlodup = nullptr;
   const int32_t* Hexp = nullptr;

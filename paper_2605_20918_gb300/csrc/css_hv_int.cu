@@ -377,6 +377,10 @@ bool css_hv_int_supported(int32_t b, int32_t n_brow, int32_t nnzb) {
   return b <= 24 && (size_t)nnzb * h_block_bytes(b) <= kHBytes && (size_t)n_brow * v_block_bytes(b) <= kVBytes;
 }
 
+size_t css_hv_int_h_bytes(int32_t b, int32_t n_brow, int32_t nnzb) {
+  return (size_t)nnzb * h_block_bytes(b) + sizeof(int32_t) * 2 * (size_t)n_brow * b;
+}
+
 size_t css_hv_int_v_bytes(int32_t n_brow, int32_t b, int32_t w) {
   const size_t exps = ((size_t)w * sizeof(int32_t) + 255) / 256 * 256;
   return exps + std::min(kVBytes, (size_t)css_ceil_div(w, kTile) * n_brow * v_block_bytes(b));

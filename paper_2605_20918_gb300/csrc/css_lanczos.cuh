@@ -101,6 +101,7 @@ css_status css_spmm_split_prepare(css_ctx* ctx, int32_t b, int32_t nnzb, const d
 css_status css_spmm_split(css_ctx* ctx, const LzArgs& a, const double* V, double* W, int variant, cudaStream_t st);
 // FP64 H * V by exact digit products on the tensor cores (css_hv_int.cu); n_brow: the largest pass's rows
 bool css_hv_int_supported(int32_t b, int32_t n_brow, int32_t nnzb);
+size_t css_hv_int_h_bytes(int32_t b, int32_t n_brow, int32_t nnzb);
 size_t css_hv_int_v_bytes(int32_t n_brow, int32_t b, int32_t w);
 css_status css_hv_int_prepare(css_ctx* ctx, int32_t b, int32_t n_brow, int32_t nnzb, const int32_t* row_ptr,
                               const int32_t* col_idx, const double* H, const void** Hdig, const int32_t** Hexp,
