@@ -110,7 +110,10 @@ css_status css_create(css_ctx** out, int device) {
 void css_destroy(css_ctx* ctx) {
   if (!ctx) return;
   cudaSetDevice(ctx->device);
-  cudaDeviceSynchronize();
+  // No device-wide synchronisation: it ends the graph capture of any other thread's context (whose call then fails),
+  // and the driver was seen to crash in it.  Every call that used the workspace has waited for its stream; what a
+  // call that ended with an error left behind, cudaFree waits for.
+  for (cudaStream_t s : ctx->side) cudaStreamSynchronize(s);
   for (auto& kv : ctx->bufs)
     if (kv.second.p) cudaFree(kv.second.p);
   for (cudaStream_t s : ctx->side) cudaStreamDestroy(s);

@@ -1588,7 +1588,7 @@ css_status css_ritz(css_ctx* ctx, double* lam, double* wgt, int32_t* n_per, int6
   *n_colours = nc;
   if (!n_per) return CSS_OK;
   std::vector<int32_t> nb(nc);
-  CSS_CU(ctx, cudaDeviceSynchronize());
+  // the call that left these results has waited for its stream
   CSS_CU(ctx, cudaMemcpy(nb.data(), ctx->last_nblk, sizeof(int32_t) * nc, cudaMemcpyDeviceToHost));
   int64_t total = 0;
   for (int32_t c = 0; c < nc; ++c) {
@@ -1616,7 +1616,7 @@ css_status css_projected(css_ctx* ctx, double* A, double* B, int32_t* nblk, int6
   const int64_t need = (int64_t)ctx->last_ncol * ctx->last_m * ctx->last_b * ctx->last_b;
   if (!A || !B || !nblk || capacity < need) return css_set_arg_error(ctx, "css_projected: capacity too small");
   CSS_CU(ctx, cudaSetDevice(ctx->device));
-  CSS_CU(ctx, cudaDeviceSynchronize());
+  // the call that left these results has waited for its stream
   CSS_CU(ctx, cudaMemcpy(A, ctx->last_A, sizeof(double) * need, cudaMemcpyDeviceToHost));
   CSS_CU(ctx, cudaMemcpy(B, ctx->last_B, sizeof(double) * need, cudaMemcpyDeviceToHost));
   CSS_CU(ctx, cudaMemcpy(nblk, ctx->last_nblk, sizeof(int32_t) * ctx->last_ncol, cudaMemcpyDeviceToHost));
