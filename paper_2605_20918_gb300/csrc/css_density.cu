@@ -1739,44 +1739,47 @@ css_status css_solve_mu(css_ctx* ctx, int32_t n_lists, const int32_t* n_per, con
     return css_set_arg_error(ctx, "css_solve_mu: kT must be finite and >= 0, n_elec finite");
   CSS_CU(ctx, cudaSetDevice(ctx->device));
   cudaStream_t st = (cudaStream_t)stream;
-  int64_t total = 0;
+  // the lists as the colours of one system (stride nmax, block width 1), solved by the kernel and the rule of
+  // css_density; lists longer than a colour's largest (4096 Ritz values) in pieces, or the few CTAs of few long lists
+  // bound the search (3 lists of 100,000 values 101.9 -> 4.9 ms; by bisection 96.4)
+  constexpr int32_t kPiece = 4096;
+  std::vector<int32_t> len;
   int32_t nmax = 1;
   for (int32_t t = 0; t < n_lists; ++t) {
     if (n_per[t] < 0) return css_set_arg_error(ctx, "css_solve_mu: negative list length");
-    total += n_per[t];
-    nmax = std::max(nmax, n_per[t]);
+    for (int64_t k = 0; k == 0 || k < n_per[t]; k += kPiece) len.push_back((int32_t)std::min<int64_t>(kPiece, n_per[t] - k));
+    nmax = std::max(nmax, std::min(kPiece, n_per[t]));
   }
-  // the lists as the colours of one system (stride nmax, block width 1), solved by the kernel
-  // and the rule of css_density
+  const int32_t n_pc = (int32_t)len.size();
   double *dl, *dw, *dpar, *dmu;
   int32_t *dn, *dsoc, *dsolve, *derr;
   unsigned* bar;
-  const size_t nn = (size_t)n_lists * nmax;
+  const size_t nn = (size_t)n_pc * nmax;
   CSS_TRY(css_ws(ctx, "smu_lam", sizeof(double) * nn, (void**)&dl));
   CSS_TRY(css_ws(ctx, "smu_wgt", sizeof(double) * nn, (void**)&dw));
-  CSS_TRY(css_ws(ctx, "smu_i", sizeof(int32_t) * (2 * (size_t)n_lists + 64), (void**)&dn));
-  dsoc = dn + n_lists;
-  dsolve = dsoc + n_lists;
+  CSS_TRY(css_ws(ctx, "smu_i", sizeof(int32_t) * (2 * (size_t)n_pc + 64), (void**)&dn));
+  dsoc = dn + n_pc;
+  dsolve = dsoc + n_pc;
   derr = dsolve + 8;
   bar = reinterpret_cast<unsigned*>(derr + 8);
   CSS_TRY(css_ws(ctx, "smu_d", sizeof(double) * 16, (void**)&dpar));
   dmu = dpar + 8;
   double* hp;
-  const size_t hbytes = sizeof(double) * 2 * nn + sizeof(int32_t) * 2 * (size_t)n_lists + 256;
+  const size_t hbytes = sizeof(double) * 2 * nn + sizeof(int32_t) * 2 * (size_t)n_pc + 256;
   CSS_TRY(css_pinned(ctx, hbytes, (void**)&hp));
   double* hl = hp;
   double* hw = hl + nn;
   int32_t* hi = reinterpret_cast<int32_t*>(hw + nn);
-  double* hd = reinterpret_cast<double*>(hi + 2 * (size_t)n_lists + 2);
+  double* hd = reinterpret_cast<double*>(hi + 2 * (size_t)n_pc + 2);
   size_t o = 0;
-  for (int32_t t = 0; t < n_lists; ++t) {
+  for (int32_t t = 0; t < n_pc; ++t) {
     for (int32_t k = 0; k < nmax; ++k) {
-      hl[(size_t)t * nmax + k] = k < n_per[t] ? lam[o + k] : 0.0;
-      hw[(size_t)t * nmax + k] = k < n_per[t] ? wgt[o + k] : 0.0;
+      hl[(size_t)t * nmax + k] = k < len[t] ? lam[o + k] : 0.0;
+      hw[(size_t)t * nmax + k] = k < len[t] ? wgt[o + k] : 0.0;
     }
-    o += n_per[t];
-    hi[t] = n_per[t];
-    hi[n_lists + t] = 0;
+    o += len[t];
+    hi[t] = len[t];
+    hi[n_pc + t] = 0;
   }
   hd[0] = kT;
   hd[1] = 0.5 * n_elec;
@@ -1784,19 +1787,19 @@ css_status css_solve_mu(css_ctx* ctx, int32_t n_lists, const int32_t* n_per, con
   hd[3] = 0.0;
   CSS_CU(ctx, cudaMemcpyAsync(dl, hl, sizeof(double) * nn, cudaMemcpyHostToDevice, st));
   CSS_CU(ctx, cudaMemcpyAsync(dw, hw, sizeof(double) * nn, cudaMemcpyHostToDevice, st));
-  CSS_CU(ctx, cudaMemcpyAsync(dn, hi, sizeof(int32_t) * 2 * (size_t)n_lists, cudaMemcpyHostToDevice, st));
+  CSS_CU(ctx, cudaMemcpyAsync(dn, hi, sizeof(int32_t) * 2 * (size_t)n_pc, cudaMemcpyHostToDevice, st));
   CSS_CU(ctx, cudaMemcpyAsync(dpar, hd, sizeof(double) * 4, cudaMemcpyHostToDevice, st));
   const int32_t one = 1;
   CSS_CU(ctx, cudaMemcpyAsync(dsolve, &one, sizeof(int32_t), cudaMemcpyHostToDevice, st));
   CSS_CU(ctx, cudaMemsetAsync(derr, 0, sizeof(int32_t) * 8 + 8 * sizeof(unsigned), st));
   int occ = 0;
   CSS_CU(ctx, mu_occupancy(1, &occ));
-  unsigned G = (unsigned)std::max(1, std::min(ctx->n_sm * std::max(occ, 1), n_lists));
+  unsigned G = (unsigned)std::max(1, std::min(ctx->n_sm * std::max(occ, 1), n_pc));
   if (G > (unsigned)ctx->n_sm) G = (unsigned)ctx->n_sm;
   double* mupart;
   CSS_TRY(css_ws(ctx, "smu_part", sizeof(double) * (2 * MU_C * (size_t)G + 16), (void**)&mupart));
   {
-    int32_t n_sys_ = 1, n_col_ = n_lists, nmax_ = nmax, b_ = 1, extra_ = 0;
+    int32_t n_sys_ = 1, n_col_ = n_pc, nmax_ = nmax, b_ = 1, extra_ = 0;
     const int32_t* nblk_ = dn;
     const int32_t* soc_ = dsoc;
     const double* lam_ = dl;
