@@ -896,7 +896,8 @@ inline int gram_threads(int32_t b) { return std::max(256, (b * b + 31) / 32 * 32
 constexpr int GLD = CSS_MAX_B + 1;
 __device__ __forceinline__ void sum_partials(const double* __restrict__ part, int32_t nch, int64_t n, int32_t b,
                                              double (*G)[GLD], double* scratch) {
-  const int32_t E = b * b, T = blockDim.x, S = max(1, T / E), t = threadIdx.x;
+  // no more sharers than partials: the sharers' sums are added one after the other (at b = 1 there would be 256)
+  const int32_t E = b * b, T = blockDim.x, S = max(1, min(T / E, nch)), t = threadIdx.x;
   if (t < S * E) {
     const int32_t y = t / E;
     const double* p = part + (t - y * E);

@@ -180,3 +180,28 @@ def test_breakdown_of_wide_blocks(torch, css, ctx, n, b, nc, m):
     assert (runs[0]["status"] == css.CSS_WARN_BREAKDOWN) == (ref["n_breakdown"] > 0)
     for r in runs[1:]:
         assert r["status"] == runs[0]["status"] and np.array_equal(r["P"], runs[0]["P"])
+
+
+# Sums of the Gram partials at narrow blocks, where many threads could share an entry: as many partials as threads and
+# fewer (1 to 40 chunks of rows).  P of the oracle, and a step at b = 1 takes no longer than one at b = 4 (1.21 times
+# as long when idle threads' zeros were added too; the least of many calls)
+@pytest.mark.parametrize("n", [3, 70, 300])
+def test_gram_sums_of_narrow_blocks(torch, css, monkeypatch, n):
+    from tests.test_gpu_parity import FP64_TOL, gpu_density
+    monkeypatch.setenv("CSS_TIMING", "1")
+    step = {}
+    with css.Context(0) as c:
+        for b in (1, 2, 4):
+            H = _dense_bsr(n, b, np.ones(n * b), 10 * n + b)
+            col = (np.arange(n) % 3).astype(np.int32)
+            s = oracle.probes(col, b, 1005)
+            kw = dict(kT=0.5, n_elec=float(n * b), m=1 if n == 3 else 6, mu=0.1, solve_mu=False)
+            ref = oracle.density(H, col, s, 3, **kw)
+            times = []
+            for _ in range(30 if n == 70 else 1):
+                got = gpu_density(torch, css, c, H, col, s, 3, precision=css.CSS_FP64, **kw)
+                times.append(c.info()["ms_rows"])
+            assert float(np.abs(got["P"] - ref["P"]).max()) < FP64_TOL
+            step[b] = min(times)
+    if n == 70:
+        assert step[1] < 1.15 * step[4], step
