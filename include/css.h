@@ -50,10 +50,11 @@ typedef enum {
 
 typedef enum {
   CSS_FP64 = 0,        /* everything in FP64.  The recurrence's H*V with b <= 24 (digits of H up to */
-                       /* 10 GiB) rounds the entries of H to 2^-63 of a power of two above their row's */
-                       /* and column's largest, those of V to 2^-63 of their column's, multiplies and  */
-                       /* adds exactly and rounds the result once: closer to the exact product in norm */
-                       /* than an FP64 sum; an entry below 2^-10 of its largest keeps under 53 bits    */
+                       /* 10 GiB, and device memory for them) rounds the entries of H to 2^-63 of a    */
+                       /* power of two above their row's and column's largest, those of V to 2^-63 of  */
+                       /* their column's, multiplies and adds exactly and rounds the result once:      */
+                       /* closer to the exact product in norm than an FP64 sum; an entry below 2^-10   */
+                       /* of its largest keeps under 53 bits                                           */
   CSS_MIXED_FP32 = 1,  /* H*V, Krylov vectors and block products in FP32 (FP32 accumulate); */
                        /* recurrence coefficients, Cholesky, eigensolve, mu, Z and P in FP64; */
                        /* implies CSS_REORTH_LOCAL (it removes an FP32-level bias of Tr P)   */
@@ -65,8 +66,8 @@ typedef enum {
   CSS_FP64_SPLIT = 3    /* as CSS_FP64, with leave to take the H*V of the block-Lanczos recurrence */
                         /* in FP32 pairs on the FMA pipe (hi + lo, error-free products, TwoSum   */
                         /* sums: about 2^-47 relative per term against 2^-53); b = 6 or 23       */
-                        /* (other b: CSS_ERR_UNSUPPORTED).  Systems whose 8-bit digits of H fit  */
-                        /* 10 GiB run the exact digit products of CSS_FP64, which are faster      */
+                        /* (other b: CSS_ERR_UNSUPPORTED).  Systems that CSS_FP64 runs with     */
+                        /* digit products run them here too: they are faster                     */
 } css_precision;
 
 /* css_density flags */
